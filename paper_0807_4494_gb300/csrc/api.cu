@@ -289,13 +289,14 @@ int run_delta(ssht_plan_t p, cudaStream_t st) {
   return 0;
 }
 
-// 3xTF32 plans that run their own column recursion make the contraction's A tiles in the
-// recursion itself (no FP64 table, no packing): the forward's tiles (rows l, K = m') with one lane
-// per column, the inverse's (rows m', K = l) with one lane per degree.  U, the spin column, and the
-// degree-lane recursion's tables are made once at plan creation.
-bool tiles_direct(const ssht_plan_s* p) {
-  return p->tc && tc_a_tiles(p->tc).A && !p->delta_shared && p->delta.method == kDeltaColumn;
-}
+// Tensor-core plans with the column recursion make the contraction's A tiles in the recursion
+// itself (no FP64 table, no packing): the forward's tiles (rows l, K = m') with one lane per column,
+// the inverse's (rows m', K = l) with one lane per degree.  U, the spin column, and the degree-lane
+// recursion's tables are made once at plan creation.  The plans of a group too, each for its own
+// spin: a sweep into the tiles writes them once, while packing them from a shared FP64 table also
+// reads that table (8 bytes an entry, the inverse's in columns).  Split-BF16, inverse + forward: B = 64,
+// L = 1024 16.0 -> 12.5 ms, B = 16, L = 2048 62.1 -> 40.6 ms (GB300).
+bool tiles_direct(const ssht_plan_s* p) { return p->tc && p->delta.method == kDeltaColumn; }
 
 // Delta and the contraction's A operand of one direction, on st.
 int make_operands(ssht_plan_t p, int forward, cudaStream_t st) {
@@ -389,7 +390,7 @@ int begin_operands(ssht_plan_t p, int forward, cudaStream_t st) {
     SSHT_CUDA(cudaEventRecord(p->ev_fork, st), "fork event");
     SSHT_CUDA(cudaStreamWaitEvent(p->aux, p->ev_fork, 0), "fork wait");
   }
-  if (p->delta_shared && p->delta_event) SSHT_CUDA(cudaStreamWaitEvent(p->aux, p->delta_event, 0), "shared Delta wait");
+  if (p->delta_shared && p->delta_event && !tiles_direct(p)) SSHT_CUDA(cudaStreamWaitEvent(p->aux, p->delta_event, 0), "shared Delta wait");
   int rc = make_operands(p, forward, p->aux);
   if (rc) return rc;
   SSHT_CUDA(cudaEventRecord(p->ev_join, p->aux), "join event");
@@ -978,7 +979,8 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     // the calls' recursions run on the plan's non-blocking stream: U must be complete first
     ce = cudaDeviceSynchronize();
     if (ce == cudaSuccess)
-      ce = lane_tables_setup(p->lane, p->delta, L, s, p->Uf, tc_inverse_tiles(p->tc).nC, tc_a_tiles(p->tc).abase);
+      ce = lane_tables_setup(p->lane, p->delta, L, s, p->Uf, tc_inverse_tiles(p->tc).nC, tc_a_tiles(p->tc).abase,
+                             p->precision == SSHT_BF16X6);
     if (ce != cudaSuccess) {
       release(p);
       return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,
@@ -1274,10 +1276,12 @@ int ssht_version(void) { return 100; }
 // Groups: many fields of uneven band-limit and spin in one call (and one CUDA graph).
 //
 // Fields are bucketed by (L, s); each bucket is one plan over its fields, which sit contiguously
-// in the caller's flat buffers in group order (ssht_group_layout).  All buckets of one L share one
-// Delta table: in recompute mode each call runs one recursion per distinct L, on its own stream,
-// and the buckets wait for it before their spin column and packing; in cache mode the tables are
-// made once here.  Buckets run on their own streams, forked from and joined to the caller's.
+// in the caller's flat buffers in group order (ssht_group_layout).  CUDA-core buckets
+// of one L share one Delta table: in recompute mode each call runs one recursion per such L, on its
+// own stream, and the buckets wait for it before their spin column; in cache mode the tables are
+// made once here.  Tensor-core buckets write their own tiles (tiles_direct): with 256 fields of L in
+// {128, .., 1024} and 20 buckets, packing every bucket's tiles from shared tables made a step
+// (inverse and forward) 39.1 ms, the sweeps into the tiles 29.4.  Buckets run on their own streams, forked from and joined to the caller's.
 // With tuning on, each bucket times every contraction form of the group's precision class
 // (FP32, 3xTF32, split-BF16 for FP32-class groups; the tensor-core forms with their own tuned
 // shape) on its own shape and keeps the fastest.
@@ -1294,6 +1298,7 @@ struct ssht_group_s {
     int L = 0;
     DeltaWork dw{};
     cudaEvent_t ev = nullptr;
+    bool table_used = false;  // some bucket of this L contracts from the table (CUDA-core plans)
   };
   // The shared recursions run one after another on one stream: each is a cooperative grid over
   // every SM, so running two at once would only make them wait for each other's SMs.
@@ -1334,8 +1339,13 @@ void group_release(ssht_group_t g) {
 int group_call(ssht_group_t g, int which, const void* in, void* out, cudaStream_t st) {
   SSHT_CUDA(cudaEventRecord(g->ev_start, st), "group fork");
   if (g->delta_mode == SSHT_DELTA_RECOMPUTE) {
-    SSHT_CUDA(cudaStreamWaitEvent(g->rec_st, g->ev_start, 0), "group fork wait");
+    // recursions into a shared table only for the band-limits whose buckets read it (a forked
+    // stream that nothing joins would spoil a capture)
+    bool forked = false;
     for (auto& h : g->holders) {
+      if (!h.table_used) continue;
+      if (!forked) SSHT_CUDA(cudaStreamWaitEvent(g->rec_st, g->ev_start, 0), "group fork wait");
+      forked = true;
       SSHT_CUDA(delta_run(h.dw, h.L, g->rec_st), "shared Delta recursion");
       SSHT_CUDA(cudaEventRecord(h.ev, g->rec_st), "shared Delta event");
     }
@@ -1343,7 +1353,7 @@ int group_call(ssht_group_t g, int which, const void* in, void* out, cudaStream_
   for (auto& b : g->buckets) {
     ssht_plan_t p = b.plan;
     SSHT_CUDA(cudaStreamWaitEvent(b.st, g->ev_start, 0), "group fork wait");
-    p->delta_event = g->delta_mode == SSHT_DELTA_RECOMPUTE ? g->holders[b.holder].ev : nullptr;
+    p->delta_event = g->delta_mode == SSHT_DELTA_RECOMPUTE && g->holders[b.holder].table_used ? g->holders[b.holder].ev : nullptr;
     int rc = set_streams(p, b.st);
     if (rc) return rc;
     const long long ci = g->coff[b.first], gi = g->goff[b.first];
@@ -1502,6 +1512,7 @@ int group_create(ssht_group_t* out, int n, const int* Ls, const int* ss, int pre
         release(p);
       }
     }
+    if (!tiles_direct(b.plan)) g->holders[b.holder].table_used = true;
     k = e;
   }
   *out = g;

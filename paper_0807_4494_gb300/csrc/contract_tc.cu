@@ -664,22 +664,24 @@ size_t tc_bytes(const TcPlan* p) { return p ? p->bytes : 0; }
 
 InvTiles tc_inverse_tiles(const TcPlan* p) {
   InvTiles t;
-  if (p && !p->bf16) {
+  if (p) {
     t.A = p->A_inv;
     t.ibase = p->ibase;
     t.nI = p->nI;
     t.nC = p->nC;
     t.ntiles = p->tiles_inv;
+    t.bf16 = p->bf16;
   }
   return t;
 }
 
 ATiles tc_a_tiles(const TcPlan* p) {
   ATiles t;
-  if (p && !p->bf16) {
+  if (p) {
     t.A = p->A;
     t.abase = p->abase;
     t.ntiles = p->tiles_A;
+    t.bf16 = p->bf16;
   }
   return t;
 }

@@ -69,17 +69,27 @@ struct ColumnParams {
   long long extent;        // entries of the table, or tiles of A (index checks)
 };
 
-// Writes A_M[l][K] = x (FP32) into row l mod 128 of tile (M, l / 128, K / 32): the 3xTF32 tiles
-// hold one FP32 part in global memory (the contraction splits it into hi + lo on arrival).
-__device__ __forceinline__ void put_a(uint8_t* A, long long tile, long long ntiles, int site, int row, int k, float x) {
-  if (!in_bounds(tile, ntiles, site)) return;
-  uint8_t* t = A + (size_t)tile * tc::kAPart;
-  *(float*)(t + tc::sw128(row, 4 * k)) = x;
+// Byte offset of (row, K) in an A tile: of the FP32 value (3xTF32 tiles, one part), or of the first
+// BF16 part (split-BF16 tiles; the second part lies at offset ^ 64, the third one part further on).
+template <bool BF>
+__device__ __forceinline__ uint32_t a_off(int row, int k) {
+  return tc::sw128(row, (BF ? 2 : 4) * k);
 }
-// The same with the swizzled offset of (row, K) in the tile already made.
+// Writes x into tile `tile` at the offset made by a_off: the FP32 value (the contraction splits it
+// into hi + lo on arrival), or its three BF16 parts.
+template <bool BF>
 __device__ __forceinline__ void put_a_at(uint8_t* A, long long tile, long long ntiles, int site, uint32_t off, float x) {
   if (!in_bounds(tile, ntiles, site)) return;
-  *(float*)(A + (size_t)tile * tc::kAPart + off) = x;
+  uint8_t* t = A + (size_t)tile * (tc::kParts<BF> * tc::kAPart);
+  if constexpr (BF) {
+    uint16_t h, m, l;
+    tc::split_bf16x3(x, &h, &m, &l);
+    *(uint16_t*)(t + off) = h;
+    *(uint16_t*)(t + (off ^ 64u)) = m;
+    *(uint16_t*)(t + tc::kAPart + off) = l;
+  } else {
+    *(float*)(t + off) = x;
+  }
 }
 
 __device__ __forceinline__ double flip_sign(double v, bool neg) {
@@ -255,7 +265,7 @@ constexpr int kTileStageFloats = 32 * 33;
 constexpr int kTileWarpBytes = kTileStageFloats * 4 + 32 * 8 + 32 * 4;  // stage, alpha[32], p[32]
 constexpr size_t kTileSmem = (size_t)kColWarps * kTileWarpBytes;
 
-template <bool SCALED>
+template <bool SCALED, bool BF>
 __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnParams P) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -291,7 +301,7 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
     const int il = l >> 7;
     const long long ilpre = 2ll * il * (il + 1);
     const long long tadd = ilpre + (m0 >> 5);
-    const uint32_t off = tc::sw128(l & 127, 4 * lane);
+    const uint32_t off = a_off<BF>(l & 127, lane);
     const size_t lrow = (size_t)l * (l + 1) / 2;  // row l of the degree-major tables
     const double md = (double)m;
     // U_l[m] of this lane's column and the tile base of its row M = m (the transposed writes)
@@ -324,7 +334,7 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
         __syncwarp();
       }
       const float x = f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur);  // y_{m'} in FP32
-      if (act) put_a_at(P.A, ab_cur + tadd, P.extent, kbColumnTile, off, (u_lane * pw[j]) * (((mp - m) & 1) ? -x : x));
+      if (act) put_a_at<BF>(P.A, ab_cur + tadd, P.extent, kbColumnTile, off, (u_lane * pw[j]) * (((mp - m) & 1) ? -x : x));
       if (mp >= m0 + 32) {
         stage[lane * 33 + j] = x;
         if (j == 0) {
@@ -335,7 +345,7 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
           const int cb = mp >> 5;
           for (int r = 0; r < 32 && m0 + r <= l; ++r) {
             const long long tile = __shfl_sync(0xffffffffu, base_lane, r) + cb;
-            if (c <= l) put_a_at(P.A, tile, P.extent, kbColumnTile, off, uc * stage[r * 33 + lane]);
+            if (c <= l) put_a_at<BF>(P.A, tile, P.extent, kbColumnTile, off, uc * stage[r * 33 + lane]);
           }
           __syncwarp();
         }
@@ -409,7 +419,7 @@ struct LaneParams {
 // Rows top .. max(m, 32 kc) are the start-up phase: lane l joins at m' = l from its first-row
 // entry.  Below 32 kc every lane of a degree that exists runs, m' < l, and the steady loop needs
 // none of the start-up tests.
-template <bool SCALED>
+template <bool SCALED, bool BF>
 __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LaneParams P) {
   const int lane = threadIdx.x & 31;
   const int L = P.L;
@@ -428,7 +438,7 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
     const bool wr = inl && l >= P.as;     // U_l vanishes below |s|: those entries stay zero
     const float um = wr ? __ldg(&P.ufT[tri_idx(m, l, L)]) : 0.f;
     const long long* ib_m = P.ibase + (size_t)m * P.nI;
-    const uint32_t off_m = tc::sw128(m & 127, 4 * lane);  // (row m, K = l) in the tiles A_{m'}[m][.]
+    const uint32_t off_m = a_off<BF>(m & 127, lane);  // (row m, K = l) in the tiles A_{m'}[m][.]
     uint8_t* const A = P.A;
     double cur = 0.0, prev = 0.0;
     int E = 0;
@@ -470,8 +480,8 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
       if (inl && mp <= l) {
         if (wr) {
           const float x = f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur);
-          put_a(A, tb, P.ntiles, kbLaneTile, mp & 127, lane, (cu * cp) * x);
-          if (mp > m) put_a_at(A, ct + kc, P.ntiles, kbLaneTile, off_m, (um * cp) * (((mp - m) & 1) ? -x : x));
+          put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off<BF>(mp & 127, lane), (cu * cp) * x);
+          if (mp > m) put_a_at<BF>(A, ct + kc, P.ntiles, kbLaneTile, off_m, (um * cp) * (((mp - m) & 1) ? -x : x));
         }
         if (mp > m) {
           const double nxt = __fma_rn(mul_small_rn(ca, (uint32_t)m, 0), cur, -prev);  // m alpha, integer pipe
@@ -504,8 +514,8 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
       if (inl) {
         if (wr) {
           const float x = f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur);
-          put_a(A, tb, P.ntiles, kbLaneTile, mp & 127, lane, (cu * cp) * x);
-          put_a_at(A, ct + kc, P.ntiles, kbLaneTile, off_m, (um * cp) * (((mp - m) & 1) ? -x : x));
+          put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off<BF>(mp & 127, lane), (cu * cp) * x);
+          put_a_at<BF>(A, ct + kc, P.ntiles, kbLaneTile, off_m, (um * cp) * (((mp - m) & 1) ? -x : x));
         }
         double c;
         if constexpr (decltype(on_fp64)::value)
@@ -531,7 +541,7 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
     // ---- the last row m' = m, if the steady loop reached it ----
     if (m < lo) {
       if ((m & 127) == 127) tb = __ldg(&ib_m[m >> 7]) + kc;
-      if (wr) put_a(A, tb, P.ntiles, kbLaneTile, m & 127, lane, (cu * cp) * f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur));
+      if (wr) put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off<BF>(m & 127, lane), (cu * cp) * f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur));
     }
   }
 }
@@ -646,7 +656,8 @@ cudaError_t column_setup(DeltaWork& w, int L, int device) {
 static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, const LaneTables* lt, ATiles t,
                                  cudaStream_t st) {
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w.barrier, 0, 4 * sizeof(unsigned int), st)) != cudaSuccess) return e;
+  unsigned int* counter = lt ? lt->counter : w.barrier;
+  if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
   ColumnParams P;
   P.L = L;
   P.ntasks = w.ntasks;
@@ -654,7 +665,7 @@ static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, con
   P.sq = w.sqrt_tab;
   P.rsq = w.sqrt_tab + (2 * (size_t)L + 4);
   P.table = w.table;
-  P.counter = w.barrier;
+  P.counter = counter;
   P.Uf = Uf;
   P.alc = lt ? lt->alc : nullptr;
   P.pc = lt ? lt->pc : nullptr;
@@ -662,10 +673,10 @@ static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, con
   P.ab2 = lt ? lt->ab2 : nullptr;
   const bool tiles = t.A != nullptr;
   P.extent = tiles ? t.ntiles : (long long)delta_offset(L);
-  if (tiles && L > 1024)
-    column_tiles_kernel<true><<<lt->col_blocks, kColThreads, kTileSmem, st>>>(P);
+  if (tiles && t.bf16)
+    (L > 1024 ? column_tiles_kernel<true, true> : column_tiles_kernel<false, true>)<<<lt->col_blocks, kColThreads, kTileSmem, st>>>(P);
   else if (tiles)
-    column_tiles_kernel<false><<<lt->col_blocks, kColThreads, kTileSmem, st>>>(P);
+    (L > 1024 ? column_tiles_kernel<true, false> : column_tiles_kernel<false, false>)<<<lt->col_blocks, kColThreads, kTileSmem, st>>>(P);
   else if (L > 1024)
     column_recursion_kernel<true><<<w.blocks, w.threads, w.smem, st>>>(P);
   else
@@ -678,14 +689,14 @@ cudaError_t column_run(const DeltaWork& w, int L, cudaStream_t st) {
 }
 
 void lane_tables_free(LaneTables& t) {
-  void* ptrs[] = {t.alc, t.pc, t.alT, t.pT, t.t1m, t.t1e, t.ufT, t.ab2, t.tasks};
+  void* ptrs[] = {t.alc, t.pc, t.alT, t.pT, t.t1m, t.t1e, t.ufT, t.ab2, t.tasks, t.counter};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   t = LaneTables();
 }
 
 cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, const float* Uf, int nC,
-                              const long long* abase) {
+                              const long long* abase, int bf16) {
   cudaError_t e;
   const size_t n = (size_t)L * (L + 1) / 2;
   const int as = s < 0 ? -s : s;
@@ -704,8 +715,9 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
   if ((e = dev_malloc(&t.t1e, n * sizeof(int))) != cudaSuccess) return e;
   if ((e = dev_malloc(&t.ufT, n * sizeof(float))) != cudaSuccess) return e;
   if ((e = dev_malloc(&t.ab2, (size_t)L * sizeof(long long))) != cudaSuccess) return e;
+  if ((e = dev_malloc(&t.counter, 4 * sizeof(unsigned int))) != cudaSuccess) return e;
   if ((e = dev_malloc(&t.tasks, std::max<size_t>(tasks.size(), 1) * sizeof(int2))) != cudaSuccess) return e;
-  t.bytes = n * (3 * sizeof(double) + sizeof(int) + 3 * sizeof(float)) + (size_t)L * sizeof(long long) +
+  t.bytes = n * (3 * sizeof(double) + sizeof(int) + 3 * sizeof(float)) + 4 * sizeof(unsigned int) + (size_t)L * sizeof(long long) +
             tasks.size() * sizeof(int2);
   if (!tasks.empty() &&
       (e = cudaMemcpy(t.tasks, tasks.data(), tasks.size() * sizeof(int2), cudaMemcpyHostToDevice)) != cudaSuccess)
@@ -722,11 +734,12 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lane_recursion_kernel<false>, kColThreads, 0)) !=
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lane_recursion_kernel<false, false>, kColThreads, 0)) !=
         cudaSuccess)
       return e;
     t.blocks = sms * std::max(1, std::min(per_sm, SSHT_LANE_CTAS));
-    const void* fns[2] = {(const void*)column_tiles_kernel<false>, (const void*)column_tiles_kernel<true>};
+    const void* fns[4] = {(const void*)column_tiles_kernel<false, false>, (const void*)column_tiles_kernel<true, false>,
+                          (const void*)column_tiles_kernel<false, true>, (const void*)column_tiles_kernel<true, true>};
     for (const void* fn : fns) {
       if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTileSmem)) != cudaSuccess)
         return e;
@@ -734,18 +747,18 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
                                     (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
         return e;
     }
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[L > 1024 ? 1 : 0], kColThreads, kTileSmem)) !=
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[(L > 1024 ? 1 : 0) + (bf16 ? 2 : 0)], kColThreads, kTileSmem)) !=
         cudaSuccess)
       return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     t.col_blocks = sms * std::min(per_sm, SSHT_COLUMN_CTAS);
   }
-  if ((e = cudaFuncSetAttribute(lane_recursion_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(lane_recursion_kernel<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
-    return e;
+  const void* lanes[4] = {(const void*)lane_recursion_kernel<false, false>, (const void*)lane_recursion_kernel<true, false>,
+                          (const void*)lane_recursion_kernel<false, true>, (const void*)lane_recursion_kernel<true, true>};
+  for (const void* fn : lanes)
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
+      return e;
   return cudaDeviceSynchronize();
 }
 
@@ -753,7 +766,7 @@ cudaError_t column_run_inverse_tiles(const DeltaWork& w, const LaneTables& t, in
                                      cudaStream_t st) {
   if (!it.A || !it.ibase || !t.alT || w.method != kDeltaColumn) return cudaErrorInvalidValue;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w.barrier, 0, 4 * sizeof(unsigned int), st)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(t.counter, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
   LaneParams P;
   P.L = L;
   P.as = s < 0 ? -s : s;
@@ -767,12 +780,12 @@ cudaError_t column_run_inverse_tiles(const DeltaWork& w, const LaneTables& t, in
   P.ufT = t.ufT;
   P.A = it.A;
   P.ibase = it.ibase;
-  P.counter = w.barrier;
+  P.counter = t.counter;
   P.ntiles = it.ntiles;
-  if (L > 1024)
-    lane_recursion_kernel<true><<<t.blocks, kColThreads, 0, st>>>(P);
+  if (it.bf16)
+    (L > 1024 ? lane_recursion_kernel<true, true> : lane_recursion_kernel<false, true>)<<<t.blocks, kColThreads, 0, st>>>(P);
   else
-    lane_recursion_kernel<false><<<t.blocks, kColThreads, 0, st>>>(P);
+    (L > 1024 ? lane_recursion_kernel<true, false> : lane_recursion_kernel<false, false>)<<<t.blocks, kColThreads, 0, st>>>(P);
   return cudaGetLastError();
 }
 

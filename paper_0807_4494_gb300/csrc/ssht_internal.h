@@ -158,21 +158,22 @@ struct TileOut {
   size_t xbytes = 0;  // the whole tile array (index checks)
 };
 TileOut tc_forward_tiles(const TcPlan* p);
-// Where the recursion can write the A operand itself (3xTF32 plans): the forward tile array and
-// its per-m tile index base; A is null for split-BF16 plans (their A comes from tc_pack_a).
+// Where the recursion writes the A operand itself: the forward tile array and its per-m tile
+// index base.
 struct ATiles {
   uint8_t* A = nullptr;
   const long long* abase = nullptr;
   long long ntiles = 0;  // tiles in A (index checks)
+  int bf16 = 0;          // split-BF16 tiles (two parts) instead of FP32 values
 };
 ATiles tc_a_tiles(const TcPlan* p);
-// The column recursion writing the A tiles of a 3xTF32 plan directly (no FP64 table):
-// A_m[l][m'] = Uf_l[m'] Delta^l_{m'm} in FP32, one value an entry, by the rescaled relation whose
+// The column recursion writing the A tiles of a tensor-core plan directly (no FP64 table):
+// A_m[l][m'] = Uf_l[m'] Delta^l_{m'm}, rounded to FP32 and stored in the plan's tile form, by the rescaled relation whose
 // tables lt holds (delta_column.cu).
 struct LaneTables;
 cudaError_t column_run_tiles(const DeltaWork& w, const LaneTables& lt, int L, const float* Uf, ATiles t,
                              cudaStream_t st);
-// The inverse contraction's A tiles (rows m', K = l) of a 3xTF32 plan: the tile array and, per
+// The inverse contraction's A tiles (rows m', K = l): the tile array and, per
 // (m, row block i), the index from which chunk kc's tile is ibase[m * nI + i] + kc.
 struct InvTiles {
   uint8_t* A = nullptr;
@@ -180,12 +181,13 @@ struct InvTiles {
   int nI = 0;
   int nC = 0;
   long long ntiles = 0;  // tiles in A (index checks)
+  int bf16 = 0;
 };
 InvTiles tc_inverse_tiles(const TcPlan* p);
 // Plan-time tables of the recursion with one lane per degree, which writes the inverse's tiles
 // directly (delta_column.cu): coefficients a(l, m'), b(l, m'), first rows (mantissa, exponent), U
 // transposed, in the triangle layout [r][l] (l >= r); its tasks (column m, chunk kc of 32 degrees).
-// Plan-time tables of the tile-writing recursions (3xTF32 plans): the rescaled relation's
+// Plan-time tables of the tile-writing recursions: the rescaled relation's
 // alpha(l, m') and p(l, m') degree-major (l(l+1)/2 + m') and in the triangle layout [m'][l], the
 // first rows and U transposed (delta_column.cu).
 struct LaneTables {
@@ -198,6 +200,7 @@ struct LaneTables {
   float* ufT = nullptr;
   long long* ab2 = nullptr;  // per M: the forward tile base less the row blocks below M's own
   int2* tasks = nullptr;
+  unsigned int* counter = nullptr;  // next task of the plan's own sweeps (plans of a group run side by side)
   int ntasks = 0;
   int blocks = 0;      // grid of the degree-lane recursion
   int col_blocks = 0;  // grid of the column recursion writing the forward tiles
@@ -205,7 +208,7 @@ struct LaneTables {
 };
 // Needs the column DeltaWork of the plan (its sqrt tables) and U (FP32) on the device; synchronises.
 cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, const float* Uf, int nC,
-                              const long long* abase);
+                              const long long* abase, int bf16);
 void lane_tables_free(LaneTables& t);
 cudaError_t column_run_inverse_tiles(const DeltaWork& w, const LaneTables& t, int L, int s, InvTiles it,
                                      cudaStream_t st);
