@@ -245,15 +245,27 @@ int run_dft(ssht_plan_t p, cufftHandle h, int sign, void* in, void* out, cudaStr
   return exec_fft(p, h, in, out, sign < 0 ? CUFFT_FORWARD : CUFFT_INVERSE, st);
 }
 
-// One fused torus pass of an FP32 plan (DFT along theta or phi with its glue), timed as FFT work.
-// in / out: a plan workspace (W1, W2) or a grid of the plan's B complex fields.
-int run_torus(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t st) {
+// The torus passes of an FP32 plan (DFT along theta or phi with its glue), timed as FFT work.  Inverse:
+// F in W1 -> samples f.
+int torus_inverse_pass(ssht_plan_t p, int step, void* f, cudaStream_t st) {
   StageScope sc(p, SSHT_STAGE_FFT, st);
-  const size_t grid = p->pair_grid_bytes();
-  const size_t ib = (in == p->W1 || in == p->W2) ? p->w_bytes : grid;
-  const size_t ob = (out == p->W1 || out == p->W2) ? p->w_bytes : grid;
-  SSHT_CUDA(torus_pass(p->torus, which, p->s, p->B, in, ib, out, ob, st), "torus pass");
-  p->launches += 1;
+  int n = 0;
+  SSHT_CUDA(torus_inverse(p->torus, p->s, p->B, p->W1, p->w_bytes, p->W2, f, p->pair_grid_bytes(), p->delta.status, p->wait_ns,
+                          st, &n, step),
+            "torus pass");
+  p->launches += n;
+  return 0;
+}
+// Forward / adjoint: samples f -> the projection's data tiles (tensor-core plans) or H in W1.
+int torus_analysis_pass(ssht_plan_t p, int step, int adjoint, const void* f, cudaStream_t st) {
+  StageScope sc(p, SSHT_STAGE_FFT, st);
+  int n = 0;
+  TileOut tiles;
+  if (p->tc) tiles = tc_forward_tiles(p->tc);
+  SSHT_CUDA(torus_analysis(p->torus, adjoint, p->s, p->B, f, p->pair_grid_bytes(), p->W1, p->W2, p->W1, p->w_bytes,
+                           p->tc ? &tiles : nullptr, p->delta.status, p->wait_ns, st, &n, step),
+            "torus pass");
+  p->launches += n;
   return 0;
 }
 
@@ -359,10 +371,9 @@ int mark_free_a(ssht_plan_t p, int forward, cudaStream_t st) {
   return 0;
 }
 
-// The inverse's A tiles of a plan whose recursions write them (3xTF32) are made as soon as the
-// previous inverse contraction has read them, without waiting for the forward contraction in
-// between: the degree-lane recursion then runs beside the forward's torus passes instead of beside
-// the next call's data packing (GB300, L = 1024, B = 64: 11.995 ms a step against 12.095).
+// The inverse's A tiles of a plan whose recursions write them are made as soon as the previous
+// inverse contraction has read them, without waiting for the forward contraction in between: the
+// degree-lane recursion (no shared memory) then fills the gaps beside the forward's packing and passes.
 #ifndef SSHT_INVERSE_OPERANDS_EARLY
 #define SSHT_INVERSE_OPERANDS_EARLY 1
 #endif
@@ -421,22 +432,21 @@ int tc_multiply(ssht_plan_t p, int forward, void* dst, cudaStream_t st) {
   return 0;
 }
 
-// Tensor-core forward / adjoint after the phi pass (in W2): the theta pass `which` (4 forward, 5
-// adjoint) writes the projection's data tiles itself (no H, no data packing), then the projection.
-int theta_to_tiles(ssht_plan_t p, int which, void* flm, cudaStream_t st) {
+// FP32-class forward (adjoint = 0) or adjoint: the torus passes, then the projection.  Tensor-core plans:
+// the theta pass writes the projection's data tiles itself (no H, no data packing).
+template <typename T>
+int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st);
+
+int analysis_fp32(ssht_plan_t p, int adjoint, const void* f, void* flm, cudaStream_t st) {
   int rc;
-  const TileOut tiles = tc_forward_tiles(p->tc);
-  {
-    StageScope sc(p, SSHT_STAGE_FFT, st);
-    SSHT_CUDA(torus_pass(p->torus, which, p->s, p->B, p->W2, p->w_bytes, nullptr, 0, st, &tiles), "torus pass");
-    p->launches += 1;
-  }
+  if ((rc = torus_analysis_pass(p, 0, adjoint, f, st)) || (rc = torus_analysis_pass(p, 1, adjoint, f, st))) return rc;
+  if (!p->tc) return project<float>(p, p->W1, flm, st);
   if ((rc = join_operands(p, st)) || (rc = tc_multiply(p, 1, flm, st))) return rc;
   return mark_free_a(p, 1, st);
 }
 
 // The SIMT projection of forward / adjoint from the folded torus sums H (in W), after the join
-// (tensor-core plans take theta_to_tiles).
+// (tensor-core plans: analysis_fp32).
 template <typename T>
 int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st) {
   int rc;
@@ -538,8 +548,8 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
   }
   if (!p->tc && (rc = mark_free(p, st))) return rc;
   if (p->torus) {
-    if ((rc = run_torus(p, 0, p->W1, p->W2, st))) return rc;
-    return run_torus(p, 1, p->W2, f, st);
+    if ((rc = torus_inverse_pass(p, 0, f, st))) return rc;
+    return torus_inverse_pass(p, 1, f, st);
   }
   rc = run_dft(p, p->fft_theta, +1, p->W1, p->W2, st);
   if (rc) return rc;
@@ -571,12 +581,7 @@ int forward_impl(ssht_plan_t p, const void* f, void* flm, cudaStream_t st) {
   const Dims& d = p->d;
   int rc = begin_operands(p, 1, st);
   if (rc) return rc;
-  if (p->torus) {
-    if ((rc = run_torus(p, 2, f, p->W2, st))) return rc;
-    if (p->tc) return theta_to_tiles(p, 4, flm, st);
-    if ((rc = run_torus(p, 4, p->W2, p->W1, st))) return rc;
-    return project<T>(p, p->W1, flm, st);
-  }
+  if (p->torus) return analysis_fp32(p, 0, f, flm, st);
   rc = analysis_front<T>(p, f, 0, st);
   if (rc) return rc;
   {
@@ -604,12 +609,7 @@ int adjoint_impl(ssht_plan_t p, const void* g, void* flm, cudaStream_t st) {
   const Dims& d = p->d;
   int rc = begin_operands(p, 1, st);
   if (rc) return rc;
-  if (p->torus) {
-    if ((rc = run_torus(p, 3, g, p->W2, st))) return rc;
-    if (p->tc) return theta_to_tiles(p, 5, flm, st);
-    if ((rc = run_torus(p, 5, p->W2, p->W1, st))) return rc;
-    return project<T>(p, p->W1, flm, st);
-  }
+  if (p->torus) return analysis_fp32(p, 1, g, flm, st);
   rc = analysis_front<T>(p, g, 1, st);
   if (rc) return rc;
   {
@@ -892,8 +892,8 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, (void**)&p->U, tri(L) * sizeof(double), "spin column"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->Uf, tri(L) * sizeof(float), "spin column (FP32)"))) return bail(rc);
   // FP64: full N x N torus rows and an M-point convolution buffer; FP32 (fused torus passes): half
-  // rows of N x L only, plus one row a field for the column pairs of the phi pass's output.
-  const size_t torus = (size_t)B * (p->f64 ? (size_t)d.N * d.N : (size_t)(d.N + 1) * d.L) * p->elem;
+  // rows of N x L, or a pass's operand tiles.
+  const size_t torus = p->f64 ? (size_t)B * d.N * d.N * p->elem : torus_workspace_bytes(L, B);
   if (pair && (rc = dalloc(p, &p->rc, (size_t)B * L * L * p->elem, "spin-pair coefficients"))) return bail(rc);
   if ((real || pair) && (ce = real_setup()) != cudaSuccess) {
     release(p);
@@ -955,7 +955,7 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
       return fail(SSHT_ECUDA, "weight spectrum setup failed");
     }
   } else {
-    ce = torus_setup(&p->torus, L, p->ph, p->device);
+    ce = torus_setup(&p->torus, L, p->device);
     if (ce != cudaSuccess) {
       release(p);
       return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,

@@ -23,8 +23,7 @@ struct BoundsRecord {
 // Where a checked access sits (the first failing one is reported by this number).
 enum BoundsSite {
   kbNone = 0,
-  kbInverseThetaIn = 1, kbInverseThetaOut, kbPhiIn, kbPhiOut, kbForwardThetaIn, kbForwardThetaOut,
-  kbAdjointThetaIn, kbAdjointThetaOut, kbPutTile,
+  kbTorusIn = 1, kbTorusOut, kbTorusTile, kbPutTile,
   kbPackVIn = 20, kbPackVOut, kbPackAIn, kbPackAOut, kbGemmA, kbGemmX, kbGemmOut,
   kbColumnTable = 40, kbColumnTile, kbLaneTable, kbLaneTile, kbColumnCoef,
   kbPairIn = 60, kbPairOut, kbRealIn, kbRealOut,

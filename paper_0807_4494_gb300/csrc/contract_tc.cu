@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
             for (int q = 0; q < 6; ++q)
 #pragma unroll
               for (int kk = 0; kk < 2; ++kk)
-                mma_bf16(dt, desc_sw128(sa + oa[pa[q]] + kk * 32), desc_sw128(sb + ob[pb[q]] + kk * 32), idesc,
+                mma_f16(dt, desc_sw128(sa + oa[pa[q]] + kk * 32), desc_sw128(sb + ob[pb[q]] + kk * 32), idesc,
                          (q == 0 && kk == 0) ? 0u : 1u);
           } else {
 #pragma unroll

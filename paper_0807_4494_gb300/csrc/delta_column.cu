@@ -254,12 +254,12 @@ __global__ void __launch_bounds__(kColThreads, 2) column_recursion_kernel(Column
 // lies in [0.15, 1] up to l = 2047 and multiplies the FP32 output; alpha and p are plan-time
 // tables (rescale_tables_kernel).  Each value is rounded to FP32 once and staged as FP32, so a
 // CTA needs half the table kernel's shared memory and three fit an SM.
-// The forward's tiles are needed only after the inverse's and the forward's torus passes, so the
-// persistent grid takes one CTA an SM and runs beside those passes, which keep two of their three
-// CTAs an SM (GB300, L = 1024, B = 64: 12.09 ms a step, against 12.11 with two CTAs an SM and 12.15
-// with three).
+// Three CTAs an SM, all that fit: a torus pass (one CTA of 213 KB an SM) cannot share an SM with the
+// sweep, so a sweep of one CTA an SM (1.61 ms instead of 0.74 at L = 1024), which ran beside the FFT
+// passes the products replaced, now only holds them up (GB300, inverse + forward: L = 1024, B = 64 9.96 ms
+// with three against 10.69 with one; L = 2048, B = 16 33.4 against 41.2).
 #ifndef SSHT_COLUMN_CTAS
-#define SSHT_COLUMN_CTAS 1
+#define SSHT_COLUMN_CTAS 3
 #endif
 constexpr int kTileStageFloats = 32 * 33;
 constexpr int kTileWarpBytes = kTileStageFloats * 4 + 32 * 8 + 32 * 4;  // stage, alpha[32], p[32]

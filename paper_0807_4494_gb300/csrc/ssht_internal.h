@@ -214,21 +214,27 @@ cudaError_t column_run_inverse_tiles(const DeltaWork& w, const LaneTables& t, in
                                      cudaStream_t st);
 
 // ---------------------------------------------------------------------------
-// Fused torus passes of FP32 plans (torus_pass.cu)
+// Fused torus passes of FP32 plans (torus_gemm.cu)
 // ---------------------------------------------------------------------------
-// Odd-length DFTs along theta and phi (Bluestein in shared memory) with the extension, phases, sin(theta) weight convolution and transpositions folded in.  Layouts (float2):
-// F half rows [B][N][L] (m + Lp, m' >= 0), h [B][L][N], f [B][L][N], X [B][(N+1)/2][L][2] (columns
-// m + Lp = 2p + j by pairs), H [B][N][L].
+// DFTs along theta and phi with the extension, phases, sin(theta) weight convolution and folds, as
+// tensor-core products.  F and H: half rows (float2) [B][N][L] (m + Lp, m' >= 0); f: samples [B][L][N].
 struct TorusPlan;
-cudaError_t torus_setup(TorusPlan** out, int L, const void* ph, int device);
+cudaError_t torus_setup(TorusPlan** out, int L, int device);  // synchronises
 void torus_destroy(TorusPlan* p);
 size_t torus_bytes(const TorusPlan* p);
-// which: 0 inverse theta (F -> h), 1 inverse phi (h -> f), 2 forward phi (f -> X, scale 1/N),
-// 3 adjoint phi (f -> X), 4 forward theta with the weight convolution (X -> H), 5 adjoint theta (X -> H).
-// which = 4 with tiles (mode != 0): the data tiles of the forward projection instead of H.
-// in_bytes / out_bytes: the extents of the buffers (the index checks of bounds-checked builds).
-cudaError_t torus_pass(const TorusPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* out,
-                       size_t out_bytes, cudaStream_t st, const TileOut* tiles = nullptr);
+// Bytes of each of the two workspaces a plan of B fields hands to the passes.
+size_t torus_workspace_bytes(int L, int B);
+// Inverse, in two steps: 0 theta (F, a workspace, is packed into `work` and then overwritten by the
+// phi pass's operand), 1 phi (from that operand to the samples out).  *_bytes: extents of the buffers
+// (the index checks of bounds-checked builds).  Timeouts of the pipeline waits set bit 2 of *status.
+cudaError_t torus_inverse(const TorusPlan* p, int s, int B, void* F, size_t f_bytes, void* work, void* out, size_t out_bytes,
+                          int* status, long long wait_ns, cudaStream_t st, int* launches, int step);
+// Forward (adjoint = 0: extension and sin(theta) weight) or adjoint, in two steps: 0 phi (f packed into
+// the workspace w1, the product into w2), 1 theta (from w2 into the projection's data tiles, or into H
+// without tiles; H may be w1).
+cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const void* f, size_t f_bytes, void* w1, void* w2,
+                           void* H, size_t h_bytes, const TileOut* tiles, int* status, long long wait_ns, cudaStream_t st,
+                           int* launches, int step);
 
 // ---------------------------------------------------------------------------
 // Torus kernels (torus.cu)

@@ -1,5 +1,5 @@
 // PTX helpers for the tcgen05 / TMEM / bulk-copy / mbarrier machinery of sm_100-family GPUs,
-// used by the tensor-core contraction (contract_tc.cu).
+// used by the tensor-core contraction (contract_tc.cu) and the torus passes (torus_gemm.cu).
 #pragma once
 
 #include <cstdint>
@@ -89,6 +89,27 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// Thread-block clusters: the rank in the cluster, a peer's shared-memory address, a barrier of the
+// whole cluster, and an arrival on a peer's mbarrier.  The arrival carries no ordinary memory accesses
+// with it (what it announces are finished tensor-memory loads and finished bulk copies): its default
+// scope is the CTA, because a release at cluster scope waits 1300 - 1800 clocks for the arriving
+// thread's earlier accesses, which made it the longest step of the pipeline.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t peer_addr(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_peer(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
@@ -98,6 +119,17 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+
+// 1-D bulk copy shared -> global, tracked by the issuing thread's bulk groups (same alignment rules).
+__device__ __forceinline__ void bulk_s2g(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// Waits until at most N of this thread's newest bulk groups still read their shared memory.
+template <int N> __device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
@@ -119,12 +151,55 @@ __device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_
                ::"r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum));
 }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 with BF16 operands (K = 16 per instruction).
-__device__ __forceinline__ void mma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
+// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 with FP16 or BF16 operands, as idesc says (K = 16 per
+// instruction).
+__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
   asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
                ::"r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum));
 }
+
+// The forms for a pair of CTAs of a cluster (cta_group::2): both allocate and free together, the
+// leader (rank 0) issues products of 256 rows -- 128 a CTA, each CTA holding its rows of A, half of the
+// rows of B and its rows of D -- and their completion arrives at the same barrier of both CTAs.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols));
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
+}
+// kind::f16, one CTA or a pair, with the descriptors (desc_sw128) given by their low words -- the
+// start address in 16-byte units, kDescLow added -- so that stepping through a tile is one addition.
+constexpr uint32_t kDescLow = 1u << 16, kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);
+template <bool PAIR>
+__device__ __forceinline__ void mma_f16_lo(uint32_t dtmem, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t accum) {
+  if constexpr (PAIR)
+    asm volatile("{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
+                 " tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n}\n"
+                 ::"r"(dtmem), "r"(alo), "r"(blo), "r"(idesc), "r"(kDescHigh), "r"(accum));
+  else
+    asm volatile("{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n mov.b64 da, {%1, %4};\n mov.b64 db, {%2, %4};\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n"
+                 ::"r"(dtmem), "r"(alo), "r"(blo), "r"(idesc), "r"(kDescHigh), "r"(accum));
+}
+// One lane of the (converged) warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
+}
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
+// Moves registers between the warpgroups of a CTA (every warp of the warpgroup executes it): N a
+// thread from here on.  The shares must add up to at most what the CTA was launched with.
+template <int N> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 
 // Arrive on an mbarrier once every tcgen05.mma issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
