@@ -427,7 +427,7 @@ int tc_pack(ssht_plan_t p, const void* src, cudaStream_t st) {
 int tc_multiply(ssht_plan_t p, int forward, void* dst, cudaStream_t st) {
   int n = 0;
   StageScope sc(p, forward ? SSHT_STAGE_PROJECT : SSHT_STAGE_INVERSE, st);
-  SSHT_CUDA(tc_gemm(p->tc, forward, dst, p->ph, p->delta.status, p->wait_ns, st, &n), "tensor-core contraction");
+  SSHT_CUDA(tc_gemm(p->tc, forward, dst, forward ? p->W1 : nullptr, p->ph, p->delta.status, p->wait_ns, st, &n), "tensor-core contraction");
   p->launches += n;
   return 0;
 }
@@ -717,8 +717,8 @@ int time_contractions(ssht_plan_t p, cudaStream_t st, float* ms) {
   int n = 0, rc = 0;
   for (int it = 0; it < 4 && !rc; ++it) {
     if (it == 1) cudaEventRecord(e0, st);
-    cudaError_t e = tc_gemm(p->tc, 0, p->W1, p->ph, p->delta.status, p->wait_ns, st, &n);
-    if (e == cudaSuccess) e = tc_gemm(p->tc, 1, p->W2, p->ph, p->delta.status, p->wait_ns, st, &n);
+    cudaError_t e = tc_gemm(p->tc, 0, p->W1, nullptr, p->ph, p->delta.status, p->wait_ns, st, &n);
+    if (e == cudaSuccess) e = tc_gemm(p->tc, 1, p->W2, p->W1, p->ph, p->delta.status, p->wait_ns, st, &n);
     if (e != cudaSuccess) rc = fail(SSHT_ECUDA, std::string("tuning contraction: ") + cudaGetErrorString(e));
   }
   cudaEventRecord(e1, st);

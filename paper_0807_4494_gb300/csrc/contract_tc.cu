@@ -1,4 +1,4 @@
-// The O(L^3) contractions on the tcgen05 tensor cores (3xTF32 split products, FP32 accumulation
+// The O(L^3) contractions on the tcgen05 tensor cores (split FP16 or BF16 products, FP32 accumulation
 // in tensor memory), for batched transforms.
 //
 // For each m >= 0 both signs of m share one matrix (eqn wignerd_sym6 gives
@@ -12,25 +12,30 @@
 //       Y_m[m', (0, part, b)] = part(H_{m m'}[b]),  Y_m[m', (1, part, b)] = (-1)^{m'} part(H_{-m m'}[b]);
 //       sf_{lm} = (-1)^s i^{m+s} P[l, (0, ., b)],  sf_{l,-m} = (-1)^s i^{-m+s} (-1)^l P[l, (1, ., b)].
 // So every m is a real GEMM with M = 128-row blocks of m' (inverse) or l (forward), K = l or m'
-// in chunks of 32, N = 2H columns, H = 2B rounded up to 16 (column sign*H + 2b + part).  Operands
-// are split x = hi + lo (TF32) and the product is hi*hi + hi*lo + lo*hi (the dropped lo*lo is
-// ~2^-22 relative).
+// in chunks of 32, N = 2H columns, H = 2B rounded up to 16 (column sign*H + 2b + part).
+//
+// Split forms.  SSHT_TF32X3 plans: x = hi + lo in two parts of 11 significant bits and the product
+// hi*hi + hi*lo + lo*hi (the dropped lo*lo is ~2^-24 relative), the arithmetic of a 3xTF32 split with the parts
+// held as FP16, which the tensor cores multiply at twice the TF32 rate and which take half the bytes.  FP16's
+// range is met by powers of two: 2^10 for A (|U Delta| < 18.1), for the data one a (row pair, chunk) -- a
+// field's real and imaginary part over 32 K -- from its largest magnitude, undone when the segment is added.
+// SSHT_BF16X6 plans: three BF16 parts, the six products down to 2^-24.
 //
 // Accumulation.  The tensor core's FP32 accumulation truncates (rounds toward zero); over the
-// 384 accumulation steps of K = 1024 that bias alone reaches ~1e-5 relative.  So each K chunk
-// accumulates into a fresh tensor-memory segment, the two small correction products first and the
-// four hi*hi products last (truncation then acts on four large steps only), and the epilogue warps
+// accumulation steps of K = 1024 that bias alone reaches ~1e-5 relative.  So each K chunk
+// accumulates into a fresh tensor-memory segment, the small correction products first and the
+// large ones last (truncation then acts on two large steps only), and the epilogue warps
 // add every segment into FP32 running sums in registers (round to nearest).
 //
-// Operands are written once per call (A also once per plan with the Delta cache) as tiles already
-// in the K-major SWIZZLE_128B layout -- 3xTF32: the FP32 values (16 KB an A tile), split into hi and
-// lo in shared memory when they arrive; split-BF16: both parts -- so the main kernel moves them with
-// 1-D bulk copies.  Main kernel: persistent, one CTA per SM, 10 warps: warp 0 lane 0 issues the bulk
-// copies (a ring of 2-4 stages), warp 1 lane 0 issues tcgen05.mma into one of two 128 x 256 FP32 accumulator
-// segments in tensor memory, warps 2-9 (two per 32-lane quarter of tensor memory, one for each
-// sign of m) read the accumulator with tcgen05.ld, apply the phases and write the outputs (the
-// inverse writes half rows m' >= 0 of F; the torus passes apply the extension).  Work items (m, row
-// block) are sorted (groups of four m, or decreasing length) and dealt to the CTAs by a greedy
+// Operands are written once per call (A also once per plan with the Delta cache) as tiles of split parts
+// already in the K-major SWIZZLE_128B layout (split-FP16: 128 bytes a row and 32 K, as many as FP32 values),
+// so that the main kernel moves them with 1-D bulk copies.  Main kernel: persistent, one CTA per SM, five
+// warpgroups: warp 0 issues the bulk copies (a ring of 2-4 stages), warp 1 issues tcgen05.mma into one of two
+// 128 x 256 FP32 accumulator segments in tensor memory (both as whole warps with an elected lane: a single
+// lane's loop took 70 clocks a product), sixteen warps (four per 32-lane quarter of tensor memory, each
+// every fourth group of 16 columns) read the accumulator with tcgen05.ld, apply the phases and write the
+// outputs (the inverse writes half rows m' >= 0 of F; the torus passes apply the extension).  Work items (m,
+// row block) are sorted (groups of four m, or decreasing length) and dealt to the CTAs by a greedy
 // schedule made on the host (schedule()).  Every wait is bounded; a
 // timeout latches a status bit and the CTA drains its copies and MMAs before leaving.
 #include "ssht_internal.h"
@@ -49,11 +54,15 @@ using namespace tc;
 
 constexpr int TM = kTileRows;              // rows per tile
 constexpr int TK = kTileK;                 // K per chunk (one 128-byte TF32 row)
-constexpr int A_PART = kAPart;             // 16 KB: one split part of an A tile
-constexpr int A_TILE = kATile;             // both parts of an A tile in shared memory (hi then lo)
+constexpr int A_PART = kAPart;             // 16 KB: one part of an A tile
 constexpr int MAX_STAGES = 4;             // pipeline depth: a plan parameter, 2 .. MAX_STAGES
-constexpr int EPI_WARPS = 8;                       // two per tensor-memory lane quarter
-constexpr int THREADS = 64 + 32 * EPI_WARPS;       // producer warp, MMA warp, epilogue warps
+constexpr int SCALE_SLOTS = 8;            // ring of the chunks' scales (MAX_STAGES + 2 would do)
+constexpr int EPI_WARPS = 16;                      // four per tensor-memory lane quarter
+// producer, MMA and two idle warps, then the epilogue's; 96 registers a thread at launch, of which the
+// first warpgroup gives some up for the epilogue's 64 running sums
+constexpr int THREADS = 128 + 32 * EPI_WARPS;
+constexpr int REGS_ISSUE = 32, REGS_EPILOGUE = 112;
+static_assert(128 * REGS_ISSUE + 32 * EPI_WARPS * REGS_EPILOGUE <= THREADS * 96, "register shares");
 
 __host__ __device__ inline long long tri_ll(long long m) { return m * (m + 1) / 2; }
 __host__ __device__ inline size_t doff(long long l) { return (size_t)(l * (l + 1) * (2 * l + 1) / 6); }
@@ -70,10 +79,13 @@ struct TcArgs {
   const Item* items;
   const uint8_t* A;       // packed A tiles
   const uint8_t* X;       // packed data tiles
+  const float* XS;        // split-FP16: their scales, [tile][NC / 2]
   const long long* xoff;  // per m: data tile index of chunk xc0(m)
   const int* xc0;         // per m: first chunk stored for m
   const float2* ph;       // e^{i pi k/N}, k in [-(N-1), N-1], at k + N - 1
-  float2* out;            // inverse: theta-DFT input E [B][N][N]; forward: flm [B][L*L]
+  float2* out;            // half rows [B][N][L] (rows by signed order; inverse: F, columns m'; forward with
+                          // `rows`: columns l >= |m|), or flm [B][L*L]
+  int rows;               // forward: half rows instead of flm
   int* status;
   long long wait_ns;      // spin limit of the pipeline waits
   long long a_tiles, x_tiles, out_n;  // extents of A, this slice's data tiles and out (index checks)
@@ -98,7 +110,7 @@ template <bool FWD, bool BF>
 __global__ void __launch_bounds__(256) pack_a_kernel(int L, int s, const Item* __restrict__ items,
                                                      const double* __restrict__ table, const float* __restrict__ Uf,
                                                      uint8_t* __restrict__ A, long long a_tiles) {
-  __shared__ __align__(16) uint8_t tile[A_TILE];
+  __shared__ __align__(16) uint8_t tile[kParts<BF> * A_PART];
   constexpr int PER = TM * TK / 256;
   const Item it = items[blockIdx.y];
   const int c = it.c0 + blockIdx.x;
@@ -124,7 +136,8 @@ __global__ void __launch_bounds__(256) pack_a_kernel(int L, int s, const Item* _
     const int r = FWD ? e / TK : e % TM, k = FWD ? e % TK : e / TM;
     const int mp = FWD ? c * TK + k : it.i * TM + r;
     const float a = u[q] * f64_to_f32_rn(d[q]);
-    put_split<BF>(tile, A_PART, r, k, ((mp - m) & 1) ? -a : a);
+    put_parts<BF>(tile, A_PART, sw128(r, 2 * k), ((mp - m) & 1) ? -a : a);
+    if (BF) *(uint16_t*)(tile + A_PART + (sw128(r, 2 * k) ^ 64u)) = 0;
   }
   __syncthreads();
   if (!in_bounds(it.atile + blockIdx.x, a_tiles, kbPackAOut)) return;
@@ -139,54 +152,110 @@ __global__ void __launch_bounds__(256) pack_a_kernel(int L, int s, const Item* _
 // ---------------------------------------------------------------------------------------------
 
 // Inverse data tiles (m, c): V_m[l, j], l = 32 c + k, rows j = sign * NC/2 + 2b (real part) and
-// 2b + 1 (imaginary part), for 16 consecutive m at once.  For every field the coefficients
-// sf_{l,+-m} of the 32 degrees of chunk c are read as runs of 16 consecutive orders (coalesced),
-// turned around in shared memory, and every tile row -- 32 consecutive K = l -- is written by one
-// warp at once; the rows of padding fields are written as zeros.  Fields run in slices of Bs
-// (blockIdx.z): slice z holds fields z Bs .. z Bs + Bs - 1 in its own tile region of xslice bytes.
+// 2b + 1 (imaginary part), for 16 consecutive m at once.  For two fields at a time the coefficients
+// sf_{l,+-m} of the 32 degrees of chunk c are read as runs of 16 consecutive orders (coalesced; the next
+// two fields' are under way meanwhile) and turned around in shared memory.  Split-FP16: a thread then takes
+// 8 K of one order, sign and field, four neighbouring threads the 32 K of a tile row, so that they find the
+// row pair's power of two with two shuffles and store 16 bytes at a time.  Split-BF16: a warp takes a row
+// pair, a lane one K.  The rows of padding fields are written as zeros.  Fields run in slices of Bs, slice z
+// in its own tile region of xslice bytes, and a CTA takes kPackFields rows' worth of fields of a slice
+// (blockIdx.z: slice and group of fields), which keeps the GPU filled at small band-limits too.
+constexpr int kPackFields = 8;
+static int pack_v_groups(int NC) { return (NC / 4 + kPackFields - 1) / kPackFields; }
+
 template <bool BF>
 __global__ void __launch_bounds__(256) pack_v_kernel(int L, int s, int Btot, int Bs, size_t xslice, int NC,
                                                      const int* __restrict__ xc0, const long long* __restrict__ xoff,
-                                                     const float2* __restrict__ flm, uint8_t* __restrict__ X) {
-  __shared__ float2 sv[32][33];
-  const int B = min(Bs, Btot - (int)blockIdx.z * Bs);
-  const long long flm_n = (long long)Btot * L * L, flm0 = (long long)blockIdx.z * Bs * L * L;
+                                                     const float2* __restrict__ flm, uint8_t* __restrict__ X,
+                                                     float* __restrict__ XS) {
+  __shared__ float2 sv[2][32][33];
+  const int half = NC / 2, nb = half / 2;  // nb: fields of a sign half, padded
+  const int groups = (nb + kPackFields - 1) / kPackFields, z = blockIdx.z / groups, bg = (blockIdx.z - z * groups) * kPackFields;
+  const int B = min(Bs, Btot - z * Bs);
+  const long long flm_n = (long long)Btot * L * L, flm0 = (long long)z * Bs * L * L;
   const long long x_tiles = (long long)(xslice / (kParts<BF> * (size_t)NC * 128));
-  flm += (size_t)blockIdx.z * Bs * L * L;
-  X += (size_t)blockIdx.z * xslice;
+  X += (size_t)z * xslice;
+  if (!BF) XS += (size_t)z * x_tiles * half;
   const int c = blockIdx.x, m0 = 16 * blockIdx.y;
   // xc0 grows with m: when chunk c is below the first stored chunk of m0, no tile of this CTA's 16
   // orders is stored (about half the grid: the degrees of chunk c all lie below m0)
   if (m0 >= L || c < xc0[m0]) return;
   const int as = s < 0 ? -s : s;
-  const int part_bytes = NC * 128, half = NC / 2, nb = half / 2;  // nb: fields of a sign half, padded
+  const int part_bytes = NC * 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int b = 0; b < nb; ++b) {
-    if (b < B) {
-      // 32 degrees l x (orders m0 .. m0 + 15, then -m0 .. -m0 - 15)
-      for (int q = threadIdx.x; q < 1024; q += 256) {
-        const int lo = q >> 5, col = q & 31, sign = col >> 4, m = m0 + (col & 15);
+  const int b_end = min(bg + kPackFields, nb);
+  // 32 degrees l x (orders m0 .. m0 + 15, then -m0 .. -m0 - 15) of a field: four values a thread
+  float2 v[2][4];
+  auto load = [&](int b) {
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = threadIdx.x + 256 * i, lo = q >> 5, col = q & 31, sign = col >> 4, m = m0 + (col & 15);
         const int l = c * TK + lo;
-        float2 v = make_float2(0.f, 0.f);
-        const long long fi = (long long)b * L * L + (long long)l * l + l + (sign ? -m : m);
-        if (m < L && l < L && l >= m && l >= as && !(sign && m == 0) && in_bounds(flm0 + fi, flm_n, kbPackVIn)) {
-          v = flm[fi];
-          if (sign && (l & 1)) v = make_float2(-v.x, -v.y);
+        float2 x = make_float2(0.f, 0.f);
+        const long long fi = flm0 + (long long)(b + f) * L * L + (long long)l * l + l + (sign ? -m : m);
+        if (b + f < B && m < L && l < L && l >= m && l >= as && !(sign && m == 0) && in_bounds(fi, flm_n, kbPackVIn)) {
+          x = __ldg(&flm[fi]);
+          if (sign && (l & 1)) x = make_float2(-x.x, -x.y);
         }
-        sv[lo][col] = v;
+        v[f][i] = x;
       }
-    }
+  };
+  load(bg);
+  for (int b = bg; b < b_end; b += 2) {
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int q = threadIdx.x + 256 * i;
+        sv[f][q >> 5][q & 31] = v[f][i];
+      }
     __syncthreads();
-    for (int cb = warp; cb < 32; cb += 8) {
-      const int sign = cb >> 4, m = m0 + (cb & 15);
-      if (m >= L || c < xc0[m]) continue;  // tile (m, c) is not stored
-      if (!in_bounds(xoff[m] + (c - xc0[m]), x_tiles, kbPackVOut) || !in_bounds(sign * half + 2 * b + 1, NC, kbPackVOut))
-        continue;
-      uint8_t* tile = X + (size_t)(xoff[m] + (c - xc0[m])) * kParts<BF> * part_bytes;
-      const float2 v = b < B ? sv[lane][cb] : make_float2(0.f, 0.f);
-      const int j = sign * half + 2 * b;
-      put_split<BF>(tile, part_bytes, j, lane, v.x);
-      put_split<BF>(tile, part_bytes, j + 1, lane, v.y);
+    if (b + 2 < b_end) load(b + 2);
+    if constexpr (BF) {
+      for (int cb = warp; cb < 64; cb += 8) {
+        const int f = cb >> 5, sign = (cb >> 4) & 1, m = m0 + (cb & 15), j = sign * half + 2 * (b + f);
+        if (m >= L || c < xc0[m] || b + f >= b_end) continue;  // tile (m, c) is not stored
+        const long long tix = xoff[m] + (c - xc0[m]);
+        if (!in_bounds(tix, x_tiles, kbPackVOut) || !in_bounds(j + 1, NC, kbPackVOut)) continue;
+        const float2 x = sv[f][lane][cb & 31];
+        put_rows2<BF>(X + (size_t)tix * kParts<BF> * part_bytes, part_bytes, j, lane, x.x, x.y, 1.f, true);
+      }
+    } else {
+      const int f = warp >> 2, cb = (warp & 3) * 8 + (lane >> 2), kq = lane & 3;
+      const int sign = cb >> 4, m = m0 + (cb & 15), j = sign * half + 2 * (b + f);
+      float x[8], y[8], amax = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float2 w = sv[f][8 * kq + k][cb];
+        x[k] = w.x;
+        y[k] = w.y;
+        amax = fmaxf(amax, fmaxf(fabsf(w.x), fabsf(w.y)));
+      }
+      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
+      float sc;
+      const float up = block_power(amax, &sc);
+      if (m < L && c >= xc0[m] && b + f < b_end) {
+        const long long tix = xoff[m] + (c - xc0[m]);
+        if (in_bounds(tix, x_tiles, kbPackVOut) && in_bounds(j + 1, NC, kbPackVOut)) {
+          uint8_t* tile = X + (size_t)tix * part_bytes;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const float* w = i ? y : x;
+            uint4 h, l;
+            split2(up * w[0], up * w[1], &h.x, &l.x);
+            split2(up * w[2], up * w[3], &h.y, &l.y);
+            split2(up * w[4], up * w[5], &h.z, &l.z);
+            split2(up * w[6], up * w[7], &h.w, &l.w);
+            const uint32_t off = sw128(j + i, 16 * kq);
+            *(uint4*)(tile + off) = h;
+            *(uint4*)(tile + (off ^ 64u)) = l;
+          }
+          if (kq == 0) XS[(size_t)tix * half + (j >> 1)] = sc;
+        }
+      }
     }
     __syncthreads();
   }
@@ -196,34 +265,22 @@ __global__ void __launch_bounds__(256) pack_v_kernel(int L, int s, int Btot, int
 // The tensor-core GEMM
 // ---------------------------------------------------------------------------------------------
 
-// Loads 4 groups of 16 columns (64 values) of this warp's 32 tensor-memory lanes, one wait.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
-  uint32_t r[64];
-#pragma unroll
-  for (int g = 0; g < 4; ++g)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[16 * g + 0]), "=r"(r[16 * g + 1]), "=r"(r[16 * g + 2]), "=r"(r[16 * g + 3]),
-                   "=r"(r[16 * g + 4]), "=r"(r[16 * g + 5]), "=r"(r[16 * g + 6]), "=r"(r[16 * g + 7]),
-                   "=r"(r[16 * g + 8]), "=r"(r[16 * g + 9]), "=r"(r[16 * g + 10]), "=r"(r[16 * g + 11]),
-                   "=r"(r[16 * g + 12]), "=r"(r[16 * g + 13]), "=r"(r[16 * g + 14]), "=r"(r[16 * g + 15])
-                 : "r"(taddr + 16 * g));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int k = 0; k < 64; ++k) v[k] = __uint_as_float(r[k]);
-}
-
 template <bool FWD, bool BF>
 __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  constexpr int GA = kParts<BF> * A_PART;  // bytes of an A tile
   const int b_part = a.NC * 128;
-  const int stage_bytes = A_TILE + 2 * b_part;  // both split parts of A and of the data tile
-  constexpr int GA = kParts<BF> * A_PART;       // bytes of an A tile in global memory
-  const int gx = kParts<BF> * b_part;           // bytes of a data tile in global memory
+  const int gx = kParts<BF> * b_part;      // bytes of a data tile
+  const int stage_bytes = GA + gx;
   const int STAGES = a.stages;
-  // full: a stage's copies have landed; ready (3xTF32): its FP32 values are split into hi + lo
-  __shared__ __align__(8) uint64_t full[MAX_STAGES], ready[MAX_STAGES], empty[MAX_STAGES], seg_full[2], seg_empty[2],
-      done_bar;
+  __shared__ __align__(8) uint64_t full[MAX_STAGES], empty[MAX_STAGES], seg_full[2], seg_empty[2], done_bar;
+  // split-FP16: the chunks' scales, filled ahead of the products.  Slot reuse needs no barrier: when the
+  // producer fills chunk n, chunk n - STAGES has been multiplied, so the epilogue has released chunk
+  // n - STAGES - 2 and read the scales of the chunk before that.
+  __shared__ __align__(16) float scales[SCALE_SLOTS][128];
+  __shared__ __align__(8) uint64_t scale_full[SCALE_SLOTS];
+  static_assert(SCALE_SLOTS > MAX_STAGES + 2 && (SCALE_SLOTS & (SCALE_SLOTS - 1)) == 0, "scale ring");
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -231,13 +288,13 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&ready[s], EPI_WARPS);
       mbar_init(&empty[s], 1);
     }
     for (int k = 0; k < 2; ++k) {
       mbar_init(&seg_full[k], 1);
       mbar_init(&seg_empty[k], EPI_WARPS);
     }
+    for (int k = 0; k < SCALE_SLOTS; ++k) mbar_init(&scale_full[k], 1);
     mbar_init(&done_bar, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -248,135 +305,126 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
   const uint32_t tbase = tmem_base;
   volatile int* abort = &abort_flag;
   const int nC = (a.L + TK - 1) / TK;
+  const int w_begin = a.sched[blockIdx.x], w_end = a.sched[blockIdx.x + 1];
 
-  if (warp == 0) {
-    if (lane == 0) {
+  if (warp < 4) {
+    regs_dec<REGS_ISSUE>();
+    if (warp == 0) {
       // ---- producer: bulk copies of the A and data tiles of every chunk ----
-      int it = 0;
-      int last_use[MAX_STAGES] = {-1, -1, -1, -1};
-      for (int w = a.sched[blockIdx.x]; w < a.sched[blockIdx.x + 1] && !*abort; ++w) {
+      const bool one = elect_one();
+      int s = 0, ph = 1, n = 0;     // stage, parity its empty barrier is waited for, chunk
+      uint32_t used = 0, uph = 0;   // stages that were filled, and the parity of their last fill
+      for (int w = w_begin; w < w_end && !*abort; ++w) {
         const Item itm = a.items[w];
-        const uint8_t* Ab = a.A + (size_t)itm.atile * GA;
-        for (int c = itm.c0; c < itm.c1; ++c, ++it) {
-          const int s = it % STAGES, u = it / STAGES;
-          if (!mbar_wait(&empty[s], (u & 1) ^ 1, abort, a.wait_ns)) {
+        const long long x0 = FWD ? (long long)itm.m * nC : a.xoff[itm.m] - a.xc0[itm.m];
+        for (int c = itm.c0; c < itm.c1; ++c, ++n) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort, a.wait_ns))) {
             *abort = 1;
             break;
           }
-          uint8_t* st = smem + s * stage_bytes;
-          mbar_expect_tx(&full[s], (uint32_t)(GA + gx));
-          // a tile index outside its array is recorded and tile 0 copied instead (the pipeline
-          // still completes; the result is wrong and the record says why)
-          const long long at = itm.atile + (c - itm.c0);
-          const uint8_t* asrc = in_bounds(at, a.a_tiles, kbGemmA) ? Ab + (size_t)(c - itm.c0) * GA : a.A;
-          bulk_g2s(st, asrc, GA, &full[s]);
-          long long xt = FWD ? (long long)itm.m * nC + c : a.xoff[itm.m] + (c - a.xc0[itm.m]);
-          if (!in_bounds(xt, a.x_tiles, kbGemmX)) xt = 0;
-          bulk_g2s(st + A_TILE, a.X + (size_t)xt * gx, (uint32_t)gx, &full[s]);
-          last_use[s] = u;
+          if (one) {
+            // a tile index outside its array is recorded and tile 0 copied instead (the pipeline
+            // still completes; the result is wrong and the record says why)
+            const long long at = itm.atile + (c - itm.c0);
+            const uint8_t* asrc = in_bounds(at, a.a_tiles, kbGemmA) ? a.A + (size_t)at * GA : a.A;
+            long long xt = x0 + c;
+            if (!in_bounds(xt, a.x_tiles, kbGemmX)) xt = 0;
+            uint8_t* st = smem + s * stage_bytes;
+            if constexpr (!BF) {
+              const int slot = n & (SCALE_SLOTS - 1);
+              mbar_expect_tx(&scale_full[slot], (uint32_t)(2 * a.NC));
+              bulk_g2s(scales[slot], a.XS + (size_t)xt * (a.NC / 2), (uint32_t)(2 * a.NC), &scale_full[slot]);
+            }
+            mbar_expect_tx(&full[s], (uint32_t)(GA + gx));
+            bulk_g2s(st, asrc, GA, &full[s]);
+            bulk_g2s(st + GA, a.X + (size_t)xt * gx, (uint32_t)gx, &full[s]);
+          }
+          used |= 1u << s;
+          uph = (uph & ~(1u << s)) | ((uint32_t)(ph ^ 1) << s);
+          if (++s == STAGES) {
+            s = 0;
+            ph ^= 1;
+          }
         }
       }
       // drain: every issued copy must have landed before the CTA leaves
-      for (int s = 0; s < STAGES; ++s)
-        if (last_use[s] >= 0) mbar_wait(&full[s], last_use[s] & 1, nullptr, kDrainNs);
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
+      for (int k = 0; k < STAGES; ++k)
+        if ((used >> k) & 1u) mbar_wait(&full[k], (uph >> k) & 1u, nullptr, kDrainNs);
+      if constexpr (!BF)
+        for (int k = max(0, n - SCALE_SLOTS); k < n; ++k)
+          mbar_wait(&scale_full[k & (SCALE_SLOTS - 1)], (k / SCALE_SLOTS) & 1, nullptr, kDrainNs);
+    } else if (warp == 1) {
       // ---- MMA issuer: one tensor-memory segment per chunk, corrections first ----
-      const uint32_t idesc = BF ? idesc_bf16(TM, a.NC) : idesc_tf32(TM, a.NC);
-      int it = 0;
-      for (int w = a.sched[blockIdx.x]; w < a.sched[blockIdx.x + 1] && !*abort; ++w) {
-        const Item itm = a.items[w];
-        bool ok = true;
-        for (int c = itm.c0; c < itm.c1; ++c, ++it) {
-          const int s = it % STAGES, u = it / STAGES;
-          const int seg = it & 1, us = it >> 1;
-          if (!mbar_wait(&seg_empty[seg], (us & 1) ^ 1, abort, a.wait_ns) ||
-              !mbar_wait(BF ? &full[s] : &ready[s], u & 1, abort, a.wait_ns)) {
+      const uint32_t idesc = BF ? idesc_bf16(TM, a.NC) : idesc_f16(TM, a.NC);
+      const bool one = elect_one();
+      const uint32_t lo0 = (smem_u32(smem) >> 4) + kDescLow;
+      int s = 0, ph = 0, seg = 0, sph = 1;
+      for (int w = w_begin; w < w_end && !*abort; ++w) {
+        const int nc = a.items[w].c1 - a.items[w].c0;
+        for (int c = 0; c < nc; ++c) {
+          const bool here = mbar_wait(&seg_empty[seg], sph, abort, a.wait_ns) && mbar_wait(&full[s], ph, abort, a.wait_ns);
+          if (!__all_sync(0xffffffffu, here)) {
             *abort = 1;
-            ok = false;
             break;
           }
           fence_after();
-          const uint32_t dt = tbase + (uint32_t)(seg * 256);
-          const uint32_t sa = smem_u32(smem + s * stage_bytes);
-          const uint32_t sb = sa + A_TILE;
-          if constexpr (BF) {
-            // parts h, m at bytes 0 and 64 of part 0, l at byte 0 of part 1; K = 16 (32 bytes)
-            // per instruction.  Products from the smallest up: h*l, l*h, m*m, h*m, m*h, h*h.
-            const uint32_t oa[3] = {0u, 64u, (uint32_t)A_PART}, ob[3] = {0u, 64u, (uint32_t)b_part};
-            const int pa[6] = {0, 2, 1, 0, 1, 0}, pb[6] = {2, 0, 1, 1, 0, 0};
+          if (one) {
+            const uint32_t dt = tbase + (uint32_t)(seg * 256);
+            const uint32_t la = lo0 + (uint32_t)(s * (stage_bytes >> 4)), lb = la + (GA >> 4);
+            if constexpr (BF) {
+              // parts h, m at bytes 0 and 64 of part 0, l at byte 0 of part 1; K = 16 (32 bytes)
+              // per instruction.  Products from the smallest up: h*l, l*h, m*m, h*m, m*h, h*h.
+              const uint32_t oa[3] = {0u, 4u, (uint32_t)(A_PART >> 4)}, ob[3] = {0u, 4u, (uint32_t)(b_part >> 4)};
+              const int pa[6] = {0, 2, 1, 0, 1, 0}, pb[6] = {2, 0, 1, 1, 0, 0};
 #pragma unroll
-            for (int q = 0; q < 6; ++q)
+              for (int q = 0; q < 6; ++q)
 #pragma unroll
-              for (int kk = 0; kk < 2; ++kk)
-                mma_f16(dt, desc_sw128(sa + oa[pa[q]] + kk * 32), desc_sw128(sb + ob[pb[q]] + kk * 32), idesc,
-                         (q == 0 && kk == 0) ? 0u : 1u);
-          } else {
+                for (int kk = 0; kk < 2; ++kk)
+                  mma_f16_lo<false>(dt, la + oa[pa[q]] + 2 * kk, lb + ob[pb[q]] + 2 * kk, idesc, (q | kk) ? 1u : 0u);
+            } else {
+              // hi at byte 0, lo at byte 64 of a row: hi*lo, lo*hi, hi*hi
 #pragma unroll
-            for (int kk = 0; kk < TK / 8; ++kk) {
-              const uint32_t ko = kk * 32;
-              mma_tf32(dt, desc_sw128(sa + ko), desc_sw128(sb + b_part + ko), idesc, kk == 0 ? 0u : 1u);  // hi * lo
-              mma_tf32(dt, desc_sw128(sa + A_PART + ko), desc_sw128(sb + ko), idesc, 1u);                 // lo * hi
+              for (int q = 0; q < 3; ++q)
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk)
+                  mma_f16_lo<false>(dt, la + (q == 1 ? 4u : 0u) + 2 * kk, lb + (q == 0 ? 4u : 0u) + 2 * kk, idesc, (q | kk) ? 1u : 0u);
             }
-#pragma unroll
-            for (int kk = 0; kk < TK / 8; ++kk) {
-              const uint32_t ko = kk * 32;
-              mma_tf32(dt, desc_sw128(sa + ko), desc_sw128(sb + ko), idesc, 1u);                          // hi * hi
-            }
+            mma_commit(&empty[s]);
+            mma_commit(&seg_full[seg]);
           }
-          mma_commit(&empty[s]);
-          mma_commit(&seg_full[seg]);
+          __syncwarp();
+          if (++s == STAGES) {
+            s = 0;
+            ph ^= 1;
+          }
+          seg ^= 1;
+          if (seg == 0) sph ^= 1;
         }
-        if (!ok) break;
       }
-      mma_commit(&done_bar);
+      if (one) mma_commit(&done_bar);
+      __syncwarp();
       mbar_wait(&done_bar, 0, nullptr, kDrainNs);  // every issued MMA has completed
     }
   } else {
     // ---- epilogue: running sums of the segments, then phases and outputs ----
-    const int q = warp & 3;                // tensor-memory lane quarter this warp may access
-    const int h = (warp - 2) >> 2;         // column half: sign of m
+    regs_inc<REGS_EPILOGUE>();
+    const int q = warp & 3;            // tensor-memory lane quarter this warp may access
+    const int cg = (warp - 4) >> 2;    // of the NC / 16 groups of 16 columns: cg, cg + 4, cg + 8, cg + 12
     const int r = q * 32 + lane;
     const int L = a.L, Lp = L - 1, NT = 2 * L - 1, B = a.B, s = a.s;
     const int H = a.NC / 2;
-    const uint32_t tq = tbase + ((uint32_t)(q * 32) << 16) + (uint32_t)(h * H);
-    // 3xTF32: the epilogue warps also split each arrived stage's FP32 values into hi + lo, one
-    // chunk ahead of the chunk they sum, so that the split of chunk c + 1 overlaps the MMAs of c
-    int nchunks = 0, conv = 0;
-    if constexpr (!BF)
-      for (int w = a.sched[blockIdx.x]; w < a.sched[blockIdx.x + 1]; ++w) nchunks += a.items[w].c1 - a.items[w].c0;
-    const int et = threadIdx.x - 64, ent = 32 * EPI_WARPS;
-    auto convert_upto = [&](int last) -> bool {
-      for (; conv < nchunks && conv <= last; ++conv) {
-        const int sc = conv % STAGES, uc = conv / STAGES;
-        if (!mbar_wait(&full[sc], uc & 1, abort, a.wait_ns)) return false;
-        uint8_t* st = smem + sc * stage_bytes;
-        split_region_tf32(st, A_PART, A_PART, et, ent);
-        split_region_tf32(st + A_TILE, b_part, b_part, et, ent);
-        fence_proxy_async();  // the split parts are read by the tensor core (async proxy)
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ready[sc]);
-      }
-      return true;
-    };
-    int it = 0;
-    for (int w = a.sched[blockIdx.x]; w < a.sched[blockIdx.x + 1] && !*abort; ++w) {
+    const uint32_t tq = tbase + ((uint32_t)(q * 32) << 16);
+    int seg = 0, sph = 0, n = 0;
+    for (int w = w_begin; w < w_end && !*abort; ++w) {
       const Item itm = a.items[w];
-      float acc[128];
+      float acc[64];
 #pragma unroll
-      for (int k = 0; k < 128; ++k) acc[k] = 0.f;
+      for (int k = 0; k < 64; ++k) acc[k] = 0.f;
       bool ok = true;
-      for (int c = itm.c0; c < itm.c1; ++c, ++it) {
-        const int seg = it & 1, us = it >> 1;
-        if constexpr (!BF) {
-          if (!convert_upto(it + 1)) {
-            *abort = 1;
-            ok = false;
-            break;
-          }
-        }
-        if (!mbar_wait(&seg_full[seg], us & 1, abort, a.wait_ns)) {
+      for (int c = itm.c0; c < itm.c1; ++c, ++n) {
+        const int slot = n & (SCALE_SLOTS - 1);
+        if ((!BF && !mbar_wait(&scale_full[slot], (n / SCALE_SLOTS) & 1, abort, a.wait_ns)) ||
+            !mbar_wait(&seg_full[seg], sph, abort, a.wait_ns)) {
           *abort = 1;
           ok = false;
           break;
@@ -384,35 +432,62 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
         fence_after();
         const uint32_t ts = tq + (uint32_t)(seg * 256);
 #pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          if (64 * g < H) {
-            float v[64];
-            tmem_ld64(ts + 64 * g, v);
+        for (int g = 0; g < 4; g += 2) {
+          uint32_t v[32];
+          const int j = 16 * (4 * g + cg);  // the groups' first columns: j and j + 64
+          if (j < a.NC) tmem_ld16_nowait(ts + j, v);
+          if (j + 64 < a.NC) tmem_ld16_nowait(ts + j + 64, v + 16);
+          tmem_wait_ld();
+          if (g == 2) {  // the segment is read: free it before the last sums
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&seg_empty[seg]);
+          }
 #pragma unroll
-            for (int k = 0; k < 64; ++k) acc[64 * g + k] += v[k];
+          for (int i = 0; i < 2; ++i) {
+            if (j + 64 * i >= a.NC) continue;
+            if constexpr (BF) {
+#pragma unroll
+              for (int k = 0; k < 16; ++k) acc[16 * (g + i) + k] += __uint_as_float(v[16 * i + k]);
+            } else {
+              const float4 s0 = *(const float4*)&scales[slot][(j + 64 * i) / 2], s1 = *(const float4*)&scales[slot][(j + 64 * i) / 2 + 4];
+              const float sc[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+#pragma unroll
+              for (int k = 0; k < 16; ++k)
+                acc[16 * (g + i) + k] = fmaf(__uint_as_float(v[16 * i + k]), sc[k >> 1], acc[16 * (g + i) + k]);
+            }
           }
         }
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&seg_empty[seg]);
+        seg ^= 1;
+        if (seg == 0) sph ^= 1;
       }
       if (!ok) break;
       const int m = itm.m;
-      if (h == 1 && m == 0) continue;
       const int rowv = itm.i * TM + r;  // m' (inverse) or l (forward)
       const bool valid = FWD ? (rowv <= Lp && rowv >= m) : (rowv <= Lp);
       if (!valid) continue;
-      const int mm = h ? -m : m;
-      const float2 pz = FWD ? ipow_signed(s, mm + s) : ipow_signed(s, -(mm + s));
-      const float rs = (h && (rowv & 1)) ? -1.f : 1.f;  // (-1)^{m'} (inverse) or (-1)^l (forward) for -m
 #pragma unroll
-      for (int b = 0; b < 64; ++b) {
-        if (b >= B) break;
-        const float xr = rs * acc[2 * b], xi = rs * acc[2 * b + 1];
-        const float2 F = make_float2(pz.x * xr - pz.y * xi, pz.x * xi + pz.y * xr);
-        const long long o = FWD ? (long long)b * L * L + (long long)rowv * rowv + rowv + mm
-                                : ((long long)b * NT + (mm + Lp)) * L + rowv;  // half row m' >= 0
-        if (in_bounds(o, a.out_n, kbGemmOut)) a.out[o] = F;
+      for (int g = 0; g < 4; ++g) {
+        const int j = 16 * (4 * g + cg);
+        if (j >= a.NC) break;
+        const int h = j >= H ? 1 : 0, b0 = (j - h * H) >> 1;  // the sign of m and the first of the group's 8 fields
+        if (h == 1 && m == 0) break;
+        const int mm = h ? -m : m;
+        // the phase, (-1)^{m'} (inverse) or (-1)^l (forward) for -m, and split-FP16's 2^14 / 2^10
+        const float2 pu = FWD ? ipow_signed(s, mm + s) : ipow_signed(s, -(mm + s));
+        const float rs = ((h && (rowv & 1)) ? -1.f : 1.f) * (BF ? 1.f : 16384.f / kAScale);
+        const float2 pz = make_float2(rs * pu.x, rs * pu.y);
+        const bool flat = FWD && !a.rows;
+        const long long o0 = flat ? (long long)rowv * rowv + rowv + mm : (long long)(mm + Lp) * L + rowv;
+        const long long ob = flat ? (long long)L * L : (long long)NT * L;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int b = b0 + k;
+          if (b >= B) break;
+          const float xr = acc[16 * g + 2 * k], xi = acc[16 * g + 2 * k + 1];
+          const long long o = o0 + b * ob;
+          if (in_bounds(o, a.out_n, kbGemmOut)) a.out[o] = make_float2(pz.x * xr - pz.y * xi, pz.x * xi + pz.y * xr);
+        }
       }
     }
   }
@@ -423,6 +498,32 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
   if (warp == 1) tmem_dealloc(tbase, 512);
 }
 
+// Forward output: half rows P [b][m + Lp][l], l >= |m|, -> flm [b][l^2 + l + m], by 32 x 32 blocks through
+// shared memory (both sides in runs of 256 bytes).  blockIdx.x: block of l, y: block of m + Lp, z: field.
+__global__ void __launch_bounds__(256) rows_to_flm_kernel(int L, const float2* __restrict__ P, float2* __restrict__ flm,
+                                                          long long p_n, long long out_n) {
+  __shared__ float2 sv[32][33];
+  const int Lp = L - 1, N = 2 * L - 1, l0 = 32 * blockIdx.x, r0 = 32 * blockIdx.y;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  // no entry of the block has l >= |m|
+  const int l1 = min(l0 + 31, Lp), m_lo = r0 - Lp, m_hi = min(r0 + 31, N - 1) - Lp;
+  if (m_lo > l1 || m_hi < -l1) return;
+  const long long pb = (long long)blockIdx.z * N * L, fb = (long long)blockIdx.z * L * L;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int r = r0 + ty + 8 * k, l = l0 + tx, m = r - Lp;
+    if (r < N && l < L && l >= m && l >= -m && in_bounds(pb + (long long)r * L + l, p_n, kbGemmOut))
+      sv[ty + 8 * k][tx] = P[pb + (long long)r * L + l];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int l = l0 + ty + 8 * k, r = r0 + tx, m = r - Lp;
+    const long long o = fb + (long long)l * l + l + m;
+    if (r < N && l < L && l >= m && l >= -m && in_bounds(o, out_n, kbGemmOut)) flm[o] = sv[tx][ty + 8 * k];
+  }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -431,7 +532,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
 
 struct TcPlan {
   int L = 0, s = 0, B = 0, NC = 0, nC = 0, nI = 0;
-  bool bf16 = false;  // split-BF16 (3 parts, 6 products) instead of 3xTF32
+  bool bf16 = false;  // split-BF16 (3 parts, 6 products) instead of split-FP16
   TcConfig cfg;
   int Bs = 0, nS = 0;        // fields per slice (one GEMM launch each) and slices
   size_t xslice = 0;         // bytes of one slice's data tiles
@@ -453,6 +554,8 @@ struct TcPlan {
   long long* ibase = nullptr;  // [m * nI + i]: tile index of chunk kc of inverse item (m, i) is ibase + kc
   uint8_t* X = nullptr;        // data tiles, nS slices of xslice bytes
   size_t xbytes = 0;
+  float* XS = nullptr;         // split-FP16: scales of the data tiles, nS slices of [tile][NC / 2]
+  size_t xsbytes = 0;
   long long* xoff = nullptr;
   int* xc0 = nullptr;
   size_t bytes = 0;
@@ -474,12 +577,12 @@ static cudaError_t gemm_attrs(K kernel, int bytes) {
 }
 
 static int nc_of(int Bs) { return 2 * (((2 * Bs + 15) / 16) * 16); }
-static size_t stage_bytes_of(int NC) { return (size_t)A_TILE + 2 * (size_t)NC * 128; }
+static size_t stage_bytes_of(int NC, bool bf16) { return (bf16 ? 2 : 1) * ((size_t)A_PART + (size_t)NC * 128); }
 
 bool tc_config_fits(const TcPlan* p, const TcConfig& c) {
   if (c.slice < 1 || c.slice > 64 || c.stages < 2 || c.stages > MAX_STAGES) return false;
   const int Bs = std::min(c.slice, p->B);
-  return (size_t)c.stages * stage_bytes_of(nc_of(Bs)) + 1024 <= (size_t)p->smem_max;
+  return (size_t)c.stages * stage_bytes_of(nc_of(Bs), p->bf16) + 1024 <= (size_t)p->smem_max;
 }
 
 // Assign the items, in list order, each to the CTA that becomes free first, with a cost of its
@@ -524,6 +627,16 @@ cudaError_t tc_configure(TcPlan* p, const TcConfig& c) {
     if ((e = tc_alloc((void**)&p->X, xslice * nS, &p->bytes)) != cudaSuccess) return e;
     p->xbytes = xslice * nS;
   }
+  const size_t xsbytes = p->bf16 ? 0 : (xslice / 128 / 2) * nS * sizeof(float);  // a float a row pair
+  if (xsbytes && (xsbytes != p->xsbytes || !p->XS)) {
+    if (p->XS) {
+      cudaFree(p->XS);
+      p->bytes -= p->xsbytes;
+      p->XS = nullptr;
+    }
+    if ((e = tc_alloc((void**)&p->XS, xsbytes, &p->bytes)) != cudaSuccess) return e;
+    p->xsbytes = xsbytes;
+  }
   p->Bs = Bs;
   p->nS = nS;
   p->NC = NC;
@@ -545,7 +658,7 @@ cudaError_t tc_configure(TcPlan* p, const TcConfig& c) {
   else std::stable_sort(fwd.begin(), fwd.end(), longest_first);
   if ((e = schedule(inv, p->grid_inv, p->items_inv, p->sched_inv)) != cudaSuccess) return e;
   if ((e = schedule(fwd, p->grid_fwd, p->items_fwd, p->sched_fwd)) != cudaSuccess) return e;
-  p->smem = (size_t)c.stages * stage_bytes_of(NC) + 1024;
+  p->smem = (size_t)c.stages * stage_bytes_of(NC, p->bf16) + 1024;
   p->cfg = c;
   return cudaSuccess;
 }
@@ -602,7 +715,7 @@ cudaError_t tc_setup(TcPlan** out, int L, int s, int B, int bf16, int device) {
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)) != cudaSuccess) goto fail;
     if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device)) != cudaSuccess) goto fail;
     p->grid = sms;
-    p->smem_max = optin - 2048;  // the kernel's static shared memory and alignment slack
+    p->smem_max = optin - 8192;  // the kernel's static shared memory and alignment slack
   }
   // the inverse leaves one SM to the recursion that writes the forward's operands meanwhile
   p->grid_inv = std::max(1, std::min(p->grid - 1, (int)inv.size()));
@@ -644,7 +757,11 @@ cudaError_t tc_setup(TcPlan** out, int L, int s, int B, int bf16, int device) {
       if ((e = prefer_shared(pack_v_kernel<false>)) != cudaSuccess) goto fail;
     }
   }
-  if ((e = tc_configure(p, TcConfig())) != cudaSuccess) goto fail;
+  {
+    TcConfig c;  // as many stages as fit
+    while (c.stages > 2 && !tc_config_fits(p, c)) --c.stages;
+    if ((e = tc_configure(p, c)) != cudaSuccess) goto fail;
+  }
   *out = p;
   return cudaSuccess;
 fail:
@@ -654,7 +771,7 @@ fail:
 
 void tc_destroy(TcPlan* p) {
   if (!p) return;
-  void* ptrs[] = {p->items_inv, p->items_fwd, p->sched_inv, p->sched_fwd, p->A, p->A_inv, p->abase, p->ibase, p->X, p->xoff, p->xc0};
+  void* ptrs[] = {p->items_inv, p->items_fwd, p->sched_inv, p->sched_fwd, p->A, p->A_inv, p->abase, p->ibase, p->X, p->XS, p->xoff, p->xc0};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete p;
@@ -702,13 +819,13 @@ cudaError_t tc_pack_a(TcPlan* p, int forward, const double* table, const float* 
 }
 
 cudaError_t tc_pack_data(TcPlan* p, const void* src, cudaStream_t st, int* launches) {
-  const dim3 g(p->nC, (p->L + 15) / 16, p->nS);
+  const dim3 g(p->nC, (p->L + 15) / 16, (unsigned)(p->nS * pack_v_groups(p->NC)));
   if (p->bf16)
     pack_v_kernel<true><<<g, 256, 0, st>>>(p->L, p->s, p->B, p->Bs, p->xslice, p->NC, p->xc0, p->xoff,
-                                           (const float2*)src, p->X);
+                                           (const float2*)src, p->X, p->XS);
   else
     pack_v_kernel<false><<<g, 256, 0, st>>>(p->L, p->s, p->B, p->Bs, p->xslice, p->NC, p->xc0, p->xoff,
-                                            (const float2*)src, p->X);
+                                            (const float2*)src, p->X, p->XS);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -722,11 +839,19 @@ TileOut tc_forward_tiles(const TcPlan* p) {
   o.Bs = p->Bs;
   o.xslice = p->xslice;
   o.xbytes = p->xbytes;
+  o.scale = p->XS;
   return o;
 }
 
-cudaError_t tc_gemm(TcPlan* p, int forward, void* out, const void* ph, int* status, long long wait_ns, cudaStream_t st,
-                    int* launches) {
+// The forward's rows l of one order lie 2l apart in flm: written from the GEMM, every 8-byte value is a
+// sector of its own, which meets its neighbours' (other orders, other CTAs) in L2 only while the output
+// is small.  From 2^22 coefficients (32 MB) on, the GEMM writes half rows, contiguous in l, into the
+// workspace and rows_to_flm_kernel transposes them (GB300, B = 64: the GEMM at L = 1024 1.68 ms direct, 0.69 by rows and 0.17 for the transposition).
+constexpr long long kRowsFrom = 1ll << 22;
+
+cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, const void* ph, int* status, long long wait_ns,
+                    cudaStream_t st, int* launches) {
+  const bool via_rows = forward && rows && (long long)p->B * p->L * p->L >= kRowsFrom;
   // one launch per slice of fields; every slice reads the same A tiles
   for (int sl = 0; sl < p->nS; ++sl) {
     TcArgs a;
@@ -739,11 +864,13 @@ cudaError_t tc_gemm(TcPlan* p, int forward, void* out, const void* ph, int* stat
     a.items = forward ? p->items_fwd : p->items_inv;
     a.A = forward ? p->A : p->A_inv;
     a.X = p->X + (size_t)sl * p->xslice;
+    a.XS = p->XS ? p->XS + (size_t)sl * (p->xslice / 256) : nullptr;
     a.xoff = p->xoff;
     a.xc0 = p->xc0;
     a.ph = (const float2*)ph;
-    const size_t per_field = forward ? (size_t)p->L * p->L : (size_t)(2 * p->L - 1) * p->L;
-    a.out = (float2*)out + (size_t)sl * p->Bs * per_field;
+    const size_t per_field = (forward && !via_rows) ? (size_t)p->L * p->L : (size_t)(2 * p->L - 1) * p->L;
+    a.out = (float2*)(via_rows ? rows : out) + (size_t)sl * p->Bs * per_field;
+    a.rows = via_rows;
     a.status = status;
     a.wait_ns = wait_ns;
     a.a_tiles = forward ? p->tiles_A : p->tiles_inv;
@@ -761,6 +888,14 @@ cudaError_t tc_gemm(TcPlan* p, int forward, void* out, const void* ph, int* stat
     *launches += 1;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+  }
+  if (via_rows) {
+    const int N = 2 * p->L - 1;
+    // fields in z, at most 65535 a launch (the library's largest batch)
+    rows_to_flm_kernel<<<dim3((p->L + 31) / 32, (N + 31) / 32, p->B), 256, 0, st>>>(
+        p->L, (const float2*)rows, (float2*)out, (long long)p->B * N * p->L, (long long)p->B * p->L * p->L);
+    *launches += 1;
+    return cudaGetLastError();
   }
   return cudaSuccess;
 }

@@ -69,27 +69,13 @@ struct ColumnParams {
   long long extent;        // entries of the table, or tiles of A (index checks)
 };
 
-// Byte offset of (row, K) in an A tile: of the FP32 value (3xTF32 tiles, one part), or of the first
-// BF16 part (split-BF16 tiles; the second part lies at offset ^ 64, the third one part further on).
-template <bool BF>
-__device__ __forceinline__ uint32_t a_off(int row, int k) {
-  return tc::sw128(row, (BF ? 2 : 4) * k);
-}
-// Writes x into tile `tile` at the offset made by a_off: the FP32 value (the contraction splits it
-// into hi + lo on arrival), or its three BF16 parts.
+// Byte offset of (row, K) in an A tile's first part.
+__device__ __forceinline__ uint32_t a_off(int row, int k) { return tc::sw128(row, 2 * k); }
+// Writes x, split, into tile `tile` at the offset made by a_off.
 template <bool BF>
 __device__ __forceinline__ void put_a_at(uint8_t* A, long long tile, long long ntiles, int site, uint32_t off, float x) {
   if (!in_bounds(tile, ntiles, site)) return;
-  uint8_t* t = A + (size_t)tile * (tc::kParts<BF> * tc::kAPart);
-  if constexpr (BF) {
-    uint16_t h, m, l;
-    tc::split_bf16x3(x, &h, &m, &l);
-    *(uint16_t*)(t + off) = h;
-    *(uint16_t*)(t + (off ^ 64u)) = m;
-    *(uint16_t*)(t + tc::kAPart + off) = l;
-  } else {
-    *(float*)(t + off) = x;
-  }
+  tc::put_parts<BF>(A + (size_t)tile * (tc::kParts<BF> * tc::kAPart), tc::kAPart, off, x);
 }
 
 __device__ __forceinline__ double flip_sign(double v, bool neg) {
@@ -301,7 +287,7 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
     const int il = l >> 7;
     const long long ilpre = 2ll * il * (il + 1);
     const long long tadd = ilpre + (m0 >> 5);
-    const uint32_t off = a_off<BF>(l & 127, lane);
+    const uint32_t off = a_off(l & 127, lane);
     const size_t lrow = (size_t)l * (l + 1) / 2;  // row l of the degree-major tables
     const double md = (double)m;
     // U_l[m] of this lane's column and the tile base of its row M = m (the transposed writes)
@@ -438,7 +424,7 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
     const bool wr = inl && l >= P.as;     // U_l vanishes below |s|: those entries stay zero
     const float um = wr ? __ldg(&P.ufT[tri_idx(m, l, L)]) : 0.f;
     const long long* ib_m = P.ibase + (size_t)m * P.nI;
-    const uint32_t off_m = a_off<BF>(m & 127, lane);  // (row m, K = l) in the tiles A_{m'}[m][.]
+    const uint32_t off_m = a_off(m & 127, lane);  // (row m, K = l) in the tiles A_{m'}[m][.]
     uint8_t* const A = P.A;
     double cur = 0.0, prev = 0.0;
     int E = 0;
@@ -480,7 +466,7 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
       if (inl && mp <= l) {
         if (wr) {
           const float x = f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur);
-          put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off<BF>(mp & 127, lane), (cu * cp) * x);
+          put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off(mp & 127, lane), (cu * cp) * x);
           if (mp > m) put_a_at<BF>(A, ct + kc, P.ntiles, kbLaneTile, off_m, (um * cp) * (((mp - m) & 1) ? -x : x));
         }
         if (mp > m) {
@@ -514,7 +500,7 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
       if (inl) {
         if (wr) {
           const float x = f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur);
-          put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off<BF>(mp & 127, lane), (cu * cp) * x);
+          put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off(mp & 127, lane), (cu * cp) * x);
           put_a_at<BF>(A, ct + kc, P.ntiles, kbLaneTile, off_m, (um * cp) * (((mp - m) & 1) ? -x : x));
         }
         double c;
@@ -541,7 +527,7 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
     // ---- the last row m' = m, if the steady loop reached it ----
     if (m < lo) {
       if ((m & 127) == 127) tb = __ldg(&ib_m[m >> 7]) + kc;
-      if (wr) put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off<BF>(m & 127, lane), (cu * cp) * f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur));
+      if (wr) put_a_at<BF>(A, tb, P.ntiles, kbLaneTile, a_off(m & 127, lane), (cu * cp) * f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur));
     }
   }
 }

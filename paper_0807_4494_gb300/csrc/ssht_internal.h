@@ -117,7 +117,7 @@ template <typename T> cudaError_t pair_gather(int L, int B, const void* in, void
 cudaError_t real_setup();
 
 // ---------------------------------------------------------------------------
-// Tensor-core contractions (contract_tc.cu), 3xTF32 or split-BF16
+// Tensor-core contractions (contract_tc.cu), split-FP16 (SSHT_TF32X3) or split-BF16
 // ---------------------------------------------------------------------------
 struct TcPlan;
 // The contraction's tunable shape: fields per GEMM launch (the N tile: 2 x 2 x slice real columns,
@@ -125,11 +125,11 @@ struct TcPlan;
 // work items (inverse: 0 grouped by m, 1 longest first; forward: 0 longest first, 1 grouped by m).
 struct TcConfig {
   int slice = 64;
-  int stages = 2;
+  int stages = 4;  // a new plan takes fewer where four do not fit
   int inv_order = 0;
   int fwd_order = 0;
 };
-// bf16 = 0: 3xTF32 split products; bf16 = 1: split-BF16 (three parts, six products).  Any batch:
+// bf16 = 0: split-FP16 (two parts, three products); bf16 = 1: split-BF16 (three parts, six products).  Any batch:
 // the fields run in slices of at most 64.
 cudaError_t tc_setup(TcPlan** out, int L, int s, int B, int bf16, int device);
 bool tc_config_fits(const TcPlan* p, const TcConfig& c);  // within the device's shared memory
@@ -144,18 +144,20 @@ cudaError_t tc_pack_a(TcPlan* p, int forward, const double* table, const float* 
 // data tiles come from their theta passes (TileOut).
 cudaError_t tc_pack_data(TcPlan* p, const void* src, cudaStream_t st, int* launches);
 // The contraction: forward = 0 writes the half rows F (float2 [B][N][L], m' >= 0) of the inverse;
-// forward = 1 writes flm (float2 [B][L*L]).  Timeouts set bit 2 of *status.
-cudaError_t tc_gemm(TcPlan* p, int forward, void* out, const void* ph, int* status, long long wait_ns, cudaStream_t st,
-                    int* launches);
+// forward = 1 writes flm (float2 [B][L*L]), large outputs by way of the workspace rows (float2 [B][N][L];
+// null: always directly).  Timeouts set bit 2 of *status.
+cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, const void* ph, int* status, long long wait_ns,
+                    cudaStream_t st, int* launches);
 // Where the forward theta pass writes the projection's data tiles directly (in place of H and
 // tc_pack_data): the tile array, its column count NC, chunks per m nC, and the split form
-// (mode 1: 3xTF32, 2: split-BF16; 0: no tiles, H is written).
+// (mode 1: split-FP16, 2: split-BF16; 0: no tiles, H is written).
 struct TileOut {
   uint8_t* X = nullptr;
   int NC = 0, nC = 0, mode = 0;
   int Bs = 64;        // fields per slice; slice z of the fields has its tiles at X + z * xslice
   size_t xslice = 0;
   size_t xbytes = 0;  // the whole tile array (index checks)
+  float* scale = nullptr;  // split-FP16: [tile][NC / 2], what undoes the power of two of a row pair
 };
 TileOut tc_forward_tiles(const TcPlan* p);
 // Where the recursion writes the A operand itself: the forward tile array and its per-m tile

@@ -5,18 +5,17 @@
 #include <cstdint>
 
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 namespace ssht {
 namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// A-operand tiles of the contraction: 128 rows x 32 K values.  In shared memory two split parts of
-// 16 KB each; in global memory one part of FP32 values for the 3xTF32 form (the contraction splits
-// them on arrival) and both parts for the split-BF16 form.
+// A-operand tiles of the contraction: 128 rows x 32 K values, 128 bytes a row and part: one part for
+// the split-FP16 form (32 hi parts, 32 lo parts), two for the split-BF16 form ([h | m] and [l | 0]).
 constexpr int kTileRows = 128, kTileK = 32;
 constexpr int kAPart = kTileRows * kTileK * 4;
-constexpr int kATile = 2 * kAPart;
 
 // Byte offset of element (row, kbyte) in a K-major tile with 128-byte rows in the SWIZZLE_128B
 // layout: 8-row x 128-byte atoms stacked along rows, the 16-byte chunk c of row r stored at
@@ -37,14 +36,14 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   return d;
 }
 
-// Instruction descriptor: D = F32, A = B = TF32, both K-major, shape M x N.
-__device__ __forceinline__ uint32_t idesc_tf32(int m, int n) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
 // Instruction descriptor: D = F32, A = B = BF16 (kind::f16), both K-major, shape M x N.
 __device__ __forceinline__ uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
+// Instruction descriptor: D = F32, A = B = FP16 (kind::f16), both K-major, shape M x N.
+__device__ __forceinline__ uint32_t idesc_f16(int m, int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 // Orders this thread's shared-memory writes (generic proxy) before later reads of the tensor core
@@ -68,14 +67,24 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   return t;
 }
 
+// The same without suspending the thread (try_wait may hold it until the phase completes).
+__device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+
 // Bounded wait for the phase of the given parity: false once limit_ns of device time has passed
-// (checked after every poll) or, if abort is not null, once *abort is set (every 256 polls).
+// (checked after every poll) or, if abort is not null, once *abort is set (every 256 polls).  Limits below
+// 10 us poll without suspending, so that a wait cannot outlast them inside one try_wait.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort, long long limit_ns) {
   const uint32_t b = smem_u32(bar);
-  if (mbar_test(b, parity)) return true;
+  const bool brief = limit_ns < 10000;
+  if (brief ? mbar_poll(b, parity) : mbar_test(b, parity)) return true;
   const unsigned long long t0 = globaltimer();
   for (unsigned i = 1;; ++i) {
-    if (mbar_test(b, parity)) return true;
+    if (brief ? mbar_poll(b, parity) : mbar_test(b, parity)) return true;
     if ((i & 255u) == 0u && abort && *abort) return false;
     if ((long long)(globaltimer() - t0) > limit_ns) return false;
   }
@@ -144,21 +153,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::tf32, issued by one thread.
-__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-               " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-               ::"r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum));
-}
-
-// D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 with FP16 or BF16 operands, as idesc says (K = 16 per
-// instruction).
-__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-               " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-               ::"r"(dtmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum));
-}
-
 // The forms for a pair of CTAs of a cluster (cta_group::2): both allocate and free together, the
 // leader (rank 0) issues products of 256 rows -- 128 a CTA, each CTA holding its rows of A, half of the
 // rows of B and its rows of D -- and their completion arrives at the same barrier of both CTAs.
@@ -207,27 +201,37 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-// 32 lanes x 32 bits, 16 consecutive columns per thread.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-               : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
+// 32 lanes x 32 bits, 16 consecutive columns per thread; tmem_wait_ld before the values are used.
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The power of two that brings a block's largest magnitude amax to [2^14, 2^15), and the scale that
+// undoes it, with a 2^-14 of the other operand's range folded in.  Magnitudes below 2^-98 share the
+// smallest one's power; an infinity or a NaN stays what it is in the parts.
+__device__ __forceinline__ float block_power(float amax, float* scale) {
+  const int e = min(max((int)(__float_as_uint(amax) >> 23), 29), 254);
+  *scale = __uint_as_float((uint32_t)(e - 28) << 23);
+  return __uint_as_float((uint32_t)(268 - e) << 23);
 }
 
-// x = hi + lo with hi rounded to TF32 (10 explicit mantissa bits, round to nearest) and lo the
-// remainder rounded the same way: the pair carries about 22 significant bits of x.
-__device__ __forceinline__ float tf32_round(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+// x = hi + lo with both parts FP16, rounded to nearest (the remainder x - hi is exact in FP32): 22 to
+// 24 significant bits while lo is a normal number.  Two values at a time.
+__device__ __forceinline__ void split2(float a, float b, uint32_t* hi, uint32_t* lo) {
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+  *hi = *reinterpret_cast<const uint32_t*>(&h);
+  *lo = *reinterpret_cast<const uint32_t*>(&l);
 }
-__device__ __forceinline__ void split_tf32(float x, float* hi, float* lo) {
-  *hi = tf32_round(x);
-  *lo = tf32_round(x - *hi);
-}
+
+// The A operand's power of two: |U Delta| <= sqrt(4095 / 4 pi) < 18.1 up to L = 2048.
+constexpr float kAScale = 1024.f;
 
 // x = h + m + l with each part rounded to BF16 (8 significant bits, round to nearest): the three
 // parts carry about 24 significant bits of x; each remainder is exact in FP32.
@@ -242,40 +246,62 @@ __device__ __forceinline__ void split_bf16x3(float x, uint16_t* h, uint16_t* m, 
   *l = __bfloat16_as_ushort(c);
 }
 
-// Writes element (row, k), k < 32, of a K-chunk operand tile as it is stored in global memory
-// (128-byte swizzled rows).  TF32 form: one part, the FP32 value itself (split into hi + lo by
-// the contraction when the tile arrives in shared memory).  BF16 split: part 0 = [h | m] (2-byte
-// elements, k at byte 2k and 64 + 2k), part 1 = [l | 0], each part part_bytes long.
+// Parts of an operand tile: 1 for split-FP16, 2 for split-BF16.
+template <bool BF> constexpr int kParts = BF ? 2 : 1;
+
+// Writes an A operand's x at the byte offset off = sw128(row, 2k) of its first part.  Split-FP16: hi, and
+// lo 64 bytes further on in the row (the swizzle flips bit 6 with it), of x times kAScale.  Split-BF16:
+// h and m likewise, l in the second part (whose other half stays zero).
 template <bool BF>
-__device__ __forceinline__ void put_split(uint8_t* tile, int part_bytes, int row, int k, float x) {
+__device__ __forceinline__ void put_parts(uint8_t* tile, int part_bytes, uint32_t off, float x) {
   if constexpr (BF) {
     uint16_t h, m, l;
     split_bf16x3(x, &h, &m, &l);
-    *(uint16_t*)(tile + sw128(row, 2 * k)) = h;
-    *(uint16_t*)(tile + sw128(row, 64 + 2 * k)) = m;
-    *(uint16_t*)(tile + part_bytes + sw128(row, 2 * k)) = l;
-    *(uint16_t*)(tile + part_bytes + sw128(row, 64 + 2 * k)) = 0;
+    *(uint16_t*)(tile + off) = h;
+    *(uint16_t*)(tile + (off ^ 64u)) = m;
+    *(uint16_t*)(tile + part_bytes + off) = l;
   } else {
     (void)part_bytes;
-    *(float*)(tile + sw128(row, 4 * k)) = x;
+    const float y = kAScale * x;
+    const __half h = __float2half_rn(y), l = __float2half_rn(y - __half2float(h));
+    *(__half*)(tile + off) = h;
+    *(__half*)(tile + (off ^ 64u)) = l;
   }
 }
 
-// Global parts of an operand tile: 1 for the TF32 form, 2 for split-BF16.
-template <bool BF> constexpr int kParts = BF ? 2 : 1;
+// block_power of the largest magnitude over the warp (amax >= 0, or a NaN).
+__device__ __forceinline__ float warp_power(float amax, float* scale) {
+  return block_power(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(amax))), scale);
+}
 
-// Splits, in shared memory, the FP32 values of an arrived 3xTF32 operand region into hi (in place)
-// and lo (lo_offset bytes further on), 16 bytes a step; the layout's swizzle permutes whole
-// 16-byte chunks, so the split goes position by position.  Threads t of nt take steps t, t + nt, ...
-__device__ __forceinline__ void split_region_tf32(uint8_t* region, int bytes, int lo_offset, int t, int nt) {
-  for (int o = 16 * t; o < bytes; o += 16 * nt) {
-    float4 x = *(const float4*)(region + o), h, l;
-    split_tf32(x.x, &h.x, &l.x);
-    split_tf32(x.y, &h.y, &l.y);
-    split_tf32(x.z, &h.z, &l.z);
-    split_tf32(x.w, &h.w, &l.w);
-    *(float4*)(region + o) = h;
-    *(float4*)(region + lo_offset + o) = l;
+// Writes two rows (j, j + 1: a field's real and imaginary part) of a data tile if `store` (warp-uniform), the
+// warp's lanes holding K = lane of both (x, y).  Split-FP16: of x and y times the block's power of two `up`;
+// neighbouring lanes exchange a value, so that each lane splits and stores two K of one row (4-byte stores).
+// Split-BF16: three 2-byte parts a value and the zero half.
+template <bool BF>
+__device__ __forceinline__ void put_rows2(uint8_t* tile, int part_bytes, int j, int lane, float x, float y, float up, bool store) {
+  if constexpr (BF) {
+    if (!store) return;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      uint16_t h, m, l;
+      split_bf16x3(i ? y : x, &h, &m, &l);
+      const uint32_t off = sw128(j + i, 2 * lane);
+      *(uint16_t*)(tile + off) = h;
+      *(uint16_t*)(tile + (off ^ 64u)) = m;
+      *(uint16_t*)(tile + part_bytes + off) = l;
+      *(uint16_t*)(tile + part_bytes + (off ^ 64u)) = 0;
+    }
+  } else {
+    const bool odd = lane & 1;
+    const float other = __shfl_xor_sync(0xffffffffu, odd ? x : y, 1);
+    uint32_t h, l;
+    split2(up * (odd ? other : x), up * (odd ? y : other), &h, &l);
+    const uint32_t off = sw128(j + (lane & 1), 4 * (lane >> 1));
+    if (store) {
+      *(uint32_t*)(tile + off) = h;
+      *(uint32_t*)(tile + (off ^ 64u)) = l;
+    }
   }
 }
 

@@ -48,8 +48,6 @@
 #include "bounds.cuh"
 #include "tc_common.cuh"
 
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -121,23 +119,6 @@ Operand operand(void* base, long long units, int chunks) {
   o.units = units;
   o.chunks = chunks;
   return o;
-}
-
-// The power of two that brings a block's largest magnitude amax to [2^14, 2^15), and the scale that
-// undoes it, with the 2^-14 of the matrices' own range folded in.  Magnitudes below 2^-98 share
-// the smallest one's power; an infinity or a NaN stays what it is in the parts.
-__device__ __forceinline__ float block_power(float amax, float* scale) {
-  const int e = min(max((int)(__float_as_uint(amax) >> 23), 29), 254);
-  *scale = __uint_as_float((uint32_t)(e - 28) << 23);
-  return __uint_as_float((uint32_t)(268 - e) << 23);
-}
-
-__device__ __forceinline__ void split2(float a, float b, uint32_t* hi, uint32_t* lo) {
-  const __half2 h = __floats2half2_rn(a, b);
-  const float2 f = __half22float2(h);
-  const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
-  *hi = *reinterpret_cast<const uint32_t*>(&h);
-  *lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
 // Scales, splits and stores the 64 K values x[0..63] of 32 rows, one a lane (K block kb): each chunk's
@@ -354,20 +335,6 @@ template <int MODE> __device__ __forceinline__ int block_chunks(const Shape& sh,
   return left >= 2 ? 2 : 1;
 }
 
-// Instruction descriptor: D = F32, A = B = FP16 (kind::f16), both K-major, shape M x N.
-__device__ __forceinline__ uint32_t idesc_f16(int m, int n) {
-  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
 // The 64 accumulator columns of epilogue warp group cg, as four groups g of 16: theta inverse and phi
 // forward take half a unit each (64 K of the next operand's rows); phi inverse and theta forward take
 // 16 rows of each half of both units, so that a thread has all four terms of its outputs.
@@ -377,33 +344,51 @@ __device__ __forceinline__ int group_col(int cg, int g) {
   return 64 * g + 16 * cg;
 }
 
-// Theta forward's stores of a thread's row m' into the data tiles of 16 orders |m| = am0, am0 + 2, ..
-// (acc: H_{+m} re, im, H_{-m} re, im, 16 each).
+// Theta forward's stores of the rows m' of a warp's lanes (one 32-K chunk of the projection) into the data
+// tiles of 16 orders |m| = am0, am0 + 2, .. (acc: H_{+m} re, im, H_{-m} re, im, 16 each); the whole warp calls
+// it.  The rows of m and -m share a power of two.  Orders past L - 1 are computed and not stored, so that
+// the 16 orders' chains of reduction, split and stores overlap.
 template <bool BF>
-__device__ __forceinline__ void put_orders(const TileOut& to, int sl, int am0, int row, int L, int pbytes, int half, int r0,
+__device__ __forceinline__ void put_orders(const TileOut& to, int sl, int am0, int row, int lane, int L, int half, int r0,
                                            bool last, int pad0, float sgn, const float* acc) {
+  const int pbytes = to.NC * 128, orders = min(16, (L - am0 + 1) >> 1);
   const size_t tb = (size_t)kParts<BF> * pbytes;
-  const int kb = row & 31;
   const long long slice_tiles = (long long)(to.xslice / tb), n = (long long)(to.xbytes / tb);
-  long long tix = sl * slice_tiles + (long long)am0 * to.nC + (row >> 5);
-  uint8_t* tile = to.X + (size_t)sl * to.xslice + ((size_t)am0 * to.nC + (row >> 5)) * tb;
+  const long long tix0 = sl * slice_tiles + (long long)am0 * to.nC + (row >> 5);
+  const bool rows_ok = in_bounds(half + r0 + 1, to.NC, kbPutTile);
+  float mine = 0.f;
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
-    if (am0 + 2 * k >= L) break;
-    if (in_bounds(tix, n, kbPutTile) && in_bounds(half + r0 + 1, to.NC, kbPutTile)) {
-      put_split<BF>(tile, pbytes, r0, kb, acc[k]);
-      put_split<BF>(tile, pbytes, r0 + 1, kb, acc[16 + k]);
-      put_split<BF>(tile, pbytes, half + r0, kb, sgn * acc[32 + k]);
-      put_split<BF>(tile, pbytes, half + r0 + 1, kb, sgn * acc[48 + k]);
-      if (last)
-        for (int rw = pad0; rw < half; ++rw) {
-          put_split<BF>(tile, pbytes, rw, kb, 0.f);
-          put_split<BF>(tile, pbytes, half + rw, kb, 0.f);
-        }
-    }
-    tix += 2 * to.nC;
-    tile += 2 * (size_t)to.nC * tb;
+    const long long tix = tix0 + 2 * k * to.nC;
+    const float v[4] = {acc[k], acc[16 + k], sgn * acc[32 + k], sgn * acc[48 + k]};
+    float sc = 0.f;
+    const float up = BF ? 1.f : warp_power(fmaxf(fmaxf(fabsf(v[0]), fabsf(v[1])), fmaxf(fabsf(v[2]), fabsf(v[3]))), &sc);
+    if (lane == k) mine = sc;
+    uint8_t* tile = to.X + (size_t)tix * tb;
+    const bool ok = k < orders && rows_ok && in_bounds(tix, n, kbPutTile);
+    put_rows2<BF>(tile, pbytes, r0, lane, v[0], v[1], up, ok);
+    put_rows2<BF>(tile, pbytes, half + r0, lane, v[2], v[3], up, ok);
   }
+  const long long tix = tix0 + 2 * lane * to.nC;  // lane k: order k's scales
+  const bool own = lane < orders && rows_ok && in_bounds(tix, n, kbPutTile);
+  if (!BF && own) {
+    float* sc = to.scale + (size_t)tix * half;
+    sc[r0 >> 1] = mine;
+    sc[(half + r0) >> 1] = mine;
+  }
+  if (last && rows_ok)  // the slice's padding rows
+    for (int k = 0; k < orders; ++k) {
+      const long long tp = tix0 + 2 * k * to.nC;
+      if (!in_bounds(tp, n, kbPutTile)) continue;
+      for (int rw = pad0; rw < half; rw += 2) {
+        put_rows2<BF>(to.X + (size_t)tp * tb, pbytes, rw, lane, 0.f, 0.f, 1.f, true);
+        put_rows2<BF>(to.X + (size_t)tp * tb, pbytes, half + rw, lane, 0.f, 0.f, 1.f, true);
+        if (!BF && lane == 0) {
+          to.scale[(size_t)tp * half + (rw >> 1)] = 0.f;
+          to.scale[(size_t)tp * half + ((half + rw) >> 1)] = 0.f;
+        }
+      }
+    }
 }
 
 // Persistent, one CTA an SM; the row blocks of a column tile are consecutive items, so that its
@@ -723,7 +708,8 @@ __device__ __forceinline__ void torus_gemm(const TgArgs& a) {
         const int cls = g < sh.gE ? 0 : 1, gi = cls ? g - sh.gE : g;
         const int am0 = 2 * (64 * gi + 16 * cg) + cls;
         const bool tiles = a.to.mode != 0;
-        if (row >= (tiles ? a.to.nC * 32 : L) || am0 >= L) continue;
+        // tiles: the lanes of a 32-K chunk that exists act together (rows past L are zeros)
+        if (am0 >= L || (tiles ? row0 >= a.to.nC * 32 : row >= L)) continue;
         // H_{+m} and H_{-m} in acc[k], acc[16 + k] and acc[32 + k], acc[48 + k]; the odd parity carries -i
         const bool live = row < L;
 #pragma unroll
@@ -752,13 +738,13 @@ __device__ __forceinline__ void torus_gemm(const TgArgs& a) {
         // half carrying (-1)^{m'} (zeros for m = 0); a slice's last field zeroes the padding rows.  The
         // rows' offsets are the same in every tile, the tiles of the 16 orders two |m| apart.
         const int sl = b / a.to.Bs, bs = b - sl * a.to.Bs, nB = min(a.to.Bs, a.B - sl * a.to.Bs);
-        const int pbytes = a.to.NC * 128, half = a.to.NC / 2;
+        const int half = a.to.NC / 2;
         if (am0 == 0) acc[32] = acc[48] = 0.f;
         const float sgn = (row & 1) ? -1.f : 1.f;
         if (a.to.mode == 2)
-          put_orders<true>(a.to, sl, am0, row, L, pbytes, half, 2 * bs, bs == nB - 1, 2 * nB, sgn, acc);
+          put_orders<true>(a.to, sl, am0, row, lane, L, half, 2 * bs, bs == nB - 1, 2 * nB, sgn, acc);
         else
-          put_orders<false>(a.to, sl, am0, row, L, pbytes, half, 2 * bs, bs == nB - 1, 2 * nB, sgn, acc);
+          put_orders<false>(a.to, sl, am0, row, lane, L, half, 2 * bs, bs == nB - 1, 2 * nB, sgn, acc);
       }
     }
     if constexpr (MODE == kThetaInverse || MODE == kPhiForward) {
