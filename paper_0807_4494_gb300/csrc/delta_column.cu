@@ -55,6 +55,7 @@ constexpr size_t kColSmem = (size_t)kColWarps * kWarpDoubles * sizeof(double);
 struct ColumnParams {
   int L;
   int ntasks;
+  int sms;                 // SMs of the device
   const int2* tasks;       // (l, b), longest first
   const double* sq;        // sqrt(k), k < 2L + 4
   const double* rsq;       // 1/sqrt(k), k >= 1
@@ -87,6 +88,17 @@ __device__ __forceinline__ int exp_of(double v) { return ((__double2hiint(v) >> 
 __device__ __forceinline__ double with_exp(double v, int e) {
   const int hi = (__double2hiint(v) & (int)0x800fffff) | ((e + 1023) << 20);
   return __hiloint2double(hi, __double2loint(v));
+}
+
+// The warp's next task: the first comes from its place in the grid -- task n to CTA n mod grid, so that
+// few tasks land on as many SMs as possible, and the CTAs that share an SM start with different warps, which
+// sit on different quarters of it -- later ones from the counter.  (All from the counter, the first CTAs took
+// eight each: at L = 128 the 319 tasks of the FP64 table ran on 40 SMs; 46 -> 41 us.)
+__device__ __forceinline__ int next_task(bool first, int sms, unsigned int* counter, int lane, int warp) {
+  if (first) return ((warp - (int)(blockIdx.x / sms)) & (kColWarps - 1)) * (int)gridDim.x + (int)blockIdx.x;
+  int t = 0;
+  if (lane == 0) t = (int)(gridDim.x * kColWarps + atomicAdd(counter, 1u));
+  return __shfl_sync(0xffffffffu, t, 0);
 }
 
 // First row of degree l for the 32 columns m = m0 + lane (the whole warp calls it, m0 a multiple of
@@ -144,10 +156,8 @@ __global__ void __launch_bounds__(kColThreads, 2) column_recursion_kernel(Column
   double* coef = stage + kStageDoubles;  // a(m') of the chunk, then b(m')
   const double* __restrict__ sq = P.sq;
   const double* __restrict__ rsq = P.rsq;
-  for (;;) {
-    int t = 0;
-    if (lane == 0) t = (int)atomicAdd(P.counter, 1u);
-    t = __shfl_sync(0xffffffffu, t, 0);
+  for (bool first = true;; first = false) {
+    const int t = next_task(first, P.sms, P.counter, lane, threadIdx.x >> 5);
     if (t >= P.ntasks) break;
     const int2 task = P.tasks[t];
     const int l = task.x, m0 = 32 * task.y, m = m0 + lane;
@@ -171,55 +181,69 @@ __global__ void __launch_bounds__(kColThreads, 2) column_recursion_kernel(Column
     const size_t row = (size_t)l + 1;
 
     // ---- rows m' = l .. m0 ----
-    for (int mp = l; mp >= m0; --mp) {
-      const int j = mp & 31;
-      if (mp == l || j == 31) {
-        // coefficients a(m'), b(m') of the chunk of m' in [mp & ~31, (mp & ~31) + 31]
-        __syncwarp();
-        const int k = (mp & ~31) + lane;
-        double a = 0.0, b = 0.0;
-        if (k >= 1 && k <= l) {
-          a = __dmul_rn(rsq[l - k + 1], rsq[l + k]);
-          b = __dmul_rn(__dmul_rn(sq[l - k], sq[l + k + 1]), a);
-        }
-        coef[lane] = a;
-        coef[32 + lane] = b;
-        __syncwarp();
+    // coefficients a(m'), b(m') of the chunk of m' in [mp & ~31, (mp & ~31) + 31]
+    auto coefficients = [&](int mp) {
+      __syncwarp();
+      const int k = (mp & ~31) + lane;
+      double a = 0.0, b = 0.0;
+      if (k >= 1 && k <= l) {
+        a = __dmul_rn(rsq[l - k + 1], rsq[l + k]);
+        b = __dmul_rn(__dmul_rn(sq[l - k], sq[l + k + 1]), a);
       }
-      const double out = (SCALED && E != 0) ? 0.0 : cur;
+      coef[lane] = a;
+      coef[32 + lane] = b;
+      __syncwarp();
+    };
+    auto write = [&](int mp, double out) {
       if (act && in_bounds((long long)delta_offset_dev(l) + (long long)(mp * row + m), P.extent, kbColumnTable))
         T[(size_t)mp * row + m] = out;
-      if (mp >= m0 + 32) {
-        // transposed entry Delta_{m m'} = (-1)^{m'-m} Delta_{m'm}, written a 32-column chunk at a time
-        stage[lane * 33 + j] = flip_sign(out, ((mp - m) & 1) != 0);
-        if (j == 0) {
-          __syncwarp();
-          const int c = mp + lane;
-          for (int r = 0; r < 32 && m0 + r <= l; ++r)
-            if (c <= l && in_bounds((long long)delta_offset_dev(l) + (long long)((m0 + r) * row + c), P.extent,
-                                    kbColumnTable))
-              T[(size_t)(m0 + r) * row + c] = stage[r * 33 + lane];
-          __syncwarp();
+      // transposed entry Delta_{m m'} = (-1)^{m'-m} Delta_{m'm}, written a 32-column chunk at a time
+      if (mp >= m0 + 32) stage[lane * 33 + (mp & 31)] = flip_sign(out, ((mp - m) & 1) != 0);
+    };
+    auto flush = [&](int mp) {  // mp a multiple of 32: its chunk is complete
+      __syncwarp();
+      const int c = mp + lane;
+#pragma unroll 4
+      for (int r = 0; r < min(32, l - m0 + 1); ++r)
+        if (c <= l && in_bounds((long long)delta_offset_dev(l) + (long long)((m0 + r) * row + c), P.extent, kbColumnTable))
+          T[(size_t)(m0 + r) * row + c] = stage[r * 33 + lane];
+      __syncwarp();
+    };
+    auto next = [&](int j) {  // the value one row down from (cur, prev)
+      const double c = mul_small_rn(coef[j], (uint32_t)m, 1);  // 2m a(m'), on the integer pipe
+      return __fma_rn(c, cur, -__dmul_rn(coef[32 + j], prev));
+    };
+    int mp = l;
+    while (mp >= m0) {
+      const int j = mp & 31;
+      if (mp == l || j == 31) coefficients(mp);
+      if (!SCALED && (mp & 3) == 3) {
+        // four rows at once: the recursion first, then the four rows' outputs, whose work overlaps (GB300:
+        // L = 257 81 -> 60 us a sweep, L = 512 178 -> 151, L = 1024 961 -> 914; m0 is a
+        // multiple of 32, so that four rows end at or above it; the update past row m0 goes unused)
+        double y[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          y[k] = cur;
+          const double nxt = next(j - k);
+          prev = cur;
+          cur = nxt;
         }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) write(mp - k, y[k]);
+        mp -= 4;
+        if (j == 3 && mp + 1 >= m0 + 32) flush(mp + 1);
+        continue;
       }
+      write(mp, (SCALED && E != 0) ? 0.0 : cur);
+      if (j == 0 && mp >= m0 + 32) flush(mp);
       if (mp > m0) {
-        const double c = mul_small_rn(coef[j], (uint32_t)m, 1);  // 2m a(m'), on the integer pipe
-        const double nxt = __fma_rn(c, cur, -__dmul_rn(coef[32 + j], prev));
+        const double nxt = next(j);
         prev = cur;
         cur = nxt;
-        if (SCALED && E != 0) {
-          const int x = exp_of(cur);
-          if (x + E >= -1021) {  // back in the normal range: fold the exponent in
-            cur = ldexp(cur, E);
-            prev = ldexp(prev, E);
-            E = 0;
-          } else if (x > 512) {  // keep the stored values far from overflow
-            cur = __dmul_rn(cur, 0x1p-512);
-            prev = __dmul_rn(prev, 0x1p-512);
-            E += 512;
-          }
-        }
+        if (SCALED && E != 0) rescale_exponent(cur, prev, E);
       }
+      --mp;
     }
   }
 }
@@ -248,7 +272,7 @@ __global__ void __launch_bounds__(kColThreads, 2) column_recursion_kernel(Column
 #define SSHT_COLUMN_CTAS 3
 #endif
 constexpr int kTileStageFloats = 32 * 33;
-constexpr int kTileWarpBytes = kTileStageFloats * 4 + 32 * 8 + 32 * 4;  // stage, alpha[32], p[32]
+constexpr int kTileWarpBytes = kTileStageFloats * 4 + 32 * 8 + 32 * 8 + 32 * 4;  // stage, alpha[32], tile base[32], p[32]
 constexpr size_t kTileSmem = (size_t)kColWarps * kTileWarpBytes;
 
 template <bool SCALED, bool BF>
@@ -257,14 +281,13 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* stage = reinterpret_cast<float*>(smraw + warp * kTileWarpBytes);
   double* alw = reinterpret_cast<double*>(smraw + warp * kTileWarpBytes + kTileStageFloats * 4);
-  float* pw = reinterpret_cast<float*>(alw + 32);
+  long long* abw = reinterpret_cast<long long*>(alw + 32);
+  float* pw = reinterpret_cast<float*>(abw + 32);
   const double* __restrict__ sq = P.sq;
   const double* __restrict__ rsq = P.rsq;
   const long long ntri = (long long)P.L * (P.L + 1) / 2;
-  for (;;) {
-    int t = 0;
-    if (lane == 0) t = (int)atomicAdd(P.counter, 1u);
-    t = __shfl_sync(0xffffffffu, t, 0);
+  for (bool first = true;; first = false) {
+    const int t = next_task(first, P.sms, P.counter, lane, threadIdx.x >> 5);
     if (t >= P.ntasks) break;
     const int2 task = P.tasks[t];
     const int l = task.x, m0 = 32 * task.y, m = m0 + lane;
@@ -297,44 +320,51 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
       u_lane = __ldg(&P.Uf[lrow + m]);
       base_lane = __ldg(&P.ab2[m]) + ilpre;
     }
-    // the base of row M = m' (a load), fetched one step ahead
-    long long ab_cur = __ldg(&P.ab2[l]), ab_next = 0;
+    // alpha(l, m'), p(l, m') and the tile base of row M = m' for a chunk of 32 consecutive m', one a lane,
+    // asked for a chunk ahead (a load one step ahead made every step as long as its latency)
+    double al_n = 0.0;
+    float p_n = 0.f;
+    long long ab_n = 0;
+    auto fetch = [&](int k0) {
+      const int k = k0 + lane;
+      if (k0 >= 0 && k <= l && in_bounds((long long)(lrow + k), ntri, kbColumnCoef)) {
+        al_n = __ldg(&P.alc[lrow + k]);
+        p_n = __ldg(&P.pc[lrow + k]);
+        ab_n = __ldg(&P.ab2[k]);
+      }
+    };
+    fetch(l & ~31);
     int mp = l;
     // one row; the coefficient m alpha of its update comes from the FP64 pipe or from the integer
     // pipe (the same exactly rounded product), alternately, so that the two pipes share the work
-    auto row = [&](auto on_fp64) {
-      if (mp > m0) ab_next = __ldg(&P.ab2[mp - 1]);
-      const int j = mp & 31;
-      if (mp == l || j == 31) {
-        // alpha(l, m') and p(l, m') of the chunk of m' in [mp & ~31, (mp & ~31) + 31]
-        __syncwarp();
-        const int k = (mp & ~31) + lane;
-        double al = 0.0;
-        float pk = 0.f;
-        if (k <= l && in_bounds((long long)(lrow + k), ntri, kbColumnCoef)) {
-          al = __ldg(&P.alc[lrow + k]);
-          pk = __ldg(&P.pc[lrow + k]);
-        }
-        alw[lane] = al;
-        pw[lane] = pk;
-        __syncwarp();
+    auto chunk = [&]() {
+      __syncwarp();
+      alw[lane] = al_n;
+      pw[lane] = p_n;
+      abw[lane] = ab_n;
+      __syncwarp();
+      if ((mp & ~31) > m0) fetch((mp & ~31) - 32);
+    };
+    // A_M[l][m'] for the columns M = m0 + r, m' = mq + lane, mq a multiple of 32: U_l[m'] p(l, m') y
+    auto flush = [&](int mq) {
+      __syncwarp();
+      const int c = mq + lane;
+      const float uc = c <= l ? __ldg(&P.Uf[lrow + c]) * __ldg(&P.pc[lrow + c]) : 0.f;
+      const int cb = mq >> 5;
+#pragma unroll 4
+      for (int r = 0; r < min(32, l - m0 + 1); ++r) {
+        const long long tile = __shfl_sync(0xffffffffu, base_lane, r) + cb;
+        if (c <= l) put_a_at<BF>(P.A, tile, P.extent, kbColumnTile, off, uc * stage[r * 33 + lane]);
       }
+      __syncwarp();
+    };
+    auto row = [&](auto on_fp64) {
+      const int j = mp & 31;
       const float x = f64_to_f32_rn((SCALED && E != 0) ? 0.0 : cur);  // y_{m'} in FP32
-      if (act) put_a_at<BF>(P.A, ab_cur + tadd, P.extent, kbColumnTile, off, (u_lane * pw[j]) * (((mp - m) & 1) ? -x : x));
+      if (act) put_a_at<BF>(P.A, abw[j] + tadd, P.extent, kbColumnTile, off, (u_lane * pw[j]) * (((mp - m) & 1) ? -x : x));
       if (mp >= m0 + 32) {
         stage[lane * 33 + j] = x;
-        if (j == 0) {
-          // A_M[l][m'] for the columns M = m0 + r, m' = mp + lane: U_l[m'] p(l, m') y
-          __syncwarp();
-          const int c = mp + lane;
-          const float uc = c <= l ? __ldg(&P.Uf[lrow + c]) * __ldg(&P.pc[lrow + c]) : 0.f;
-          const int cb = mp >> 5;
-          for (int r = 0; r < 32 && m0 + r <= l; ++r) {
-            const long long tile = __shfl_sync(0xffffffffu, base_lane, r) + cb;
-            if (c <= l) put_a_at<BF>(P.A, tile, P.extent, kbColumnTile, off, uc * stage[r * 33 + lane]);
-          }
-          __syncwarp();
-        }
+        if (j == 0) flush(mp);
       }
       if (mp > m0) {
         double c;
@@ -347,14 +377,41 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
         cur = nxt;
         if (SCALED && E != 0) rescale_exponent(cur, prev, E);
       }
-      ab_cur = ab_next;
       --mp;
     };
-    for (;;) {
-      row(std::true_type{});
-      if (mp < m0) break;
-      row(std::false_type{});
-      if (mp < m0) break;
+    // four rows at once (rows 4k + 3 .. 4k): the recursion first, then the rows' outputs, whose chains of
+    // rounding, splitting and stores overlap (GB300, against row after row: L = 1024 784 -> 655 us a sweep,
+    // L = 257 90 -> 74).  The update past row m0 goes unused.
+    auto four = [&]() {
+      const int j = mp & 31;
+      double y[4], c[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) c[k] = (k & 1) ? mul_small_rn(alw[j - k], (uint32_t)m, 0) : __dmul_rn(md, alw[j - k]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        y[k] = cur;
+        const double nxt = __fma_rn(c[k], cur, -prev);
+        prev = cur;
+        cur = nxt;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float x = f64_to_f32_rn(y[k]);
+        if (act) put_a_at<BF>(P.A, abw[j - k] + tadd, P.extent, kbColumnTile, off, (u_lane * pw[j - k]) * (((mp - k - m) & 1) ? -x : x));
+        if (mp >= m0 + 32) stage[lane * 33 + j - k] = x;
+      }
+      if (j == 3 && mp >= m0 + 32) flush(mp - 3);
+      mp -= 4;
+    };
+    while (mp >= m0) {
+      if ((mp & 31) == 31 || mp == l) chunk();
+      if (!SCALED && (mp & 3) == 3) {
+        four();
+      } else if (mp & 1) {
+        row(std::true_type{});
+      } else {
+        row(std::false_type{});
+      }
     }
   }
 }
@@ -382,6 +439,7 @@ __host__ __device__ __forceinline__ size_t tri_idx(long long r, long long l, lon
 
 struct LaneParams {
   int L, as, nI, ntasks;
+  int sms;                  // SMs of the device
   const int2* tasks;        // (m, kc), longest first
   const double* alpha;      // alpha(l, m') at tri_idx(m', l)
   const float* p;           // p(l, m') at tri_idx(m', l)
@@ -410,10 +468,8 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
   const int lane = threadIdx.x & 31;
   const int L = P.L;
   const int ntri = L * (L + 1) / 2;
-  for (;;) {
-    int t = 0;
-    if (lane == 0) t = (int)atomicAdd(P.counter, 1u);
-    t = __shfl_sync(0xffffffffu, t, 0);
+  for (bool first = true;; first = false) {
+    const int t = next_task(first, P.sms, P.counter, lane, threadIdx.x >> 5);
     if (t >= P.ntasks) break;
     const int2 task = P.tasks[t];
     const int m = task.x, kc = task.y;
@@ -532,6 +588,113 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
   }
 }
 
+// The same sweep for small band-limits, where a warp has at most a task or two and a step lasts as long
+// as its chain of instructions: four rows at a time, the recursion first and then their outputs, whose
+// chains overlap, with the rows' loads (alpha, p, U, tile base) issued four rows ahead.  Two CTAs an SM are
+// room enough for its registers.  GB300: L = 257 104 -> 80 us a sweep, L = 512 221 -> 175; L = 1024 788 -> 905, where
+// the variant above, with twice the warps, is taken.
+template <bool BF>
+__global__ void __launch_bounds__(kColThreads, 2) lane_recursion_deep_kernel(LaneParams P) {
+  const int lane = threadIdx.x & 31;
+  const int L = P.L;
+  const int ntri = L * (L + 1) / 2;
+  constexpr int D = 4;
+  for (bool first = true;; first = false) {
+    const int t = next_task(first, P.sms, P.counter, lane, threadIdx.x >> 5);
+    if (t >= P.ntasks) break;
+    const int2 task = P.tasks[t];
+    const int m = task.x, kc = task.y;
+    const int l = 32 * kc + lane;
+    const int top = min(32 * kc + 31, L - 1);
+    const bool inl = l < L && l >= m;     // degree l exists and has column m
+    const bool wr = inl && l >= P.as;     // U_l vanishes below |s|: those entries stay zero
+    const float um = wr ? __ldg(&P.ufT[tri_idx(m, l, L)]) : 0.f;
+    const double y0 = inl ? __ldg(&P.t1m[tri_idx(m, l, L)]) : 0.0;  // y_l = Delta_{l m}
+    const long long* ib_m = P.ibase + (size_t)m * P.nI;
+    const uint32_t off_m = a_off(m & 127, lane);  // (row m, K = l) in the tiles A_{m'}[m][.]
+    const double md = (double)m;
+    double cur = 0.0, prev = 0.0, ca[D];
+    float cp[D], cu[D];
+    long long ct[D];
+    int kidx = top * L - top * (top - 1) / 2 + (l - top);  // tri_idx of the next row to ask for
+    int ask = top;
+    const long long* ibr = P.ibase + (size_t)top * P.nI + (m >> 7);
+    auto fetch = [&](int q) {  // row `ask` into slot q
+      ca[q] = 0.0;
+      cp[q] = cu[q] = 0.f;
+      ct[q] = 0;
+      if (ask >= m) {
+        if (inl && ask <= l && in_bounds(kidx, ntri, kbLaneTable)) {
+          ca[q] = __ldg(&P.alpha[kidx]);
+          cp[q] = __ldg(&P.p[kidx]);
+          cu[q] = __ldg(&P.ufT[kidx]);
+        }
+        ct[q] = __ldg(ibr);
+        --ask;
+        kidx -= L - (ask + 1);
+        ibr -= P.nI;
+      }
+    };
+#pragma unroll
+    for (int q = 0; q < D; ++q) fetch(q);
+    long long tb = 0, tbn = __ldg(&ib_m[top >> 7]);  // tiles of row m' of column m: this and the next row block
+    int mp = top;
+    while (mp >= m) {
+      if (mp < 32 * kc && mp - 3 > m && (mp & 127) != 127 && (mp >> 7) == ((mp - 3) >> 7)) {
+        // four rows at once, every lane under way: the recursion first, then the rows' outputs, whose
+        // chains of rounding, splitting and stores overlap
+        double y[D], c[D];
+#pragma unroll
+        for (int q = 0; q < D; ++q) c[q] = (q & 1) ? mul_small_rn(ca[q], (uint32_t)m, 0) : __dmul_rn(md, ca[q]);
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+          y[q] = cur;
+          const double nxt = __fma_rn(c[q], cur, -prev);
+          prev = cur;
+          cur = nxt;
+        }
+        if (wr) {
+#pragma unroll
+          for (int q = 0; q < D; ++q) {
+            const float x = f64_to_f32_rn(y[q]);
+            put_a_at<BF>(P.A, tb, P.ntiles, kbLaneTile, a_off((mp - q) & 127, lane), (cu[q] * cp[q]) * x);
+            put_a_at<BF>(P.A, ct[q] + kc, P.ntiles, kbLaneTile, off_m, (um * cp[q]) * (((mp - q - m) & 1) ? -x : x));
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < D; ++q) fetch(q);
+        mp -= D;
+        continue;
+      }
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        if (mp >= m) {
+          if (mp == top || (mp & 127) == 127) {
+            tb = tbn + kc;
+            if (mp >> 7) tbn = __ldg(&ib_m[(mp >> 7) - 1]);
+          }
+          if (mp == l && inl) {
+            cur = y0;
+            prev = 0.0;
+          }
+          if (inl && mp <= l) {
+            if (wr) {
+              const float x = f64_to_f32_rn(cur);
+              put_a_at<BF>(P.A, tb, P.ntiles, kbLaneTile, a_off(mp & 127, lane), (cu[q] * cp[q]) * x);
+              if (mp > m) put_a_at<BF>(P.A, ct[q] + kc, P.ntiles, kbLaneTile, off_m, (um * cp[q]) * (((mp - m) & 1) ? -x : x));
+            }
+            const double nxt = __fma_rn(__dmul_rn(md, ca[q]), cur, -prev);  // not used after row m
+            prev = cur;
+            cur = nxt;
+          }
+          fetch(q);
+          --mp;
+        }
+      }
+    }
+  }
+}
+
 // Plan-time tables of the tile-writing recursions: the first rows (one warp per degree and block
 // of 32 columns, the arithmetic of the column recursion), the rescaled relation's alpha(l, m') and
 // p(l, m'), and U transposed.
@@ -621,6 +784,7 @@ cudaError_t column_setup(DeltaWork& w, int L, int device) {
   w.method = kDeltaColumn;
   w.threads = kColThreads;
   w.blocks = sms * std::min(per_sm, 2);
+  w.sms = sms;
   w.smem = kColSmem;
   w.ntasks = (int)tasks.size();
   if ((e = dev_malloc(&w.table, delta_offset(L) * sizeof(double))) != cudaSuccess) return e;
@@ -647,6 +811,7 @@ static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, con
   ColumnParams P;
   P.L = L;
   P.ntasks = w.ntasks;
+  P.sms = w.sms;
   P.tasks = w.tasks;
   P.sq = w.sqrt_tab;
   P.rsq = w.sqrt_tab + (2 * (size_t)L + 4);
@@ -724,6 +889,10 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
         cudaSuccess)
       return e;
     t.blocks = sms * std::max(1, std::min(per_sm, SSHT_LANE_CTAS));
+    // the variant of four rows a step while its two CTAs an SM have room for half of the tasks at once
+    // (up to L = 550 or so; between the L = 512 and L = 1024 figures beside it)
+    t.deep = t.ntasks <= 2 * 2 * sms * kColWarps;
+    if (t.deep) t.blocks = 2 * sms;
     const void* fns[4] = {(const void*)column_tiles_kernel<false, false>, (const void*)column_tiles_kernel<true, false>,
                           (const void*)column_tiles_kernel<false, true>, (const void*)column_tiles_kernel<true, true>};
     for (const void* fn : fns) {
@@ -739,7 +908,8 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     t.col_blocks = sms * std::min(per_sm, SSHT_COLUMN_CTAS);
   }
-  const void* lanes[4] = {(const void*)lane_recursion_kernel<false, false>, (const void*)lane_recursion_kernel<true, false>,
+  const void* lanes[6] = {(const void*)lane_recursion_deep_kernel<false>, (const void*)lane_recursion_deep_kernel<true>,
+                          (const void*)lane_recursion_kernel<false, false>, (const void*)lane_recursion_kernel<true, false>,
                           (const void*)lane_recursion_kernel<false, true>, (const void*)lane_recursion_kernel<true, true>};
   for (const void* fn : lanes)
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -758,6 +928,7 @@ cudaError_t column_run_inverse_tiles(const DeltaWork& w, const LaneTables& t, in
   P.as = s < 0 ? -s : s;
   P.nI = it.nI;
   P.ntasks = t.ntasks;
+  P.sms = w.sms;
   P.tasks = t.tasks;
   P.alpha = t.alT;
   P.p = t.pT;
@@ -768,7 +939,11 @@ cudaError_t column_run_inverse_tiles(const DeltaWork& w, const LaneTables& t, in
   P.ibase = it.ibase;
   P.counter = t.counter;
   P.ntiles = it.ntiles;
-  if (it.bf16)
+  if (t.deep && it.bf16)
+    lane_recursion_deep_kernel<true><<<t.blocks, kColThreads, 0, st>>>(P);
+  else if (t.deep)
+    lane_recursion_deep_kernel<false><<<t.blocks, kColThreads, 0, st>>>(P);
+  else if (it.bf16)
     (L > 1024 ? lane_recursion_kernel<true, true> : lane_recursion_kernel<false, true>)<<<t.blocks, kColThreads, 0, st>>>(P);
   else
     (L > 1024 ? lane_recursion_kernel<true, false> : lane_recursion_kernel<false, false>)<<<t.blocks, kColThreads, 0, st>>>(P);

@@ -61,6 +61,7 @@ struct DeltaWork {
   unsigned int* barrier = nullptr;  // grid barrier counter
   int* status = nullptr;          // latched status word
   int blocks = 0;                 // cooperative grid size
+  int sms = 0;                    // SMs of the device (column method)
   int threads = 0;
   size_t smem = 0;
   size_t bytes = 0;   // device memory held (table, slabs, tables, words)
@@ -204,6 +205,7 @@ struct LaneTables {
   int2* tasks = nullptr;
   unsigned int* counter = nullptr;  // next task of the plan's own sweeps (plans of a group run side by side)
   int ntasks = 0;
+  bool deep = false;   // the variant for small band-limits
   int blocks = 0;      // grid of the degree-lane recursion
   int col_blocks = 0;  // grid of the column recursion writing the forward tiles
   size_t bytes = 0;
