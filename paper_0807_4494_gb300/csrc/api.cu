@@ -128,6 +128,7 @@ struct ssht_plan_s {
   size_t bytes = 0;
   TcPlan* tc = nullptr;    // tensor-core contraction (precisions SSHT_TF32X3, SSHT_BF16X6)
   TorusPlan* torus = nullptr;  // fused torus passes of FP32 plans (FP64 plans: cuFFT Z2Z + glue)
+  DirectPlan* direct = nullptr;  // torus products of FP64 plans of small band-limit, in place of the FFTs
   // The Delta recursion (and the A packing) of a call runs on a second stream, forked from the
   // caller's stream at the start of the call and joined before the contraction, so that the
   // Delta-independent work of the call (the torus stage of forward/adjoint, data packing) runs
@@ -432,6 +433,20 @@ int tc_multiply(ssht_plan_t p, int forward, void* dst, cudaStream_t st) {
   return 0;
 }
 
+// One torus product of an FP64 plan of small band-limit, timed as FFT work; which: 0, 1 the inverse's theta
+// and phi, 2 phi of forward and adjoint, 3, 4 theta of forward and adjoint.
+int direct_pass(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t st) {
+  StageScope sc(p, SSHT_STAGE_FFT, st);
+  cudaError_t e;
+  if (which == 0) e = direct_inverse(p->direct, p->s, p->B, in, out, nullptr, st, 0);
+  else if (which == 1) e = direct_inverse(p->direct, p->s, p->B, nullptr, const_cast<void*>(in), out, st, 1);
+  else if (which == 2) e = direct_analysis(p->direct, 0, p->s, p->B, in, out, nullptr, st, 0);
+  else e = direct_analysis(p->direct, which == 4, p->s, p->B, nullptr, const_cast<void*>(in), out, st, 1);
+  SSHT_CUDA(e, "torus product");
+  p->launches += 1;
+  return 0;
+}
+
 // FP32-class forward (adjoint = 0) or adjoint: the torus passes, then the projection.  Tensor-core plans:
 // the theta pass writes the projection's data tiles itself (no H, no data packing).
 template <typename T>
@@ -542,7 +557,7 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
     if ((rc = join_operands(p, st))) return rc;
     StageScope sc(p, SSHT_STAGE_INVERSE, st);
     SSHT_CUDA(contract_inverse_simt<T>(d, p->s, p->B, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W1, p->w_bytes,
-                                       p->ph64, p->torus ? 1 : 0, st),
+                                       p->ph64, p->torus || p->direct ? 1 : 0, st),
               "inverse contraction");
     p->launches += 1;
   }
@@ -550,6 +565,10 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
   if (p->torus) {
     if ((rc = torus_inverse_pass(p, 0, f, st))) return rc;
     return torus_inverse_pass(p, 1, f, st);
+  }
+  if (p->direct) {
+    if ((rc = direct_pass(p, 0, p->W1, p->W2, st))) return rc;
+    return direct_pass(p, 1, p->W2, f, st);
   }
   rc = run_dft(p, p->fft_theta, +1, p->W1, p->W2, st);
   if (rc) return rc;
@@ -582,6 +601,10 @@ int forward_impl(ssht_plan_t p, const void* f, void* flm, cudaStream_t st) {
   int rc = begin_operands(p, 1, st);
   if (rc) return rc;
   if (p->torus) return analysis_fp32(p, 0, f, flm, st);
+  if (p->direct) {
+    if ((rc = direct_pass(p, 2, f, p->W2, st)) || (rc = direct_pass(p, 3, p->W2, p->W1, st))) return rc;
+    return project<T>(p, p->W1, flm, st);
+  }
   rc = analysis_front<T>(p, f, 0, st);
   if (rc) return rc;
   {
@@ -610,6 +633,10 @@ int adjoint_impl(ssht_plan_t p, const void* g, void* flm, cudaStream_t st) {
   int rc = begin_operands(p, 1, st);
   if (rc) return rc;
   if (p->torus) return analysis_fp32(p, 1, g, flm, st);
+  if (p->direct) {
+    if ((rc = direct_pass(p, 2, g, p->W2, st)) || (rc = direct_pass(p, 4, p->W2, p->W1, st))) return rc;
+    return project<T>(p, p->W1, flm, st);
+  }
   rc = analysis_front<T>(p, g, 1, st);
   if (rc) return rc;
   {
@@ -801,6 +828,7 @@ void release(ssht_plan_t p) {
   }
   if (p->tc) tc_destroy(p->tc);
   if (p->torus) torus_destroy(p->torus);
+  if (p->direct) direct_destroy(p->direct);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
   if (p->ev_free) cudaEventDestroy(p->ev_free);
@@ -893,7 +921,8 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, (void**)&p->Uf, tri(L) * sizeof(float), "spin column (FP32)"))) return bail(rc);
   // FP64: full N x N torus rows and an M-point convolution buffer; FP32 (fused torus passes): half
   // rows of N x L, or a pass's operand tiles.
-  const size_t torus = p->f64 ? (size_t)B * d.N * d.N * p->elem : torus_workspace_bytes(L, B);
+  const bool direct = p->f64 && direct_wanted(L, B);  // L^2 products twice over fit N x N rows but for L = 1
+  const size_t torus = p->f64 ? (size_t)B * std::max(d.N * d.N, 2) * p->elem : torus_workspace_bytes(L, B);
   if (pair && (rc = dalloc(p, &p->rc, (size_t)B * L * L * p->elem, "spin-pair coefficients"))) return bail(rc);
   if ((real || pair) && (ce = real_setup()) != cudaSuccess) {
     release(p);
@@ -906,7 +935,7 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, &p->W1, torus, "torus workspace 1"))) return bail(rc);
   if ((rc = dalloc(p, &p->W2, torus, "torus workspace 2"))) return bail(rc);
   p->w_bytes = torus;
-  if (p->f64) {
+  if (p->f64 && !direct) {
     if ((rc = dalloc(p, &p->W3, (size_t)B * d.N * d.M * p->elem, "convolution workspace"))) return bail(rc);
     if ((rc = dalloc(p, &p->khat, (size_t)d.M * p->elem, "weight spectrum"))) return bail(rc);
   }
@@ -936,6 +965,16 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if (p->f64) {
     if ((rc = make_fft(p, &p->fft_phi, &p->have_phi, d.N, (size_t)B * d.L, "cuFFT phi plan"))) return bail(rc);
     if ((rc = make_fft(p, &p->fft_theta, &p->have_theta, d.N, (size_t)B * d.N, "cuFFT theta plan"))) return bail(rc);
+  }
+  if (direct) {  // the FFT plans above serve the triangular forward only
+    ce = direct_setup(&p->direct, L);
+    if (ce != cudaSuccess) {
+      release(p);
+      return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,
+                  std::string("torus product setup: ") + cudaGetErrorString(ce));
+    }
+    p->bytes += direct_bytes(p->direct);
+  } else if (p->f64) {
     if ((rc = make_fft(p, &p->fft_conv, &p->have_conv, d.M, (size_t)B * d.N, "cuFFT convolution plan")))
       return bail(rc);
     // Weight spectrum: FFT of the even part of w(p) = int_0^pi sin(t) e^{ipt} dt.

@@ -241,6 +241,22 @@ cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const 
                            int* launches, int step);
 
 // ---------------------------------------------------------------------------
+// Torus passes of FP64 plans of small band-limit (torus_direct.cu)
+// ---------------------------------------------------------------------------
+// The same folded products as the FP32 plans' passes, in FP64 on CUDA cores.  F, H: half rows (double2)
+// [B][N][L]; work: 2 B L^2 double2; f: samples [B][L][N].
+struct DirectPlan;
+bool direct_wanted(int L, int B);  // whether a plan of this band-limit and batch takes them instead of the FFTs
+cudaError_t direct_setup(DirectPlan** out, int L);  // synchronises
+void direct_destroy(DirectPlan* p);
+size_t direct_bytes(const DirectPlan* p);
+// step 0: theta (F -> work), 1: phi (work -> f).
+cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* F, void* work, void* f, cudaStream_t st, int step);
+// step 0: phi (f -> work), 1: theta (work -> H; adjoint = 0 with the extension and the sin(theta) weight).
+cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* f, void* work, void* H, cudaStream_t st,
+                            int step);
+
+// ---------------------------------------------------------------------------
 // Torus kernels (torus.cu)
 // ---------------------------------------------------------------------------
 // g[b][m+Lp][t] (theta-synthesis output, N per row) -> h[b][t][m mod N] * e^{i pi m / N}, t < L.

@@ -1,0 +1,280 @@
+// Torus passes of FP64 plans of small band-limit: the folded cosine and sine products of the torus stage
+// (torus_gemm.cu gives the identities) in FP64 on CUDA cores, in place of cuFFT's transforms of odd length
+// and the kernels between them.
+//
+// Matrices are stored [k][row], so that a warp's lanes (32 rows) read them coalesced, and a data column is
+// read by the whole warp at one address.  A CTA computes 32 rows of one unit -- one order |m| (both signs), or
+// one ring -- as two complex columns, 4 FP64 multiply-adds a k; its eight warps take an eighth of the k's each
+// and add up at the end, which keeps every quarter of every SM busy down to the smallest band-limits.
+//
+// What bounds it: the FP64 pipe, 8 B L^3 flops a pass.  That grows faster than the FFTs' N^2 log N, but
+// those are far from any bound at these sizes (odd, often prime lengths; 11 launches an inverse + forward).
+// 1.07 TFLOP/s at L = 128, B = 16 (0.85 of the FP64 pipe's rate).
+#include "ssht_internal.h"
+#include "torus_matrices.cuh"
+
+#include <algorithm>
+
+namespace ssht {
+namespace {
+
+constexpr int kWarps = 8;
+
+// Matrices, each L x L, [k][row].
+enum Matrix { kCosKX = 0, kSinKX, kCosXK, kSinXK, kWeightE, kWeightO, kMatrices };
+
+__global__ void direct_matrices_kernel(int L, const double2* __restrict__ cs, const double2* __restrict__ T,
+                                       double* __restrict__ out) {
+  const int N = 2 * L - 1;
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (long long)L * L) return;
+  const int k = (int)(e / L), r = (int)(e % L);
+  const size_t n = (size_t)L * L;
+  // order k at node r, and order r at node k; sin vanishes at the node theta = pi
+  const double2 a = cs[(int)(((long long)k * (2 * r + 1)) % (2 * N))], b = cs[(int)(((long long)r * (2 * k + 1)) % (2 * N))];
+  out[kCosKX * n + e] = a.x;
+  out[kSinKX * n + e] = r == L - 1 ? 0.0 : a.y;
+  out[kCosXK * n + e] = b.x;
+  out[kSinXK * n + e] = k == L - 1 ? 0.0 : b.y;
+  out[kWeightE * n + e] = weight_entry(true, L, cs, T, r, k);
+  out[kWeightO * n + e] = weight_entry(false, L, cs, T, r, k);
+}
+
+struct Pair {
+  double2 a, b;
+};
+
+// Sum of the eight warps' pairs for lane's row, in warp 0 (all threads call it).
+__device__ __forceinline__ Pair reduce_warps(Pair v, int warp, int lane) {
+  __shared__ double2 part[kWarps][2][32];
+  part[warp][0][lane] = v.a;
+  part[warp][1][lane] = v.b;
+  __syncthreads();
+  Pair r;
+  r.a = r.b = make_double2(0.0, 0.0);
+  if (warp == 0)
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const double2 a = part[w][0][lane], b = part[w][1][lane];
+      r.a.x += a.x;
+      r.a.y += a.y;
+      r.b.x += b.x;
+      r.b.y += b.y;
+    }
+  return r;
+}
+
+__device__ __forceinline__ void axpy(double2& acc, double a, double2 x) {
+  acc.x = fma(a, x.x, acc.x);
+  acc.y = fma(a, x.y, acc.y);
+}
+
+// theta inverse: F [b][m + Lp][m'] -> work E, O [2][b][m][t] = x_m +- x_{-m} (m = 0: x_0, 0).
+__global__ void __launch_bounds__(32 * kWarps) direct_theta_inverse_kernel(int L, int s, int B, const double* __restrict__ M,
+                                                                           const double2* __restrict__ F, double2* __restrict__ work) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
+  const int t = 32 * blockIdx.y + lane, b = blockIdx.x / L, m = blockIdx.x - b * L;
+  const bool odd = (m + s) & 1;
+  const double* A = M + (size_t)(odd ? kSinKX : kCosKX) * L * L;
+  const double2* Fp = F + ((size_t)b * N + L - 1 + m) * L;
+  const double2* Fm = F + ((size_t)b * N + L - 1 - m) * L;
+  Pair v;
+  v.a = v.b = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k = warp; k < L; k += kWarps) {
+    double a = t < L ? __ldg(&A[(size_t)k * L + t]) : 0.0;
+    if (k == 0) a *= 0.5;  // the sum is doubled below
+    axpy(v.a, a, __ldg(&Fp[k]));
+    axpy(v.b, a, __ldg(&Fm[k]));
+  }
+  v = reduce_warps(v, warp, lane);
+  if (warp || t >= L) return;
+  double2 e = v.a, o = make_double2(0.0, 0.0);
+  if (m > 0) {
+    e = make_double2(v.a.x + v.b.x, v.a.y + v.b.y);
+    o = make_double2(v.a.x - v.b.x, v.a.y - v.b.y);
+  }
+  if (odd) {  // times i
+    e = make_double2(-e.y, e.x);
+    o = make_double2(-o.y, o.x);
+  }
+  const size_t at = ((size_t)b * L + m) * L + t;
+  work[at] = make_double2(2.0 * e.x, 2.0 * e.y);
+  work[(size_t)B * L * L + at] = make_double2(2.0 * o.x, 2.0 * o.y);
+}
+
+// phi inverse: E, O [2][b][m][t] -> f[b][t][p] = E + iO, f[b][t][N-1-p] = E - iO.
+__global__ void __launch_bounds__(32 * kWarps) direct_phi_inverse_kernel(int L, int B, const double* __restrict__ M,
+                                                                         const double2* __restrict__ work, double2* __restrict__ f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
+  const int p = 32 * blockIdx.y + lane, b = blockIdx.x / L, t = blockIdx.x - b * L;
+  const double* C = M + (size_t)kCosKX * L * L;
+  const double* S = M + (size_t)kSinKX * L * L;
+  const double2* E = work + (size_t)b * L * L + t;
+  const double2* O = E + (size_t)B * L * L;
+  Pair v;
+  v.a = v.b = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k = warp; k < L; k += kWarps) {
+    const double c = p < L ? __ldg(&C[(size_t)k * L + p]) : 0.0, sn = p < L ? __ldg(&S[(size_t)k * L + p]) : 0.0;
+    axpy(v.a, c, __ldg(&E[(size_t)k * L]));
+    axpy(v.b, sn, __ldg(&O[(size_t)k * L]));
+  }
+  v = reduce_warps(v, warp, lane);
+  if (warp || p >= L) return;
+  double2* row = f + ((size_t)b * L + t) * N;
+  row[p] = make_double2(v.a.x - v.b.y, v.a.y + v.b.x);
+  if (p < L - 1) row[N - 1 - p] = make_double2(v.a.x + v.b.y, v.a.y - v.b.x);
+}
+
+// phi of forward and adjoint: f [b][t][p] -> P, Q [2][b][t][m].  A warp folds 32 of its k's at a time.
+__global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, int B, const double* __restrict__ M,
+                                                                         const double2* __restrict__ f, double2* __restrict__ work) {
+  __shared__ double2 fold[kWarps][2][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
+  const int m = 32 * blockIdx.y + lane, b = blockIdx.x / L, t = blockIdx.x - b * L;
+  const double* C = M + (size_t)kCosXK * L * L;
+  const double* S = M + (size_t)kSinXK * L * L;
+  const double2* row = f + ((size_t)b * L + t) * N;
+  const int per = (L + kWarps - 1) / kWarps, k_end = min(L, (warp + 1) * per);
+  Pair v;
+  v.a = v.b = make_double2(0.0, 0.0);
+  for (int k0 = warp * per; k0 < k_end; k0 += 32) {
+    const int p = k0 + lane;
+    double2 e = make_double2(0.0, 0.0), o = e;
+    if (p < k_end) {
+      e = row[p];
+      if (p < L - 1) {
+        const double2 y = row[N - 1 - p];
+        o = make_double2(e.x - y.x, e.y - y.y);
+        e = make_double2(e.x + y.x, e.y + y.y);
+      }
+    }
+    __syncwarp();
+    fold[warp][0][lane] = e;
+    fold[warp][1][lane] = o;
+    __syncwarp();
+    const int n = min(32, k_end - k0);
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+      const double c = m < L ? __ldg(&C[(size_t)(k0 + i) * L + m]) : 0.0, sn = m < L ? __ldg(&S[(size_t)(k0 + i) * L + m]) : 0.0;
+      axpy(v.a, c, fold[warp][0][i]);
+      axpy(v.b, sn, fold[warp][1][i]);
+    }
+  }
+  v = reduce_warps(v, warp, lane);
+  if (warp || m >= L) return;
+  const size_t at = ((size_t)b * L + t) * L + m;
+  work[at] = v.a;
+  work[(size_t)B * L * L + at] = v.b;
+}
+
+// theta of forward (weight matrices) and adjoint (cosines and sines, the fold of m' < 0): P, Q -> H [b][m + Lp][m'].
+__global__ void __launch_bounds__(32 * kWarps) direct_theta_forward_kernel(int L, int s, int B, int adjoint,
+                                                                           const double* __restrict__ M,
+                                                                           const double2* __restrict__ work, double2* __restrict__ H) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
+  const int mp = 32 * blockIdx.y + lane, b = blockIdx.x / L, m = blockIdx.x - b * L;
+  const bool odd = (m + s) & 1;
+  const double* A = M + (size_t)(adjoint ? (odd ? kSinXK : kCosXK) : (odd ? kWeightO : kWeightE)) * L * L;
+  const double2* P = work + (size_t)b * L * L + m;
+  const double2* Q = P + (size_t)B * L * L;
+  Pair v;
+  v.a = v.b = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int k = warp; k < L; k += kWarps) {
+    const double a = mp < L ? __ldg(&A[(size_t)k * L + mp]) : 0.0;
+    axpy(v.a, a, __ldg(&P[(size_t)k * L]));
+    axpy(v.b, a, __ldg(&Q[(size_t)k * L]));
+  }
+  v = reduce_warps(v, warp, lane);
+  if (warp || mp >= L) return;
+  const double w = adjoint && mp > 0 ? 2.0 : 1.0;
+  double2 hp = make_double2(w * (v.a.x + v.b.y), w * (v.a.y - v.b.x)), hm = make_double2(w * (v.a.x - v.b.y), w * (v.a.y + v.b.x));
+  if (odd) {  // times -i
+    hp = make_double2(hp.y, -hp.x);
+    hm = make_double2(hm.y, -hm.x);
+  }
+  H[((size_t)b * N + L - 1 + m) * L + mp] = hp;
+  if (m > 0) H[((size_t)b * N + L - 1 - m) * L + mp] = hm;
+}
+
+}  // namespace
+
+struct DirectPlan {
+  int L = 0;
+  double* mats = nullptr;
+  size_t bytes = 0;
+};
+
+// Where the products beat the FFTs: for little work (B L^3 <= 2^23), where the FFTs' 11 launches and short
+// rows set the time, and up to L = 208 where N has a prime factor above 127, for which cuFFT changes to its slow
+// general transform.  GB300, torus stage of an inverse and a forward, FFTs against products: L = 64, B = 1 141 and
+// 43 us; L = 160, B = 1 329 and 162; L = 129, B = 4 (N = 257) 588 and 342; L = 192, B = 8 (N = 383) 2125 and 1633; beyond the
+// line L = 256, B = 1 372 and 515; L = 128, B = 16 (N = 255) 813 and 1008; L = 224, B = 4 (N = 3 149) 1267 and 1306.
+bool direct_wanted(int L, int B) {
+  if ((long long)B * L * L * L <= (1ll << 23)) return true;
+  int n = 2 * L - 1, largest = 1;
+  for (int q = 3; q * q <= n; q += 2)
+    while (n % q == 0) {
+      largest = std::max(largest, q);
+      n /= q;
+    }
+  return L <= 208 && std::max(largest, n) > 127;
+}
+
+cudaError_t direct_setup(DirectPlan** out, int L) {
+  *out = nullptr;
+  DirectPlan* p = new DirectPlan();
+  p->L = L;
+  const size_t n = (size_t)L * L, ncs = 2 * (size_t)(2 * L - 1);
+  double2* tmp = nullptr;
+  cudaError_t e = dev_malloc(&p->mats, kMatrices * n * sizeof(double));
+  if (e == cudaSuccess) {
+    p->bytes = kMatrices * n * sizeof(double);
+    e = dev_malloc(&tmp, (ncs + n) * sizeof(double2));
+  }
+  if (e == cudaSuccess) {
+    node_table_kernel<<<(unsigned)((ncs + 255) / 256), 256>>>(2 * L - 1, tmp);
+    weight_prefix_kernel<<<(unsigned)((L + 31) / 32), 32>>>(L, tmp, tmp + ncs);
+    direct_matrices_kernel<<<(unsigned)((n + 255) / 256), 256>>>(L, tmp, tmp + ncs, p->mats);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  }
+  if (tmp) cudaFree(tmp);
+  if (e != cudaSuccess) {
+    direct_destroy(p);
+    return e;
+  }
+  *out = p;
+  return cudaSuccess;
+}
+
+void direct_destroy(DirectPlan* p) {
+  if (!p) return;
+  if (p->mats) cudaFree(p->mats);
+  delete p;
+}
+
+size_t direct_bytes(const DirectPlan* p) { return p ? p->bytes : 0; }
+
+cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* F, void* work, void* f, cudaStream_t st, int step) {
+  const dim3 grid((unsigned)B * p->L, (p->L + 31) / 32);
+  if (step == 0)
+    direct_theta_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, p->mats, (const double2*)F, (double2*)work);
+  else
+    direct_phi_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)work, (double2*)f);
+  return cudaGetLastError();
+}
+
+cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* f, void* work, void* H, cudaStream_t st,
+                            int step) {
+  const dim3 grid((unsigned)B * p->L, (p->L + 31) / 32);
+  if (step == 0)
+    direct_phi_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)f, (double2*)work);
+  else
+    direct_theta_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, adjoint, p->mats, (const double2*)work, (double2*)H);
+  return cudaGetLastError();
+}
+
+}  // namespace ssht

@@ -47,6 +47,7 @@
 #include "ssht_internal.h"
 #include "bounds.cuh"
 #include "tc_common.cuh"
+#include "torus_matrices.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -777,35 +778,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) torus_g
 enum Matrix { kCosTheta = 0, kSinTheta, kCosPhiInv, kSinPhiInv, kCosPhiFwd, kSinPhiFwd, kWeightEven, kWeightOdd, kCosAdj, kSinAdj,
               kMatrices };
 
-// cs[r] = (cos, sin)(pi r / N), r < 2N
-__global__ void node_table_kernel(int N, double2* cs) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < 2 * N) cs[r] = make_double2(cospi((double)r / N), sinpi((double)r / N));
-}
-
-// Prefix sums over even p = 2q >= 0 of w_e(p) e^{ip x_t}, w_e(p) = 2/(1-p^2): T[q * L + t], q < L.
-__global__ void weight_prefix_kernel(int L, const double2* __restrict__ cs, double2* __restrict__ T) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, N = 2 * L - 1;
-  if (t >= L) return;
-  double2 sum = make_double2(0.0, 0.0);
-  const int step = (int)((2ll * (2 * t + 1)) % (2 * N));
-  int r = 0;
-  for (int q = 0; q < L; ++q) {
-    const double p = 2.0 * q, w = 2.0 / (1.0 - p * p);
-    const double2 e = cs[r];
-    sum.x += w * e.x;
-    sum.y += w * e.y;
-    T[(size_t)q * L + t] = sum;
-    r += step;
-    if (r >= 2 * N) r -= 2 * N;
-  }
-}
-
-// Entry (row, k) of matrix `which`.  The weight matrices: with the extension about theta = pi (ring
-// t = L-1 once, and zero for the odd parity) the DFT of column t is F_{m''} = c_t cos(m'' x_t) / N or
-// -i c_t sin(m'' x_t) / N, and H_{m'} = (2 - delta_{m'0}) 2 pi sum_{|m''| < L} F_{m''} w_e(m'' - m').  The sum is
-// e^{im' x} sum_p w_e(p) e^{ip x} over -(L-1) - m' <= p <= L-1 - m': prefix sums of both signs of p.  The
-// phi pass's 1/N rides along.
+// Entry (row, k) of matrix `which`.
 __device__ double matrix_entry(int which, const Shape& sh, const double2* cs, const double2* T, int row, int k) {
   const int L = sh.L, N = sh.N;
   auto at = [&](int order, int node) { return cs[(int)(((long long)order * (2 * node + 1)) % (2 * N))]; };
@@ -832,12 +805,7 @@ __device__ double matrix_entry(int which, const Shape& sh, const double2* cs, co
     default: break;
   }
   // kWeightEven, kWeightOdd: row m', k = t
-  if (k >= L || (which == kWeightOdd && (k == L - 1 || row == 0))) return 0.0;
-  const double2 up = T[(size_t)((L - 1 - row) / 2) * L + k], dn = T[(size_t)((L - 1 + row) / 2) * L + k];
-  const double sr = up.x + dn.x - 2.0, si = up.y - dn.y;  // sum over p of w_e(p) e^{ipx}; w_e(0) = 2 counted once
-  const double2 e = at(row, k);
-  const double c = (row == 0 ? 1.0 : 2.0) * 6.283185307179586476925 * (k == L - 1 ? 1.0 : 2.0) / ((double)N * N);
-  return c * (which == kWeightEven ? e.x * sr - e.y * si : e.x * si + e.y * sr);
+  return k >= L ? 0.0 : weight_entry(which == kWeightEven, L, cs, T, row, k);
 }
 
 // Tiles [i][chunk] of 128 rows x 32 K of one matrix times `scale`, split; a thread writes 8 K of a row.

@@ -1,0 +1,48 @@
+// Plan-time tables of the torus passes' matrices, shared by the tensor-core products (torus_gemm.cu) and
+// the FP64 ones (torus_direct.cu): cos and sin of the multiples of pi/N and the sin(theta) weight's matrices.
+#pragma once
+
+namespace ssht {
+namespace {
+
+// cs[r] = (cos, sin)(pi r / N), r < 2N
+static __global__ void node_table_kernel(int N, double2* cs) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r < 2 * N) cs[r] = make_double2(cospi((double)r / N), sinpi((double)r / N));
+}
+
+// Prefix sums over even p = 2q >= 0 of w_e(p) e^{ip x_t}, w_e(p) = 2/(1-p^2): T[q * L + t], q < L.
+static __global__ void weight_prefix_kernel(int L, const double2* __restrict__ cs, double2* __restrict__ T) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, N = 2 * L - 1;
+  if (t >= L) return;
+  double2 sum = make_double2(0.0, 0.0);
+  const int step = (int)((2ll * (2 * t + 1)) % (2 * N));
+  int r = 0;
+  for (int q = 0; q < L; ++q) {
+    const double p = 2.0 * q, w = 2.0 / (1.0 - p * p);
+    const double2 e = cs[r];
+    sum.x += w * e.x;
+    sum.y += w * e.y;
+    T[(size_t)q * L + t] = sum;
+    r += step;
+    if (r >= 2 * N) r -= 2 * N;
+  }
+}
+
+// Entry (m', t) of a weight matrix (parity even or odd).  With the extension about theta = pi (ring
+// t = L-1 once, and zero for the odd parity) the DFT of column t is F_{m''} = c_t cos(m'' x_t) / N or
+// -i c_t sin(m'' x_t) / N, and H_{m'} = (2 - delta_{m'0}) 2 pi sum_{|m''| < L} F_{m''} w_e(m'' - m').  The sum is
+// e^{im' x} sum_p w_e(p) e^{ip x} over -(L-1) - m' <= p <= L-1 - m': prefix sums of both signs of p.  The
+// phi pass's 1/N rides along; the odd parity's factor -i does not.
+__device__ __forceinline__ double weight_entry(bool even, int L, const double2* cs, const double2* T, int mp, int t) {
+  const int N = 2 * L - 1;
+  if (!even && (t == L - 1 || mp == 0)) return 0.0;
+  const double2 up = T[(size_t)((L - 1 - mp) / 2) * L + t], dn = T[(size_t)((L - 1 + mp) / 2) * L + t];
+  const double sr = up.x + dn.x - 2.0, si = up.y - dn.y;  // sum over p of w_e(p) e^{ipx}; w_e(0) = 2 counted once
+  const double2 e = cs[(int)(((long long)mp * (2 * t + 1)) % (2 * N))];
+  const double c = (mp == 0 ? 1.0 : 2.0) * 6.283185307179586476925 * (t == L - 1 ? 1.0 : 2.0) / ((double)N * N);
+  return c * (even ? e.x * sr - e.y * si : e.x * si + e.y * sr);
+}
+
+}  // namespace
+}  // namespace ssht
