@@ -153,18 +153,21 @@ __global__ void __launch_bounds__(256) pack_a_kernel(int L, int s, const Item* _
 
 // Inverse data tiles (m, c): V_m[l, j], l = 32 c + k, rows j = sign * NC/2 + 2b (real part) and
 // 2b + 1 (imaginary part), for 16 consecutive m at once.  For two fields at a time the coefficients
-// sf_{l,+-m} of the 32 degrees of chunk c are read as runs of 16 consecutive orders (coalesced; the next
-// two fields' are under way meanwhile) and turned around in shared memory.  Split-FP16: a thread then takes
+// sf_{l,+-m} of the 32 degrees of chunk c are read as runs of 16 consecutive orders (coalesced)
+// and turned around in shared memory.  Split-FP16: a thread then takes
 // 8 K of one order, sign and field, four neighbouring threads the 32 K of a tile row, so that they find the
 // row pair's power of two with two shuffles and store 16 bytes at a time.  Split-BF16: a warp takes a row
 // pair, a lane one K.  The rows of padding fields are written as zeros.  Fields run in slices of Bs, slice z
 // in its own tile region of xslice bytes, and a CTA takes kPackFields rows' worth of fields of a slice
-// (blockIdx.z: slice and group of fields), which keeps the GPU filled at small band-limits too.
+// (blockIdx.z: slice and group of fields), which keeps the GPU filled at small band-limits too.  Bound by HBM
+// traffic (1.1 GB at L = 1024, B = 64: 0.16 ms) and by how many loads are in flight: six CTAs on an SM (40
+// registers) take 0.28 ms where three with the next fields' loads under way (80 registers) took 0.47 and
+// a CTA of 64 KB staging with bulk stores 0.66; at L = 512, B = 32 42 us, 68 before.
 constexpr int kPackFields = 8;
 static int pack_v_groups(int NC) { return (NC / 4 + kPackFields - 1) / kPackFields; }
 
 template <bool BF>
-__global__ void __launch_bounds__(256) pack_v_kernel(int L, int s, int Btot, int Bs, size_t xslice, int NC,
+__global__ void __launch_bounds__(256, 6) pack_v_kernel(int L, int s, int Btot, int Bs, size_t xslice, int NC,
                                                      const int* __restrict__ xc0, const long long* __restrict__ xoff,
                                                      const float2* __restrict__ flm, uint8_t* __restrict__ X,
                                                      float* __restrict__ XS) {
@@ -184,35 +187,31 @@ __global__ void __launch_bounds__(256) pack_v_kernel(int L, int s, int Btot, int
   const int part_bytes = NC * 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b_end = min(bg + kPackFields, nb);
-  // 32 degrees l x (orders m0 .. m0 + 15, then -m0 .. -m0 - 15) of a field: four values a thread
-  float2 v[2][4];
-  auto load = [&](int b) {
+  // 32 degrees l x (orders m0 .. m0 + 15, then -m0 .. -m0 - 15) of a field: four values a thread, whose
+  // places in a field are the same for every field
+  int at[4];
+  unsigned have = 0, neg = 0;
 #pragma unroll
-    for (int f = 0; f < 2; ++f)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int q = threadIdx.x + 256 * i, lo = q >> 5, col = q & 31, sign = col >> 4, m = m0 + (col & 15);
-        const int l = c * TK + lo;
-        float2 x = make_float2(0.f, 0.f);
-        const long long fi = flm0 + (long long)(b + f) * L * L + (long long)l * l + l + (sign ? -m : m);
-        if (b + f < B && m < L && l < L && l >= m && l >= as && !(sign && m == 0) && in_bounds(fi, flm_n, kbPackVIn)) {
-          x = __ldg(&flm[fi]);
-          if (sign && (l & 1)) x = make_float2(-x.x, -x.y);
-        }
-        v[f][i] = x;
-      }
-  };
-  load(bg);
+  for (int i = 0; i < 4; ++i) {
+    const int q = threadIdx.x + 256 * i, lo = q >> 5, col = q & 31, sign = col >> 4, m = m0 + (col & 15);
+    const int l = c * TK + lo;
+    at[i] = l * l + l + (sign ? -m : m);
+    if (m < L && l < L && l >= m && l >= as && !(sign && m == 0)) have |= 1u << i;
+    if (sign && (l & 1)) neg |= 1u << i;
+  }
   for (int b = bg; b < b_end; b += 2) {
 #pragma unroll
-    for (int f = 0; f < 2; ++f)
+    for (int f = 0; f < 2; ++f) {
+      const long long f0 = flm0 + (long long)(b + f) * L * L;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int q = threadIdx.x + 256 * i;
-        sv[f][q >> 5][q & 31] = v[f][i];
+        float2 x = make_float2(0.f, 0.f);
+        if (((have >> i) & 1u) && b + f < B && in_bounds(f0 + at[i], flm_n, kbPackVIn)) x = __ldg(&flm[f0 + at[i]]);
+        sv[f][q >> 5][q & 31] = ((neg >> i) & 1u) ? make_float2(-x.x, -x.y) : x;
       }
+    }
     __syncthreads();
-    if (b + 2 < b_end) load(b + 2);
     if constexpr (BF) {
       for (int cb = warp; cb < 64; cb += 8) {
         const int f = cb >> 5, sign = (cb >> 4) & 1, m = m0 + (cb & 15), j = sign * half + 2 * (b + f);

@@ -172,107 +172,115 @@ __device__ __forceinline__ void store_rows64(const Operand& o, uint8_t* stage, i
 }
 
 // ---------------------------------------------------------------------------------------------
-// Packing of the operands that no pass's epilogue writes: a CTA takes 16 rows (a warp each) and 64 K
+// Packing of the operands that no pass's epilogue writes: a CTA takes 16 rows (a warp each) and 128 K
 // ---------------------------------------------------------------------------------------------
 
-// Largest magnitude of each of the four terms over the CTA's 16 warps.
-__device__ __forceinline__ void block_max4(float (&amax)[4], float (*sm)[4], int warp, int lane) {
+// A warp's lanes hold four terms (the real and imaginary parts of a sum and a difference, each a row of its
+// own) of K = 2 lane and 2 lane + 1 in each of two 64-K blocks, v[block][term][2]; the CTA's 16 warps are the 16
+// rows of the blocks that share a power of two.  The split parts are put together in shared memory in the
+// tiles' layout and leave as 2 KB bulk copies, one a term and chunk (stored by the threads, 4 bytes a lane,
+// the packing of L = 1024, B = 64 took 0.456 ms, now 0.397 by theta and 0.442 by phi; at L = 512, B = 32 60 us
+// and 53 / 55 us; bound by HBM traffic and the conversions).  Term i goes to rows row0[i] .. row0[i] + 15 of unit[i].
+__device__ __forceinline__ void pack_rows16(const Operand& o, const float (&v)[2][4][2], int kb0, const long long (&unit)[4],
+                                            const int (&row0)[4], uint8_t* sm, float (*smax)[8]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t mx[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) amax[i] = fmaxf(amax[i], __shfl_xor_sync(0xffffffffu, amax[i], d));
+  for (int i = 0; i < 8; ++i) {
+    const float m = fmaxf(fabsf(v[i >> 2][i & 3][0]), fabsf(v[i >> 2][i & 3][1]));
+    mx[i] = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+  }
   if (lane == 0) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sm[warp][i] = amax[i];
+    for (int i = 0; i < 8; ++i) smax[warp][i] = __uint_as_float(mx[i]);
   }
   __syncthreads();
+  const uint32_t off = sw128(warp, 4 * (lane & 15));
+  float mine = 0.f;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    float m = sm[lane & 15][i];
-#pragma unroll
-    for (int d = 8; d > 0; d >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, d));
-    amax[i] = m;
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(smax[lane & 15][i]));
+    float sc;
+    const float up = block_power(__uint_as_float(m), &sc);
+    if (lane == i) mine = sc;
+    uint32_t h, l;
+    split2(up * v[i >> 2][i & 3][0], up * v[i >> 2][i & 3][1], &h, &l);
+    // [term][block][chunk]: 16 rows of 128 bytes
+    uint8_t* t = sm + (((i & 3) * 4 + 2 * (i >> 2) + (lane >> 4)) << 11);
+    *(uint32_t*)(t + off) = h;
+    *(uint32_t*)(t + (off ^ 64u)) = l;
   }
-}
-
-// Splits and stores K = 2 lane and 2 lane + 1 of the block's row `row`; its first row stores the scale.
-__device__ __forceinline__ void store_pair(const Operand& o, long long unit, int kb, int row, int lane, float amax, float a,
-                                           float b) {
-  if (!in_bounds(unit, o.units, kbTorusTile) || !in_bounds(kb, o.chunks / 2, kbTorusTile)) return;
-  float sc;
-  const float up = block_power(amax, &sc);
-  if (lane == 0 && (row & 15) == 0) o.scale[((size_t)unit * (o.chunks / 2) + kb) * 8 + (row >> 4)] = sc;
-  uint8_t* t = o.x + ((size_t)unit * o.chunks + 2 * kb + (lane >> 4)) * kUnitBytes;
-  uint32_t h, l;
-  split2(a * up, b * up, &h, &l);
-  *(uint32_t*)(t + sw128(row, 4 * (lane & 15))) = h;
-  *(uint32_t*)(t + sw128(row, 64 + 4 * (lane & 15))) = l;
+  const int nkb = o.chunks / 2;
+  if (warp == 0 && lane < 8 && kb0 + (lane >> 2) < nkb) {
+    const int i = lane & 3;
+    if (in_bounds(unit[i], o.units, kbTorusTile))
+      o.scale[((size_t)unit[i] * nkb + kb0 + (lane >> 2)) * 8 + (row0[i] >> 4)] = mine;
+  }
+  fence_proxy_async();
+  __syncthreads();
+  if (warp == 0) {
+    if (lane < 16 && kb0 + ((lane >> 1) & 1) < nkb) {
+      const int i = lane >> 2;
+      if (in_bounds(unit[i], o.units, kbTorusTile))
+        bulk_s2g(o.x + ((size_t)unit[i] * o.chunks + 2 * kb0 + (lane & 3)) * kUnitBytes + row0[i] * 128, sm + (lane << 11), 2048);
+    }
+    bulk_commit();
+    bulk_wait_read<0>();
+  }
 }
 
 // F half rows [b][m + Lp][m'] -> theta-inverse units F_m +- F_{-m} (m = 0: F_0 and 0); a CTA takes 16
-// orders |m| of one parity.  blockIdx.x: (b, parity, 16 orders), blockIdx.y: 64 K.
+// orders |m| of one parity.  blockIdx.x: (b, parity, 16 orders), blockIdx.y: 128 K.
 __global__ void __launch_bounds__(512) pack_theta_kernel(Shape sh, int B, const float2* __restrict__ F, Operand o,
                                                          long long in_n) {
-  __shared__ float sm[16][4];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kb = blockIdx.y;
+  __shared__ __align__(1024) uint8_t sm[16 * 2048];
+  __shared__ float smax[16][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kb0 = 2 * blockIdx.y;
   const int nq = ((sh.L + 1) / 2 + 15) / 16, nqo = (sh.L / 2 + 15) / 16;  // blocks of even and of odd orders
   const int b = blockIdx.x / (nq + nqo), r = blockIdx.x - b * (nq + nqo), odd = r >= nq ? 1 : 0;
-  const int q = 16 * (r - odd * nq) + warp, am = 2 * q + odd;
+  const int q0 = 16 * (r - odd * nq), am = 2 * (q0 + warp) + odd;
   const long long rp = ((long long)b * sh.N + sh.L - 1 + am) * sh.L, rm = ((long long)b * sh.N + sh.L - 1 - am) * sh.L;
-  float2 e[2], d[2];
-  float amax[4] = {0.f, 0.f, 0.f, 0.f};
+  float v[2][4][2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int k = 64 * kb + 2 * lane + i;
+  for (int i = 0; i < 4; ++i) {
+    const int k = 64 * (kb0 + (i >> 1)) + 2 * lane + (i & 1);
     float2 x = make_float2(0.f, 0.f), y = x;
-    if (am < sh.L && k < sh.L && in_bounds(rp + k, in_n, kbTorusIn)) x = F[rp + k];
-    if (am < sh.L && k < sh.L && am > 0 && in_bounds(rm + k, in_n, kbTorusIn)) y = F[rm + k];
-    e[i] = make_float2(x.x + y.x, x.y + y.y);
-    d[i] = am > 0 ? make_float2(x.x - y.x, x.y - y.y) : make_float2(0.f, 0.f);
-    amax[0] = fmaxf(amax[0], fabsf(e[i].x));
-    amax[1] = fmaxf(amax[1], fabsf(e[i].y));
-    amax[2] = fmaxf(amax[2], fabsf(d[i].x));
-    amax[3] = fmaxf(amax[3], fabsf(d[i].y));
+    if (am < sh.L && k < sh.L && in_bounds(rp + k, in_n, kbTorusIn)) x = __ldg(&F[rp + k]);
+    if (am < sh.L && k < sh.L && am > 0 && in_bounds(rm + k, in_n, kbTorusIn)) y = __ldg(&F[rm + k]);
+    v[i >> 1][0][i & 1] = x.x + y.x;
+    v[i >> 1][1][i & 1] = x.y + y.y;
+    v[i >> 1][2][i & 1] = am > 0 ? x.x - y.x : 0.f;
+    v[i >> 1][3][i & 1] = am > 0 ? x.y - y.y : 0.f;
   }
-  block_max4(amax, sm, warp, lane);
-  const int g = (odd ? sh.gE : 0) + (q >> 6), row = q & 63;
-  const long long unit = 2 * ((long long)b * sh.G() + g);
-  store_pair(o, unit, kb, row, lane, amax[0], e[0].x, e[1].x);
-  store_pair(o, unit + 1, kb, row, lane, amax[1], e[0].y, e[1].y);
-  store_pair(o, unit, kb, 64 + row, lane, amax[2], d[0].x, d[1].x);
-  store_pair(o, unit + 1, kb, 64 + row, lane, amax[3], d[0].y, d[1].y);
+  const long long unit = 2 * ((long long)b * sh.G() + (odd ? sh.gE : 0) + (q0 >> 6));
+  const int row = q0 & 63;
+  pack_rows16(o, v, kb0, {unit, unit + 1, unit, unit + 1}, {row, row, 64 + row, 64 + row}, sm, smax);
 }
 
 // Samples f [b][t][p] -> phi-forward units: sums and differences of mirrored samples (p = L - 1 is
-// its own mirror image); a CTA takes 16 rings.  blockIdx.x: (b, 16 rings), blockIdx.y: 64 K.
+// its own mirror image); a CTA takes 16 rings.  blockIdx.x: (b, 16 rings), blockIdx.y: 128 K.
 __global__ void __launch_bounds__(512) pack_phi_kernel(Shape sh, int B, const float2* __restrict__ f, Operand o,
                                                        long long in_n) {
-  __shared__ float sm[16][4];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kb = blockIdx.y;
-  const int nt = (sh.L + 15) / 16, b = blockIdx.x / nt, t = 16 * (blockIdx.x - b * nt) + warp;
+  __shared__ __align__(1024) uint8_t sm[16 * 2048];
+  __shared__ float smax[16][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kb0 = 2 * blockIdx.y;
+  const int nt = (sh.L + 15) / 16, b = blockIdx.x / nt, t0 = 16 * (blockIdx.x - b * nt), t = t0 + warp;
   const long long at = ((long long)b * sh.L + t) * sh.N;
-  float2 e[2], d[2];
-  float amax[4] = {0.f, 0.f, 0.f, 0.f};
+  float v[2][4][2];
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int p = 64 * kb + 2 * lane + i;
+  for (int i = 0; i < 4; ++i) {
+    const int p = 64 * (kb0 + (i >> 1)) + 2 * lane + (i & 1);
     float2 x = make_float2(0.f, 0.f), y = x;
-    if (t < sh.L && p < sh.L && in_bounds(at + p, in_n, kbTorusIn)) x = f[at + p];
-    if (t < sh.L && p < sh.L - 1 && in_bounds(at + sh.N - 1 - p, in_n, kbTorusIn)) y = f[at + sh.N - 1 - p];
-    e[i] = make_float2(x.x + y.x, x.y + y.y);
-    d[i] = p < sh.L - 1 ? make_float2(x.x - y.x, x.y - y.y) : make_float2(0.f, 0.f);
-    amax[0] = fmaxf(amax[0], fabsf(e[i].x));
-    amax[1] = fmaxf(amax[1], fabsf(e[i].y));
-    amax[2] = fmaxf(amax[2], fabsf(d[i].x));
-    amax[3] = fmaxf(amax[3], fabsf(d[i].y));
+    if (t < sh.L && p < sh.L && in_bounds(at + p, in_n, kbTorusIn)) x = __ldg(&f[at + p]);
+    if (t < sh.L && p < sh.L - 1 && in_bounds(at + sh.N - 1 - p, in_n, kbTorusIn)) y = __ldg(&f[at + sh.N - 1 - p]);
+    v[i >> 1][0][i & 1] = x.x + y.x;
+    v[i >> 1][1][i & 1] = x.y + y.y;
+    v[i >> 1][2][i & 1] = p < sh.L - 1 ? x.x - y.x : 0.f;
+    v[i >> 1][3][i & 1] = p < sh.L - 1 ? x.y - y.y : 0.f;
   }
-  block_max4(amax, sm, warp, lane);
-  const long long half = o.units / 2, unit = (long long)b * sh.nT + (t >> 6);
-  const int row = t & 63;
-  store_pair(o, unit, kb, row, lane, amax[0], e[0].x, e[1].x);
-  store_pair(o, unit, kb, 64 + row, lane, amax[1], e[0].y, e[1].y);
-  store_pair(o, half + unit, kb, row, lane, amax[2], d[0].x, d[1].x);
-  store_pair(o, half + unit, kb, 64 + row, lane, amax[3], d[0].y, d[1].y);
+  const long long half = o.units / 2, unit = (long long)b * sh.nT + (t0 >> 6);
+  const int row = t0 & 63;
+  pack_rows16(o, v, kb0, {unit, unit, half + unit, half + unit}, {row, 64 + row, row, 64 + row}, sm, smax);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -898,6 +906,7 @@ cudaError_t torus_setup(TorusPlan** out, int L, int device) {
     }
     if ((e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, device)) != cudaSuccess) goto fail;
     p->pair = sh.nI > 1;
+    if ((e = prefer_shared(pack_theta_kernel)) != cudaSuccess || (e = prefer_shared(pack_phi_kernel)) != cudaSuccess) goto fail;
     if ((e = gemm_attr<kThetaInverse>()) != cudaSuccess || (e = gemm_attr<kPhiInverse>()) != cudaSuccess ||
         (e = gemm_attr<kPhiForward>()) != cudaSuccess || (e = gemm_attr<kThetaForward>()) != cudaSuccess)
       goto fail;
@@ -966,7 +975,7 @@ cudaError_t torus_inverse(const TorusPlan* p, int s, int B, void* F, size_t f_by
   TgArgs a{};
   if (step == 0) {
     const int blocks = ((sh.L + 1) / 2 + 15) / 16 + (sh.L / 2 + 15) / 16;
-    pack_theta_kernel<<<dim3((unsigned)(B * blocks), (unsigned)(sh.nKs / 2)), 512, 0, st>>>(sh, B, (const float2*)F, x, (long long)(f_bytes / sizeof(float2)));
+    pack_theta_kernel<<<dim3((unsigned)(B * blocks), (unsigned)((sh.nKs / 2 + 1) / 2)), 512, 0, st>>>(sh, B, (const float2*)F, x, (long long)(f_bytes / sizeof(float2)));
     a.in = x;
     a.out = y;
     *launches += 2;
@@ -987,7 +996,7 @@ cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const 
   const Operand y = operand(w2, pass_units(sh, kThetaForward, B), sh.nKs);
   TgArgs a{};
   if (step == 0) {
-    pack_phi_kernel<<<dim3((unsigned)(B * ((sh.L + 15) / 16)), (unsigned)(sh.nKs / 2)), 512, 0, st>>>(sh, B, (const float2*)f, x, (long long)(f_bytes / sizeof(float2)));
+    pack_phi_kernel<<<dim3((unsigned)(B * ((sh.L + 15) / 16)), (unsigned)((sh.nKs / 2 + 1) / 2)), 512, 0, st>>>(sh, B, (const float2*)f, x, (long long)(f_bytes / sizeof(float2)));
     a.in = x;
     a.out = y;
     *launches += 2;
