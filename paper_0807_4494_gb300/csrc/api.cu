@@ -78,16 +78,6 @@ const char* cufft_name(cufftResult r) {
     }                                                                                              \
   } while (0)
 
-// Smallest 2^a 3^b 5^c 7^d >= n (a length cuFFT handles with its fast radices).
-int good_fft_size(int n) {
-  for (int m = n > 1 ? n : 1;; ++m) {
-    int r = m;
-    for (int p : {2, 3, 5, 7})
-      while (r % p == 0) r /= p;
-    if (r == 1) return m;
-  }
-}
-
 bool is_device_pointer(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -112,10 +102,9 @@ struct ssht_plan_s {
   void* W2 = nullptr;
   size_t w_bytes = 0;  // each of W1, W2
   void* W3 = nullptr;
-  void* khat = nullptr;
   void* ph = nullptr;       // phase table, element precision
   double2* ph64 = nullptr;  // phase table, FP64
-  cufftHandle fft_phi = 0, fft_theta = 0, fft_conv = 0;
+  cufftHandle fft_phi = 0, fft_theta = 0;
   bool have_phi = false, have_theta = false, have_conv = false;
   void* stage_in = nullptr;
   size_t stage_in_bytes = 0;
@@ -128,7 +117,8 @@ struct ssht_plan_s {
   size_t bytes = 0;
   TcPlan* tc = nullptr;    // tensor-core contraction (precisions SSHT_TF32X3, SSHT_BF16X6)
   TorusPlan* torus = nullptr;  // fused torus passes of FP32 plans (FP64 plans: cuFFT Z2Z + glue)
-  DirectPlan* direct = nullptr;  // torus products of FP64 plans of small band-limit, in place of the FFTs
+  DigitPlan* digits = nullptr;   // torus products of FP64 plans
+  DirectPlan* direct = nullptr;  // ... and of those with little work
   // The Delta recursion (and the A packing) of a call runs on a second stream, forked from the
   // caller's stream at the start of the call and joined before the contraction, so that the
   // Delta-independent work of the call (the torus stage of forward/adjoint, data packing) runs
@@ -232,18 +222,10 @@ int dalloc(ssht_plan_t p, void** ptr, size_t bytes, const char* what) {
   return 0;
 }
 
-int exec_fft(const ssht_plan_t p, cufftHandle h, void* in, void* out, int dir, cudaStream_t st) {
+int run_dft(ssht_plan_t p, cufftHandle h, void* in, void* out, cudaStream_t st) {
   StageScope sc(p, SSHT_STAGE_FFT, st);
-  if (p->f64) {
-    SSHT_FFT(cufftExecZ2Z(h, (cufftDoubleComplex*)in, (cufftDoubleComplex*)out, dir), "cufftExecZ2Z");
-  } else {
-    SSHT_FFT(cufftExecC2C(h, (cufftComplex*)in, (cufftComplex*)out, dir), "cufftExecC2C");
-  }
+  SSHT_FFT(cufftExecZ2Z(h, (cufftDoubleComplex*)in, (cufftDoubleComplex*)out, CUFFT_FORWARD), "cufftExecZ2Z");
   return 0;
-}
-
-int run_dft(ssht_plan_t p, cufftHandle h, int sign, void* in, void* out, cudaStream_t st) {
-  return exec_fft(p, h, in, out, sign < 0 ? CUFFT_FORWARD : CUFFT_INVERSE, st);
 }
 
 // The torus passes of an FP32 plan (DFT along theta or phi with its glue), timed as FFT work.  Inverse:
@@ -273,7 +255,7 @@ int torus_analysis_pass(ssht_plan_t p, int step, int adjoint, const void* f, cud
 int make_fft(ssht_plan_t p, cufftHandle* h, bool* have, int n, size_t batch, const char* what) {
   if (batch > (size_t)0x7fffffff) return fail(SSHT_EUNSUPPORTED, std::string(what) + ": batch too large");
   int nn = n;
-  SSHT_FFT(cufftPlanMany(h, 1, &nn, nullptr, 1, n, nullptr, 1, n, p->f64 ? CUFFT_Z2Z : CUFFT_C2C, (int)batch), what);
+  SSHT_FFT(cufftPlanMany(h, 1, &nn, nullptr, 1, n, nullptr, 1, n, CUFFT_Z2Z, (int)batch), what);
   *have = true;
   size_t ws = 0;
   if (cufftGetSize(*h, &ws) == CUFFT_SUCCESS) p->bytes += ws;
@@ -283,7 +265,6 @@ int make_fft(ssht_plan_t p, cufftHandle* h, bool* have, int n, size_t batch, con
 int set_streams(ssht_plan_t p, cudaStream_t st) {
   if (p->have_phi) SSHT_FFT(cufftSetStream(p->fft_phi, st), "cufftSetStream");
   if (p->have_theta) SSHT_FFT(cufftSetStream(p->fft_theta, st), "cufftSetStream");
-  if (p->have_conv) SSHT_FFT(cufftSetStream(p->fft_conv, st), "cufftSetStream");
   return 0;
 }
 
@@ -433,17 +414,22 @@ int tc_multiply(ssht_plan_t p, int forward, void* dst, cudaStream_t st) {
   return 0;
 }
 
-// One torus product of an FP64 plan of small band-limit, timed as FFT work; which: 0, 1 the inverse's theta
-// and phi, 2 phi of forward and adjoint, 3, 4 theta of forward and adjoint.
-int direct_pass(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t st) {
+// One torus product of an FP64 plan, timed as FFT work; which: 0, 1 the inverse's theta and phi, 2 phi of
+// forward and adjoint, 3, 4 theta of forward and adjoint.  W1 (half rows) <-> W2 <-> samples.
+int fp64_pass(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t st) {
   StageScope sc(p, SSHT_STAGE_FFT, st);
   cudaError_t e;
-  if (which == 0) e = direct_inverse(p->direct, p->s, p->B, in, out, nullptr, st, 0);
-  else if (which == 1) e = direct_inverse(p->direct, p->s, p->B, nullptr, const_cast<void*>(in), out, st, 1);
-  else if (which == 2) e = direct_analysis(p->direct, 0, p->s, p->B, in, out, nullptr, st, 0);
-  else e = direct_analysis(p->direct, which == 4, p->s, p->B, nullptr, const_cast<void*>(in), out, st, 1);
+  if (p->digits) {
+    const size_t fb = p->pair_grid_bytes();
+    e = digits_pass(p->digits, which, p->s, p->B, in, which == 2 ? fb : p->w_bytes, p->W3, p->W1, p->w_bytes, out,
+                    which == 1 ? fb : p->w_bytes, p->delta.status, p->wait_ns, st);
+  } else if (which < 2) {
+    e = direct_inverse(p->direct, p->s, p->B, in, out, st, which);
+  } else {
+    e = direct_analysis(p->direct, which == 4, p->s, p->B, in, out, st, which - 2 > 0);
+  }
   SSHT_CUDA(e, "torus product");
-  p->launches += 1;
+  p->launches += !p->digits ? 1 : which == 1 ? 3 : 2;
   return 0;
 }
 
@@ -557,7 +543,7 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
     if ((rc = join_operands(p, st))) return rc;
     StageScope sc(p, SSHT_STAGE_INVERSE, st);
     SSHT_CUDA(contract_inverse_simt<T>(d, p->s, p->B, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W1, p->w_bytes,
-                                       p->ph64, p->torus || p->direct ? 1 : 0, st),
+                                       st),
               "inverse contraction");
     p->launches += 1;
   }
@@ -566,85 +552,39 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
     if ((rc = torus_inverse_pass(p, 0, f, st))) return rc;
     return torus_inverse_pass(p, 1, f, st);
   }
-  if (p->direct) {
-    if ((rc = direct_pass(p, 0, p->W1, p->W2, st))) return rc;
-    return direct_pass(p, 1, p->W2, f, st);
-  }
-  rc = run_dft(p, p->fft_theta, +1, p->W1, p->W2, st);
+  if ((rc = fp64_pass(p, 0, p->W1, p->W2, st))) return rc;
+  return fp64_pass(p, 1, p->W2, f, st);
+}
+
+// Front of the triangular forward: phi DFT, extension into the theta-DFT input, theta DFT in place in W1.
+int analysis_front(ssht_plan_t p, const void* f, cudaStream_t st) {
+  const Dims& d = p->d;
+  int rc = run_dft(p, p->fft_phi, const_cast<void*>(f), p->W2, st);
   if (rc) return rc;
   {
     StageScope sc(p, SSHT_STAGE_TORUS, st);
-    SSHT_CUDA(inv_theta_to_phi<T>(d, p->B, p->W2, p->W1, p->ph, st), "theta-to-phi transpose");
+    SSHT_CUDA(fwd_phi_to_theta(d, p->s, p->B, p->W2, p->W1, p->ph64, st), "phi-to-theta extension");
     p->launches += 1;
   }
-  return run_dft(p, p->fft_phi, +1, p->W1, f, st);
+  return run_dft(p, p->fft_theta, p->W1, p->W1, st);
 }
 
-// Shared front of the forward transform (mode 0) and the adjoint (mode 1): phi DFT,
-// extension (or zero rings) into the theta-DFT input, theta DFT in place in W1.
+// Forward, or (adjoint) the adjoint.
 template <typename T>
-int analysis_front(ssht_plan_t p, const void* f, int mode, cudaStream_t st) {
-  const Dims& d = p->d;
-  int rc = run_dft(p, p->fft_phi, -1, const_cast<void*>(f), p->W2, st);
-  if (rc) return rc;
-  {
-    StageScope sc(p, SSHT_STAGE_TORUS, st);
-    SSHT_CUDA(fwd_phi_to_theta<T>(d, p->s, p->B, mode, p->W2, p->W1, p->ph, st), "phi-to-theta extension");
-    p->launches += 1;
-  }
-  return run_dft(p, p->fft_theta, -1, p->W1, p->W1, st);
-}
-
-template <typename T>
-int forward_impl(ssht_plan_t p, const void* f, void* flm, cudaStream_t st) {
-  const Dims& d = p->d;
+int analysis_impl(ssht_plan_t p, int adjoint, const void* f, void* flm, cudaStream_t st) {
   int rc = begin_operands(p, 1, st);
   if (rc) return rc;
-  if (p->torus) return analysis_fp32(p, 0, f, flm, st);
-  if (p->direct) {
-    if ((rc = direct_pass(p, 2, f, p->W2, st)) || (rc = direct_pass(p, 3, p->W2, p->W1, st))) return rc;
-    return project<T>(p, p->W1, flm, st);
-  }
-  rc = analysis_front<T>(p, f, 0, st);
-  if (rc) return rc;
-  {
-    StageScope sc(p, SSHT_STAGE_TORUS, st);
-    SSHT_CUDA(fwd_theta_to_conv<T>(d, p->B, p->W1, p->W3, p->ph, st), "weight convolution input");
-    p->launches += 1;
-  }
-  if ((rc = exec_fft(p, p->fft_conv, p->W3, p->W3, CUFFT_FORWARD, st))) return rc;
-  {
-    StageScope sc(p, SSHT_STAGE_TORUS, st);
-    SSHT_CUDA(conv_multiply<T>(d, p->B, p->W3, p->khat, st), "weight convolution product");
-    p->launches += 1;
-  }
-  if ((rc = exec_fft(p, p->fft_conv, p->W3, p->W3, CUFFT_INVERSE, st))) return rc;
-  {
-    StageScope sc(p, SSHT_STAGE_TORUS, st);
-    SSHT_CUDA(conv_to_project<T>(d, p->B, p->W3, p->W1, st), "weight convolution output");
-    p->launches += 1;
-  }
+  if (p->torus) return analysis_fp32(p, adjoint, f, flm, st);
+  if ((rc = fp64_pass(p, 2, f, p->W2, st)) || (rc = fp64_pass(p, adjoint ? 4 : 3, p->W2, p->W1, st))) return rc;
   return project<T>(p, p->W1, flm, st);
 }
-
+template <typename T>
+int forward_impl(ssht_plan_t p, const void* f, void* flm, cudaStream_t st) {
+  return analysis_impl<T>(p, 0, f, flm, st);
+}
 template <typename T>
 int adjoint_impl(ssht_plan_t p, const void* g, void* flm, cudaStream_t st) {
-  const Dims& d = p->d;
-  int rc = begin_operands(p, 1, st);
-  if (rc) return rc;
-  if (p->torus) return analysis_fp32(p, 1, g, flm, st);
-  if (p->direct) {
-    if ((rc = direct_pass(p, 2, g, p->W2, st)) || (rc = direct_pass(p, 4, p->W2, p->W1, st))) return rc;
-    return project<T>(p, p->W1, flm, st);
-  }
-  rc = analysis_front<T>(p, g, 1, st);
-  if (rc) return rc;
-  {
-    StageScope sc(p, SSHT_STAGE_TORUS, st);
-    SSHT_CUDA(adj_theta_fold<T>(d, p->s, p->B, p->W1, p->W2, p->ph, st), "adjoint fold");
-    p->launches += 1;
-  }
-  return project<T>(p, p->W2, flm, st);
+  return analysis_impl<T>(p, 1, g, flm, st);
 }
 
 // Real spin-0 fields, two to a complex field: which = 0 inverse, 1 forward, 2 adjoint.
@@ -829,6 +769,7 @@ void release(ssht_plan_t p) {
   if (p->tc) tc_destroy(p->tc);
   if (p->torus) torus_destroy(p->torus);
   if (p->direct) direct_destroy(p->direct);
+  if (p->digits) digits_destroy(p->digits);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
   if (p->ev_free) cudaEventDestroy(p->ev_free);
@@ -837,10 +778,9 @@ void release(ssht_plan_t p) {
   if (p->aux) cudaStreamDestroy(p->aux);
   if (p->have_phi) cufftDestroy(p->fft_phi);
   if (p->have_theta) cufftDestroy(p->fft_theta);
-  if (p->have_conv) cufftDestroy(p->fft_conv);
   if (!p->delta_shared) delta_free(p->delta);
   lane_tables_free(p->lane);
-  void* ptrs[] = {p->U, p->Uf, p->W1, p->W2, p->W3, p->khat, p->ph, p->ph64, p->stage_in, p->stage_out, p->rc, p->rg};
+  void* ptrs[] = {p->U, p->Uf, p->W1, p->W2, p->W3, p->ph, p->ph64, p->stage_in, p->stage_out, p->rc, p->rg};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete p;
@@ -885,7 +825,6 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   p->d.L = L;
   p->d.Lp = L - 1;
   p->d.N = 2 * L - 1;
-  p->d.M = good_fft_size(4 * L - 3);
   p->s = s;
   p->B = B;
   p->precision = desc->precision;
@@ -919,9 +858,8 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   }
   if ((rc = dalloc(p, (void**)&p->U, tri(L) * sizeof(double), "spin column"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->Uf, tri(L) * sizeof(float), "spin column (FP32)"))) return bail(rc);
-  // FP64: full N x N torus rows and an M-point convolution buffer; FP32 (fused torus passes): half
-  // rows of N x L, or a pass's operand tiles.
-  const bool direct = p->f64 && direct_wanted(L, B);  // L^2 products twice over fit N x N rows but for L = 1
+  // FP64: full N x N torus rows (the triangular forward's; the products' half rows, and L x L twice over, fit
+  // but for L = 1) and the digits of a pass's data; FP32: half rows of N x L, or a pass's operand tiles.
   const size_t torus = p->f64 ? (size_t)B * std::max(d.N * d.N, 2) * p->elem : torus_workspace_bytes(L, B);
   if (pair && (rc = dalloc(p, &p->rc, (size_t)B * L * L * p->elem, "spin-pair coefficients"))) return bail(rc);
   if ((real || pair) && (ce = real_setup()) != cudaSuccess) {
@@ -935,10 +873,8 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, &p->W1, torus, "torus workspace 1"))) return bail(rc);
   if ((rc = dalloc(p, &p->W2, torus, "torus workspace 2"))) return bail(rc);
   p->w_bytes = torus;
-  if (p->f64 && !direct) {
-    if ((rc = dalloc(p, &p->W3, (size_t)B * d.N * d.M * p->elem, "convolution workspace"))) return bail(rc);
-    if ((rc = dalloc(p, &p->khat, (size_t)d.M * p->elem, "weight spectrum"))) return bail(rc);
-  }
+  const bool direct = p->f64 && direct_wanted(L, B);
+  if (p->f64 && !direct && (rc = dalloc(p, &p->W3, digits_workspace_bytes(L, s, B), "torus product workspace"))) return bail(rc);
   if ((rc = dalloc(p, &p->ph, (size_t)(2 * d.N - 1) * p->elem, "phase table"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->ph64, (size_t)(2 * d.N - 1) * sizeof(double2), "phase table"))) return bail(rc);
 
@@ -966,42 +902,13 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     if ((rc = make_fft(p, &p->fft_phi, &p->have_phi, d.N, (size_t)B * d.L, "cuFFT phi plan"))) return bail(rc);
     if ((rc = make_fft(p, &p->fft_theta, &p->have_theta, d.N, (size_t)B * d.N, "cuFFT theta plan"))) return bail(rc);
   }
-  if (direct) {  // the FFT plans above serve the triangular forward only
-    ce = direct_setup(&p->direct, L);
-    if (ce != cudaSuccess) {
-      release(p);
-      return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,
-                  std::string("torus product setup: ") + cudaGetErrorString(ce));
-    }
-    p->bytes += direct_bytes(p->direct);
-  } else if (p->f64) {
-    if ((rc = make_fft(p, &p->fft_conv, &p->have_conv, d.M, (size_t)B * d.N, "cuFFT convolution plan")))
-      return bail(rc);
-    // Weight spectrum: FFT of the even part of w(p) = int_0^pi sin(t) e^{ipt} dt.
-    cufftHandle k1;
-    int nn = d.M;
-    cufftResult r = cufftPlan1d(&k1, nn, CUFFT_Z2Z, 1);
-    if (r != CUFFT_SUCCESS) {
-      release(p);
-      return fail(SSHT_ECUDA, std::string("cuFFT weight plan: ") + cufft_name(r));
-    }
-    ce = make_weight_kernel<double>(d, p->khat, 0);
-    if (ce == cudaSuccess) r = cufftExecZ2Z(k1, (cufftDoubleComplex*)p->khat, (cufftDoubleComplex*)p->khat, CUFFT_FORWARD);
-    cudaError_t se = cudaDeviceSynchronize();
-    cufftDestroy(k1);
-    if (ce != cudaSuccess || r != CUFFT_SUCCESS || se != cudaSuccess) {
-      release(p);
-      return fail(SSHT_ECUDA, "weight spectrum setup failed");
-    }
-  } else {
-    ce = torus_setup(&p->torus, L, p->device);
-    if (ce != cudaSuccess) {
-      release(p);
-      return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,
-                  std::string("torus pass setup: ") + cudaGetErrorString(ce));
-    }
-    p->bytes += torus_bytes(p->torus);
+  ce = direct ? direct_setup(&p->direct, L) : p->f64 ? digits_setup(&p->digits, L, p->device) : torus_setup(&p->torus, L, p->device);
+  if (ce != cudaSuccess) {
+    release(p);
+    return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,
+                std::string("torus pass setup: ") + cudaGetErrorString(ce));
   }
+  p->bytes += direct_bytes(p->direct) + digits_bytes(p->digits) + torus_bytes(p->torus);
   if (desc->precision == SSHT_TF32X3 || desc->precision == SSHT_BF16X6) {
     ce = tc_setup(&p->tc, L, s, B, desc->precision == SSHT_BF16X6 ? 1 : 0, p->device);
     if (ce != cudaSuccess) {
@@ -1149,7 +1056,7 @@ int ssht_forward_triangular(ssht_plan_t p, const void* f, void* flm, void* strea
     dst = p->rc;
   }
   if ((rc = begin_operands(p, 1, st))) return rc;
-  if ((rc = analysis_front<double>(p, src, 0, st))) return rc;
+  if ((rc = analysis_front(p, src, st))) return rc;
   if ((rc = join_operands(p, st))) return rc;
   {
     StageScope sc(p, SSHT_STAGE_PROJECT, st);
@@ -1290,7 +1197,7 @@ int ssht_debug_fail_allocation(int n) {
 int ssht_debug_bounds(long long* count, int* site, long long* index, long long* extent) {
   if (!kBoundsChecked) return fail(SSHT_EUNSUPPORTED, "ssht_debug_bounds: this library was built without index checks");
   SSHT_CUDA(cudaDeviceSynchronize(), "synchronize");
-  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass, bounds_take_contract_tc, bounds_take_delta_column,
+  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass, bounds_take_torus_digits, bounds_take_contract_tc, bounds_take_delta_column,
                                           bounds_take_real, bounds_take_contract_simt};
   BoundsRecord first{};
   long long total = 0;

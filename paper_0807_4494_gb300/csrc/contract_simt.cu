@@ -4,9 +4,7 @@
 //   F_{m m'} = (-1)^s i^{-(m+s)} sum_{l >= max(|m|, m', |s|)} U_l[m'] Delta^l_{m' m} sf_lm,
 //   U_l[m'] = sqrt((2l+1)/4pi) Delta^l_{m',-s}.
 // Both signs of m share the products U Delta (Delta^l_{m',-m} = (-1)^{l+m'} Delta^l_{m' m}, eqn
-// wignerd_sym6), and so do the fields of a thread.  The result is written as the
-// input of the theta synthesis: F_{m m'} e^{i pi m'/N} at k = m' and, by eqn Ffourier_sym,
-// (-1)^{m+s} F_{m m'} e^{-i pi m'/N} at k = N - m' (the phase of eqn idft_spatial).
+// wignerd_sym6), and so do the fields of a thread.
 //
 // Projection (forward transform and adjoint), for l >= |s|:
 //   sf_lm = (-1)^s i^{m+s} sum_{m'=0}^{l} U_l[m'] Delta^l_{m' m} H_{m m'}
@@ -62,8 +60,7 @@ __global__ void __launch_bounds__(32 * kWarps) inverse_kernel(int L, int s, int 
                                                               const double* __restrict__ U,
                                                               const typename Cplx<T>::type* __restrict__ flm,
                                                               typename Cplx<T>::type* __restrict__ E,
-                                                              const double2* __restrict__ ph, int half, long long in_n,
-                                                              long long out_n) {
+                                                              long long in_n, long long out_n) {
   using C = typename Cplx<T>::type;
   __shared__ C part[kWarps][2 * FB][32];
   const int Lp = L - 1, N = 2 * L - 1;
@@ -98,7 +95,7 @@ __global__ void __launch_bounds__(32 * kWarps) inverse_kernel(int L, int s, int 
 #pragma unroll
   for (int j = 0; j < 2 * FB; ++j) part[warp][j][lane] = acc[j];
   __syncthreads();
-  // the warps' sums, phases and outputs: one (field, sign) a warp
+  // the warps' sums and outputs: one (field, sign) a warp
   for (int j = warp; j < 2 * FB; j += kWarps) {
     const int b = b0 + (j >> 1), sgn = j & 1;
     if (b >= B || mp > Lp || (sgn && m == 0)) continue;
@@ -111,25 +108,8 @@ __global__ void __launch_bounds__(32 * kWarps) inverse_kernel(int L, int s, int 
     const int mm = sgn ? -m : m;
     // +m: (-1)^{m'-m}; -m: (-1)^m (the row m of the table stands for Delta_{m' m})
     const C F = times_ik<C>(s, sgn ? m : mp - m, -(mm + s), ar, ai);
-    if (half) {
-      const long long o = ((long long)b * N + (mm + Lp)) * L + mp;
-      if (in_bounds(o, out_n, kbSimtOut)) E[o] = F;
-      continue;
-    }
-    const double Fr = F.x, Fi = F.y;
-    C v;
-    // theta phase e^{+-i pi m'/N}
-    const double2 eth = ph[(N - 1) + mp], ethc = ph[(N - 1) - mp];
-    const double sig = ((mm + s) & 1) ? -1.0 : 1.0;  // (-1)^{m+s}
-    const long long o = ((long long)b * N + (mm + Lp)) * N;
-    v.x = (T)(Fr * eth.x - Fi * eth.y);
-    v.y = (T)(Fr * eth.y + Fi * eth.x);
-    if (in_bounds(o + mp, out_n, kbSimtOut)) E[o + mp] = v;
-    if (mp > 0) {
-      v.x = (T)(sig * (Fr * ethc.x - Fi * ethc.y));
-      v.y = (T)(sig * (Fr * ethc.y + Fi * ethc.x));
-      if (in_bounds(o + N - mp, out_n, kbSimtOut)) E[o + N - mp] = v;
-    }
+    const long long o = ((long long)b * N + (mm + Lp)) * L + mp;
+    if (in_bounds(o, out_n, kbSimtOut)) E[o] = F;
   }
 }
 
@@ -225,10 +205,10 @@ __global__ void __launch_bounds__(32 * kWarps) project_kernel(int L, int s, int 
 
 template <typename T, int FB>
 static void launch_inverse(const Dims& d, int s, int B, const double* table, const double* U, const void* flm, size_t flm_bytes,
-                           void* E, size_t e_bytes, const double2* ph, int half, cudaStream_t st) {
+                           void* E, size_t e_bytes, cudaStream_t st) {
   using C = typename Cplx<T>::type;
   const dim3 grid((d.L + 31) / 32, d.L, (B + FB - 1) / FB);
-  inverse_kernel<T, FB><<<grid, 32 * kWarps, 0, st>>>(d.L, s, B, table, U, (const C*)flm, (C*)E, ph, half,
+  inverse_kernel<T, FB><<<grid, 32 * kWarps, 0, st>>>(d.L, s, B, table, U, (const C*)flm, (C*)E,
                                                       (long long)(flm_bytes / sizeof(C)), (long long)(e_bytes / sizeof(C)));
 }
 
@@ -245,12 +225,11 @@ static void launch_project(const Dims& d, int s, int B, const double* table, con
 // products U Delta and the loads of the table (a field is 4 of 5 FP64 instructions alone, 16 of 17 at 4).
 template <typename T>
 cudaError_t contract_inverse_simt(const Dims& d, int s, int B, const double* table, const double* U,
-                                  const void* flm, size_t flm_bytes, void* E, size_t e_bytes, const double2* ph, int half,
-                                  cudaStream_t st) {
-  if (B == 1) launch_inverse<T, 1>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, ph, half, st);
-  else if (B == 2) launch_inverse<T, 2>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, ph, half, st);
-  else if (sizeof(T) == 8 || B <= 4) launch_inverse<T, 4>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, ph, half, st);
-  else launch_inverse<T, sizeof(T) == 8 ? 4 : 8>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, ph, half, st);
+                                  const void* flm, size_t flm_bytes, void* E, size_t e_bytes, cudaStream_t st) {
+  if (B == 1) launch_inverse<T, 1>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, st);
+  else if (B == 2) launch_inverse<T, 2>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, st);
+  else if (sizeof(T) == 8 || B <= 4) launch_inverse<T, 4>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, st);
+  else launch_inverse<T, sizeof(T) == 8 ? 4 : 8>(d, s, B, table, U, flm, flm_bytes, E, e_bytes, st);
   return cudaGetLastError();
 }
 
@@ -267,9 +246,9 @@ cudaError_t contract_project_simt(const Dims& d, int s, int B, const double* tab
 }
 
 template cudaError_t contract_inverse_simt<double>(const Dims&, int, int, const double*, const double*, const void*, size_t, void*,
-                                                   size_t, const double2*, int, cudaStream_t);
+                                                   size_t, cudaStream_t);
 template cudaError_t contract_inverse_simt<float>(const Dims&, int, int, const double*, const double*, const void*, size_t, void*,
-                                                  size_t, const double2*, int, cudaStream_t);
+                                                  size_t, cudaStream_t);
 template cudaError_t contract_project_simt<double>(const Dims&, int, int, const double*, const double*, const void*, size_t, void*,
                                                    size_t, cudaStream_t);
 template cudaError_t contract_project_simt<float>(const Dims&, int, int, const double*, const double*, const void*, size_t, void*,

@@ -29,7 +29,6 @@ struct Dims {
   int L;   // exclusive band-limit
   int Lp;  // L - 1, the paper's inclusive band-limit
   int N;   // 2L - 1 torus samples per axis
-  int M;   // length of the zero-padded weight convolution, >= 4L - 3
 };
 
 // Records the message returned by ssht_last_error() and returns code.
@@ -87,13 +86,10 @@ cudaError_t delta_spin_column(const double* table, int L, int s, double* U, floa
 // ---------------------------------------------------------------------------
 // SIMT contractions (contract_simt.cu); T is double or float
 // ---------------------------------------------------------------------------
-// Inverse: half = 0 writes the theta-DFT input E[b][m + Lp][k], k = m' mod N, of the extended,
-// phase-shifted F (eqn fourier_coeff, eqn Ffourier_sym, eqn idft_spatial phase); half = 1 writes
-// the half rows F[b][m + Lp][m'], 0 <= m' < L, without phases (the torus passes' input).
+// Inverse: the half rows F[b][m + Lp][m'], 0 <= m' < L, of F (eqn fourier_coeff), the torus passes' input.
 template <typename T>
 cudaError_t contract_inverse_simt(const Dims& d, int s, int B, const double* table, const double* U,
-                                  const void* flm, size_t flm_bytes, void* E, size_t e_bytes, const double2* ph, int half,
-                                  cudaStream_t st);
+                                  const void* flm, size_t flm_bytes, void* F, size_t f_bytes, cudaStream_t st);
 // Projection: flm[b][l*l+l+m] = (-1)^s i^{m+s} c_l sum_{m'>=0} Delta_{m'm} Delta_{m',-s} H[b][m+Lp][m']
 template <typename T>
 cudaError_t contract_project_simt(const Dims& d, int s, int B, const double* table, const double* U,
@@ -241,53 +237,37 @@ cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const 
                            int* launches, int step);
 
 // ---------------------------------------------------------------------------
-// Torus passes of FP64 plans of small band-limit (torus_direct.cu)
+// Torus passes of FP64 plans (torus_digits.cu, torus_direct.cu)
 // ---------------------------------------------------------------------------
-// The same folded products as the FP32 plans' passes, in FP64 on CUDA cores.  F, H: half rows (double2)
-// [B][N][L]; work: 2 B L^2 double2; f: samples [B][L][N].
+// The same folded products as the FP32 plans' passes, on tensor cores with both operands in fixed-point digits,
+// or, with little work, in FP64 on CUDA cores.  F, H: half rows (double2) [B][m + L - 1][m']; E, O: [2][B][m][t];
+// P, Q: [2][B][t][m]; samples [B][t][p].
+struct DigitPlan;
+cudaError_t digits_setup(DigitPlan** out, int L, int device);  // synchronises
+void digits_destroy(DigitPlan* p);
+size_t digits_bytes(const DigitPlan* p);
+size_t digits_workspace_bytes(int L, int s, int B);
+// One pass: 0 theta of the inverse, F -> E, O; 1 its phi, E, O -> samples, by way of mid (E, O's size); 2 phi of forward
+// and adjoint, samples -> P, Q; 3 theta of the forward (with the extension and the sin(theta) weight), 4 of the adjoint, P, Q -> H.
+cudaError_t digits_pass(const DigitPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* work, void* mid,
+                        size_t mid_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st);
+
 struct DirectPlan;
-bool direct_wanted(int L, int B);  // whether a plan of this band-limit and batch takes them instead of the FFTs
+bool direct_wanted(int L, int B);  // whether a plan of this band-limit and batch takes the CUDA cores
 cudaError_t direct_setup(DirectPlan** out, int L);  // synchronises
 void direct_destroy(DirectPlan* p);
 size_t direct_bytes(const DirectPlan* p);
-// step 0: theta (F -> work), 1: phi (work -> f).
-cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* F, void* work, void* f, cudaStream_t st, int step);
-// step 0: phi (f -> work), 1: theta (work -> H; adjoint = 0 with the extension and the sin(theta) weight).
-cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* f, void* work, void* H, cudaStream_t st,
-                            int step);
+// step 0: theta (F -> E, O), 1: phi (E, O -> samples).
+cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, void* out, cudaStream_t st, int step);
+// step 0: phi (samples -> P, Q), 1: theta (P, Q -> H; adjoint = 0 with the extension and the sin(theta) weight).
+cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, void* out, cudaStream_t st, int step);
 
 // ---------------------------------------------------------------------------
 // Torus kernels (torus.cu)
 // ---------------------------------------------------------------------------
-// g[b][m+Lp][t] (theta-synthesis output, N per row) -> h[b][t][m mod N] * e^{i pi m / N}, t < L.
-template <typename T>
-cudaError_t inv_theta_to_phi(const Dims& d, int B, const void* g, void* h, const void* ph, cudaStream_t st);
-// X[b][t][k] (phi-DFT of the samples) -> ext[b][m+Lp][t'] (theta-DFT input).
-// mode 0: forward (per-m parity extension, factor e^{-i pi m/N}/N);
-// mode 1: adjoint (zero rings t' >= L, factor e^{-i pi m/N}).
-template <typename T>
-cudaError_t fwd_phi_to_theta(const Dims& d, int s, int B, int mode, const void* X, void* ext, const void* ph,
-                             cudaStream_t st);
-// Fk[b][m+Lp][k'] (theta-DFT) -> zero-padded conv input cx[b][m+Lp][j], j = m'' mod M,
-// value F_{m m''} = Fk[k'(m'')] e^{-i pi m''/N} / N.
-template <typename T>
-cudaError_t fwd_theta_to_conv(const Dims& d, int B, const void* Fk, void* cx, const void* ph, cudaStream_t st);
-// Pointwise product of the conv spectrum with the weight spectrum (real kernel, length M).
-template <typename T>
-cudaError_t conv_multiply(const Dims& d, int B, void* cx, const void* khat, cudaStream_t st);
-// Conv output y[b][m+Lp][j] -> H[b][m+Lp][m'] = c_{m'} y[m'] / M, m' in [0, Lp], c_0 = 2pi, else 4pi.
-template <typename T>
-cudaError_t conv_to_project(const Dims& d, int B, const void* y, void* H, cudaStream_t st);
-// Adjoint: Fk (theta-DFT of the zero-padded rings) -> folded H[b][m+Lp][m'], m' in [0, Lp]:
-// H'_{m m'} + (-1)^{m+s} H'_{m,-m'} (m' > 0), H'_{m 0} (m' = 0), H'_{m m'} = Fk[k'(m')] e^{-i pi m'/N}.
-template <typename T>
-cudaError_t adj_theta_fold(const Dims& d, int s, int B, const void* Fk, void* H, const void* ph, cudaStream_t st);
-// Weight kernel kappa[p mod M] = w_e(p) = 2/(1-p^2) for even |p| <= 2Lp (0 otherwise); its FFT is
-// the spectrum used by conv_multiply.  The phase table ph[k + N - 1] = e^{i pi k/N}, |k| < N, is
-// complex in the element precision T (double2 or float2).
-template <typename T>
-cudaError_t make_weight_kernel(const Dims& d, void* kappa, cudaStream_t st);
-
+// X[b][t][k] (phi-DFT of the samples) -> ext[b][m+Lp][t'] (theta-DFT input): the per-m parity extension, factor
+// e^{-i pi m/N}/N, with the phase table ph[k + N - 1] = e^{i pi k/N}, |k| < N.
+cudaError_t fwd_phi_to_theta(const Dims& d, int s, int B, const void* X, void* ext, const double2* ph, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Index checks of bounds-checked builds (bounds.cuh): each translation unit's record, copied out
@@ -297,6 +277,7 @@ struct BoundsRecord;
 cudaError_t bounds_take_torus_pass(BoundsRecord* r);
 cudaError_t bounds_take_contract_tc(BoundsRecord* r);
 cudaError_t bounds_take_delta_column(BoundsRecord* r);
+cudaError_t bounds_take_torus_digits(BoundsRecord* r);
 cudaError_t bounds_take_real(BoundsRecord* r);
 cudaError_t bounds_take_contract_simt(BoundsRecord* r);
 

@@ -1,15 +1,13 @@
-// Torus passes of FP64 plans of small band-limit: the folded cosine and sine products of the torus stage
-// (torus_gemm.cu gives the identities) in FP64 on CUDA cores, in place of cuFFT's transforms of odd length
-// and the kernels between them.
+// Torus passes of FP64 plans with little work: the folded cosine and sine products of the torus stage
+// (torus_gemm.cu gives the identities) in FP64 on CUDA cores, four launches an inverse + forward.
 //
 // Matrices are stored [k][row], so that a warp's lanes (32 rows) read them coalesced, and a data column is
 // read by the whole warp at one address.  A CTA computes 32 rows of one unit -- one order |m| (both signs), or
 // one ring -- as two complex columns, 4 FP64 multiply-adds a k; its eight warps take an eighth of the k's each
 // and add up at the end, which keeps every quarter of every SM busy down to the smallest band-limits.
 //
-// What bounds it: the FP64 pipe, 8 B L^3 flops a pass.  That grows faster than the FFTs' N^2 log N, but
-// those are far from any bound at these sizes (odd, often prime lengths; 11 launches an inverse + forward).
-// 1.07 TFLOP/s at L = 128, B = 16 (0.85 of the FP64 pipe's rate).
+// What bounds it: launches and latency at the smallest sizes, then the FP64 pipe, 8 B L^3 flops a pass
+// (1.07 TFLOP/s at L = 128, B = 16, 0.85 of its rate).  L = 64, B = 1: 43 us, by FFTs 141.
 #include "ssht_internal.h"
 #include "torus_matrices.cuh"
 
@@ -207,21 +205,11 @@ struct DirectPlan {
   size_t bytes = 0;
 };
 
-// Where the products beat the FFTs: for little work (B L^3 <= 2^23), where the FFTs' 11 launches and short
-// rows set the time, and up to L = 208 where N has a prime factor above 127, for which cuFFT changes to its slow
-// general transform.  GB300, torus stage of an inverse and a forward, FFTs against products: L = 64, B = 1 141 and
-// 43 us; L = 160, B = 1 329 and 162; L = 129, B = 4 (N = 257) 588 and 342; L = 192, B = 8 (N = 383) 2125 and 1633; beyond the
-// line L = 256, B = 1 372 and 515; L = 128, B = 16 (N = 255) 813 and 1008; L = 224, B = 4 (N = 3 149) 1267 and 1306.
-bool direct_wanted(int L, int B) {
-  if ((long long)B * L * L * L <= (1ll << 23)) return true;
-  int n = 2 * L - 1, largest = 1;
-  for (int q = 3; q * q <= n; q += 2)
-    while (n % q == 0) {
-      largest = std::max(largest, q);
-      n /= q;
-    }
-  return L <= 208 && std::max(largest, n) > 127;
-}
+// Where these products beat those of digits: for little work, where the digits' nine launches set the time, and
+// at band-limits that fill little of their tiles.  GB300, torus stage of an inverse and a forward in us, digits against these: L = 64, B = 1
+// 95 and 43; L = 96, B = 1 101 and 56; L = 128, B = 1 107 and 102; L = 16, B = 4096 2127 and 1727; L = 32, B = 128 193 and 185;
+// beyond the line L = 96, B = 2 104 and 85, L = 64, B = 8 98 and 103 (the two meet there); L = 144, B = 1 115 and 132; L = 128, B = 4 114 and 283.
+bool direct_wanted(int L, int B) { return L <= 32 || (long long)B * L * L * L <= (1ll << 21); }
 
 cudaError_t direct_setup(DirectPlan** out, int L) {
   *out = nullptr;
@@ -258,22 +246,21 @@ void direct_destroy(DirectPlan* p) {
 
 size_t direct_bytes(const DirectPlan* p) { return p ? p->bytes : 0; }
 
-cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* F, void* work, void* f, cudaStream_t st, int step) {
+cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, void* out, cudaStream_t st, int step) {
   const dim3 grid((unsigned)B * p->L, (p->L + 31) / 32);
   if (step == 0)
-    direct_theta_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, p->mats, (const double2*)F, (double2*)work);
+    direct_theta_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, p->mats, (const double2*)in, (double2*)out);
   else
-    direct_phi_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)work, (double2*)f);
+    direct_phi_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)in, (double2*)out);
   return cudaGetLastError();
 }
 
-cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* f, void* work, void* H, cudaStream_t st,
-                            int step) {
+cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, void* out, cudaStream_t st, int step) {
   const dim3 grid((unsigned)B * p->L, (p->L + 31) / 32);
   if (step == 0)
-    direct_phi_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)f, (double2*)work);
+    direct_phi_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)in, (double2*)out);
   else
-    direct_theta_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, adjoint, p->mats, (const double2*)work, (double2*)H);
+    direct_theta_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, adjoint, p->mats, (const double2*)in, (double2*)out);
   return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
-"""FP64 plans on both sides of the rule that chooses the torus stage -- products or FFTs (the batch and
-the factors of N = 2L - 1 decide) -- against the FP64 oracle in all three directions.
+"""FP64 plans on both sides of the rule that chooses the torus stage -- products on CUDA cores or of digits on
+tensor cores -- against the FP64 oracle in all three directions; the digits' scaling over the exponent range.
 
 Bound 1e-12 max-norm, that of the FP64 parity tests at L <= 256."""
 import numpy as np
@@ -22,10 +22,12 @@ def rel(a, b):
     return float(np.abs(a - b).max() / np.abs(b).max())
 
 
-# (L, s, B): smallest sizes; edges of 32 rows; N = 199 prime with a large batch (products); N = 255 = 3 5 17
-# and N = 189 = 3^3 7 with B L^3 just below and above 2^23 (products, FFTs); L = 209 (N = 3 139), above the line
+# (L, s, B): smallest sizes; edges of 32 rows and k's and of 128 rows; B L^3 on both sides of 2^21 (128, 1 and 129, 1); data
+# tiles of 16 and 32 columns with a last one not full; more than 512 k's (two segments of sums, and packing in two reads)
 @pytest.mark.parametrize("L,s,B", [(1, 0, 3), (2, -1, 2), (3, 2, 1), (32, 1, 2), (33, -2, 1), (65, 0, 2), (100, 2, 10),
-                                   (128, 1, 4), (128, -1, 5), (95, 0, 9), (95, 2, 10), (203, 1, 1), (209, 0, 1)])
+                                   (128, 1, 4), (128, -1, 5), (95, 0, 9), (95, 2, 10), (203, 1, 1), (209, 0, 1),
+                                   (32, -1, 80), (33, 0, 64), (33, -2, 70), (127, 1, 2), (128, 0, 1), (129, 2, 1), (161, 1, 7),
+                                   (513, 1, 1)])
 def test_both_torus_stages_match_oracle(L, s, B):
     from paper_0807_4494_gb300 import ssht
     flm = inputs.coeffs(L, s, B, seed=L + B)
@@ -39,3 +41,30 @@ def test_both_torus_stages_match_oracle(L, s, B):
     assert rel(f.cpu().numpy(), T.inverse(flm, L, s)) < 1e-12
     assert rel(fwd, T.forward(g, L, s)) < 1e-12
     assert rel(adj, T.adjoint(g, L, s)) < 1e-12
+
+
+def test_powers_of_two_and_non_finite_rows():
+    """Fixed point with a row's own power of two: scaling a field by 2^k scales the outputs exactly, and a field
+    with a NaN or an infinity leaves the other fields' outputs as they are."""
+    from paper_0807_4494_gb300 import ssht
+    L, s, B = 140, 1, 5
+    x = torch.from_numpy(inputs.coeffs(L, s, B, seed=3)).cuda()
+    plan = ssht.Plan(L, s, B, precision="fp64")
+    f = plan.inverse(x)
+    y, a = plan.forward(f), plan.adjoint(f)
+    for k in (-900, -300, 37, 800):
+        fk = plan.inverse(x * 2.0 ** k)
+        assert torch.equal(fk, f * 2.0 ** k)
+        assert torch.equal(plan.forward(fk), y * 2.0 ** k)
+        assert torch.equal(plan.adjoint(fk), a * 2.0 ** k)
+    bad = x.clone()
+    bad[1, 7] = float("nan")
+    bad[3, 9] = float("inf")
+    fb = plan.inverse(bad)
+    yb = plan.forward(fb)
+    plan.check()
+    keep = [0, 2, 4]
+    assert torch.equal(fb[keep], f[keep]) and torch.equal(yb[keep], y[keep])
+    for b in (1, 3):
+        assert not torch.isfinite(torch.view_as_real(fb[b])).any()
+        assert not torch.isfinite(torch.view_as_real(yb[b])).all()
