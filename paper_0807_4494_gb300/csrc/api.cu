@@ -119,6 +119,7 @@ struct ssht_plan_s {
   TorusPlan* torus = nullptr;  // fused torus passes of FP32 plans (FP64 plans: cuFFT Z2Z + glue)
   DigitPlan* digits = nullptr;   // torus products of FP64 plans
   DirectPlan* direct = nullptr;  // ... and of those with little work
+  bool contract_digits = false;  // FP64 contractions on tensor cores
   // The Delta recursion (and the A packing) of a call runs on a second stream, forked from the
   // caller's stream at the start of the call and joined before the contraction, so that the
   // Delta-independent work of the call (the torus stage of forward/adjoint, data packing) runs
@@ -454,9 +455,14 @@ int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st) {
   if ((rc = join_operands(p, st))) return rc;
   {
     StageScope sc(p, SSHT_STAGE_PROJECT, st);
-    SSHT_CUDA(contract_project_simt<T>(p->d, p->s, p->B, p->delta.table, p->U, H, p->w_bytes, flm, p->pair_coeff_bytes(), st),
-              "projection");
-    p->launches += 1;
+    if (p->contract_digits)
+      SSHT_CUDA(contract_digits(1, p->d.L, p->s, p->B, p->delta.sms, p->delta.table, p->U, H, p->w_bytes, p->W3, flm,
+                                p->pair_coeff_bytes(), p->delta.status, p->wait_ns, st),
+                "projection");
+    else
+      SSHT_CUDA(contract_project_simt<T>(p->d, p->s, p->B, p->delta.table, p->U, H, p->w_bytes, flm, p->pair_coeff_bytes(), st),
+                "projection");
+    p->launches += p->contract_digits ? 2 : 1;
   }
   return mark_free(p, st);
 }
@@ -542,10 +548,15 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
   } else {
     if ((rc = join_operands(p, st))) return rc;
     StageScope sc(p, SSHT_STAGE_INVERSE, st);
-    SSHT_CUDA(contract_inverse_simt<T>(d, p->s, p->B, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W1, p->w_bytes,
-                                       st),
-              "inverse contraction");
-    p->launches += 1;
+    if (p->contract_digits)
+      SSHT_CUDA(contract_digits(0, d.L, p->s, p->B, p->delta.sms, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W3, p->W1,
+                                p->w_bytes, p->delta.status, p->wait_ns, st),
+                "inverse contraction");
+    else
+      SSHT_CUDA(contract_inverse_simt<T>(d, p->s, p->B, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W1, p->w_bytes,
+                                         st),
+                "inverse contraction");
+    p->launches += p->contract_digits ? 2 : 1;
   }
   if (!p->tc && (rc = mark_free(p, st))) return rc;
   if (p->torus) {
@@ -874,7 +885,18 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, &p->W2, torus, "torus workspace 2"))) return bail(rc);
   p->w_bytes = torus;
   const bool direct = p->f64 && direct_wanted(L, B);
-  if (p->f64 && !direct && (rc = dalloc(p, &p->W3, digits_workspace_bytes(L, s, B), "torus product workspace"))) return bail(rc);
+  p->contract_digits = p->f64 && !direct && contract_digits_wanted(L, B);
+  if (p->f64 && !direct) {
+    size_t w3 = digits_workspace_bytes(L, s, B);
+    if (p->contract_digits) {
+      w3 = std::max(w3, contract_digits_bytes(L, B));
+      if ((ce = contract_digits_setup()) != cudaSuccess) {
+        release(p);
+        return fail(SSHT_ECUDA, std::string("contraction setup: ") + cudaGetErrorString(ce));
+      }
+    }
+    if ((rc = dalloc(p, &p->W3, w3, "operand digits"))) return bail(rc);
+  }
   if ((rc = dalloc(p, &p->ph, (size_t)(2 * d.N - 1) * p->elem, "phase table"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->ph64, (size_t)(2 * d.N - 1) * sizeof(double2), "phase table"))) return bail(rc);
 
@@ -1197,7 +1219,7 @@ int ssht_debug_fail_allocation(int n) {
 int ssht_debug_bounds(long long* count, int* site, long long* index, long long* extent) {
   if (!kBoundsChecked) return fail(SSHT_EUNSUPPORTED, "ssht_debug_bounds: this library was built without index checks");
   SSHT_CUDA(cudaDeviceSynchronize(), "synchronize");
-  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass, bounds_take_torus_digits, bounds_take_contract_tc, bounds_take_delta_column,
+  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass, bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc, bounds_take_delta_column,
                                           bounds_take_real, bounds_take_contract_simt};
   BoundsRecord first{};
   long long total = 0;

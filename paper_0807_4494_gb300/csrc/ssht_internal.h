@@ -262,6 +262,15 @@ cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, vo
 // step 0: phi (samples -> P, Q), 1: theta (P, Q -> H; adjoint = 0 with the extension and the sin(theta) weight).
 cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, void* out, cudaStream_t st, int step);
 
+// The contractions of FP64 plans on tensor cores (contract_digits.cu): the same results as
+// contract_inverse_simt (forward = 0) and contract_project_simt, with a workspace for the data columns.
+bool contract_digits_wanted(int L, int B);
+size_t contract_digits_bytes(int L, int B);
+cudaError_t contract_digits_setup();
+cudaError_t contract_digits(int forward, int L, int s, int B, int sms, const double* table, const double* U, const void* in,
+                            size_t in_bytes, void* work, void* out, size_t out_bytes, int* status, long long wait_ns,
+                            cudaStream_t st);
+
 // ---------------------------------------------------------------------------
 // Torus kernels (torus.cu)
 // ---------------------------------------------------------------------------
@@ -278,6 +287,7 @@ cudaError_t bounds_take_torus_pass(BoundsRecord* r);
 cudaError_t bounds_take_contract_tc(BoundsRecord* r);
 cudaError_t bounds_take_delta_column(BoundsRecord* r);
 cudaError_t bounds_take_torus_digits(BoundsRecord* r);
+cudaError_t bounds_take_contract_digits(BoundsRecord* r);
 cudaError_t bounds_take_real(BoundsRecord* r);
 cudaError_t bounds_take_contract_simt(BoundsRecord* r);
 

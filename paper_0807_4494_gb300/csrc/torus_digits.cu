@@ -21,16 +21,13 @@
 #include <cstdint>
 
 #include "bounds.cuh"
+#include "digits.cuh"
 #include "ssht_internal.h"
-#include "tc_common.cuh"
 #include "torus_matrices.cuh"
 
 namespace ssht {
 namespace {
 
-using namespace tc;
-
-constexpr int kDigits = 8;
 constexpr int kChunkK = 32;                                  // k's of a tile
 constexpr int kMatTile = 128 * kChunkK * kDigits * 2;        // four parts of 128 rows x 128 bytes: two digits' 32 k's
 template <int PAIRS> constexpr int kDataTile = 2 * PAIRS * kChunkK * kDigits * 2;  // PAIRS complex columns
@@ -39,7 +36,6 @@ constexpr int kStages = 2;
 constexpr int kSegChunks = 16;                               // chunks whose sums stay exact: 512 k
 constexpr int kEpiWarps = 16, kThreads = 128 + 32 * kEpiWarps;
 constexpr int kRegsIssue = 32, kRegsEpilogue = 112;          // 128 * 32 + 512 * 112 = 640 * 96
-constexpr int kNotFinite = 1 << 20;                          // exponent of a row that holds an infinity or a NaN
 template <int PAIRS> constexpr size_t kSmem = (size_t)kStages * kStageBytes<PAIRS> + 1024;
 
 enum Pass { kThetaInverse = 0, kPhiInverse, kPhiForward, kThetaForward, kThetaAdjoint };
@@ -68,69 +64,6 @@ Sets sets_of(int pass, int L, int s, int B, int pairs) {
 }
 
 __host__ __device__ inline int chunks_of(int L) { return (L + kChunkK - 1) / kChunkK; }
-
-// Exponent field of x (1 for denormals and zero), or kNotFinite.
-__device__ __forceinline__ int exponent_of(double x) {
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return e == 0x7ff ? kNotFinite : max(e, 1);
-}
-
-// x in units of 2^(e - 1077), rounded to nearest, e >= its own exponent field: at most 55 bits.
-__device__ __forceinline__ long long fixed_point(double x, int e) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)(u >> 52) & 0x7ff;
-  unsigned long long m = (u & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
-  const int sh = e - max(ex, 1);
-  m = sh > 55 ? 0ull : sh > 0 ? ((m << 2) + (1ull << (sh - 1))) >> sh : m << 2;
-  return (u >> 63) ? -(long long)m : (long long)m;
-}
-
-// The digits of eight consecutive k's of a row go to 16 bytes a digit: with 64 sum_i 128^i added, digit i is
-// the plain field of seven bits less 64 (the top one takes 0 .. 128), and 0x6400 + n is the FP16 number 1024 + n.
-template <int PART_BYTES>
-__device__ __forceinline__ void put_digits(uint8_t* tile, int row, int piece, const double (&x)[8], int e) {
-  unsigned long long v[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = (unsigned long long)(fixed_point(x[k], e) + 0x81020408102040ll);
-  const __half2 bias = __float2half2_rn(1088.f);
-#pragma unroll
-  for (int i = 0; i < kDigits; ++i) {
-    uint32_t w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      uint32_t a = (uint32_t)(v[2 * k] >> (7 * (7 - i))), b = (uint32_t)(v[2 * k + 1] >> (7 * (7 - i)));
-      if (i > 0) {
-        a &= 127u;
-        b &= 127u;
-      }
-      const uint32_t bits = 0x64006400u + a + (b << 16);
-      const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&bits), bias);
-      w[k] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    *(uint4*)(tile + (i >> 1) * PART_BYTES + sw128(row, 64 * (i & 1) + 16 * piece)) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-// (hi 2^28 + lo) 2^e, rounded to nearest.  Integer instructions: a conversion or product on the FP64 pipe takes a warp 64 clocks.
-__device__ __forceinline__ double assemble(long long hi, long long lo, int e) {
-  long long h = hi + (lo >> 28);
-  unsigned l = (unsigned)lo & 0xfffffffu;
-  const bool neg = h < 0;
-  if (neg) {
-    h = -h - (l ? 1 : 0);
-    l = (0u - l) & 0xfffffffu;
-  }
-  const int z = min(__clzll(h), 28);
-  unsigned long long m = ((unsigned long long)h << z) | (l >> (28 - z));
-  const int c = __clzll((long long)m);
-  if (m) m <<= c;
-  m = (m >> 11) + ((m >> 10) & 1);
-  const int E = e + (28 - z) - c + 63 + 1023;
-  if (m == 0 && E < kNotFinite / 2) return 0.0;
-  if (E >= 1 && E <= 2045) return __longlong_as_double((long long)(((unsigned long long)(E - 1) << 52) + m) | (neg ? (1ll << 63) : 0ll));
-  if (E >= kNotFinite / 2) return __longlong_as_double(0x7ff8000000000000ll);
-  return (neg ? -1.0 : 1.0) * scalbn((double)m, E - 1023 - 52);
-}
 
 // ---------------------------------------------------------------------------------------------
 // Matrices
@@ -162,7 +95,7 @@ __global__ void __launch_bounds__(128) digit_matrices_kernel(int L, const double
     double x[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) x[k] = entry(which, L, cs, T, r, 8 * g + k);
-    put_digits<128 * 128>(t + (size_t)(g >> 2) * kMatTile, r & 127, g & 3, x, e);
+    put_digits<kDigits, 128 * 128>(t + (size_t)(g >> 2) * kMatTile, r & 127, g & 3, x, e);
   }
 }
 
@@ -282,7 +215,7 @@ __global__ void __launch_bounds__(kPackThreads) digit_pack_kernel(const __grid_c
       const int tile = (set ? a.q.tiles[0] : 0) + col / PAIRS, row = 2 * (col % PAIRS) + (r & 1), e = top[so][r];
       if (!in_bounds(tile, a.q.all(), kbTorusTile)) continue;
       if (g == 0) a.exps[tile * 2 * PAIRS + row] = e;
-      put_digits<2 * PAIRS * 128>(a.x + ((size_t)tile * nc + (g >> 2)) * kDataTile<PAIRS>, row, g & 3, x[r], e);
+      put_digits<kDigits, 2 * PAIRS * 128>(a.x + ((size_t)tile * nc + (g >> 2)) * kDataTile<PAIRS>, row, g & 3, x[r], e);
     }
   }
 }
@@ -315,9 +248,6 @@ __device__ __forceinline__ Item item_of(const GemmArgs& a, int w) {
   t.u = t.j >= a.q.tiles[0];
   return t;
 }
-
-// Whether the CTA still works, the same answer for the whole (converged) warp.
-__device__ __forceinline__ bool going(volatile int* abort) { return !__any_sync(0xffffffffu, *abort); }
 
 template <int PASS, int PAIRS>
 __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_constant__ GemmArgs a) {

@@ -1,5 +1,6 @@
 """FP64 plans on both sides of the rule that chooses the torus stage -- products on CUDA cores or of digits on
-tensor cores -- against the FP64 oracle in all three directions; the digits' scaling over the exponent range.
+tensor cores -- and of the one that chooses the contractions, against the FP64 oracle in all three directions; the
+digits' scaling over the exponent range.
 
 Bound 1e-12 max-norm, that of the FP64 parity tests at L <= 256."""
 import numpy as np
@@ -23,11 +24,14 @@ def rel(a, b):
 
 
 # (L, s, B): smallest sizes; edges of 32 rows and k's and of 128 rows; B L^3 on both sides of 2^21 (128, 1 and 129, 1); data
-# tiles of 16 and 32 columns with a last one not full; more than 512 k's (two segments of sums, and packing in two reads)
+# tiles of 16 and 32 columns with a last one not full; more than 512 k's (two segments of sums, and packing in two reads);
+# contractions of digits (B L^3 > 2^23, 64 <= L <= 512): one to nine fields in groups of four, edges of 32 k's and 128 rows, |s|
+# beyond the first row blocks
 @pytest.mark.parametrize("L,s,B", [(1, 0, 3), (2, -1, 2), (3, 2, 1), (32, 1, 2), (33, -2, 1), (65, 0, 2), (100, 2, 10),
                                    (128, 1, 4), (128, -1, 5), (95, 0, 9), (95, 2, 10), (203, 1, 1), (209, 0, 1),
                                    (32, -1, 80), (33, 0, 64), (33, -2, 70), (127, 1, 2), (128, 0, 1), (129, 2, 1), (161, 1, 7),
-                                   (513, 1, 1)])
+                                   (513, 1, 1), (128, 0, 5), (129, 2, 4), (129, -64, 5), (64, 1, 33), (64, -63, 33), (100, 0, 9),
+                                   (257, -2, 1), (384, 1, 1), (512, 0, 1)])
 def test_both_torus_stages_match_oracle(L, s, B):
     from paper_0807_4494_gb300 import ssht
     flm = inputs.coeffs(L, s, B, seed=L + B)
