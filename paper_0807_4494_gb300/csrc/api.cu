@@ -1011,8 +1011,15 @@ int ssht_inverse(ssht_plan_t p, const void* flm, void* f, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   if ((rc = set_streams(p, st))) return rc;
   IO io;
-  if ((rc = io_begin(p, flm, p->coeff_bytes(), f, p->grid_bytes(), st, &io))) return rc;
-  if (p->real)
+  // spin pairs from host memory: the inverse reads the coefficients of spin s only, so those alone cross the host
+  // link, to where pair_gather would put them (L = 512, 24 pairs: 50 of 100 MB; inverse and forward 1.88 -> 1.63 ms)
+  const bool half = p->pair && flm && f && !is_device_pointer(flm);
+  if ((rc = io_begin(p, half ? p->rc : flm, p->coeff_bytes(), f, p->grid_bytes(), st, &io))) return rc;
+  if (half) {
+    const size_t n = (size_t)p->d.L * p->d.L * p->elem;
+    SSHT_CUDA(cudaMemcpy2DAsync(p->rc, n, flm, 2 * n, n, p->B, cudaMemcpyHostToDevice, st), "input copy to device");
+    rc = p->f64 ? inverse_impl<double>(p, p->rc, io.out_dev, st) : inverse_impl<float>(p, p->rc, io.out_dev, st);
+  } else if (p->real)
     rc = p->f64 ? real_call<double>(p, 0, io.in_dev, io.out_dev, st) : real_call<float>(p, 0, io.in_dev, io.out_dev, st);
   else if (p->pair)
     rc = p->f64 ? pair_call<double>(p, 0, io.in_dev, io.out_dev, st) : pair_call<float>(p, 0, io.in_dev, io.out_dev, st);
