@@ -227,15 +227,18 @@ def quadrant_entries(L):
 
 
 def torus_M(L):
-    """FFT length of the torus passes' Bluestein DFTs of length N = 2L - 1."""
+    """Power of two for a Bluestein DFT of the torus' odd length N = 2L - 1, the work a transform of fast
+    Fourier passes would count (the torus passes here are matrix products)."""
     M = 128
     while M < 2 * (2 * L - 1) - 1:
         M *= 2
     return M
 
 
-def fft_flops(M):
-    return 5.0 * M * np.log2(M)
+def torus_pass_flops(L, B):
+    """Real products and sums of one torus pass: per field L cosine or sine sums of length L for 2L complex
+    columns (orders, or rings of both parities), 2 flops a real part."""
+    return 8.0 * B * float(L) ** 3
 
 
 KERNEL_SOURCES = {
@@ -249,10 +252,11 @@ KERNEL_SOURCES = {
     "tc_gemm_kernel<inverse>": ["paper_0807_4494_gb300/csrc/contract_tc.cu"],
     "tc_gemm_kernel<forward>": ["paper_0807_4494_gb300/csrc/contract_tc.cu"],
     "pack_v_kernel": ["paper_0807_4494_gb300/csrc/contract_tc.cu"],
-    "inverse_theta_kernel": ["paper_0807_4494_gb300/csrc/torus_pass.cu"],
-    "phi_kernel<+1>": ["paper_0807_4494_gb300/csrc/torus_pass.cu"],
-    "phi_kernel<-1>": ["paper_0807_4494_gb300/csrc/torus_pass.cu"],
-    "forward_theta_kernel": ["paper_0807_4494_gb300/csrc/torus_pass.cu"],
+    "torus_gemm_kernel<theta inverse>": ["paper_0807_4494_gb300/csrc/torus_gemm.cu", "paper_0807_4494_gb300/csrc/tc_common.cuh"],
+    "torus_gemm_kernel<phi inverse>": ["paper_0807_4494_gb300/csrc/torus_gemm.cu", "paper_0807_4494_gb300/csrc/tc_common.cuh"],
+    "torus_gemm_kernel<phi forward>": ["paper_0807_4494_gb300/csrc/torus_gemm.cu", "paper_0807_4494_gb300/csrc/tc_common.cuh"],
+    "torus_gemm_kernel<theta forward>": ["paper_0807_4494_gb300/csrc/torus_gemm.cu", "paper_0807_4494_gb300/csrc/tc_common.cuh"],
+    "digit_contract_kernel": ["paper_0807_4494_gb300/csrc/contract_digits.cu", "paper_0807_4494_gb300/csrc/digits.cuh"],
     "inverse_kernel (SIMT)": ["paper_0807_4494_gb300/csrc/contract_simt.cu"],
     "project_kernel (SIMT)": ["paper_0807_4494_gb300/csrc/contract_simt.cu"],
 }
@@ -270,7 +274,7 @@ def split_trace(trace, steps):
         out.setdefault(names[k % 4], []).append(d)
     rec_inv = [t1 - t0 for name, lane, t0, t1 in trace if name == "delta_inverse"]
     rec = [t1 - t0 for name, lane, t0, t1 in trace if name == "delta"]
-    if rec_inv:  # 3xTF32 plans: the recursions writing the A tiles of each direction
+    if rec_inv:  # tensor-core plans: the recursions writing the A tiles of each direction
         out["recursion_inverse"] = rec_inv
         if rec:
             out["recursion_forward"] = rec
@@ -289,7 +293,7 @@ def split_trace(trace, steps):
 def kernel_rooflines(times, L, s, B, prec, recursion, pk):
     """Achieved fraction of each kernel's bound: algorithmic work of one launch over its live
     average duration.  Algorithmic bytes count each operand once (a lower bound on DRAM traffic)."""
-    N, M = 2 * L - 1, torus_M(L)
+    N = 2 * L - 1
     macs = B * contraction_macs(L, s)
     quad = quadrant_entries(L)
     res = {}
@@ -317,12 +321,12 @@ def kernel_rooflines(times, L, s, B, prec, recursion, pk):
         return e
 
     tc = prec in ("tf32x3", "bf16x6")
-    # bytes of one real operand value in the contraction's tiles in global memory: 3xTF32 tiles
-    # hold the FP32 value (split into hi + lo in shared memory), split-BF16 tiles the two parts
+    # bytes of one real operand value in the contraction's tiles in global memory: two FP16 parts, or three
+    # BF16 parts and a gap
     tv = 4.0 if prec == "tf32x3" else 8.0
     for key, v in times.items():
         ms = v["ms"]
-        if key == "recursion_inverse" and tc and recursion != "risbo" and prec == "tf32x3":
+        if key == "recursion_inverse" and tc and recursion != "risbo":
             u = lane_updates(L)
             res[key] = entry("lane_recursion_kernel", ms, 2.5 * u, pk["fp64_tflops"], None, quad * tv,
                              {"fp64_instr_frac": (1.5 * u / (ms / 1e3)) / (pk["fp64_tflops"][0] * 1e12 / 2.0),
@@ -337,10 +341,10 @@ def kernel_rooflines(times, L, s, B, prec, recursion, pk):
                                  {"fp64_instr_frac": ((4.0 * nh + 5.0 * ni) / (ms / 1e3)) / (pk["fp64_tflops"][0] * 1e12 / 2.0)})
             else:
                 u = column_updates(L)
-                # tile output (3xTF32): the rescaled relation's FMA, and the coefficient product at
+                # tile output (tensor-core plans): the rescaled relation's FMA, and the coefficient product at
                 # every other row (the integer pipe makes it at the others); FP64 table: b y and
                 # the FMA, the coefficient on the integer pipe
-                direct = prec == "tf32x3"
+                direct = tc
                 ni, nf = (1.5, 2.5) if direct else (2.0, 3.0)
                 res[key] = entry("column_tiles_kernel" if direct else "column_recursion_kernel (table)", ms,
                                  nf * u, pk["fp64_tflops"], None, quad * (tv if direct else 8.0),
@@ -349,7 +353,7 @@ def kernel_rooflines(times, L, s, B, prec, recursion, pk):
                                       u, ni, nf, "the A tiles (%d B an entry)" % tv if direct else "the FP64 table"),
                                   "fp64_probe_tflops": FP64_PROBE_TFLOPS})
         elif key in ("contraction_inverse", "contraction_forward") and tc:
-            nprod, pkey = (3, "tf32_tflops") if prec == "tf32x3" else (6, "bf16_tflops_sustained")
+            nprod, pkey = (3 if prec == "tf32x3" else 6), "bf16_tflops_sustained"
             fwd = key.endswith("forward")
             data = B * (N * L if fwd else L * L) * 2.0 * tv
             outb = B * (L * L if fwd else N * L) * 8.0
@@ -359,18 +363,23 @@ def kernel_rooflines(times, L, s, B, prec, recursion, pk):
         elif key in ("contraction_inverse", "contraction_forward"):
             fwd = key.endswith("forward")
             pkey = "fp64_tflops" if prec == "fp64" else "fp32_tflops"
-            res[key] = entry(("project_kernel" if fwd else "inverse_kernel") + " (SIMT)", ms, 4.0 * macs, pk[pkey], None,
+            digits = prec == "fp64" and 64 <= L <= 512 and B * L ** 3 > 1 << 23
+            kern = "digit_contract_kernel" if digits else "project_kernel (SIMT)" if fwd else "inverse_kernel (SIMT)"
+            if digits:
+                pkey = "bf16_tflops_sustained"
+            res[key] = entry(kern, ms, (44 if digits else 1) * 4.0 * macs, pk[pkey], None,
                              quad * 8.0 + B * (L * L + N * L) * (16.0 if prec == "fp64" else 8.0))
         elif key == "pack_data":
             res[key] = entry("pack_v_kernel", ms, None, None, None, B * L * L * (8.0 + 2.0 * tv))
         elif key in ("theta_inverse", "phi_inverse", "phi_forward", "theta_forward") and prec != "fp64":
             rows = B * L
-            nfft = 4 if key == "theta_forward" else 2
-            outb = B * L * (N + 1) * (2.0 * tv if (key == "theta_forward" and tc) else 8.0)
-            kern = {"theta_inverse": "inverse_theta_kernel", "phi_inverse": "phi_kernel<+1>",
-                    "phi_forward": "phi_kernel<-1>", "theta_forward": "forward_theta_kernel"}[key]
-            res[key] = entry(kern, ms, rows * nfft * fft_flops(M), pk["fp32_tflops"], None, B * L * N * 8.0 + outb,
-                             {"work": "%d rows x %d FFTs of %d points (5 M log2 M flops each)" % (rows, nfft, M)})
+            outb = rows * (N + 1) * (2.0 * tv if (key == "theta_forward" and tc) else 8.0)
+            kern = "torus_gemm_kernel<%s>" % key.replace("_", " ")
+            res[key] = entry(kern, ms, 3.0 * torus_pass_flops(L, B), pk["bf16_tflops_sustained"], None, rows * N * 8.0 + outb,
+                             {"useful_tflops": torus_pass_flops(L, B) / (ms / 1e3) / 1e12, "issued_products": 3,
+                              "work": "folded cosine and sine products, 8 B L^3 flops, three split-FP16 products each%s" % (
+                                  "" if key.startswith("theta_f") or key.startswith("phi_inv") else
+                                  "; the bracket includes the packing of the operand")})
     return res
 
 
@@ -571,7 +580,7 @@ def run_ssht(args):
         check = {"inverse": e_inv, "forward": e_fwd, "roundtrip": rt, "fields_checked": fields,
                  "measure": "max|x - oracle| / max|oracle|"}
 
-    # the other split form of the tensor-core contraction on the same workload (3xTF32 <-> split-BF16)
+    # the other split form of the tensor-core contraction on the same workload (split FP16 <-> split BF16)
     alt = None
     if not args.no_alt and prec in ("tf32x3", "bf16x6"):
         other = "bf16x6" if prec == "tf32x3" else "tf32x3"
@@ -632,9 +641,8 @@ def run_ssht(args):
                              "note": "the table-writing sweep timed by itself (ssht_wigner_delta)"}
     stage_ms = {k: round(v[0] / args.steps, 4) for k, v in stages.items() if v[1] > 0}
 
-    # column pairing along theta (two phi-frequency columns of opposite parity in one DFT): the
-    # inverse theta pass transforms pairs, the adjoint's theta pass one column at a time, each
-    # with two FFTs of the same length -- their time per column shows what the pairing saves
+    # the parity of a phi-frequency column along theta halves its sums (cosines or sines of m' >= 0 only), in
+    # the inverse's theta pass as in the adjoint's: their time per column
     pairing = None
     if prec != "fp64":
         plan.profile(True)
@@ -649,11 +657,10 @@ def run_ssht(args):
         theta_inv = kern.get("theta_inverse", {}).get("ms")
         if theta_adj and theta_inv:
             cols = B * (2 * L - 1)
-            pairing = {"theta_inverse_paired_ms": theta_inv, "theta_adjoint_unpaired_ms": theta_adj,
-                       "us_per_column_paired": 1e3 * theta_inv / cols, "us_per_column_unpaired": 1e3 * theta_adj / cols,
-                       "unpaired_over_paired": theta_adj / theta_inv,
-                       "note": "same DFT length and FFT count per transformed sequence; the adjoint's theta pass "
-                               "also writes the data tiles, the inverse's the phi input"}
+            pairing = {"theta_inverse_ms": theta_inv, "theta_adjoint_ms": theta_adj,
+                       "us_per_column_inverse": 1e3 * theta_inv / cols, "us_per_column_adjoint": 1e3 * theta_adj / cols,
+                       "note": "both fold the columns by parity; the adjoint's theta pass writes the data tiles, the "
+                               "inverse's bracket includes the packing of its operand"}
         del adj_out
 
     # the plain FP64 GPU transform of the same workload (the mixed-precision form must beat it)
@@ -767,7 +774,7 @@ def run_fp64(args, torch, inputs, ssht, world, device, stream, rank, pk, inv_ora
         plan.check()
         ms = max_over_ranks(e0.elapsed_time(e1), world, device)
         # FP64 plans make the same table in both calls; the forward call's sweep waits beside the
-        # inverse's cuFFT passes for room on the SMs, so its bracket measures that wait: the
+        # inverse's torus passes for room on the SMs, so its bracket measures that wait: the
         # inverse call's bracket is the sweep
         times = {k: v for k, v in split_trace(trace, nrep).items()
                  if k in ("recursion_inverse", "contraction_inverse", "contraction_forward")}

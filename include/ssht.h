@@ -62,9 +62,10 @@ extern "C" {
 
 /* Arithmetic of the O(L^3) contraction.  The Delta recursion is FP64 in every mode. */
 typedef enum {
-  SSHT_FP64 = 0,   /* FP64 everywhere (CUDA cores); double I/O                          */
+  SSHT_FP64 = 0,   /* FP64 (its sums also as exact products of digits on tensor cores) */
   SSHT_FP32 = 1,   /* FP32 contraction on CUDA cores with FP64 Delta; float I/O          */
-  SSHT_TF32X3 = 2, /* contraction on tcgen05 tensor cores, 3xTF32 split products         */
+  SSHT_TF32X3 = 2, /* contraction on tcgen05 tensor cores, the 3xTF32 products of two   */
+                   /* 11-bit parts (held as FP16 with powers of two)                    */
   SSHT_BF16X6 = 3  /* contraction on tcgen05 tensor cores, 3-way BF16 split, 6 products  */
 } ssht_precision;
 
@@ -114,7 +115,8 @@ typedef struct ssht_plan_s* ssht_plan_t;
 
 /* Create an FP64 plan with the Delta recursion run in every call.
  * out: receives the plan; L, s, batch as in ssht_plan_desc.
- * Allocates the plan's device workspace (see ssht_plan_workspace_bytes) and cuFFT plans. */
+ * Allocates the plan's device workspace (see ssht_plan_workspace_bytes) and, for the triangular
+ * forward of FP64 plans, cuFFT plans. */
 SSHT_API int ssht_plan(ssht_plan_t* out, int L, int s, int batch);
 
 /* Create a plan from a descriptor (precision and Delta mode).  With SSHT_DELTA_CACHE the
@@ -190,10 +192,10 @@ SSHT_API int ssht_plan_check(ssht_plan_t plan);
                                 /* whose recursion writes the A tiles, the forward's      */
 #define SSHT_STAGE_INVERSE 1    /* inverse contraction (eqn fourier_coeff)                */
 #define SSHT_STAGE_PROJECT 2    /* forward / adjoint contraction (harmonic projection)    */
-#define SSHT_STAGE_FFT 3        /* torus DFTs: fused torus passes (FP32 plans) or cuFFT   */
-#define SSHT_STAGE_TORUS 4      /* extension, phase, transpose and weight-product kernels */
+#define SSHT_STAGE_FFT 3        /* torus DFTs: cosine and sine products, with packing     */
+#define SSHT_STAGE_TORUS 4      /* extension kernel of the triangular forward             */
 #define SSHT_STAGE_PACK 5       /* operand packing for the tensor-core contraction        */
-#define SSHT_STAGE_DELTA_INVERSE 6 /* the recursion writing the inverse's A tiles (3xTF32) */
+#define SSHT_STAGE_DELTA_INVERSE 6 /* the recursion writing the inverse's A tiles          */
 #define SSHT_NUM_STAGES 7
 
 /* Enable (1) or disable (0) per-stage timing: each stage of each later call is bracketed by
@@ -226,9 +228,9 @@ typedef struct ssht_group_s* ssht_group_t;
 
 /* Create a group of n fields with band-limits L[i] (1..2048) and spins s[i] (|s[i]| < L[i]).
  * Fields are bucketed by (L, s) and each bucket is transformed by one plan of the given
- * precision and Delta mode; buckets of the same L share one Delta table (recompute mode: one
- * recursion per distinct L per call; cache mode: made here).  tune != 0 (FP32-class
- * precisions only) times the FP32, 3xTF32 and split-BF16 contractions on each bucket, the
+ * precision and Delta mode; CUDA-core buckets of the same L share one Delta table (recompute mode: one
+ * recursion per such L per call; cache mode: made here), tensor-core buckets make their own operands.  tune != 0 (FP32-class
+ * precisions only) times the FP32, split-FP16 and split-BF16 contractions on each bucket, the
  * tensor-core forms each with their own tuned shape (SSHT_FLAG_TUNE, SSHT_TUNE_CACHE), and keeps
  * the fastest.  Synchronises the device. */
 SSHT_API int ssht_group_create(ssht_group_t* out, int n, const int* L, const int* s, int precision,
@@ -280,7 +282,7 @@ SSHT_API int ssht_debug_noalloc_wait_limit(long long ns);
 
 /* Index checks of the bounds-checked build (the paper has no counterpart; the library compiled
  * with -DSSHT_DEBUG, `python -m paper_0807_4494_gb300.build --debug`): in that build every checked
- * global access of the kernels (torus passes, packing, tensor-core contraction, recursions writing
+ * global access of the kernels (torus passes, packing, tensor-core contractions, recursions writing
  * the tiles, real-field and spin-pair kernels, SIMT contractions) tests its index against the extent
  * of its buffer and skips it when it lies outside.  *count receives the number of such accesses
  * since the last call, *site / *index / *extent the first one's site (an internal number), index
@@ -296,7 +298,7 @@ SSHT_API int ssht_plan_tile_config(ssht_plan_t plan, int* cfg);
 
 /* Spin limit of the plan's device-side waits, in nanoseconds of the device clock (default 10^9, one
  * second): the Risbo recursion's hand-offs between CTAs (SSHT_FLAG_RISBO plans) and the
- * tensor-core contraction's pipeline waits.  A wait that exceeds it latches SSHT_ETIMEOUT in the
+ * pipeline waits of the tensor-core contractions and torus products.  A wait that exceeds it latches SSHT_ETIMEOUT in the
  * plan (read by ssht_plan_check), makes the kernel's other CTAs leave at their next wait, and leaves
  * the outputs of that call incomplete; copies and tensor-core operations already issued are waited
  * for before a CTA leaves, with the default limit.  A tiny limit makes the waits give up at once

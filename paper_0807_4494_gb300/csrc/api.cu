@@ -111,12 +111,12 @@ struct ssht_plan_s {
   void* stage_out = nullptr;
   size_t stage_out_bytes = 0;
   bool delta_ready = false;
-  bool u_fixed = false;  // U / Uf made once at creation (3xTF32 plans with the recursion writing the A tiles)
+  bool u_fixed = false;  // U / Uf made once at creation (plans whose recursion writes the A tiles)
   long long wait_ns = kDefaultWaitNs;  // spin limit of the device-side waits
-  LaneTables lane;  // tables of the recursion that writes the inverse's A tiles (3xTF32, own recursion)
+  LaneTables lane;  // tables of the recursion that writes the inverse's A tiles
   size_t bytes = 0;
   TcPlan* tc = nullptr;    // tensor-core contraction (precisions SSHT_TF32X3, SSHT_BF16X6)
-  TorusPlan* torus = nullptr;  // fused torus passes of FP32 plans (FP64 plans: cuFFT Z2Z + glue)
+  TorusPlan* torus = nullptr;  // torus products of FP32-class plans
   DigitPlan* digits = nullptr;   // torus products of FP64 plans
   DirectPlan* direct = nullptr;  // ... and of those with little work
   bool contract_digits = false;  // FP64 contractions on tensor cores
@@ -229,7 +229,7 @@ int run_dft(ssht_plan_t p, cufftHandle h, void* in, void* out, cudaStream_t st) 
   return 0;
 }
 
-// The torus passes of an FP32 plan (DFT along theta or phi with its glue), timed as FFT work.  Inverse:
+// The torus passes of an FP32-class plan (products along theta or phi), timed as FFT work.  Inverse:
 // F in W1 -> samples f.
 int torus_inverse_pass(ssht_plan_t p, int step, void* f, cudaStream_t st) {
   StageScope sc(p, SSHT_STAGE_FFT, st);
@@ -376,7 +376,7 @@ int begin_operands(ssht_plan_t p, int forward, cudaStream_t st) {
     // ... and the other direction's contraction: it cannot share an SM with the recursion, so
     // queued behind a running recursion it would wait for the whole sweep, while run first
     // (about 1 ms) it lets the torus passes that follow it overlap the recursion (not for the
-    // inverse's tiles of a 3xTF32 plan, see above)
+    // inverse's tiles of a tensor-core plan, see above)
     const bool early = SSHT_INVERSE_OPERANDS_EARLY && !forward && tiles_direct(p);
     if (p->tc && !early && p->afree_valid[1 - forward] && p->afree_capture[1 - forward] == cap)
       SSHT_CUDA(cudaStreamWaitEvent(p->aux, p->ev_free_a[1 - forward], 0), "other contraction wait");
@@ -1226,8 +1226,8 @@ int ssht_debug_fail_allocation(int n) {
 int ssht_debug_bounds(long long* count, int* site, long long* index, long long* extent) {
   if (!kBoundsChecked) return fail(SSHT_EUNSUPPORTED, "ssht_debug_bounds: this library was built without index checks");
   SSHT_CUDA(cudaDeviceSynchronize(), "synchronize");
-  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass, bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc, bounds_take_delta_column,
-                                          bounds_take_real, bounds_take_contract_simt};
+  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass,  bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc,
+                                          bounds_take_delta_column, bounds_take_real, bounds_take_contract_simt};
   BoundsRecord first{};
   long long total = 0;
   for (auto f : take) {
@@ -1258,7 +1258,7 @@ int ssht_version(void) { return 100; }
 // {128, .., 1024} and 20 buckets, packing every bucket's tiles from shared tables made a step
 // (inverse and forward) 39.1 ms, the sweeps into the tiles 29.4.  Buckets run on their own streams, forked from and joined to the caller's.
 // With tuning on, each bucket times every contraction form of the group's precision class
-// (FP32, 3xTF32, split-BF16 for FP32-class groups; the tensor-core forms with their own tuned
+// (FP32, split-FP16, split-BF16 for FP32-class groups; the tensor-core forms with their own tuned
 // shape) on its own shape and keeps the fastest.
 // ---------------------------------------------------------------------------------------------
 

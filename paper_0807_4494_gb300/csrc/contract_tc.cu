@@ -53,7 +53,7 @@ namespace {
 using namespace tc;
 
 constexpr int TM = kTileRows;              // rows per tile
-constexpr int TK = kTileK;                 // K per chunk (one 128-byte TF32 row)
+constexpr int TK = kTileK;                 // K per chunk (two FP16 parts: 128 bytes a row)
 constexpr int A_PART = kAPart;             // 16 KB: one part of an A tile
 constexpr int MAX_STAGES = 4;             // pipeline depth: a plan parameter, 2 .. MAX_STAGES
 constexpr int SCALE_SLOTS = 8;            // ring of the chunks' scales (MAX_STAGES + 2 would do)

@@ -61,7 +61,7 @@ struct ColumnParams {
   const double* rsq;       // 1/sqrt(k), k >= 1
   double* table;           // quadrant table, entry (l, m', m) at offset(l) + m'(l+1) + m
   unsigned int* counter;   // next task (zeroed before the launch)
-  // tile output (3xTF32 plans): A_m[l][m'] = Uf_l[m'] Delta^l_{m'm} into the forward tile layout
+  // tile output (tensor-core plans): A_m[l][m'] = Uf_l[m'] Delta^l_{m'm} into the forward tile layout
   const float* Uf;         // U_l[m'] in FP32 at l(l+1)/2 + m'
   const double* alc;       // alpha(l, m') of the rescaled relation at l(l+1)/2 + m'
   const float* pc;         // p(l, m') at l(l+1)/2 + m'
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kColThreads, 2) column_recursion_kernel(Column
   }
 }
 
-// The same walk writing the A tiles of a 3xTF32 plan instead of the table.  With x = Delta_{m'm}
+// The same walk writing the A tiles of a tensor-core plan instead of the table.  With x = Delta_{m'm}
 // in lane m at step m' (row), the entry serves two tiles: A_{m'}[l][m] = U_l[m] (-1)^{m'-m} x, a
 // row of 32 consecutive K values across the warp (written at once), for every row m' >= 32b; and
 // A_m[l][m'] = U_l[m'] x, which goes through the transposition block like the table's transposed
@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kColThreads, 3) column_tiles_kernel(ColumnPara
 }
 
 // ---------------------------------------------------------------------------------------------
-// One lane per degree: the inverse contraction's A tiles (rows m', K = l), 3xTF32 plans.
+// One lane per degree: the inverse contraction's A tiles (rows m', K = l), tensor-core plans.
 //
 // The inverse's tile rows run along K = l, so here a warp takes 32 consecutive degrees
 // l = 32 kc + lane and one column m and walks m' from the top degree down to m, lane l starting
