@@ -120,6 +120,7 @@ struct ssht_plan_s {
   DigitPlan* digits = nullptr;   // torus products of FP64 plans
   DirectPlan* direct = nullptr;  // ... and of those with little work
   bool contract_digits = false;  // FP64 contractions on tensor cores
+  int sms = 0;                   // of the plan's device
   // The Delta recursion (and the A packing) of a call runs on a second stream, forked from the
   // caller's stream at the start of the call and joined before the contraction, so that the
   // Delta-independent work of the call (the torus stage of forward/adjoint, data packing) runs
@@ -456,7 +457,7 @@ int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st) {
   {
     StageScope sc(p, SSHT_STAGE_PROJECT, st);
     if (p->contract_digits)
-      SSHT_CUDA(contract_digits(1, p->d.L, p->s, p->B, p->delta.sms, p->delta.table, p->U, H, p->w_bytes, p->W3, flm,
+      SSHT_CUDA(contract_digits(1, p->d.L, p->s, p->B, p->sms, p->delta.table, p->U, H, p->w_bytes, p->W3, flm,
                                 p->pair_coeff_bytes(), p->delta.status, p->wait_ns, st),
                 "projection");
     else
@@ -549,7 +550,7 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
     if ((rc = join_operands(p, st))) return rc;
     StageScope sc(p, SSHT_STAGE_INVERSE, st);
     if (p->contract_digits)
-      SSHT_CUDA(contract_digits(0, d.L, p->s, p->B, p->delta.sms, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W3, p->W1,
+      SSHT_CUDA(contract_digits(0, d.L, p->s, p->B, p->sms, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W3, p->W1,
                                 p->w_bytes, p->delta.status, p->wait_ns, st),
                 "inverse contraction");
     else
@@ -890,7 +891,9 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     size_t w3 = digits_workspace_bytes(L, s, B);
     if (p->contract_digits) {
       w3 = std::max(w3, contract_digits_bytes(L, B));
-      if ((ce = contract_digits_setup()) != cudaSuccess) {
+      ce = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
+      if (ce == cudaSuccess) ce = contract_digits_setup();
+      if (ce != cudaSuccess) {
         release(p);
         return fail(SSHT_ECUDA, std::string("contraction setup: ") + cudaGetErrorString(ce));
       }

@@ -47,6 +47,20 @@ def test_both_torus_stages_match_oracle(L, s, B):
     assert rel(adj, T.adjoint(g, L, s)) < 1e-12
 
 
+@pytest.mark.parametrize("recursion,delta_mode", [("risbo", "recompute"), ("risbo", "cache"), ("column", "cache")])
+def test_digit_contractions_of_every_table(recursion, delta_mode):
+    """The contractions of digits read the table of either recursion, made in the call or kept."""
+    from paper_0807_4494_gb300 import ssht
+    L, s, B = 140, -1, 4
+    flm = inputs.coeffs(L, s, B, seed=5)
+    plan = ssht.Plan(L, s, B, precision="fp64", recursion=recursion, delta_mode=delta_mode)
+    f = plan.inverse(torch.from_numpy(flm).cuda())
+    back = plan.forward(f).cpu().numpy()
+    plan.check()
+    assert rel(f.cpu().numpy(), T.inverse(flm, L, s)) < 1e-12
+    assert rel(back, flm) < 1e-12
+
+
 def test_powers_of_two_and_non_finite_rows():
     """Fixed point with a row's own power of two: scaling a field by 2^k scales the outputs exactly, and a field
     with a NaN or an infinity leaves the other fields' outputs as they are."""
@@ -72,3 +86,39 @@ def test_powers_of_two_and_non_finite_rows():
     for b in (1, 3):
         assert not torch.isfinite(torch.view_as_real(fb[b])).any()
         assert not torch.isfinite(torch.view_as_real(yb[b])).all()
+
+
+def test_real_pair_and_group_forms_of_digit_plans():
+    """Real fields against the oracle; a group's buckets (concurrent, and replayed from a capture) bit for bit
+    against plans of their own."""
+    from paper_0807_4494_gb300 import ssht
+    L, B = 140, 8
+    flm = inputs.coeffs(L, 0, B, seed=9, real=True)
+    plan = ssht.Plan(L, 0, B, precision="fp64", real=True)
+    f = plan.inverse(torch.from_numpy(flm).cuda())
+    back = plan.forward(f).cpu().numpy()
+    plan.check()
+    for b in range(B):
+        assert rel(f[b].cpu().numpy(), T.inverse(flm[b], L, 0).real) < 1e-12
+        assert rel(back[b], flm[b]) < 1e-12
+
+    Ls, ss = [140] * 4 + [210] * 2 + [40] * 3 + [140] * 5, [0] * 4 + [-1] * 2 + [2] * 3 + [1] * 5
+    x = [torch.from_numpy(inputs.coeffs(l, s, 1, seed=i)[0]).cuda() for i, (l, s) in enumerate(zip(Ls, ss))]
+    g = ssht.Group(Ls, ss, precision="fp64", tune=False)
+    flat = g.pack_coeffs(x)
+    grid, out = g.inverse(flat), None
+    out = g.forward(grid)
+    grid2, out2 = g.empty_grid(), g.empty_coeffs()
+    g.capture(flat, grid2, out2)
+    g.replay()
+    torch.cuda.synchronize()
+    g.check()
+    assert torch.equal(grid2, grid) and torch.equal(out2, out)
+    fs, bs = g.unpack_grid(grid), g.unpack_coeffs(out)
+    for l, s in set(zip(Ls, ss)):
+        idx = [i for i in range(len(Ls)) if (Ls[i], ss[i]) == (l, s)]
+        p = ssht.Plan(l, s, len(idx), precision="fp64")
+        want = p.inverse(torch.stack([x[i] for i in idx]))
+        wb = p.forward(want)
+        for k, i in enumerate(idx):
+            assert torch.equal(fs[i], want[k]) and torch.equal(bs[i], wb[k])
