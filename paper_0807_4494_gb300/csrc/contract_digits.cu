@@ -155,6 +155,9 @@ __device__ __forceinline__ Item item_of(const GemmArgs& a, int w) {
   return t;
 }
 
+// Column of accumulator d: the even ones, then the odd ones.
+__device__ __forceinline__ constexpr uint32_t acc_col(int d) { return kCols * (d >> 1) + (d & 1) * 5 * kCols; }
+
 template <bool FWD>
 __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __grid_constant__ GemmArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -216,8 +219,9 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       for (int k = 0; k < kStages; ++k)
         if ((used >> k) & 1u) mbar_wait(&data_full[k], (uph >> k) & 1u, nullptr, kDrainNs);
     } else if (warp == 1) {
-      // ---- MMA issuer: digits i of A and j of the data into accumulator i + j <= 8 ----
-      const uint32_t idesc = idesc_f16(128, kCols);
+      // ---- MMA issuer: digits i of A and j of the data into accumulator i + j <= 8.  A part of the data tile
+      // holds two digits, so the even (or the odd) ones are the rows of one operand, and with the accumulators of one
+      // parity side by side one product takes digit i times all of them ----
       const bool one = elect_one();
       const uint32_t lo0 = (smem_u32(smem) >> 4) + kDescLow;
       int s = 0, ph = 0, buf = 0, bph = 1;
@@ -238,12 +242,17 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-              for (int j = 0; j < kDigits; ++j)
-#pragma unroll
-                for (int i = 0; i < kADigits - j; ++i)
-                  mma_f16_lo<false>(dt + (uint32_t)(kCols * (i + j)), la + (i >> 1) * (kAPart >> 4) + (i & 1) * 4 + 2 * kk,
-                                    lb + (j >> 1) * (kXPart >> 4) + (j & 1) * 4 + 2 * kk, idesc,
-                                    kk == 0 && (j == 0) ? more : 1u);
+              for (int i = 0; i < kADigits; ++i) {
+                const int jm = kDigits - 1 < kADigits - 1 - i ? kDigits - 1 : kADigits - 1 - i, even = jm / 2 + 1, odd = (jm + 1) / 2;
+                const uint32_t da = la + (i >> 1) * (kAPart >> 4) + (i & 1) * 4 + 2 * kk, init = kk == 0 && i == 0 ? more : 1u;
+                mma_f16_lo<false>(dt + acc_col(i), da, lb + 2 * kk, idesc_f16(128, kCols * even), init);
+                if (i == 1) {  // accumulator 8 has its first product here
+                  mma_f16_lo<false>(dt + acc_col(2), da, lb + 4 + 2 * kk, idesc_f16(128, kCols * (odd - 1)), 1u);
+                  mma_f16_lo<false>(dt + acc_col(8), da, lb + (odd - 1) * (kXPart >> 4) + 4 + 2 * kk, idesc_f16(128, kCols), kk == 0 ? more : 1u);
+                } else if (odd) {
+                  mma_f16_lo<false>(dt + acc_col(i + 1), da, lb + 4 + 2 * kk, idesc_f16(128, kCols * odd), init);
+                }
+              }
             mma_commit(&empty[s]);
             if (c + 1 == t.c1) mma_commit(&acc_full[buf]);
           }
@@ -279,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       fence_after();
       uint32_t v[kADigits][4];
 #pragma unroll
-      for (int d = 0; d < kADigits; ++d) tmem_ld4_nowait(tq + 256 * buf + kCols * d, v[d]);
+      for (int d = 0; d < kADigits; ++d) tmem_ld4_nowait(tq + 256 * buf + acc_col(d), v[d]);
       tmem_wait_ld();
       fence_before();
       __syncwarp();

@@ -11,11 +11,11 @@
 // 64-bit integers and rounded once to FP64.  The transforms' error is what it was with FFTs (round trip against
 // exact sums 2.3e-13 at L = 512, 2.8e-14 at L = 129, with both).
 //
-// What bounds it: reading the operands' digits from shared memory, 6 KB a product of 128 x 64 x 16 (53 clocks), 72 of them in
-// 32 k's, and below L = 300 launches, the first loads and the epilogue (10 us a pass).  It replaces FFTs of odd
+// What bounds it: the tensor cores (36 digit products of 128 x 64 x 16 in 15 instructions, 1150 clocks, and 132 KB of operands
+// read from shared memory, 1060), and below L = 300 launches, the first loads and the epilogue (10 us a pass).  It replaces FFTs of odd
 // length and the kernels between them, which the FP64 pipe bounds: that pipe does two multiply-adds a clock on
-// an SM.  Torus stage of an inverse and a forward, before and now: L = 512, B = 1 1003 and 232 us (a product 43 us, a
-// packing 12); L = 129, B = 4 587 and 122; L = 256, B = 8 2088 and 276; L = 1024, B = 1 5.26 and 1.25 ms; L = 2048, B = 1 16.5 and 8.0.
+// an SM.  Torus stage of an inverse and a forward, before and now: L = 512, B = 1 1003 and 200 us (a product 35 us, 43 with
+// an instruction for each pair of digits; a packing 12); L = 129, B = 4 587 and 105; L = 256, B = 8 2088 and 245.
 // The tile is 128 rows x 32 complex columns: eight accumulators of 64 columns fill the tensor memory.
 #include <algorithm>
 #include <cstdint>
@@ -249,6 +249,10 @@ __device__ __forceinline__ Item item_of(const GemmArgs& a, int w) {
   return t;
 }
 
+// Column of accumulator d: the even ones, then the odd ones.
+template <int COLS>
+__device__ __forceinline__ constexpr uint32_t acc_col(int d) { return COLS * (d >> 1) + (d & 1) * 4 * COLS; }
+
 template <int PASS, int PAIRS>
 __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_constant__ GemmArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -311,8 +315,9 @@ __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_co
       for (int k = 0; k < kStages; ++k)
         if ((used >> k) & 1u) mbar_wait(&full[k], (uph >> k) & 1u, nullptr, kDrainNs);
     } else if (warp == 1) {
-      // ---- MMA issuer: per 16 k's the 36 digit products, digits i + j into accumulator i + j ----
-      const uint32_t idesc = idesc_f16(128, COLS);
+      // ---- MMA issuer: per 16 k's the 36 digit products, digits i + j into accumulator i + j.  A part of the data
+      // tile holds two digits, so the even (or the odd) ones are the rows of one operand, and with the accumulators of one parity
+      // side by side one product takes digit i of the matrix times all of them ----
       const bool one = elect_one();
       const uint32_t lo0 = (smem_u32(smem) >> 4) + kDescLow;
       int s = 0, ph = 0, sph = 1;
@@ -331,12 +336,12 @@ __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_co
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-              for (int i = 0; i < kDigits; ++i)
-#pragma unroll
-                for (int j = 0; j < kDigits - i; ++j)
-                  mma_f16_lo<false>(tbase + (uint32_t)(COLS * (i + j)), la + (i >> 1) * (128 * 128 >> 4) + (i & 1) * 4 + 2 * kk,
-                                    lb + (j >> 1) * (COLS * 128 >> 4) + (j & 1) * 4 + 2 * kk, idesc,
-                                    first && kk == 0 && i == 0 ? 0u : 1u);
+              for (int i = 0; i < kDigits; ++i) {
+                const int jm = kDigits - 1 - i, even = jm / 2 + 1, odd = (jm + 1) / 2;
+                const uint32_t da = la + (i >> 1) * (128 * 128 >> 4) + (i & 1) * 4 + 2 * kk, init = first && kk == 0 && i == 0 ? 0u : 1u;
+                mma_f16_lo<false>(tbase + acc_col<COLS>(i), da, lb + 2 * kk, idesc_f16(128, COLS * even), init);
+                if (odd) mma_f16_lo<false>(tbase + acc_col<COLS>(i + 1), da, lb + 4 + 2 * kk, idesc_f16(128, COLS * odd), init);
+              }
             mma_commit(&empty[s]);
             if (last) mma_commit(&seg_full);
           }
@@ -377,7 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_co
           for (int d = 0; d < kDigits; d += 4) {
             int v[4][8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tmem_ld8_nowait(tq + COLS * (d + k) + 8 * h, (uint32_t*)v[k]);
+            for (int k = 0; k < 4; ++k) tmem_ld8_nowait(tq + acc_col<COLS>(d + k) + 8 * h, (uint32_t*)v[k]);
             tmem_wait_ld();
             // whole numbers of at most (d + 1) 2^21: the pairs' sums stay below 2^31
 #pragma unroll
@@ -555,7 +560,7 @@ static cudaError_t run_tiles(const DigitPlan* p, int mat, int s, int B, const vo
 }
 
 // Tiles of 16 complex columns where those of 32 would leave half of the SMs without one: L = 129, B = 4 (66 and
-// 130 tiles) 21.8 us a product with 32, 17.4 with 16; L = 8, B = 4 13.6 and 9.9.
+// 130 tiles) 21.8 us a product with 32, 17.4 with 16 (13.5 since the digits are taken together).
 template <int PASS>
 static cudaError_t run(const DigitPlan* p, int mat, int s, int B, const void* in, size_t in_bytes, void* work, void* out,
                        size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
