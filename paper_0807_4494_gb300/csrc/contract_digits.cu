@@ -7,10 +7,12 @@
 // warps, a thread one row and eight k's at a time.  A's entries have one power of two for all of them (|A| <= sqrt((2L - 1) / 4 pi))
 // and nine digits, so that they keep 2^-58 of that bound; a data column has its own and eight.  44 products of digits a chunk.
 //
-// What bounds it: making A's digits (half of the issue slots at 18 warps, 6300 clocks a chunk of 4096 entries), then the
-// products' reads of them from shared memory (88 of 32 clocks a chunk) and the FP64 pipe's products U Delta (2048) -- one an
-// entry, where CUDA cores need four more a field.  L = 512, B = 1 280 us the inverse and 306 the projection, 517 and 482 on CUDA
-// cores; L = 256, B = 8 97 and 121, about 440 each there.  Taken back: the conversion to integers by F2I (307 and 333 us: it runs at the FP64 pipe's rate).
+// What bounds it: making A's digits, 6000 clocks a chunk of 4096 entries -- loads, one FP64 product an entry (2048 clocks; CUDA
+// cores need four more a field) and the integer instructions behind it, with 60 % of the issue slots busy; the
+// tensor cores' part (1440) is beside it.  L = 512, B = 1: 270 us the inverse and 288 the projection, 517 and 482 on CUDA
+// cores; L = 256, B = 8 91 and 112, about 440 each there.  The next chunk's FP64 products stand one by one among the integer
+// instructions (281 and 286 us before).  Taken back: the conversion to integers by F2I (307 and 333 us: it runs at the FP64 pipe's
+// rate), fewer instructions to take the digits out (280 and 299: within the noise).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -322,8 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       return true;
     };
 
-    // the values of a chunk are loaded while the one before is made: Delta and U of eight k's (masked ones
-    // from a valid place)
+    // Delta and U of eight k's of a chunk (masked ones from a valid place)
     double d[8], u[8];
     auto fetch = [&](const Item& t, int c) {
       const int r = 128 * t.i + row;
@@ -359,31 +360,47 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       }
       return false;
     };
-    Item pending, t;
+    // where the loads are: one chunk ahead of the products U Delta, two ahead of the digits
+    Item ft;
+    int fw = blockIdx.x, fc = 0;
+    bool loads = next_item(fw, ft);
+    auto next_loads = [&] {
+      if (loads && ++fc >= ft.c1) {
+        fw += gridDim.x;
+        loads = next_item(fw, ft);
+        fc = ft.c0;
+      }
+      if (loads) fetch(ft, fc);
+    };
+    Item pending, t = ft;
     pending.m = -1;
-    int w = blockIdx.x;
-    bool more = next_item(w, t);
-    if (more) fetch(t, t.c0);
+    int w = fw;
+    bool more = loads;
+    double x[8];
+    if (more) {
+      fc = ft.c0;
+      fetch(ft, fc);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = u[i] * d[i];
+      next_loads();
+    }
     while (more && going(abort)) {
-      Item nt = t;
       bool ok = true;
       for (int c = t.c0; c < t.c1; ++c) {
-        double x[8];
+        // the next chunk's products, one by one among the integer instructions: the FP64 pipe holds a warp for 64 clocks
+        unsigned long long v[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = u[i] * d[i];
-        if (c + 1 < t.c1) {
-          fetch(t, c + 1);
-        } else {
-          w += gridDim.x;
-          more = next_item(w, nt);
-          if (more) fetch(nt, nt.c0);
+        for (int i = 0; i < 8; ++i) {
+          v[i] = (unsigned long long)fixed_point<7 * kADigits - 54>(x[i], a.aexp);
+          x[i] = u[i] * d[i];
         }
+        next_loads();
         if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort, a.wait_ns))) {
           *abort = 1;
           ok = false;
           break;
         }
-        put_digits<kADigits, kAPart>(smem + s * kStageBytes, row, piece, x, a.aexp);
+        put_integers<kADigits, kAPart>(smem + s * kStageBytes, row, piece, v);
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[s]);
@@ -400,7 +417,8 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       }
       if (!ok) break;
       pending = t;
-      t = nt;
+      w += gridDim.x;
+      more = next_item(w, t);
     }
     __syncwarp();
     if (pending.m >= 0 && going(abort)) drain(pending);
@@ -452,10 +470,10 @@ cudaError_t run(int L, int s, int B, int sms, const double* table, const double*
 
 }  // namespace
 
-// Where they beat the CUDA cores' contractions, an inverse and a projection in us, these and those: L = 512, B = 1 621 and 1006, B = 4 653
-// and 3041; L = 256, B = 1 144 and 168, B = 8 260 and 881; L = 192, B = 8 181 and 413; L = 129, B = 4 83 and 92; L = 64, B = 64 154 and 208.
-// Below B L^3 = 2^23 few items, of few chunks, leave the launch and the epilogue (L = 192, B = 1 109 and 98; L = 160, B = 1 86 and 63), and
-// below L = 64 half of a tile's rows are empty (L = 40, B = 96 156 and 126).
+// Where they beat the CUDA cores' contractions, an inverse and a projection in us, these and those: L = 512, B = 1 594 and 1006,
+// B = 4 627 and 3041; L = 256, B = 1 136 and 168, B = 8 245 and 881; L = 192, B = 8 173 and 413; L = 129, B = 4 75 and 92; L = 64,
+// B = 64 151 and 208.  Below B L^3 = 2^23 few items, of few chunks, leave the launch and the epilogue (L = 192, B = 1 109 and 98;
+// L = 160, B = 1 86 and 63), and below L = 64 half of a tile's rows are empty (L = 40, B = 96 156 and 126).
 bool contract_digits_wanted(int L, int B) { return L >= 64 && L <= kMaxL && (long long)B * L * L * L > (1ll << 23); }
 
 size_t contract_digits_bytes(int L, int B) {

@@ -36,11 +36,10 @@ __device__ __forceinline__ long long fixed_point(double x, int e) {
 // bits less 64 (the top one takes 0 .. 128), and 0x6400 + n is the FP16 number 1024 + n.  Two digits share a part's
 // 128-byte row.
 template <int DIGITS, int PART_BYTES>
-__device__ __forceinline__ void put_digits(uint8_t* tile, int row, int piece, const double (&x)[8], int e) {
-  constexpr unsigned long long kMiddle = DIGITS == 8 ? 0x81020408102040ll : 0x4081020408102040ll;
-  unsigned long long v[8];
+__device__ __forceinline__ void put_integers(uint8_t* tile, int row, int piece, unsigned long long (&v)[8]) {
+  constexpr unsigned long long kMiddle = DIGITS == 8 ? 0x81020408102040ull : 0x4081020408102040ull;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) v[k] = (unsigned long long)fixed_point<7 * DIGITS - 54>(x[k], e) + kMiddle;
+  for (int k = 0; k < 8; ++k) v[k] += kMiddle;
   const __half2 bias = __float2half2_rn(1088.f);
 #pragma unroll
   for (int i = 0; i < DIGITS; ++i) {
@@ -59,6 +58,14 @@ __device__ __forceinline__ void put_digits(uint8_t* tile, int row, int piece, co
     }
     *(uint4*)(tile + (i >> 1) * PART_BYTES + sw128(row, 64 * (i & 1) + 16 * piece)) = make_uint4(w[0], w[1], w[2], w[3]);
   }
+}
+
+template <int DIGITS, int PART_BYTES>
+__device__ __forceinline__ void put_digits(uint8_t* tile, int row, int piece, const double (&x)[8], int e) {
+  unsigned long long v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = (unsigned long long)fixed_point<7 * DIGITS - 54>(x[k], e);
+  put_integers<DIGITS, PART_BYTES>(tile, row, piece, v);
 }
 
 // (hi 2^28 + lo) 2^e, rounded to nearest.  Integer instructions: a conversion or product on the FP64 pipe takes a warp 64 clocks.
