@@ -2,7 +2,7 @@
 // fixed-point digits held as FP16 (digits.cuh; torus_digits.cu says why the sums are exact).
 //
 // For an order m the inverse is F_{+-m}[m'] = sum_l A[m', l] sf_{l,+-m}, the projection sf_{l,+-m} = sum_m' A[m', l] H_{+-m}[m'], with
-// A[m', l] = U_l[m'] Delta^l_{m' m} up to signs.  A work item is 128 rows (m' or l) of one order and four fields: 16
+// A[m', l] = U_l[m'] Delta^l_{m' m} up to signs.  A work item is 128 rows (m' or l) of one order and four or eight fields: 16 or 32
 // columns (field, sign of m, part).  A CTA makes the digits of A itself, from the FP64 table into the tensor cores' shared memory: 16
 // warps, a thread one row and eight k's at a time.  A's entries have one power of two for all of them (|A| <= sqrt((2L - 1) / 4 pi))
 // and nine digits, so that they keep 2^-58 of that bound; a data column has its own and eight.  44 products of digits a chunk.
@@ -10,7 +10,7 @@
 // What bounds it: making A's digits, 6000 clocks a chunk of 4096 entries -- loads, one FP64 product an entry (2048 clocks; CUDA
 // cores need four more a field) and the integer instructions behind it, with 60 % of the issue slots busy; the
 // tensor cores' part (1440) is beside it.  L = 512, B = 1: 270 us the inverse and 288 the projection, 517 and 482 on CUDA
-// cores; L = 256, B = 8 91 and 112, about 440 each there.  The next chunk's FP64 products stand one by one among the integer
+// cores; L = 256, B = 8 176 both (245 in two items of four fields), 881 there.  The next chunk's FP64 products stand one by one among the integer
 // instructions (281 and 286 us before).  Taken back: the conversion to integers by F2I (307 and 333 us: it runs at the FP64 pipe's
 // rate), fewer instructions to take the digits out (280 and 299: within the noise).
 #include <algorithm>
@@ -24,11 +24,14 @@
 namespace ssht {
 namespace {
 
-constexpr int kADigits = 9, kFields = 4, kCols = 4 * kFields;
-constexpr int kAPart = 128 * 128, kXPart = kCols * 128;           // two digits' 32 k's
-constexpr int kATile9 = (kADigits + 1) / 2 * kAPart, kXTile = kDigits / 2 * kXPart;
-constexpr int kStageBytes = kATile9 + kXTile, kStages = 2;
-constexpr size_t kSmem = (size_t)kStages * kStageBytes + 1024;
+constexpr int kADigits = 9, kStages = 2;
+constexpr int kAPart = 128 * 128, kATile9 = (kADigits + 1) / 2 * kAPart;  // a part: two digits' 32 k's
+// Fields of a work item: four or eight.
+template <int FIELDS> constexpr int kCols = 4 * FIELDS;
+template <int FIELDS> constexpr int kXPart = kCols<FIELDS> * 128;
+template <int FIELDS> constexpr int kXTile = kDigits / 2 * kXPart<FIELDS>;
+template <int FIELDS> constexpr int kStageBytes = kATile9 + kXTile<FIELDS>;
+template <int FIELDS> constexpr size_t kSmem = (size_t)kStages * kStageBytes<FIELDS> + 1024;
 constexpr int kGenWarps = 16, kThreads = 128 + 32 * kGenWarps;
 constexpr int kRegsIssue = 32, kRegsGen = 112;                    // 128 * 32 + 512 * 112 = 640 * 96
 constexpr int kMaxL = 512;                                        // an item's sums are one segment of at most 512 k's
@@ -45,7 +48,7 @@ __device__ __forceinline__ double2 times_ik(int s, int e, int k, double x, doubl
 }
 
 // ---------------------------------------------------------------------------------------------
-// Data columns: tiles [m][field / 4][chunk] of 16 rows
+// Data columns: tiles [m][field / FIELDS][chunk] of 4 FIELDS rows
 // ---------------------------------------------------------------------------------------------
 // A CTA takes kSources (field, order |m|), each two complex columns -- four rows -- of all k: their largest
 // exponents, then their digits.  The lanes run along orders (inverse: sf_{l,+-m}, contiguous in m) or k (projection: H).
@@ -59,7 +62,7 @@ struct PackArgs {
   int* exps;
 };
 
-template <bool FWD>
+template <bool FWD, int FIELDS>
 __global__ void __launch_bounds__(kPackThreads) digit_columns_kernel(const __grid_constant__ PackArgs a) {
   __shared__ int top[kSources][4];
   const int L = a.L, nc = chunks_of(L), pieces = 4 * nc, items = kSources * pieces, as = a.s < 0 ? -a.s : a.s;
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(kPackThreads) digit_columns_kernel(const __gri
       const int b = (int)(src / L), m = (int)(src - (long long)b * L);
       if (!FWD && (g >> 2) < m / 32) continue;  // below the order: no item reads it
       if (phase == 0 || items > kPackThreads) load(b, m, g);  // else its values are still here
-      const size_t tile = (size_t)m * a.groups + b / kFields;
+      const size_t tile = (size_t)m * a.groups + b / FIELDS;
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         if (phase == 0) {
@@ -109,9 +112,9 @@ __global__ void __launch_bounds__(kPackThreads) digit_columns_kernel(const __gri
           for (int k = 0; k < 8; ++k) e = max(e, exponent_of(x[r][k]));
           if (e > *(volatile int*)&top[so][r]) atomicMax(&top[so][r], e);
         } else {
-          const int row = 4 * (b % kFields) + r, e = top[so][r];
-          if ((g >> 2) == nc - 1 && (g & 3) == 0) a.exps[tile * kCols + row] = e;
-          put_digits<kDigits, kXPart>(a.x + (tile * nc + (g >> 2)) * kXTile, row, g & 3, x[r], e);
+          const int row = 4 * (b % FIELDS) + r, e = top[so][r];
+          if ((g >> 2) == nc - 1 && (g & 3) == 0) a.exps[tile * kCols<FIELDS> + row] = e;
+          put_digits<kDigits, kXPart<FIELDS>>(a.x + (tile * nc + (g >> 2)) * kXTile<FIELDS>, row, g & 3, x[r], e);
         }
       }
     }
@@ -134,7 +137,7 @@ struct GemmArgs {
   long long wait_ns;
 };
 
-// Work item w: order m, row block i, fields 4 g .. 4 g + 3, chunks c0 .. c1 - 1 (none: nothing to do).  The row
+// Work item w: order m, row block i, fields FIELDS g on, chunks c0 .. c1 - 1 (none: nothing to do).  The row
 // blocks with the longest sums come first, so that every CTA gets its share of each.
 struct Item {
   int m, i, g, c0, c1;
@@ -158,15 +161,18 @@ __device__ __forceinline__ Item item_of(const GemmArgs& a, int w) {
 }
 
 // Column of accumulator d: the even ones, then the odd ones.
-__device__ __forceinline__ constexpr uint32_t acc_col(int d) { return kCols * (d >> 1) + (d & 1) * 5 * kCols; }
+template <int FIELDS>
+__device__ __forceinline__ constexpr uint32_t acc_col(int d) { return kCols<FIELDS> * (d >> 1) + (d & 1) * 5 * kCols<FIELDS>; }
 
-template <bool FWD>
+template <bool FWD, int FIELDS>
 __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __grid_constant__ GemmArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   __shared__ __align__(8) uint64_t full[kStages], data_full[kStages], empty[kStages], acc_full[2], acc_empty[2], done_bar;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
+  constexpr int COLS = kCols<FIELDS>, STAGE = kStageBytes<FIELDS>, XTILE = kXTile<FIELDS>, XPART = kXPart<FIELDS>;
+  constexpr bool kTwo = FIELDS == 4;  // two sets of accumulators fit the tensor memory
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 1) tmem_alloc(&tmem_base, 512);
   if (threadIdx.x == 0) {
@@ -199,15 +205,15 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       uint32_t used = 0, uph = 0;  // stages that were filled, and the parity of their last fill
       for (int w = blockIdx.x; w < a.nitems && going(abort); w += gridDim.x) {
         const Item t = item_of<FWD>(a, w);
-        const uint8_t* x = a.x + ((size_t)t.m * a.groups + t.g) * nc * kXTile;
+        const uint8_t* x = a.x + ((size_t)t.m * a.groups + t.g) * nc * XTILE;
         for (int c = t.c0; c < t.c1; ++c) {
           if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort, a.wait_ns))) {
             *abort = 1;
             break;
           }
           if (one) {
-            mbar_expect_tx(&data_full[s], (uint32_t)kXTile);
-            bulk_g2s(smem + s * kStageBytes + kATile9, x + (size_t)c * kXTile, kXTile, &data_full[s]);
+            mbar_expect_tx(&data_full[s], (uint32_t)XTILE);
+            bulk_g2s(smem + s * STAGE + kATile9, x + (size_t)c * XTILE, XTILE, &data_full[s]);
           }
           used |= 1u << s;
           uph = (uph & ~(1u << s)) | ((uint32_t)(ph ^ 1) << s);
@@ -239,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
           }
           fence_after();
           if (one) {
-            const uint32_t la = lo0 + (uint32_t)(s * (kStageBytes >> 4)), lb = la + (kATile9 >> 4), dt = tbase + 256u * buf;
+            const uint32_t la = lo0 + (uint32_t)(s * (STAGE >> 4)), lb = la + (kATile9 >> 4), dt = tbase + 256u * buf;
             const uint32_t more = c > t.c0 ? 1u : 0u;
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
@@ -247,12 +253,12 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
               for (int i = 0; i < kADigits; ++i) {
                 const int jm = kDigits - 1 < kADigits - 1 - i ? kDigits - 1 : kADigits - 1 - i, even = jm / 2 + 1, odd = (jm + 1) / 2;
                 const uint32_t da = la + (i >> 1) * (kAPart >> 4) + (i & 1) * 4 + 2 * kk, init = kk == 0 && i == 0 ? more : 1u;
-                mma_f16_lo<false>(dt + acc_col(i), da, lb + 2 * kk, idesc_f16(128, kCols * even), init);
+                mma_f16_lo<false>(dt + acc_col<FIELDS>(i), da, lb + 2 * kk, idesc_f16(128, COLS * even), init);
                 if (i == 1) {  // accumulator 8 has its first product here
-                  mma_f16_lo<false>(dt + acc_col(2), da, lb + 4 + 2 * kk, idesc_f16(128, kCols * (odd - 1)), 1u);
-                  mma_f16_lo<false>(dt + acc_col(8), da, lb + (odd - 1) * (kXPart >> 4) + 4 + 2 * kk, idesc_f16(128, kCols), kk == 0 ? more : 1u);
+                  mma_f16_lo<false>(dt + acc_col<FIELDS>(2), da, lb + 4 + 2 * kk, idesc_f16(128, COLS * (odd - 1)), 1u);
+                  mma_f16_lo<false>(dt + acc_col<FIELDS>(8), da, lb + (odd - 1) * (XPART >> 4) + 4 + 2 * kk, idesc_f16(128, COLS), kk == 0 ? more : 1u);
                 } else if (odd) {
-                  mma_f16_lo<false>(dt + acc_col(i + 1), da, lb + 4 + 2 * kk, idesc_f16(128, kCols * odd), init);
+                  mma_f16_lo<false>(dt + acc_col<FIELDS>(i + 1), da, lb + 4 + 2 * kk, idesc_f16(128, COLS * odd), init);
                 }
               }
             mma_commit(&empty[s]);
@@ -264,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
             ph ^= 1;
           }
         }
-        buf ^= 1;
+        if (kTwo) buf ^= 1;
         if (buf == 0) bph ^= 1;
       }
       // every issued product has completed before the CTA leaves
@@ -279,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
     // a thread's row and piece of eight k's: lanes along the table's contiguous m'
     const int row = FWD ? gt >> 2 : gt & 127, piece = FWD ? gt & 3 : gt >> 7;
     const int q = warp & 3, cg = (warp - 4) >> 2;
-    const uint32_t tq = tbase + ((uint32_t)(q * 32) << 16) + 4 * cg;
+    const uint32_t tq = tbase + ((uint32_t)(q * 32) << 16) + FIELDS * cg;
     int s = 0, ph = 1, buf = 0, bph = 0;
 
     auto drain = [&](const Item& t) {  // false: gave up
@@ -288,38 +294,45 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
         return false;
       }
       fence_after();
-      uint32_t v[kADigits][4];
+      const uint32_t acc = tq + 256 * buf;
+      const int r = 128 * t.i + 32 * q + lane, m = t.m;
 #pragma unroll
-      for (int d = 0; d < kADigits; ++d) tmem_ld4_nowait(tq + 256 * buf + acc_col(d), v[d]);
-      tmem_wait_ld();
-      fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[buf]);
-      buf ^= 1;
-      if (buf == 0) bph ^= 1;
-      const int r = 128 * t.i + 32 * q + lane, b = kFields * t.g + cg;
-      if (b >= a.B || r >= L || (FWD && r < t.m)) return true;
-      const int4 e = __ldg((const int4*)(a.xexp + ((size_t)t.m * a.groups + t.g) * kCols + 4 * cg));
-      const int xe[4] = {e.x, e.y, e.z, e.w};
-      double z[4];
+      for (int f = 0; f < FIELDS / 4; ++f) {
+        uint32_t v[kADigits][4];
+        __syncwarp();
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        int d[kADigits];  // whole numbers of at most min(i + 1, 8) 2^21
+        for (int d = 0; d < kADigits; ++d) tmem_ld4_nowait(acc + acc_col<FIELDS>(d) + 4 * f, v[d]);
+        tmem_wait_ld();
+        if (f + 1 == FIELDS / 4) {  // all is read
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[buf]);
+          if (kTwo) buf ^= 1;
+          if (buf == 0) bph ^= 1;
+        }
+        const int b = FIELDS * t.g + cg * (FIELDS / 4) + f;
+        if (b >= a.B || r >= L || (FWD && r < m)) continue;
+        const int4 e = __ldg((const int4*)(a.xexp + ((size_t)m * a.groups + t.g) * COLS + FIELDS * cg + 4 * f));
+        const int xe[4] = {e.x, e.y, e.z, e.w};
+        double z[4];
 #pragma unroll
-        for (int i = 0; i < kADigits; ++i) d[i] = __float2int_rn(__uint_as_float(v[i][k]));
-        const long long hi = (long long)(d[0] * 128 + d[1]) * 16384 + (d[2] * 128 + d[3]);
-        const long long lo = ((long long)(d[4] * 128 + d[5]) * 16384 + (d[6] * 128 + d[7])) * 128 + d[8];
-        z[k] = assemble(hi * 128, lo, a.aexp + xe[k] - 2112);
-      }
-      const int m = t.m;
-      if (FWD) {  // +m: (-1)^m; -m: (-1)^{l+m}
-        const long long o = (long long)b * L * L + (long long)r * r + r + m;
-        if (in_bounds(o, a.out_n, kbSimtOut)) a.out[o] = times_ik(a.s, m, m + a.s, z[0], z[1]);
-        if (m > 0 && in_bounds(o - 2 * m, a.out_n, kbSimtOut)) a.out[o - 2 * m] = times_ik(a.s, r + m, a.s - m, z[2], z[3]);
-      } else {  // +m: (-1)^{m'-m}; -m: (-1)^m
-        const long long o = ((long long)b * (2 * L - 1) + L - 1 + m) * L + r, on = o - 2ll * m * L;
-        if (in_bounds(o, a.out_n, kbSimtOut)) a.out[o] = times_ik(a.s, r - m, -(m + a.s), z[0], z[1]);
-        if (m > 0 && in_bounds(on, a.out_n, kbSimtOut)) a.out[on] = times_ik(a.s, m, m - a.s, z[2], z[3]);
+        for (int k = 0; k < 4; ++k) {
+          int d[kADigits];  // whole numbers of at most min(i + 1, 8) 2^21
+#pragma unroll
+          for (int i = 0; i < kADigits; ++i) d[i] = __float2int_rn(__uint_as_float(v[i][k]));
+          const long long hi = (long long)(d[0] * 128 + d[1]) * 16384 + (d[2] * 128 + d[3]);
+          const long long lo = ((long long)(d[4] * 128 + d[5]) * 16384 + (d[6] * 128 + d[7])) * 128 + d[8];
+          z[k] = assemble(hi * 128, lo, a.aexp + xe[k] - 2112);
+        }
+        if (FWD) {  // +m: (-1)^m; -m: (-1)^{l+m}
+          const long long o = (long long)b * L * L + (long long)r * r + r + m;
+          if (in_bounds(o, a.out_n, kbSimtOut)) a.out[o] = times_ik(a.s, m, m + a.s, z[0], z[1]);
+          if (m > 0 && in_bounds(o - 2 * m, a.out_n, kbSimtOut)) a.out[o - 2 * m] = times_ik(a.s, r + m, a.s - m, z[2], z[3]);
+        } else {  // +m: (-1)^{m'-m}; -m: (-1)^m
+          const long long o = ((long long)b * (2 * L - 1) + L - 1 + m) * L + r, on = o - 2ll * m * L;
+          if (in_bounds(o, a.out_n, kbSimtOut)) a.out[o] = times_ik(a.s, r - m, -(m + a.s), z[0], z[1]);
+          if (m > 0 && in_bounds(on, a.out_n, kbSimtOut)) a.out[on] = times_ik(a.s, m, m - a.s, z[2], z[3]);
+        }
       }
       return true;
     };
@@ -400,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
           ok = false;
           break;
         }
-        put_integers<kADigits, kAPart>(smem + s * kStageBytes, row, piece, v);
+        put_integers<kADigits, kAPart>(smem + s * STAGE, row, piece, v);
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) mbar_arrive(&full[s]);
@@ -430,9 +443,12 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
   if (warp == 1) tmem_dealloc(tbase, 512);
 }
 
-int groups_of(int B) { return (B + kFields - 1) / kFields; }
+// Four fields an item (two sets of accumulators then fit the tensor memory), or eight beyond that: A's digits, the larger
+// part of the work, are made once for them (L = 256, B = 8 245 -> 176 us, L = 64, B = 64 151 -> 127).
+int fields_of(int B) { return B > 4 ? 8 : 4; }
+int groups_of(int B) { return (B + fields_of(B) - 1) / fields_of(B); }
 
-template <bool FWD>
+template <bool FWD, int FIELDS>
 cudaError_t run(int L, int s, int B, int sms, const double* table, const double* U, const void* in, size_t in_bytes, void* work,
                 void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
   PackArgs k{};
@@ -443,8 +459,8 @@ cudaError_t run(int L, int s, int B, int sms, const double* table, const double*
   k.in = (const double2*)in;
   k.in_n = (long long)(in_bytes / sizeof(double2));
   k.x = (uint8_t*)work;
-  k.exps = (int*)((uint8_t*)work + (size_t)L * k.groups * chunks_of(L) * kXTile);
-  digit_columns_kernel<FWD><<<(unsigned)(((long long)B * L + kSources - 1) / kSources), kPackThreads, 0, st>>>(k);
+  k.exps = (int*)((uint8_t*)work + (size_t)L * k.groups * chunks_of(L) * kXTile<FIELDS>);
+  digit_columns_kernel<FWD, FIELDS><<<(unsigned)(((long long)B * L + kSources - 1) / kSources), kPackThreads, 0, st>>>(k);
   GemmArgs a{};
   a.L = L;
   a.s = s;
@@ -464,37 +480,43 @@ cudaError_t run(int L, int s, int B, int sms, const double* table, const double*
   a.out_n = (long long)(out_bytes / sizeof(double2));
   a.status = status;
   a.wait_ns = wait_ns;
-  digit_contract_kernel<FWD><<<(unsigned)std::min(a.nitems, sms), kThreads, kSmem, st>>>(a);
+  digit_contract_kernel<FWD, FIELDS><<<(unsigned)std::min(a.nitems, sms), kThreads, kSmem<FIELDS>, st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 // Where they beat the CUDA cores' contractions, an inverse and a projection in us, these and those: L = 512, B = 1 594 and 1006,
-// B = 4 627 and 3041; L = 256, B = 1 136 and 168, B = 8 245 and 881; L = 192, B = 8 173 and 413; L = 129, B = 4 75 and 92; L = 64,
-// B = 64 151 and 208.  Below B L^3 = 2^23 few items, of few chunks, leave the launch and the epilogue (L = 192, B = 1 109 and 98;
+// B = 4 627 and 3041; L = 256, B = 1 136 and 168, B = 8 176 and 881; L = 192, B = 8 133 and 413; L = 129, B = 4 75 and 92; L = 64,
+// B = 64 127 and 208.  Below B L^3 = 2^23 few items, of few chunks, leave the launch and the epilogue (L = 192, B = 1 109 and 98;
 // L = 160, B = 1 86 and 63), and below L = 64 half of a tile's rows are empty (L = 40, B = 96 156 and 126).
 bool contract_digits_wanted(int L, int B) { return L >= 64 && L <= kMaxL && (long long)B * L * L * L > (1ll << 23); }
 
 size_t contract_digits_bytes(int L, int B) {
-  return (size_t)L * groups_of(B) * (chunks_of(L) * (size_t)kXTile + kCols * sizeof(int));
+  const size_t cols = 4 * fields_of(B);
+  return (size_t)L * groups_of(B) * cols * (chunks_of(L) * (size_t)(kDigits * 64) + sizeof(int));
+}
+
+template <bool FWD, int FIELDS>
+static cudaError_t kernel_attr() {
+  cudaError_t e = prefer_shared(digit_contract_kernel<FWD, FIELDS>);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(digit_contract_kernel<FWD, FIELDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem<FIELDS>);
 }
 
 cudaError_t contract_digits_setup() {
-  cudaError_t e = prefer_shared(digit_contract_kernel<false>);
-  if (e == cudaSuccess) e = prefer_shared(digit_contract_kernel<true>);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(digit_contract_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(digit_contract_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  cudaError_t e = kernel_attr<false, 4>();
+  if (e == cudaSuccess) e = kernel_attr<true, 4>();
+  if (e == cudaSuccess) e = kernel_attr<false, 8>();
+  if (e == cudaSuccess) e = kernel_attr<true, 8>();
   return e;
 }
 
 cudaError_t contract_digits(int forward, int L, int s, int B, int sms, const double* table, const double* U, const void* in,
                             size_t in_bytes, void* work, void* out, size_t out_bytes, int* status, long long wait_ns,
                             cudaStream_t st) {
-  return forward ? run<true>(L, s, B, sms, table, U, in, in_bytes, work, out, out_bytes, status, wait_ns, st)
-                 : run<false>(L, s, B, sms, table, U, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
+  auto go = fields_of(B) == 8 ? (forward ? run<true, 8> : run<false, 8>) : (forward ? run<true, 4> : run<false, 4>);
+  return go(L, s, B, sms, table, U, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
 }
 
 SSHT_BOUNDS_TU(contract_digits)

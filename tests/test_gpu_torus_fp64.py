@@ -25,12 +25,12 @@ def rel(a, b):
 
 # (L, s, B): smallest sizes; edges of 32 rows and k's and of 128 rows; B L^3 on both sides of 2^21 (128, 1 and 129, 1); data
 # tiles of 16 and 32 columns with a last one not full; more than 512 k's (two segments of sums, and packing in two reads);
-# contractions of digits (B L^3 > 2^23, 64 <= L <= 512): one to nine fields in groups of four, edges of 32 k's and 128 rows, |s|
+# contractions of digits (B L^3 > 2^23, 64 <= L <= 512): one to 33 fields in groups of four or eight, edges of 32 k's and 128 rows, |s|
 # beyond the first row blocks
 @pytest.mark.parametrize("L,s,B", [(1, 0, 3), (2, -1, 2), (3, 2, 1), (32, 1, 2), (33, -2, 1), (65, 0, 2), (100, 2, 10),
                                    (128, 1, 4), (128, -1, 5), (95, 0, 9), (95, 2, 10), (203, 1, 1), (209, 0, 1),
                                    (32, -1, 80), (33, 0, 64), (33, -2, 70), (127, 1, 2), (128, 0, 1), (129, 2, 1), (161, 1, 7),
-                                   (513, 1, 1), (128, 0, 5), (129, 2, 4), (129, -64, 5), (64, 1, 33), (64, -63, 33), (100, 0, 9),
+                                   (513, 1, 1), (128, 0, 5), (128, 1, 8), (128, 2, 17), (129, 2, 4), (129, -64, 5), (64, 1, 33), (64, -63, 33), (100, 0, 9),
                                    (257, -2, 1), (384, 1, 1), (512, 0, 1)])
 def test_both_torus_stages_match_oracle(L, s, B):
     from paper_0807_4494_gb300 import ssht
