@@ -588,8 +588,8 @@ __global__ void __launch_bounds__(kColThreads, 4) lane_recursion_kernel(LanePara
   }
 }
 
-// The same sweep for small band-limits, where a warp has at most a task or two and a step lasts as long
-// as its chain of instructions: four rows at a time, the recursion first and then their outputs, whose
+// The same sweep for small band-limits (L <= 1024: it reads no exponents), where a warp has at most a task or two
+// and a step lasts as long as its chain of instructions: four rows at a time, the recursion first and then their outputs, whose
 // chains overlap, with the rows' loads (alpha, p, U, tile base) issued four rows ahead.  Two CTAs an SM are
 // room enough for its registers.  GB300: L = 257 104 -> 80 us a sweep, L = 512 221 -> 175; L = 1024 788 -> 905, where
 // the variant above, with twice the warps, is taken.
@@ -890,8 +890,9 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
       return e;
     t.blocks = sms * std::max(1, std::min(per_sm, SSHT_LANE_CTAS));
     // the variant of four rows a step while its two CTAs an SM have room for half of the tasks at once
-    // (up to L = 550 or so; between the L = 512 and L = 1024 figures beside it)
-    t.deep = t.ntasks <= 2 * 2 * sms * kColWarps;
+    // (up to L = 550 or so, further for spins near L, whose tasks are few; between the L = 512 and L = 1024
+    // figures beside it), and only where first rows need no exponents of their own
+    t.deep = L <= 1024 && t.ntasks <= 2 * 2 * sms * kColWarps;
     if (t.deep) t.blocks = 2 * sms;
     const void* fns[4] = {(const void*)column_tiles_kernel<false, false>, (const void*)column_tiles_kernel<true, false>,
                           (const void*)column_tiles_kernel<false, true>, (const void*)column_tiles_kernel<true, true>};
