@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256) pack_a_kernel(int L, int s, const Item* _
 // and turned around in shared memory.  Split-FP16: a thread then takes
 // 8 K of one order, sign and field, four neighbouring threads the 32 K of a tile row, so that they find the
 // row pair's power of two with two shuffles and store 16 bytes at a time.  Split-BF16: a warp takes a row
-// pair, a lane one K.  The rows of padding fields are written as zeros.  Fields run in slices of Bs, slice z
+// pair, a lane one K.  The rows of padding fields stay as tc_configure zeroed them.  Fields run in slices of Bs, slice z
 // in its own tile region of xslice bytes, and a CTA takes kPackFields rows' worth of fields of a slice
 // (blockIdx.z: slice and group of fields), which keeps the GPU filled at small band-limits too.  Bound by HBM
 // traffic (1.1 GB at L = 1024, B = 64: 0.16 ms) and by how many loads are in flight: six CTAs on an SM (40
@@ -182,11 +182,11 @@ __global__ void __launch_bounds__(256, 6) pack_v_kernel(int L, int s, int Btot, 
   const int c = blockIdx.x, m0 = 16 * blockIdx.y;
   // xc0 grows with m: when chunk c is below the first stored chunk of m0, no tile of this CTA's 16
   // orders is stored (about half the grid: the degrees of chunk c all lie below m0)
-  if (m0 >= L || c < xc0[m0]) return;
+  if (m0 >= L || c < xc0[m0] || bg >= B) return;
   const int as = s < 0 ? -s : s;
   const int part_bytes = NC * 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b_end = min(bg + kPackFields, nb);
+  const int b_end = min(bg + kPackFields, B);
   // 32 degrees l x (orders m0 .. m0 + 15, then -m0 .. -m0 - 15) of a field: four values a thread, whose
   // places in a field are the same for every field
   int at[4];
@@ -636,6 +636,12 @@ cudaError_t tc_configure(TcPlan* p, const TcConfig& c) {
     if ((e = tc_alloc((void**)&p->XS, xsbytes, &p->bytes)) != cudaSuccess) return e;
     p->xsbytes = xsbytes;
   }
+  // The rows of padding fields are the same in every tile of a slice, in both directions: zeroed here,
+  // written by no call.  (Zeroed by every call, they were most of the tiles' writes with few fields: the
+  // cached forward of one field at L = 128 took 59 us with split FP16 and 72 with split BF16, now 39 and 41.)
+  if ((e = cudaMemset(p->X, 0, p->xbytes)) != cudaSuccess) return e;
+  if (p->xsbytes && (e = cudaMemset(p->XS, 0, p->xsbytes)) != cudaSuccess) return e;
+  if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;  // the calls' streams do not wait for the legacy one
   p->Bs = Bs;
   p->nS = nS;
   p->NC = NC;

@@ -359,7 +359,7 @@ __device__ __forceinline__ int group_col(int cg, int g) {
 // the 16 orders' chains of reduction, split and stores overlap.
 template <bool BF>
 __device__ __forceinline__ void put_orders(const TileOut& to, int sl, int am0, int row, int lane, int L, int half, int r0,
-                                           bool last, int pad0, float sgn, const float* acc) {
+                                           float sgn, const float* acc) {
   const int pbytes = to.NC * 128, orders = min(16, (L - am0 + 1) >> 1);
   const size_t tb = (size_t)kParts<BF> * pbytes;
   const long long slice_tiles = (long long)(to.xslice / tb), n = (long long)(to.xbytes / tb);
@@ -385,19 +385,6 @@ __device__ __forceinline__ void put_orders(const TileOut& to, int sl, int am0, i
     sc[r0 >> 1] = mine;
     sc[(half + r0) >> 1] = mine;
   }
-  if (last && rows_ok)  // the slice's padding rows
-    for (int k = 0; k < orders; ++k) {
-      const long long tp = tix0 + 2 * k * to.nC;
-      if (!in_bounds(tp, n, kbPutTile)) continue;
-      for (int rw = pad0; rw < half; rw += 2) {
-        put_rows2<BF>(to.X + (size_t)tp * tb, pbytes, rw, lane, 0.f, 0.f, 1.f, true);
-        put_rows2<BF>(to.X + (size_t)tp * tb, pbytes, half + rw, lane, 0.f, 0.f, 1.f, true);
-        if (!BF && lane == 0) {
-          to.scale[(size_t)tp * half + (rw >> 1)] = 0.f;
-          to.scale[(size_t)tp * half + ((half + rw) >> 1)] = 0.f;
-        }
-      }
-    }
 }
 
 // Persistent, one CTA an SM; the row blocks of a column tile are consecutive items, so that its
@@ -744,16 +731,16 @@ __device__ __forceinline__ void torus_gemm(const TgArgs& a) {
           continue;
         }
         // the projection's data tiles (|m|, m' / 32): rows sign * NC/2 + 2b + part, K = m', the negative
-        // half carrying (-1)^{m'} (zeros for m = 0); a slice's last field zeroes the padding rows.  The
+        // half carrying (-1)^{m'} (zeros for m = 0; padding rows stay as the plan zeroed them).  The
         // rows' offsets are the same in every tile, the tiles of the 16 orders two |m| apart.
-        const int sl = b / a.to.Bs, bs = b - sl * a.to.Bs, nB = min(a.to.Bs, a.B - sl * a.to.Bs);
+        const int sl = b / a.to.Bs, bs = b - sl * a.to.Bs;
         const int half = a.to.NC / 2;
         if (am0 == 0) acc[32] = acc[48] = 0.f;
         const float sgn = (row & 1) ? -1.f : 1.f;
         if (a.to.mode == 2)
-          put_orders<true>(a.to, sl, am0, row, lane, L, half, 2 * bs, bs == nB - 1, 2 * nB, sgn, acc);
+          put_orders<true>(a.to, sl, am0, row, lane, L, half, 2 * bs, sgn, acc);
         else
-          put_orders<false>(a.to, sl, am0, row, lane, L, half, 2 * bs, bs == nB - 1, 2 * nB, sgn, acc);
+          put_orders<false>(a.to, sl, am0, row, lane, L, half, 2 * bs, sgn, acc);
       }
     }
     if constexpr (MODE == kThetaInverse || MODE == kPhiForward) {
