@@ -119,6 +119,7 @@ struct ssht_plan_s {
   TorusPlan* torus = nullptr;  // torus products of FP32-class plans
   DigitPlan* digits = nullptr;   // torus products of FP64 plans
   DirectPlan* direct = nullptr;  // ... and of those with little work
+  SmallPlan* small = nullptr;    // torus products of small band-limits, any precision
   bool contract_digits = false;  // FP64 contractions on tensor cores
   int sms = 0;                   // of the plan's device
   // The Delta recursion (and the A packing) of a call runs on a second stream, forked from the
@@ -435,21 +436,38 @@ int fp64_pass(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t 
   return 0;
 }
 
-// FP32-class forward (adjoint = 0) or adjoint: the torus passes, then the projection.  Tensor-core plans:
-// the theta pass writes the projection's data tiles itself (no H, no data packing).
-template <typename T>
-int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st);
-
-int analysis_fp32(ssht_plan_t p, int adjoint, const void* f, void* flm, cudaStream_t st) {
+// The torus stage: half rows in W1 -> samples f.
+int torus_to_samples(ssht_plan_t p, void* f, cudaStream_t st) {
   int rc;
-  if ((rc = torus_analysis_pass(p, 0, adjoint, f, st)) || (rc = torus_analysis_pass(p, 1, adjoint, f, st))) return rc;
-  if (!p->tc) return project<float>(p, p->W1, flm, st);
-  if ((rc = join_operands(p, st)) || (rc = tc_multiply(p, 1, flm, st))) return rc;
-  return mark_free_a(p, 1, st);
+  if (p->small) {
+    StageScope sc(p, SSHT_STAGE_FFT, st);
+    SSHT_CUDA(small_inverse(p->small, p->s, p->B, p->W1, p->w_bytes, f, p->pair_grid_bytes(), st), "torus product");
+    p->launches += 1;
+    return 0;
+  }
+  if (p->torus) return (rc = torus_inverse_pass(p, 0, f, st)) ? rc : torus_inverse_pass(p, 1, f, st);
+  return (rc = fp64_pass(p, 0, p->W1, p->W2, st)) ? rc : fp64_pass(p, 1, p->W2, f, st);
+}
+
+// Forward / adjoint: samples f -> H in W1, or (tensor-core plans) the projection's data tiles (no H, no data
+// packing).
+int torus_from_samples(ssht_plan_t p, int adjoint, const void* f, cudaStream_t st) {
+  int rc;
+  if (p->small) {
+    StageScope sc(p, SSHT_STAGE_FFT, st);
+    TileOut tiles;
+    if (p->tc) tiles = tc_forward_tiles(p->tc);
+    SSHT_CUDA(small_analysis(p->small, adjoint, p->s, p->B, f, p->pair_grid_bytes(), p->W1, p->w_bytes, p->tc ? &tiles : nullptr, st),
+              "torus product");
+    p->launches += 1;
+    return 0;
+  }
+  if (p->torus) return (rc = torus_analysis_pass(p, 0, adjoint, f, st)) ? rc : torus_analysis_pass(p, 1, adjoint, f, st);
+  return (rc = fp64_pass(p, 2, f, p->W2, st)) ? rc : fp64_pass(p, adjoint ? 4 : 3, p->W2, p->W1, st);
 }
 
 // The SIMT projection of forward / adjoint from the folded torus sums H (in W), after the join
-// (tensor-core plans: analysis_fp32).
+// (tensor-core plans: analysis_impl).
 template <typename T>
 int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st) {
   int rc;
@@ -560,12 +578,7 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
     p->launches += p->contract_digits ? 2 : 1;
   }
   if (!p->tc && (rc = mark_free(p, st))) return rc;
-  if (p->torus) {
-    if ((rc = torus_inverse_pass(p, 0, f, st))) return rc;
-    return torus_inverse_pass(p, 1, f, st);
-  }
-  if ((rc = fp64_pass(p, 0, p->W1, p->W2, st))) return rc;
-  return fp64_pass(p, 1, p->W2, f, st);
+  return torus_to_samples(p, f, st);
 }
 
 // Front of the triangular forward: phi DFT, extension into the theta-DFT input, theta DFT in place in W1.
@@ -585,10 +598,10 @@ int analysis_front(ssht_plan_t p, const void* f, cudaStream_t st) {
 template <typename T>
 int analysis_impl(ssht_plan_t p, int adjoint, const void* f, void* flm, cudaStream_t st) {
   int rc = begin_operands(p, 1, st);
-  if (rc) return rc;
-  if (p->torus) return analysis_fp32(p, adjoint, f, flm, st);
-  if ((rc = fp64_pass(p, 2, f, p->W2, st)) || (rc = fp64_pass(p, adjoint ? 4 : 3, p->W2, p->W1, st))) return rc;
-  return project<T>(p, p->W1, flm, st);
+  if (rc || (rc = torus_from_samples(p, adjoint, f, st))) return rc;
+  if (!p->tc) return project<T>(p, p->W1, flm, st);
+  if ((rc = join_operands(p, st)) || (rc = tc_multiply(p, 1, flm, st))) return rc;
+  return mark_free_a(p, 1, st);
 }
 template <typename T>
 int forward_impl(ssht_plan_t p, const void* f, void* flm, cudaStream_t st) {
@@ -781,6 +794,7 @@ void release(ssht_plan_t p) {
   if (p->tc) tc_destroy(p->tc);
   if (p->torus) torus_destroy(p->torus);
   if (p->direct) direct_destroy(p->direct);
+  if (p->small) small_destroy(p->small);
   if (p->digits) digits_destroy(p->digits);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
@@ -871,8 +885,13 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, (void**)&p->U, tri(L) * sizeof(double), "spin column"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->Uf, tri(L) * sizeof(float), "spin column (FP32)"))) return bail(rc);
   // FP64: full N x N torus rows (the triangular forward's; the products' half rows, and L x L twice over, fit
-  // but for L = 1) and the digits of a pass's data; FP32: half rows of N x L, or a pass's operand tiles.
-  const size_t torus = p->f64 ? (size_t)B * std::max(d.N * d.N, 2) * p->elem : torus_workspace_bytes(L, B);
+  // but for L = 1) and the digits of a pass's data; FP32: half rows of N x L, or a pass's operand tiles (small
+  // band-limits have none; tuning writes a contraction's output to the second workspace).
+  const bool small = small_wanted(L, B, p->f64);
+  const size_t half_rows = (size_t)B * d.N * L * p->elem;
+  const size_t torus = p->f64 ? (size_t)B * std::max(d.N * d.N, 2) * p->elem : small ? half_rows : torus_workspace_bytes(L, B);
+  const bool tensor = desc->precision == SSHT_TF32X3 || desc->precision == SSHT_BF16X6;
+  const size_t second = p->f64 || !small ? torus : tensor ? p->pair_coeff_bytes() : 0;
   if (pair && (rc = dalloc(p, &p->rc, (size_t)B * L * L * p->elem, "spin-pair coefficients"))) return bail(rc);
   if ((real || pair) && (ce = real_setup()) != cudaSuccess) {
     release(p);
@@ -883,11 +902,11 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     if ((rc = dalloc(p, &p->rg, p->pair_grid_bytes(), "real-field pair samples"))) return bail(rc);
   }
   if ((rc = dalloc(p, &p->W1, torus, "torus workspace 1"))) return bail(rc);
-  if ((rc = dalloc(p, &p->W2, torus, "torus workspace 2"))) return bail(rc);
+  if ((rc = dalloc(p, &p->W2, second, "torus workspace 2"))) return bail(rc);
   p->w_bytes = torus;
-  const bool direct = p->f64 && direct_wanted(L, B);
-  p->contract_digits = p->f64 && !direct && contract_digits_wanted(L, B);
-  if (p->f64 && !direct) {
+  const bool direct = p->f64 && !small && direct_wanted(L, B);
+  p->contract_digits = p->f64 && !direct && !small && contract_digits_wanted(L, B);
+  if (p->f64 && !direct && !small) {
     size_t w3 = digits_workspace_bytes(L, s, B);
     if (p->contract_digits) {
       w3 = std::max(w3, contract_digits_bytes(L, B));
@@ -927,14 +946,17 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     if ((rc = make_fft(p, &p->fft_phi, &p->have_phi, d.N, (size_t)B * d.L, "cuFFT phi plan"))) return bail(rc);
     if ((rc = make_fft(p, &p->fft_theta, &p->have_theta, d.N, (size_t)B * d.N, "cuFFT theta plan"))) return bail(rc);
   }
-  ce = direct ? direct_setup(&p->direct, L) : p->f64 ? digits_setup(&p->digits, L, p->device) : torus_setup(&p->torus, L, p->device);
+  ce = small    ? small_setup(&p->small, L, p->f64, p->device)
+       : direct ? direct_setup(&p->direct, L)
+       : p->f64 ? digits_setup(&p->digits, L, p->device)
+                : torus_setup(&p->torus, L, p->device);
   if (ce != cudaSuccess) {
     release(p);
     return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA,
                 std::string("torus pass setup: ") + cudaGetErrorString(ce));
   }
-  p->bytes += direct_bytes(p->direct) + digits_bytes(p->digits) + torus_bytes(p->torus);
-  if (desc->precision == SSHT_TF32X3 || desc->precision == SSHT_BF16X6) {
+  p->bytes += small_bytes(p->small) + direct_bytes(p->direct) + digits_bytes(p->digits) + torus_bytes(p->torus);
+  if (tensor) {
     ce = tc_setup(&p->tc, L, s, B, desc->precision == SSHT_BF16X6 ? 1 : 0, p->device);
     if (ce != cudaSuccess) {
       release(p);
@@ -1229,7 +1251,7 @@ int ssht_debug_fail_allocation(int n) {
 int ssht_debug_bounds(long long* count, int* site, long long* index, long long* extent) {
   if (!kBoundsChecked) return fail(SSHT_EUNSUPPORTED, "ssht_debug_bounds: this library was built without index checks");
   SSHT_CUDA(cudaDeviceSynchronize(), "synchronize");
-  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass,  bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc,
+  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass,  bounds_take_torus_small, bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc,
                                           bounds_take_delta_column, bounds_take_real, bounds_take_contract_simt};
   BoundsRecord first{};
   long long total = 0;

@@ -237,7 +237,7 @@ cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const 
                            int* launches, int step);
 
 // ---------------------------------------------------------------------------
-// Torus passes of FP64 plans (torus_digits.cu, torus_direct.cu)
+// Torus passes of FP64 plans (torus_digits.cu, torus_direct.cu) and of small band-limits (torus_small.cu)
 // ---------------------------------------------------------------------------
 // The same folded products as the FP32 plans' passes, on tensor cores with both operands in fixed-point digits,
 // or, with little work, in FP64 on CUDA cores.  F, H: half rows (double2) [B][m + L - 1][m']; E, O: [2][B][m][t];
@@ -251,6 +251,18 @@ size_t digits_workspace_bytes(int L, int s, int B);
 // and adjoint, samples -> P, Q; 3 theta of the forward (with the extension and the sin(theta) weight), 4 of the adjoint, P, Q -> H.
 cudaError_t digits_pass(const DigitPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* work, void* mid,
                         size_t mid_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st);
+
+// Small band-limits, FP64 and FP32-class plans (torus_small.cu): theta and phi in one launch on CUDA cores, no workspace.
+struct SmallPlan;
+bool small_wanted(int L, int B, bool f64);  // whether a plan takes this form
+cudaError_t small_setup(SmallPlan** out, int L, bool f64, int device);  // synchronises
+void small_destroy(SmallPlan* p);
+size_t small_bytes(const SmallPlan* p);
+cudaError_t small_inverse(const SmallPlan* p, int s, int B, const void* F, size_t f_bytes, void* out, size_t out_bytes,
+                          cudaStream_t st);
+// Samples -> H, or the projection's data tiles (FP32-class tensor-core plans).
+cudaError_t small_analysis(const SmallPlan* p, int adjoint, int s, int B, const void* f, size_t f_bytes, void* H, size_t h_bytes,
+                           const TileOut* tiles, cudaStream_t st);
 
 struct DirectPlan;
 bool direct_wanted(int L, int B);  // whether a plan of this band-limit and batch takes the CUDA cores
@@ -287,6 +299,7 @@ cudaError_t bounds_take_torus_pass(BoundsRecord* r);
 cudaError_t bounds_take_contract_tc(BoundsRecord* r);
 cudaError_t bounds_take_delta_column(BoundsRecord* r);
 cudaError_t bounds_take_torus_digits(BoundsRecord* r);
+cudaError_t bounds_take_torus_small(BoundsRecord* r);
 cudaError_t bounds_take_contract_digits(BoundsRecord* r);
 cudaError_t bounds_take_real(BoundsRecord* r);
 cudaError_t bounds_take_contract_simt(BoundsRecord* r);

@@ -1,4 +1,4 @@
-// Torus passes of FP64 plans with little work: the folded cosine and sine products of the torus stage
+// Torus passes of FP64 plans above L = 32 with little work: the folded cosine and sine products of the torus stage
 // (torus_gemm.cu gives the identities) in FP64 on CUDA cores, four launches an inverse + forward.
 //
 // Matrices are stored [k][row], so that a warp's lanes (32 rows) read them coalesced, and a data column is
@@ -18,25 +18,7 @@ namespace {
 
 constexpr int kWarps = 8;
 
-// Matrices, each L x L, [k][row].
-enum Matrix { kCosKX = 0, kSinKX, kCosXK, kSinXK, kWeightE, kWeightO, kMatrices };
-
-__global__ void direct_matrices_kernel(int L, const double2* __restrict__ cs, const double2* __restrict__ T,
-                                       double* __restrict__ out) {
-  const int N = 2 * L - 1;
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)L * L) return;
-  const int k = (int)(e / L), r = (int)(e % L);
-  const size_t n = (size_t)L * L;
-  // order k at node r, and order r at node k; sin vanishes at the node theta = pi
-  const double2 a = cs[(int)(((long long)k * (2 * r + 1)) % (2 * N))], b = cs[(int)(((long long)r * (2 * k + 1)) % (2 * N))];
-  out[kCosKX * n + e] = a.x;
-  out[kSinKX * n + e] = r == L - 1 ? 0.0 : a.y;
-  out[kCosXK * n + e] = b.x;
-  out[kSinXK * n + e] = k == L - 1 ? 0.0 : b.y;
-  out[kWeightE * n + e] = weight_entry(true, L, cs, T, r, k);
-  out[kWeightO * n + e] = weight_entry(false, L, cs, T, r, k);
-}
+using namespace folded;
 
 struct Pair {
   double2 a, b;
@@ -205,31 +187,17 @@ struct DirectPlan {
   size_t bytes = 0;
 };
 
-// Where these products beat those of digits: for little work, where the digits' nine launches set the time, and
-// at band-limits that fill little of their tiles.  GB300, torus stage of an inverse and a forward in us, digits against these: L = 64, B = 1
-// 95 and 43; L = 96, B = 1 101 and 56; L = 128, B = 1 107 and 102; L = 16, B = 4096 2127 and 1727; L = 32, B = 128 193 and 185;
-// beyond the line L = 96, B = 2 104 and 85, L = 64, B = 8 98 and 103 (the two meet there); L = 144, B = 1 115 and 132; L = 128, B = 4 114 and 283.
-bool direct_wanted(int L, int B) { return L <= 32 || (long long)B * L * L * L <= (1ll << 21); }
+// Where these products beat those of digits: for little work, where the digits' nine launches set the time.  (Up to
+// L = 32 one launch does both passes: torus_small.cu.)  GB300, torus stage of an inverse and a forward in us, digits against these: L = 64, B = 1
+// 95 and 43; L = 96, B = 1 101 and 56; L = 128, B = 1 107 and 102; beyond the line L = 96, B = 2 104 and 85, L = 64, B = 8
+// 98 and 103 (the two meet there); L = 144, B = 1 115 and 132; L = 128, B = 4 114 and 283.
+bool direct_wanted(int L, int B) { return (long long)B * L * L * L <= (1ll << 21); }
 
 cudaError_t direct_setup(DirectPlan** out, int L) {
   *out = nullptr;
   DirectPlan* p = new DirectPlan();
   p->L = L;
-  const size_t n = (size_t)L * L, ncs = 2 * (size_t)(2 * L - 1);
-  double2* tmp = nullptr;
-  cudaError_t e = dev_malloc(&p->mats, kMatrices * n * sizeof(double));
-  if (e == cudaSuccess) {
-    p->bytes = kMatrices * n * sizeof(double);
-    e = dev_malloc(&tmp, (ncs + n) * sizeof(double2));
-  }
-  if (e == cudaSuccess) {
-    node_table_kernel<<<(unsigned)((ncs + 255) / 256), 256>>>(2 * L - 1, tmp);
-    weight_prefix_kernel<<<(unsigned)((L + 31) / 32), 32>>>(L, tmp, tmp + ncs);
-    direct_matrices_kernel<<<(unsigned)((n + 255) / 256), 256>>>(L, tmp, tmp + ncs, p->mats);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  }
-  if (tmp) cudaFree(tmp);
+  const cudaError_t e = make_matrices(L, &p->mats, &p->bytes);
   if (e != cudaSuccess) {
     direct_destroy(p);
     return e;

@@ -18,8 +18,8 @@
 // A pass is 8 B L^3 flops (24 B L^3 as split products), against two to four FFTs of 4L .. 8L points a row
 // for the odd length (Bluestein's algorithm in shared memory, the passes this replaces).  GB300, alone, the
 // four passes of an inverse and a forward (theta, phi, phi, theta), products against FFTs: L = 1024, B = 64
-// 1.13, 1.18, 1.18, 1.17 ms against 2.08, 1.27, 1.64, 2.88; the cubic form is the faster one for every
-// L the library takes (L = 2048, B = 16: inverse + forward 40.6 -> 33.4 ms as a whole).
+// 1.13, 1.18, 1.18, 1.17 ms against 2.08, 1.27, 1.64, 2.88; L = 2048, B = 16: inverse + forward 40.6 -> 33.4 ms as
+// a whole.  Small band-limits, which would fill little of the tiles, take torus_small.cu (small_wanted).
 //
 // Precision.  Both operands are split x = hi + lo into two FP16 values (22 to 24 significant bits,
 // the parts of an 11-bit significand each, as in a 3xTF32 split, at twice its rate) and the product

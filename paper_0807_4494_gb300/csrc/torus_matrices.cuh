@@ -1,5 +1,6 @@
-// Plan-time tables of the torus passes' matrices, shared by the tensor-core products (torus_gemm.cu) and
-// the FP64 ones (torus_direct.cu): cos and sin of the multiples of pi/N and the sin(theta) weight's matrices.
+// Plan-time tables of the torus passes' matrices, shared by the products of every form (torus_gemm.cu,
+// torus_digits.cu, torus_direct.cu, torus_small.cu): cos and sin of the multiples of pi/N and the sin(theta)
+// weight's matrices.
 #pragma once
 
 namespace ssht {
@@ -43,6 +44,48 @@ __device__ __forceinline__ double weight_entry(bool even, int L, const double2* 
   const double c = (mp == 0 ? 1.0 : 2.0) * 6.283185307179586476925 * (t == L - 1 ? 1.0 : 2.0) / ((double)N * N);
   return c * (even ? e.x * sr - e.y * si : e.x * si + e.y * sr);
 }
+
+// The folded products' matrices for CUDA cores, each L x L, [k][row], in the element type: order k at node row,
+// order row at node k, and the weight's.  sin vanishes at the node theta = pi.
+namespace folded {
+enum Matrix { kCosKX = 0, kSinKX, kCosXK, kSinXK, kWeightE, kWeightO, kMatrices };
+
+template <typename T>
+__global__ void matrices_kernel(int L, const double2* __restrict__ cs, const double2* __restrict__ tab, T* __restrict__ out) {
+  const int N = 2 * L - 1;
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (long long)L * L) return;
+  const int k = (int)(e / L), r = (int)(e % L);
+  const size_t n = (size_t)L * L;
+  const double2 a = cs[(int)(((long long)k * (2 * r + 1)) % (2 * N))], b = cs[(int)(((long long)r * (2 * k + 1)) % (2 * N))];
+  out[kCosKX * n + e] = (T)a.x;
+  out[kSinKX * n + e] = r == L - 1 ? T(0) : (T)a.y;
+  out[kCosXK * n + e] = (T)b.x;
+  out[kSinXK * n + e] = k == L - 1 ? T(0) : (T)b.y;
+  out[kWeightE * n + e] = (T)weight_entry(true, L, cs, tab, r, k);
+  out[kWeightO * n + e] = (T)weight_entry(false, L, cs, tab, r, k);
+}
+
+// Allocates and fills them; synchronises.
+template <typename T>
+cudaError_t make_matrices(int L, T** mats, size_t* bytes) {
+  const size_t n = (size_t)L * L, ncs = 2 * (size_t)(2 * L - 1);
+  double2* tmp = nullptr;
+  cudaError_t e = dev_malloc(mats, kMatrices * n * sizeof(T));
+  if (e != cudaSuccess) return e;
+  *bytes = kMatrices * n * sizeof(T);
+  e = dev_malloc(&tmp, (ncs + n) * sizeof(double2));
+  if (e == cudaSuccess) {
+    node_table_kernel<<<(unsigned)((ncs + 255) / 256), 256>>>(2 * L - 1, tmp);
+    weight_prefix_kernel<<<(unsigned)((L + 31) / 32), 32>>>(L, tmp, tmp + ncs);
+    matrices_kernel<T><<<(unsigned)((n + 255) / 256), 256>>>(L, tmp, tmp + ncs, *mats);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  }
+  if (tmp) cudaFree(tmp);
+  return e;
+}
+}  // namespace folded
 
 }  // namespace
 }  // namespace ssht
