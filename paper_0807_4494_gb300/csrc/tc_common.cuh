@@ -222,11 +222,12 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // The power of two that brings a block's largest magnitude amax to [2^14, 2^15), and the scale that
-// undoes it, with a 2^-14 of the other operand's range folded in.  Magnitudes below 2^-98 share the
-// smallest one's power; an infinity or a NaN stays what it is in the parts.
+// undoes it, with a 2^-14 of the other operand's range folded in (below 2^-126 a denormal number).
+// Magnitudes below 2^-112 share 2^127, which leaves the smallest normal number 2^1 and so both of its parts
+// whole; an infinity or a NaN stays what it is in the parts.
 __device__ __forceinline__ float block_power(float amax, float* scale) {
-  const int e = min(max((int)(__float_as_uint(amax) >> 23), 29), 254);
-  *scale = __uint_as_float((uint32_t)(e - 28) << 23);
+  const int e = min(max((int)(__float_as_uint(amax) >> 23), 14), 254);
+  *scale = __uint_as_float(e > 28 ? (uint32_t)(e - 28) << 23 : 1u << (e - 6));
   return __uint_as_float((uint32_t)(268 - e) << 23);
 }
 
