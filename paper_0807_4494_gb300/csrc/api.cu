@@ -102,6 +102,7 @@ struct ssht_plan_s {
   void* W2 = nullptr;
   size_t w_bytes = 0;  // each of W1, W2
   void* W3 = nullptr;
+  size_t w3_bytes = 0;
   void* ph = nullptr;       // phase table, element precision
   double2* ph64 = nullptr;  // phase table, FP64
   cufftHandle fft_phi = 0, fft_theta = 0;
@@ -422,14 +423,14 @@ int tc_multiply(ssht_plan_t p, int forward, void* dst, cudaStream_t st) {
 int fp64_pass(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t st) {
   StageScope sc(p, SSHT_STAGE_FFT, st);
   cudaError_t e;
+  const size_t fb = p->pair_grid_bytes(), ib = which == 2 ? fb : p->w_bytes, ob = which == 1 ? fb : p->w_bytes;
   if (p->digits) {
-    const size_t fb = p->pair_grid_bytes();
-    e = digits_pass(p->digits, which, p->s, p->B, in, which == 2 ? fb : p->w_bytes, p->W3, p->W1, p->w_bytes, out,
-                    which == 1 ? fb : p->w_bytes, p->delta.status, p->wait_ns, st);
+    e = digits_pass(p->digits, which, p->s, p->B, in, ib, p->W3, p->w3_bytes, p->W1, p->w_bytes, out, ob, p->delta.status,
+                    p->wait_ns, st);
   } else if (which < 2) {
-    e = direct_inverse(p->direct, p->s, p->B, in, out, st, which);
+    e = direct_inverse(p->direct, p->s, p->B, in, ib, out, ob, st, which);
   } else {
-    e = direct_analysis(p->direct, which == 4, p->s, p->B, in, out, st, which - 2 > 0);
+    e = direct_analysis(p->direct, which == 4, p->s, p->B, in, ib, out, ob, st, which - 2 > 0);
   }
   SSHT_CUDA(e, "torus product");
   p->launches += !p->digits ? 1 : which == 1 ? 3 : 2;
@@ -475,7 +476,7 @@ int project(ssht_plan_t p, const void* H, void* flm, cudaStream_t st) {
   {
     StageScope sc(p, SSHT_STAGE_PROJECT, st);
     if (p->contract_digits)
-      SSHT_CUDA(contract_digits(1, p->d.L, p->s, p->B, p->sms, p->delta.table, p->U, H, p->w_bytes, p->W3, flm,
+      SSHT_CUDA(contract_digits(1, p->d.L, p->s, p->B, p->sms, p->delta.table, p->U, H, p->w_bytes, p->W3, p->w3_bytes, flm,
                                 p->pair_coeff_bytes(), p->delta.status, p->wait_ns, st),
                 "projection");
     else
@@ -568,8 +569,8 @@ int inverse_impl(ssht_plan_t p, const void* flm, void* f, cudaStream_t st) {
     if ((rc = join_operands(p, st))) return rc;
     StageScope sc(p, SSHT_STAGE_INVERSE, st);
     if (p->contract_digits)
-      SSHT_CUDA(contract_digits(0, d.L, p->s, p->B, p->sms, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W3, p->W1,
-                                p->w_bytes, p->delta.status, p->wait_ns, st),
+      SSHT_CUDA(contract_digits(0, d.L, p->s, p->B, p->sms, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W3, p->w3_bytes,
+                                p->W1, p->w_bytes, p->delta.status, p->wait_ns, st),
                 "inverse contraction");
     else
       SSHT_CUDA(contract_inverse_simt<T>(d, p->s, p->B, p->delta.table, p->U, flm, p->pair_coeff_bytes(), p->W1, p->w_bytes,
@@ -918,6 +919,7 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
       }
     }
     if ((rc = dalloc(p, &p->W3, w3, "operand digits"))) return bail(rc);
+    p->w3_bytes = w3;
   }
   if ((rc = dalloc(p, &p->ph, (size_t)(2 * d.N - 1) * p->elem, "phase table"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->ph64, (size_t)(2 * d.N - 1) * sizeof(double2), "phase table"))) return bail(rc);
@@ -1251,8 +1253,9 @@ int ssht_debug_fail_allocation(int n) {
 int ssht_debug_bounds(long long* count, int* site, long long* index, long long* extent) {
   if (!kBoundsChecked) return fail(SSHT_EUNSUPPORTED, "ssht_debug_bounds: this library was built without index checks");
   SSHT_CUDA(cudaDeviceSynchronize(), "synchronize");
-  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass,  bounds_take_torus_small, bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc,
-                                          bounds_take_delta_column, bounds_take_real, bounds_take_contract_simt};
+  cudaError_t (*take[])(BoundsRecord*) = {bounds_take_torus_pass,   bounds_take_torus_small,     bounds_take_torus_direct,
+                                          bounds_take_torus_digits, bounds_take_contract_digits, bounds_take_contract_tc,
+                                          bounds_take_delta_column, bounds_take_real,            bounds_take_contract_simt};
   BoundsRecord first{};
   long long total = 0;
   for (auto f : take) {

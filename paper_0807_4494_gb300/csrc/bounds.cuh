@@ -27,7 +27,8 @@ enum BoundsSite {
   kbPackVIn = 20, kbPackVOut, kbPackAIn, kbPackAOut, kbGemmA, kbGemmX, kbGemmOut,
   kbColumnTable = 40, kbColumnTile, kbLaneTable, kbLaneTile, kbColumnCoef,
   kbPairIn = 60, kbPairOut, kbRealIn, kbRealOut,
-  kbSimtIn = 80, kbSimtOut,
+  kbSimtIn = 80, kbSimtOut, kbSimtTable,
+  kbDigitTile = 90, kbDigitExp, kbDigitTable,
 };
 
 #if defined(SSHT_DEBUG) && defined(__CUDACC__)

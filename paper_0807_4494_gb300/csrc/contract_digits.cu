@@ -60,6 +60,7 @@ struct PackArgs {
   long long in_n;
   uint8_t* x;
   int* exps;
+  long long x_n, exps_n;  // tiles and exponents of the workspace
 };
 
 template <bool FWD, int FIELDS>
@@ -113,8 +114,9 @@ __global__ void __launch_bounds__(kPackThreads) digit_columns_kernel(const __gri
           if (e > *(volatile int*)&top[so][r]) atomicMax(&top[so][r], e);
         } else {
           const int row = 4 * (b % FIELDS) + r, e = top[so][r];
-          if ((g >> 2) == nc - 1 && (g & 3) == 0) a.exps[tile * kCols<FIELDS> + row] = e;
-          put_digits<kDigits, kXPart<FIELDS>>(a.x + (tile * nc + (g >> 2)) * kXTile<FIELDS>, row, g & 3, x[r], e);
+          const long long ei = (long long)tile * kCols<FIELDS> + row, xi = (long long)tile * nc + (g >> 2);
+          if ((g >> 2) == nc - 1 && (g & 3) == 0 && in_bounds(ei, a.exps_n, kbDigitExp)) a.exps[ei] = e;
+          if (in_bounds(xi, a.x_n, kbDigitTile)) put_digits<kDigits, kXPart<FIELDS>>(a.x + (size_t)xi * kXTile<FIELDS>, row, g & 3, x[r], e);
         }
       }
     }
@@ -131,6 +133,7 @@ struct GemmArgs {
   const double* U;
   const uint8_t* x;
   const int* xexp;
+  long long x_n, exps_n;  // tiles and exponents of the workspace
   double2* out;
   long long out_n;
   int* status;
@@ -205,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
       uint32_t used = 0, uph = 0;  // stages that were filled, and the parity of their last fill
       for (int w = blockIdx.x; w < a.nitems && going(abort); w += gridDim.x) {
         const Item t = item_of<FWD>(a, w);
-        const uint8_t* x = a.x + ((size_t)t.m * a.groups + t.g) * nc * XTILE;
+        const long long x0 = ((long long)t.m * a.groups + t.g) * nc;
         for (int c = t.c0; c < t.c1; ++c) {
           if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort, a.wait_ns))) {
             *abort = 1;
@@ -213,7 +216,9 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
           }
           if (one) {
             mbar_expect_tx(&data_full[s], (uint32_t)XTILE);
-            bulk_g2s(smem + s * STAGE + kATile9, x + (size_t)c * XTILE, XTILE, &data_full[s]);
+            // (a tile outside the workspace is recorded and tile 0 copied instead: the pipeline still completes)
+            const long long xi = in_bounds(x0 + c, a.x_n, kbDigitTile) ? x0 + c : 0;
+            bulk_g2s(smem + s * STAGE + kATile9, a.x + (size_t)xi * XTILE, XTILE, &data_full[s]);
           }
           used |= 1u << s;
           uph = (uph & ~(1u << s)) | ((uint32_t)(ph ^ 1) << s);
@@ -312,7 +317,9 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
         }
         const int b = FIELDS * t.g + cg * (FIELDS / 4) + f;
         if (b >= a.B || r >= L || (FWD && r < m)) continue;
-        const int4 e = __ldg((const int4*)(a.xexp + ((size_t)m * a.groups + t.g) * COLS + FIELDS * cg + 4 * f));
+        const long long ei = ((long long)m * a.groups + t.g) * COLS + FIELDS * cg + 4 * f;
+        if (!in_bounds(ei + 3, a.exps_n, kbDigitExp)) continue;
+        const int4 e = __ldg((const int4*)(a.xexp + ei));
         const int xe[4] = {e.x, e.y, e.z, e.w};
         double z[4];
 #pragma unroll
@@ -347,8 +354,9 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int mp = k0 + 4 * i <= last ? k0 + 4 * i : 0;
-          d[i] = __ldg(&a.table[o + mp]);
-          u[i] = __ldg(&a.U[ou + mp]);
+          const bool here = in_bounds(o + mp, doff32(L), kbDigitTable) && in_bounds(ou + mp, tri32(L), kbDigitTable);
+          d[i] = __ldg(&a.table[here ? o + mp : 0]);
+          u[i] = __ldg(&a.U[here ? ou + mp : 0]);
           if (k0 + 4 * i > last) u[i] = 0.0;
         }
       } else {  // row m' = r; k = l
@@ -356,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_contract_kernel(const __gri
         int o = doff32(l0) + t.m * (l0 + 1) + r, ou = tri32(l0) + r;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const bool in = l0 + i >= from && l0 + i < L;
+          const bool in = l0 + i >= from && l0 + i < L && in_bounds(o, doff32(L), kbDigitTable) && in_bounds(ou, tri32(L), kbDigitTable);
           d[i] = __ldg(&a.table[in ? o : 0]);
           u[i] = __ldg(&a.U[in ? ou : 0]);
           if (!in) u[i] = 0.0;
@@ -450,7 +458,7 @@ int groups_of(int B) { return (B + fields_of(B) - 1) / fields_of(B); }
 
 template <bool FWD, int FIELDS>
 cudaError_t run(int L, int s, int B, int sms, const double* table, const double* U, const void* in, size_t in_bytes, void* work,
-                void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
+                size_t work_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
   PackArgs k{};
   k.L = L;
   k.s = s;
@@ -459,7 +467,10 @@ cudaError_t run(int L, int s, int B, int sms, const double* table, const double*
   k.in = (const double2*)in;
   k.in_n = (long long)(in_bytes / sizeof(double2));
   k.x = (uint8_t*)work;
-  k.exps = (int*)((uint8_t*)work + (size_t)L * k.groups * chunks_of(L) * kXTile<FIELDS>);
+  k.x_n = (long long)L * k.groups * chunks_of(L);
+  k.exps_n = (long long)L * k.groups * kCols<FIELDS>;
+  k.exps = (int*)((uint8_t*)work + (size_t)k.x_n * kXTile<FIELDS>);
+  if ((size_t)k.x_n * kXTile<FIELDS> + (size_t)k.exps_n * sizeof(int) > work_bytes) return cudaErrorInvalidValue;
   digit_columns_kernel<FWD, FIELDS><<<(unsigned)(((long long)B * L + kSources - 1) / kSources), kPackThreads, 0, st>>>(k);
   GemmArgs a{};
   a.L = L;
@@ -476,6 +487,8 @@ cudaError_t run(int L, int s, int B, int sms, const double* table, const double*
   a.U = U;
   a.x = k.x;
   a.xexp = k.exps;
+  a.x_n = k.x_n;
+  a.exps_n = k.exps_n;
   a.out = (double2*)out;
   a.out_n = (long long)(out_bytes / sizeof(double2));
   a.status = status;
@@ -513,10 +526,10 @@ cudaError_t contract_digits_setup() {
 }
 
 cudaError_t contract_digits(int forward, int L, int s, int B, int sms, const double* table, const double* U, const void* in,
-                            size_t in_bytes, void* work, void* out, size_t out_bytes, int* status, long long wait_ns,
-                            cudaStream_t st) {
+                            size_t in_bytes, void* work, size_t work_bytes, void* out, size_t out_bytes, int* status,
+                            long long wait_ns, cudaStream_t st) {
   auto go = fields_of(B) == 8 ? (forward ? run<true, 8> : run<false, 8>) : (forward ? run<true, 4> : run<false, 4>);
-  return go(L, s, B, sms, table, U, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
+  return go(L, s, B, sms, table, U, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st);
 }
 
 SSHT_BOUNDS_TU(contract_digits)

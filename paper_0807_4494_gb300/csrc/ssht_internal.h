@@ -249,8 +249,8 @@ size_t digits_bytes(const DigitPlan* p);
 size_t digits_workspace_bytes(int L, int s, int B);
 // One pass: 0 theta of the inverse, F -> E, O; 1 its phi, E, O -> samples, by way of mid (E, O's size); 2 phi of forward
 // and adjoint, samples -> P, Q; 3 theta of the forward (with the extension and the sin(theta) weight), 4 of the adjoint, P, Q -> H.
-cudaError_t digits_pass(const DigitPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* work, void* mid,
-                        size_t mid_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st);
+cudaError_t digits_pass(const DigitPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* work,
+                        size_t work_bytes, void* mid, size_t mid_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st);
 
 // Small band-limits, FP64 and FP32-class plans (torus_small.cu): theta and phi in one launch on CUDA cores, no workspace.
 struct SmallPlan;
@@ -270,9 +270,11 @@ cudaError_t direct_setup(DirectPlan** out, int L);  // synchronises
 void direct_destroy(DirectPlan* p);
 size_t direct_bytes(const DirectPlan* p);
 // step 0: theta (F -> E, O), 1: phi (E, O -> samples).
-cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, void* out, cudaStream_t st, int step);
+cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, size_t in_bytes, void* out, size_t out_bytes,
+                           cudaStream_t st, int step);
 // step 0: phi (samples -> P, Q), 1: theta (P, Q -> H; adjoint = 0 with the extension and the sin(theta) weight).
-cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, void* out, cudaStream_t st, int step);
+cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, size_t in_bytes, void* out,
+                            size_t out_bytes, cudaStream_t st, int step);
 
 // The contractions of FP64 plans on tensor cores (contract_digits.cu): the same results as
 // contract_inverse_simt (forward = 0) and contract_project_simt, with a workspace for the data columns.
@@ -280,8 +282,8 @@ bool contract_digits_wanted(int L, int B);
 size_t contract_digits_bytes(int L, int B);
 cudaError_t contract_digits_setup();
 cudaError_t contract_digits(int forward, int L, int s, int B, int sms, const double* table, const double* U, const void* in,
-                            size_t in_bytes, void* work, void* out, size_t out_bytes, int* status, long long wait_ns,
-                            cudaStream_t st);
+                            size_t in_bytes, void* work, size_t work_bytes, void* out, size_t out_bytes, int* status,
+                            long long wait_ns, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Torus kernels (torus.cu)
@@ -300,6 +302,7 @@ cudaError_t bounds_take_contract_tc(BoundsRecord* r);
 cudaError_t bounds_take_delta_column(BoundsRecord* r);
 cudaError_t bounds_take_torus_digits(BoundsRecord* r);
 cudaError_t bounds_take_torus_small(BoundsRecord* r);
+cudaError_t bounds_take_torus_direct(BoundsRecord* r);
 cudaError_t bounds_take_contract_digits(BoundsRecord* r);
 cudaError_t bounds_take_real(BoundsRecord* r);
 cudaError_t bounds_take_contract_simt(BoundsRecord* r);

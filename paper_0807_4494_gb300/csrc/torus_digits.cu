@@ -290,8 +290,10 @@ __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_co
       uint32_t used = 0, uph = 0;  // stages that were filled, and the parity of their last fill
       for (int w = blockIdx.x; w < a.ntiles && going(abort); w += gridDim.x) {
         const Item t = item_of(a, w);
-        const uint8_t* m = a.A[t.u] + (size_t)t.i * nc * kMatTile;
-        const uint8_t* x = a.x + (size_t)t.j * nc * DATA;
+        // (a tile outside its array is recorded and the first one copied instead: the pipeline still completes)
+        const bool here = in_bounds(t.i, a.mblocks, kbDigitTile) && in_bounds(t.j, a.q.all(), kbDigitTile);
+        const uint8_t* m = a.A[t.u] + (size_t)(here ? t.i : 0) * nc * kMatTile;
+        const uint8_t* x = a.x + (size_t)(here ? t.j : 0) * nc * DATA;
         for (int c = 0; c < nc; ++c) {
           if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort, a.wait_ns))) {
             *abort = 1;
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1) digit_gemm_kernel(const __grid_co
       if (!ok) break;
       const int row = t.i * 128 + q * 32 + lane;
       const int col0 = (t.j - (t.u ? a.q.tiles[0] : 0)) * PAIRS + PER / 2 * cg;
-      if (row >= L) continue;
+      if (row >= L || !in_bounds(row, 128 * a.mblocks, kbDigitExp) || !in_bounds(t.j, a.q.all(), kbDigitExp)) continue;
       const int ea = a.aexp[t.u][row] - 2105;
       const int* xe = a.xexp + (size_t)t.j * COLS + PER * cg;
 #pragma unroll
@@ -523,11 +525,12 @@ void digits_destroy(DigitPlan* p) {
 size_t digits_bytes(const DigitPlan* p) { return p ? p->bytes : 0; }
 
 template <int PASS, int PAIRS>
-static cudaError_t run_tiles(const DigitPlan* p, int mat, int s, int B, const void* in, size_t in_bytes, void* work, void* out,
-                       size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
+static cudaError_t run_tiles(const DigitPlan* p, int mat, int s, int B, const void* in, size_t in_bytes, void* work,
+                             size_t work_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
   const int L = p->L, rows = (L + 127) / 128 * 128;
   const Sets q = sets_of(PASS, L, s, B, PAIRS);
   const size_t tile_bytes = (size_t)q.all() * chunks_of(L) * kDataTile<PAIRS>;
+  if (tile_bytes + (size_t)q.all() * 2 * PAIRS * sizeof(int) > work_bytes) return cudaErrorInvalidValue;
   PackArgs k{};
   k.L = L;
   k.s = s;
@@ -562,23 +565,23 @@ static cudaError_t run_tiles(const DigitPlan* p, int mat, int s, int B, const vo
 // Tiles of 16 complex columns where those of 32 would leave half of the SMs without one: L = 129, B = 4 (66 and
 // 130 tiles) 21.8 us a product with 32, 17.4 with 16 (13.5 since the digits are taken together).
 template <int PASS>
-static cudaError_t run(const DigitPlan* p, int mat, int s, int B, const void* in, size_t in_bytes, void* work, void* out,
-                       size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
+static cudaError_t run(const DigitPlan* p, int mat, int s, int B, const void* in, size_t in_bytes, void* work,
+                             size_t work_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
   const int tiles = (p->L + 127) / 128 * sets_of(PASS, p->L, s, B, 32).all();
-  return 2 * tiles <= p->sms ? run_tiles<PASS, 16>(p, mat, s, B, in, in_bytes, work, out, out_bytes, status, wait_ns, st)
-                             : run_tiles<PASS, 32>(p, mat, s, B, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
+  return 2 * tiles <= p->sms ? run_tiles<PASS, 16>(p, mat, s, B, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st)
+                             : run_tiles<PASS, 32>(p, mat, s, B, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st);
 }
 
-cudaError_t digits_pass(const DigitPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* work, void* mid,
-                        size_t mid_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
+cudaError_t digits_pass(const DigitPlan* p, int which, int s, int B, const void* in, size_t in_bytes, void* work,
+                        size_t work_bytes, void* mid, size_t mid_bytes, void* out, size_t out_bytes, int* status, long long wait_ns, cudaStream_t st) {
   switch (which) {
-    case kThetaInverse: return run<kThetaInverse>(p, kCosKX, s, B, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
-    case kPhiForward: return run<kPhiForward>(p, kCosXK, s, B, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
-    case kThetaForward: return run<kThetaForward>(p, kWeightE, s, B, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
-    case kThetaAdjoint: return run<kThetaAdjoint>(p, kCosXK, s, B, in, in_bytes, work, out, out_bytes, status, wait_ns, st);
+    case kThetaInverse: return run<kThetaInverse>(p, kCosKX, s, B, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st);
+    case kPhiForward: return run<kPhiForward>(p, kCosXK, s, B, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st);
+    case kThetaForward: return run<kThetaForward>(p, kWeightE, s, B, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st);
+    case kThetaAdjoint: return run<kThetaAdjoint>(p, kCosXK, s, B, in, in_bytes, work, work_bytes, out, out_bytes, status, wait_ns, st);
     default: break;
   }
-  cudaError_t e = run<kPhiInverse>(p, kCosKX, s, B, in, in_bytes, work, mid, mid_bytes, status, wait_ns, st);
+  cudaError_t e = run<kPhiInverse>(p, kCosKX, s, B, in, in_bytes, work, work_bytes, mid, mid_bytes, status, wait_ns, st);
   if (e != cudaSuccess) return e;
   const long long rings = (long long)B * p->L;
   digit_join_kernel<<<(unsigned)((rings * p->L + 255) / 256), 256, 0, st>>>(p->L, rings, (const double2*)mid,

@@ -8,6 +8,7 @@
 //
 // What bounds it: launches and latency at the smallest sizes, then the FP64 pipe, 8 B L^3 flops a pass
 // (1.07 TFLOP/s at L = 128, B = 16, 0.85 of its rate).  L = 64, B = 1: 43 us, by FFTs 141.
+#include "bounds.cuh"
 #include "ssht_internal.h"
 #include "torus_matrices.cuh"
 
@@ -44,6 +45,14 @@ __device__ __forceinline__ Pair reduce_warps(Pair v, int warp, int lane) {
   return r;
 }
 
+// Element i of a buffer of n, zero outside (checked builds).
+__device__ __forceinline__ double2 load(const double2* p, long long i, long long n) {
+  return in_bounds(i, n, kbTorusIn) ? __ldg(&p[i]) : make_double2(0.0, 0.0);
+}
+__device__ __forceinline__ void store(double2* p, long long i, long long n, double2 v) {
+  if (in_bounds(i, n, kbTorusOut)) p[i] = v;
+}
+
 __device__ __forceinline__ void axpy(double2& acc, double a, double2 x) {
   acc.x = fma(a, x.x, acc.x);
   acc.y = fma(a, x.y, acc.y);
@@ -51,21 +60,21 @@ __device__ __forceinline__ void axpy(double2& acc, double a, double2 x) {
 
 // theta inverse: F [b][m + Lp][m'] -> work E, O [2][b][m][t] = x_m +- x_{-m} (m = 0: x_0, 0).
 __global__ void __launch_bounds__(32 * kWarps) direct_theta_inverse_kernel(int L, int s, int B, const double* __restrict__ M,
-                                                                           const double2* __restrict__ F, double2* __restrict__ work) {
+                                                                           const double2* __restrict__ F, long long in_n,
+                                                                           double2* __restrict__ work, long long out_n) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
   const int t = 32 * blockIdx.y + lane, b = blockIdx.x / L, m = blockIdx.x - b * L;
   const bool odd = (m + s) & 1;
   const double* A = M + (size_t)(odd ? kSinKX : kCosKX) * L * L;
-  const double2* Fp = F + ((size_t)b * N + L - 1 + m) * L;
-  const double2* Fm = F + ((size_t)b * N + L - 1 - m) * L;
+  const long long fp = ((long long)b * N + L - 1 + m) * L, fm = fp - 2ll * m * L;
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = warp; k < L; k += kWarps) {
     double a = t < L ? __ldg(&A[(size_t)k * L + t]) : 0.0;
     if (k == 0) a *= 0.5;  // the sum is doubled below
-    axpy(v.a, a, __ldg(&Fp[k]));
-    axpy(v.b, a, __ldg(&Fm[k]));
+    axpy(v.a, a, load(F, fp + k, in_n));
+    axpy(v.b, a, load(F, fm + k, in_n));
   }
   v = reduce_warps(v, warp, lane);
   if (warp || t >= L) return;
@@ -78,44 +87,45 @@ __global__ void __launch_bounds__(32 * kWarps) direct_theta_inverse_kernel(int L
     e = make_double2(-e.y, e.x);
     o = make_double2(-o.y, o.x);
   }
-  const size_t at = ((size_t)b * L + m) * L + t;
-  work[at] = make_double2(2.0 * e.x, 2.0 * e.y);
-  work[(size_t)B * L * L + at] = make_double2(2.0 * o.x, 2.0 * o.y);
+  const long long at = ((long long)b * L + m) * L + t;
+  store(work, at, out_n, make_double2(2.0 * e.x, 2.0 * e.y));
+  store(work, (long long)B * L * L + at, out_n, make_double2(2.0 * o.x, 2.0 * o.y));
 }
 
 // phi inverse: E, O [2][b][m][t] -> f[b][t][p] = E + iO, f[b][t][N-1-p] = E - iO.
 __global__ void __launch_bounds__(32 * kWarps) direct_phi_inverse_kernel(int L, int B, const double* __restrict__ M,
-                                                                         const double2* __restrict__ work, double2* __restrict__ f) {
+                                                                         const double2* __restrict__ work, long long in_n,
+                                                                         double2* __restrict__ f, long long out_n) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
   const int p = 32 * blockIdx.y + lane, b = blockIdx.x / L, t = blockIdx.x - b * L;
   const double* C = M + (size_t)kCosKX * L * L;
   const double* S = M + (size_t)kSinKX * L * L;
-  const double2* E = work + (size_t)b * L * L + t;
-  const double2* O = E + (size_t)B * L * L;
+  const long long e0 = (long long)b * L * L + t, o0 = e0 + (long long)B * L * L;
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = warp; k < L; k += kWarps) {
     const double c = p < L ? __ldg(&C[(size_t)k * L + p]) : 0.0, sn = p < L ? __ldg(&S[(size_t)k * L + p]) : 0.0;
-    axpy(v.a, c, __ldg(&E[(size_t)k * L]));
-    axpy(v.b, sn, __ldg(&O[(size_t)k * L]));
+    axpy(v.a, c, load(work, e0 + (long long)k * L, in_n));
+    axpy(v.b, sn, load(work, o0 + (long long)k * L, in_n));
   }
   v = reduce_warps(v, warp, lane);
   if (warp || p >= L) return;
-  double2* row = f + ((size_t)b * L + t) * N;
-  row[p] = make_double2(v.a.x - v.b.y, v.a.y + v.b.x);
-  if (p < L - 1) row[N - 1 - p] = make_double2(v.a.x + v.b.y, v.a.y - v.b.x);
+  const long long row = ((long long)b * L + t) * N;
+  store(f, row + p, out_n, make_double2(v.a.x - v.b.y, v.a.y + v.b.x));
+  if (p < L - 1) store(f, row + N - 1 - p, out_n, make_double2(v.a.x + v.b.y, v.a.y - v.b.x));
 }
 
 // phi of forward and adjoint: f [b][t][p] -> P, Q [2][b][t][m].  A warp folds 32 of its k's at a time.
 __global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, int B, const double* __restrict__ M,
-                                                                         const double2* __restrict__ f, double2* __restrict__ work) {
+                                                                         const double2* __restrict__ f, long long in_n,
+                                                                         double2* __restrict__ work, long long out_n) {
   __shared__ double2 fold[kWarps][2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
   const int m = 32 * blockIdx.y + lane, b = blockIdx.x / L, t = blockIdx.x - b * L;
   const double* C = M + (size_t)kCosXK * L * L;
   const double* S = M + (size_t)kSinXK * L * L;
-  const double2* row = f + ((size_t)b * L + t) * N;
+  const long long row = ((long long)b * L + t) * N;
   const int per = (L + kWarps - 1) / kWarps, k_end = min(L, (warp + 1) * per);
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
@@ -123,9 +133,9 @@ __global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, 
     const int p = k0 + lane;
     double2 e = make_double2(0.0, 0.0), o = e;
     if (p < k_end) {
-      e = row[p];
+      e = load(f, row + p, in_n);
       if (p < L - 1) {
-        const double2 y = row[N - 1 - p];
+        const double2 y = load(f, row + N - 1 - p, in_n);
         o = make_double2(e.x - y.x, e.y - y.y);
         e = make_double2(e.x + y.x, e.y + y.y);
       }
@@ -144,28 +154,28 @@ __global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, 
   }
   v = reduce_warps(v, warp, lane);
   if (warp || m >= L) return;
-  const size_t at = ((size_t)b * L + t) * L + m;
-  work[at] = v.a;
-  work[(size_t)B * L * L + at] = v.b;
+  const long long at = ((long long)b * L + t) * L + m;
+  store(work, at, out_n, v.a);
+  store(work, (long long)B * L * L + at, out_n, v.b);
 }
 
 // theta of forward (weight matrices) and adjoint (cosines and sines, the fold of m' < 0): P, Q -> H [b][m + Lp][m'].
 __global__ void __launch_bounds__(32 * kWarps) direct_theta_forward_kernel(int L, int s, int B, int adjoint,
                                                                            const double* __restrict__ M,
-                                                                           const double2* __restrict__ work, double2* __restrict__ H) {
+                                                                           const double2* __restrict__ work, long long in_n,
+                                                                           double2* __restrict__ H, long long out_n) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = 2 * L - 1;
   const int mp = 32 * blockIdx.y + lane, b = blockIdx.x / L, m = blockIdx.x - b * L;
   const bool odd = (m + s) & 1;
   const double* A = M + (size_t)(adjoint ? (odd ? kSinXK : kCosXK) : (odd ? kWeightO : kWeightE)) * L * L;
-  const double2* P = work + (size_t)b * L * L + m;
-  const double2* Q = P + (size_t)B * L * L;
+  const long long p0 = (long long)b * L * L + m, q0 = p0 + (long long)B * L * L;
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = warp; k < L; k += kWarps) {
     const double a = mp < L ? __ldg(&A[(size_t)k * L + mp]) : 0.0;
-    axpy(v.a, a, __ldg(&P[(size_t)k * L]));
-    axpy(v.b, a, __ldg(&Q[(size_t)k * L]));
+    axpy(v.a, a, load(work, p0 + (long long)k * L, in_n));
+    axpy(v.b, a, load(work, q0 + (long long)k * L, in_n));
   }
   v = reduce_warps(v, warp, lane);
   if (warp || mp >= L) return;
@@ -175,8 +185,8 @@ __global__ void __launch_bounds__(32 * kWarps) direct_theta_forward_kernel(int L
     hp = make_double2(hp.y, -hp.x);
     hm = make_double2(hm.y, -hm.x);
   }
-  H[((size_t)b * N + L - 1 + m) * L + mp] = hp;
-  if (m > 0) H[((size_t)b * N + L - 1 - m) * L + mp] = hm;
+  store(H, ((long long)b * N + L - 1 + m) * L + mp, out_n, hp);
+  if (m > 0) store(H, ((long long)b * N + L - 1 - m) * L + mp, out_n, hm);
 }
 
 }  // namespace
@@ -214,22 +224,29 @@ void direct_destroy(DirectPlan* p) {
 
 size_t direct_bytes(const DirectPlan* p) { return p ? p->bytes : 0; }
 
-cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, void* out, cudaStream_t st, int step) {
+cudaError_t direct_inverse(const DirectPlan* p, int s, int B, const void* in, size_t in_bytes, void* out, size_t out_bytes,
+                           cudaStream_t st, int step) {
   const dim3 grid((unsigned)B * p->L, (p->L + 31) / 32);
+  const long long in_n = (long long)(in_bytes / sizeof(double2)), out_n = (long long)(out_bytes / sizeof(double2));
   if (step == 0)
-    direct_theta_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, p->mats, (const double2*)in, (double2*)out);
+    direct_theta_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, p->mats, (const double2*)in, in_n, (double2*)out, out_n);
   else
-    direct_phi_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)in, (double2*)out);
+    direct_phi_inverse_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)in, in_n, (double2*)out, out_n);
   return cudaGetLastError();
 }
 
-cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, void* out, cudaStream_t st, int step) {
+cudaError_t direct_analysis(const DirectPlan* p, int adjoint, int s, int B, const void* in, size_t in_bytes, void* out,
+                            size_t out_bytes, cudaStream_t st, int step) {
   const dim3 grid((unsigned)B * p->L, (p->L + 31) / 32);
+  const long long in_n = (long long)(in_bytes / sizeof(double2)), out_n = (long long)(out_bytes / sizeof(double2));
   if (step == 0)
-    direct_phi_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)in, (double2*)out);
+    direct_phi_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, B, p->mats, (const double2*)in, in_n, (double2*)out, out_n);
   else
-    direct_theta_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, adjoint, p->mats, (const double2*)in, (double2*)out);
+    direct_theta_forward_kernel<<<grid, 32 * kWarps, 0, st>>>(p->L, s, B, adjoint, p->mats, (const double2*)in, in_n, (double2*)out,
+                                                              out_n);
   return cudaGetLastError();
 }
+
+SSHT_BOUNDS_TU(torus_direct)
 
 }  // namespace ssht
