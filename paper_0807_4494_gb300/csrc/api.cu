@@ -100,7 +100,7 @@ struct ssht_plan_s {
   float* Uf = nullptr;  // U in FP32 (tensor-core operand packing)
   void* W1 = nullptr;
   void* W2 = nullptr;
-  size_t w_bytes = 0;  // each of W1, W2
+  size_t w_bytes = 0;  // of W1 (FP64 plans: of W2 too)
   void* W3 = nullptr;
   size_t w3_bytes = 0;
   void* ph = nullptr;       // phase table, element precision
@@ -118,6 +118,7 @@ struct ssht_plan_s {
   size_t bytes = 0;
   TcPlan* tc = nullptr;    // tensor-core contraction (precisions SSHT_TF32X3, SSHT_BF16X6)
   TorusPlan* torus = nullptr;  // torus products of FP32-class plans
+  int torus_fields = 0;        // fields of a slice of theirs
   DigitPlan* digits = nullptr;   // torus products of FP64 plans
   DirectPlan* direct = nullptr;  // ... and of those with little work
   SmallPlan* small = nullptr;    // torus products of small band-limits, any precision
@@ -232,27 +233,46 @@ int run_dft(ssht_plan_t p, cufftHandle h, void* in, void* out, cudaStream_t st) 
   return 0;
 }
 
-// The torus passes of an FP32-class plan (products along theta or phi), timed as FFT work.  Inverse:
-// F in W1 -> samples f.
-int torus_inverse_pass(ssht_plan_t p, int step, void* f, cudaStream_t st) {
-  StageScope sc(p, SSHT_STAGE_FFT, st);
-  int n = 0;
-  SSHT_CUDA(torus_inverse(p->torus, p->s, p->B, p->W1, p->w_bytes, p->W2, f, p->pair_grid_bytes(), p->delta.status, p->wait_ns,
-                          st, &n, step),
-            "torus pass");
-  p->launches += n;
+// The torus passes of an FP32-class plan (products along theta or phi), timed as FFT work, by slices of fields.
+// Inverse: F in W1 -> samples f.
+int torus_inverse_passes(ssht_plan_t p, void* f, cudaStream_t st) {
+  const size_t row = (size_t)p->d.N * p->d.L * p->elem;  // of a field's half rows, and of its samples
+  const bool whole = p->torus_fields == p->B;
+  for (int b0 = 0; b0 < p->B; b0 += p->torus_fields) {
+    const int n = std::min(p->torus_fields, p->B - b0);
+    char* F = (char*)p->W1 + b0 * row;
+    void* y = whole ? p->W1 : (char*)p->W2 + torus_operand_bytes(p->torus, p->torus_fields);
+    for (int step = 0; step < 2; ++step) {
+      StageScope sc(p, SSHT_STAGE_FFT, st);
+      int k = 0;
+      SSHT_CUDA(torus_inverse(p->torus, p->s, n, F, p->w_bytes - b0 * row, p->W2, y, (char*)f + b0 * row, p->pair_grid_bytes() - b0 * row,
+                              p->delta.status, p->wait_ns, st, &k, step),
+                "torus pass");
+      p->launches += k;
+    }
+  }
   return 0;
 }
 // Forward / adjoint: samples f -> the projection's data tiles (tensor-core plans) or H in W1.
-int torus_analysis_pass(ssht_plan_t p, int step, int adjoint, const void* f, cudaStream_t st) {
-  StageScope sc(p, SSHT_STAGE_FFT, st);
-  int n = 0;
+int torus_analysis_passes(ssht_plan_t p, int adjoint, const void* f, cudaStream_t st) {
+  const size_t row = (size_t)p->d.N * p->d.L * p->elem;
+  const bool whole = p->torus_fields == p->B;
   TileOut tiles;
   if (p->tc) tiles = tc_forward_tiles(p->tc);
-  SSHT_CUDA(torus_analysis(p->torus, adjoint, p->s, p->B, f, p->pair_grid_bytes(), p->W1, p->W2, p->W1, p->w_bytes,
-                           p->tc ? &tiles : nullptr, p->delta.status, p->wait_ns, st, &n, step),
-            "torus pass");
-  p->launches += n;
+  for (int b0 = 0; b0 < p->B; b0 += p->torus_fields) {
+    const int n = std::min(p->torus_fields, p->B - b0);
+    void* x = whole ? p->W1 : p->W2;
+    void* y = whole ? p->W2 : (char*)p->W2 + torus_operand_bytes(p->torus, p->torus_fields);
+    for (int step = 0; step < 2; ++step) {
+      StageScope sc(p, SSHT_STAGE_FFT, st);
+      int k = 0;
+      SSHT_CUDA(torus_analysis(p->torus, adjoint, p->s, n, (const char*)f + b0 * row, p->pair_grid_bytes() - b0 * row, x, y,
+                               (char*)p->W1 + b0 * row, p->w_bytes - b0 * row, p->tc ? &tiles : nullptr, b0, p->delta.status,
+                               p->wait_ns, st, &k, step),
+                "torus pass");
+      p->launches += k;
+    }
+  }
   return 0;
 }
 
@@ -446,7 +466,7 @@ int torus_to_samples(ssht_plan_t p, void* f, cudaStream_t st) {
     p->launches += 1;
     return 0;
   }
-  if (p->torus) return (rc = torus_inverse_pass(p, 0, f, st)) ? rc : torus_inverse_pass(p, 1, f, st);
+  if (p->torus) return torus_inverse_passes(p, f, st);
   return (rc = fp64_pass(p, 0, p->W1, p->W2, st)) ? rc : fp64_pass(p, 1, p->W2, f, st);
 }
 
@@ -463,7 +483,7 @@ int torus_from_samples(ssht_plan_t p, int adjoint, const void* f, cudaStream_t s
     p->launches += 1;
     return 0;
   }
-  if (p->torus) return (rc = torus_analysis_pass(p, 0, adjoint, f, st)) ? rc : torus_analysis_pass(p, 1, adjoint, f, st);
+  if (p->torus) return torus_analysis_passes(p, adjoint, f, st);
   return (rc = fp64_pass(p, 2, f, p->W2, st)) ? rc : fp64_pass(p, adjoint ? 4 : 3, p->W2, p->W1, st);
 }
 
@@ -886,13 +906,20 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
   if ((rc = dalloc(p, (void**)&p->U, tri(L) * sizeof(double), "spin column"))) return bail(rc);
   if ((rc = dalloc(p, (void**)&p->Uf, tri(L) * sizeof(float), "spin column (FP32)"))) return bail(rc);
   // FP64: full N x N torus rows (the triangular forward's; the products' half rows, and L x L twice over, fit
-  // but for L = 1) and the digits of a pass's data; FP32: half rows of N x L, or a pass's operand tiles (small
-  // band-limits have none; tuning writes a contraction's output to the second workspace).
+  // but for L = 1) and the digits of a pass's data; FP32: half rows of N x L and the passes' operands (small
+  // band-limits have none); tuning writes a contraction's output to the second workspace.
   const bool small = small_wanted(L, B, p->f64);
-  const size_t half_rows = (size_t)B * d.N * L * p->elem;
-  const size_t torus = p->f64 ? (size_t)B * std::max(d.N * d.N, 2) * p->elem : small ? half_rows : torus_workspace_bytes(L, B);
   const bool tensor = desc->precision == SSHT_TF32X3 || desc->precision == SSHT_BF16X6;
-  const size_t second = p->f64 || !small ? torus : tensor ? p->pair_coeff_bytes() : 0;
+  TorusWork work;
+  if (p->f64) {
+    work.w1 = work.w2 = (size_t)B * std::max(d.N * d.N, 2) * p->elem;
+  } else if (small) {
+    work.w1 = (size_t)B * d.N * L * p->elem;
+  } else {
+    work = torus_work(L, B);
+    p->torus_fields = work.fields;
+  }
+  if (tensor) work.w2 = std::max(work.w2, p->pair_coeff_bytes());
   if (pair && (rc = dalloc(p, &p->rc, (size_t)B * L * L * p->elem, "spin-pair coefficients"))) return bail(rc);
   if ((real || pair) && (ce = real_setup()) != cudaSuccess) {
     release(p);
@@ -902,9 +929,9 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     if ((rc = dalloc(p, &p->rc, p->pair_coeff_bytes(), "real-field pair coefficients"))) return bail(rc);
     if ((rc = dalloc(p, &p->rg, p->pair_grid_bytes(), "real-field pair samples"))) return bail(rc);
   }
-  if ((rc = dalloc(p, &p->W1, torus, "torus workspace 1"))) return bail(rc);
-  if ((rc = dalloc(p, &p->W2, second, "torus workspace 2"))) return bail(rc);
-  p->w_bytes = torus;
+  if ((rc = dalloc(p, &p->W1, work.w1, "torus workspace 1"))) return bail(rc);
+  if ((rc = dalloc(p, &p->W2, work.w2, "torus workspace 2"))) return bail(rc);
+  p->w_bytes = work.w1;
   const bool direct = p->f64 && !small && direct_wanted(L, B);
   p->contract_digits = p->f64 && !direct && !small && contract_digits_wanted(L, B);
   if (p->f64 && !direct && !small) {

@@ -222,18 +222,24 @@ struct TorusPlan;
 cudaError_t torus_setup(TorusPlan** out, int L, int device);  // synchronises
 void torus_destroy(TorusPlan* p);
 size_t torus_bytes(const TorusPlan* p);
-// Bytes of each of the two workspaces a plan of B fields hands to the passes.
-size_t torus_workspace_bytes(int L, int B);
-// Inverse, in two steps: 0 theta (F, a workspace, is packed into `work` and then overwritten by the
-// phi pass's operand), 1 phi (from that operand to the samples out).  *_bytes: extents of the buffers
+// What a plan of B fields holds for the passes: workspaces of w1 (F and H too) and w2 bytes, and how many fields a slice
+// has.  All in one slice: the passes' operands lie one in each workspace; several: both in w2, torus_operand_bytes apart.
+struct TorusWork {
+  size_t w1 = 0, w2 = 0;
+  int fields = 0;
+};
+TorusWork torus_work(int L, int B);
+size_t torus_operand_bytes(const TorusPlan* p, int B);
+// Inverse of a slice of B fields, in two steps: 0 theta (F is packed into x_work, the product goes to y_work, which may
+// be F), 1 phi (from y_work to the samples out).  *_bytes: extents of the buffers from the slice on
 // (the index checks of bounds-checked builds).  Timeouts of the pipeline waits set bit 2 of *status.
-cudaError_t torus_inverse(const TorusPlan* p, int s, int B, void* F, size_t f_bytes, void* work, void* out, size_t out_bytes,
-                          int* status, long long wait_ns, cudaStream_t st, int* launches, int step);
+cudaError_t torus_inverse(const TorusPlan* p, int s, int B, const void* F, size_t f_bytes, void* x_work, void* y_work, void* out,
+                          size_t out_bytes, int* status, long long wait_ns, cudaStream_t st, int* launches, int step);
 // Forward (adjoint = 0: extension and sin(theta) weight) or adjoint, in two steps: 0 phi (f packed into
-// the workspace w1, the product into w2), 1 theta (from w2 into the projection's data tiles, or into H
-// without tiles; H may be w1).
-cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const void* f, size_t f_bytes, void* w1, void* w2,
-                           void* H, size_t h_bytes, const TileOut* tiles, int* status, long long wait_ns, cudaStream_t st,
+// x_work, the product into y_work), 1 theta (from y_work into the projection's data tiles, the slice's first field being
+// field b0 there, or into H without tiles; H may be x_work).
+cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const void* f, size_t f_bytes, void* x_work, void* y_work,
+                           void* H, size_t h_bytes, const TileOut* tiles, int b0, int* status, long long wait_ns, cudaStream_t st,
                            int* launches, int step);
 
 // ---------------------------------------------------------------------------

@@ -288,7 +288,8 @@ __global__ void __launch_bounds__(512) pack_phi_kernel(Shape sh, int B, const fl
 // ---------------------------------------------------------------------------------------------
 struct TgArgs {
   Shape sh;
-  int s, B;
+  int s, B;               // B: fields of this slice
+  int b0;                 // its first field (theta forward into tiles)
   int stages;
   int ntiles;             // work items: column tile * row_tiles + row tile
   int row_tiles;          // row blocks, or pairs of them
@@ -733,7 +734,7 @@ __device__ __forceinline__ void torus_gemm(const TgArgs& a) {
         // the projection's data tiles (|m|, m' / 32): rows sign * NC/2 + 2b + part, K = m', the negative
         // half carrying (-1)^{m'} (zeros for m = 0; padding rows stay as the plan zeroed them).  The
         // rows' offsets are the same in every tile, the tiles of the 16 orders two |m| apart.
-        const int sl = b / a.to.Bs, bs = b - sl * a.to.Bs;
+        const int sl = (a.b0 + b) / a.to.Bs, bs = a.b0 + b - sl * a.to.Bs;
         const int half = a.to.NC / 2;
         if (am0 == 0) acc[32] = acc[48] = 0.f;
         const float sgn = (row & 1) ? -1.f : 1.f;
@@ -859,11 +860,36 @@ static long long pass_units(const Shape& sh, int pass, int B) {
 }
 static int pass_chunks(const Shape& sh, int pass) { return pass == kPhiInverse ? sh.nKm() : sh.nKs; }
 
-size_t torus_workspace_bytes(int L, int B) {
-  const Shape sh = make_shape(L);
-  size_t n = (size_t)B * sh.N * sh.L * sizeof(float2);  // F and H half rows
-  for (int p = 0; p < 4; ++p) n = std::max(n, operand_bytes(pass_units(sh, p, B), pass_chunks(sh, p)));
+// Bytes of one field's operand: the largest of the four passes'.
+static size_t field_bytes(const Shape& sh) {
+  size_t n = 0;
+  for (int p = 0; p < 4; ++p) n = std::max(n, operand_bytes(pass_units(sh, p, 1), pass_chunks(sh, p)));
   return n;
+}
+
+size_t torus_operand_bytes(const TorusPlan* p, int B) { return field_bytes(p->sh) * B; }
+
+// The passes hold two operands at a time.  As long as these stay within kWhole all fields go at once, one operand in
+// place of the half rows (which are read by then).  Beyond that, where a field's operand is the larger
+// (padding: 3.9 times at L = 65, 1.5 at L = 257, none from L = 1024 on), the fields run in slices whose operands share
+// kSlice bytes, which is thousands of fields at L = 65 and more than a hundred at L = 513, so that every launch still
+// fills the GPU: a plan then holds little more than its half rows.  Held by an FP32 plan, all fields at once and in slices:
+// L = 65, B = 20000 10.5 and 3.4 GB, L = 300, B = 2000 8.0 and 4.9; inverse and forward 24.8 and 25.0 ms, 113.3 and 113.5.
+TorusWork torus_work(int L, int B) {
+  constexpr size_t kWhole = 4ull << 30, kSlice = 2ull << 30;
+  const Shape sh = make_shape(L);
+  const size_t half = (size_t)sh.N * sh.L * sizeof(float2), op = field_bytes(sh);
+  TorusWork w;
+  if (2 * op * B <= kWhole || 10 * op <= 11 * half) {
+    w.fields = B;
+    w.w1 = w.w2 = std::max(half, op) * B;
+  } else {
+    const int most = (int)std::max<size_t>(1, kSlice / (2 * op)), n = (B + most - 1) / most;
+    w.fields = (B + n - 1) / n;
+    w.w1 = half * B;
+    w.w2 = 2 * op * w.fields;
+  }
+  return w;
 }
 
 template <int MODE>
@@ -954,11 +980,11 @@ static cudaError_t launch(const TorusPlan* p, TgArgs& a, int s, int B, int col_t
   return cudaGetLastError();
 }
 
-cudaError_t torus_inverse(const TorusPlan* p, int s, int B, void* F, size_t f_bytes, void* work, void* out, size_t out_bytes,
-                          int* status, long long wait_ns, cudaStream_t st, int* launches, int step) {
+cudaError_t torus_inverse(const TorusPlan* p, int s, int B, const void* F, size_t f_bytes, void* x_work, void* y_work, void* out,
+                          size_t out_bytes, int* status, long long wait_ns, cudaStream_t st, int* launches, int step) {
   const Shape& sh = p->sh;
-  const Operand x = operand(work, pass_units(sh, kThetaInverse, B), sh.nKs);
-  const Operand y = operand(F, pass_units(sh, kPhiInverse, B), sh.nKm());  // in place of F, read by then
+  const Operand x = operand(x_work, pass_units(sh, kThetaInverse, B), sh.nKs);
+  const Operand y = operand(y_work, pass_units(sh, kPhiInverse, B), sh.nKm());
   TgArgs a{};
   if (step == 0) {
     const int blocks = ((sh.L + 1) / 2 + 15) / 16 + (sh.L / 2 + 15) / 16;
@@ -975,12 +1001,12 @@ cudaError_t torus_inverse(const TorusPlan* p, int s, int B, void* F, size_t f_by
   return launch<kPhiInverse>(p, a, s, B, B * sh.nT, kCosPhiInv, status, wait_ns, st);
 }
 
-cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const void* f, size_t f_bytes, void* w1, void* w2,
-                           void* H, size_t h_bytes, const TileOut* tiles, int* status, long long wait_ns, cudaStream_t st,
+cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const void* f, size_t f_bytes, void* x_work, void* y_work,
+                           void* H, size_t h_bytes, const TileOut* tiles, int b0, int* status, long long wait_ns, cudaStream_t st,
                            int* launches, int step) {
   const Shape& sh = p->sh;
-  const Operand x = operand(w1, pass_units(sh, kPhiForward, B), sh.nKs);
-  const Operand y = operand(w2, pass_units(sh, kThetaForward, B), sh.nKs);
+  const Operand x = operand(x_work, pass_units(sh, kPhiForward, B), sh.nKs);
+  const Operand y = operand(y_work, pass_units(sh, kThetaForward, B), sh.nKs);
   TgArgs a{};
   if (step == 0) {
     pack_phi_kernel<<<dim3((unsigned)(B * ((sh.L + 15) / 16)), (unsigned)((sh.nKs / 2 + 1) / 2)), 512, 0, st>>>(sh, B, (const float2*)f, x, (long long)(f_bytes / sizeof(float2)));
@@ -990,6 +1016,7 @@ cudaError_t torus_analysis(const TorusPlan* p, int adjoint, int s, int B, const 
     return launch<kPhiForward>(p, a, s, B, 2 * ((B * sh.nT + 1) / 2), kCosPhiFwd, status, wait_ns, st);
   }
   a.in = y;
+  a.b0 = b0;
   if (tiles) a.to = *tiles;
   a.f = (float2*)H;
   a.f_n = (long long)(h_bytes / sizeof(float2));
