@@ -233,15 +233,18 @@ cudaError_t contract_inverse_simt(const Dims& d, int s, int B, const double* tab
   return cudaGetLastError();
 }
 
-// Fields times degrees a warp: 4 (FP64) or 8 (FP32), whose sums fill the lanes.
+// Degrees a warp: FP64 four with one field, two with two, one beyond, whose sums fill the lanes; FP32, which has more
+// room in its pipe than in its loads of the table, two up to four fields and one beyond.  GB300, FP32, one field, by 1, 2, 4
+// and 8 degrees, us: L = 256 29, 25, 29, 46; L = 1024 1394, 1133, 1539, 2949; L = 2048 10227, 8372, 11295, 21927; two fields
+// by 1, 2 and 4: L = 256 35, 33, 39; L = 1024 2012, 1686, 2103.
 template <typename T>
 cudaError_t contract_project_simt(const Dims& d, int s, int B, const double* table, const double* U,
                                   const void* H, size_t h_bytes, void* flm, size_t flm_bytes, cudaStream_t st) {
-  constexpr int V = sizeof(T) == 8 ? 4 : 8;
-  if (B == 1) launch_project<T, 1, V>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
-  else if (B == 2) launch_project<T, 2, V / 2>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
-  else if (sizeof(T) == 8 || B <= 4) launch_project<T, 4, V / 4>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
-  else launch_project<T, sizeof(T) == 8 ? 4 : 8, 1>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
+  constexpr bool f64 = sizeof(T) == 8;
+  if (B == 1) launch_project<T, 1, f64 ? 4 : 2>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
+  else if (B == 2) launch_project<T, 2, 2>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
+  else if (f64 || B <= 4) launch_project<T, 4, f64 ? 1 : 2>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
+  else launch_project<T, f64 ? 4 : 8, 1>(d, s, B, table, U, H, h_bytes, flm, flm_bytes, st);
   return cudaGetLastError();
 }
 
