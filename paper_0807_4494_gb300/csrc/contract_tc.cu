@@ -158,22 +158,19 @@ __global__ void __launch_bounds__(256) pack_a_kernel(int L, int s, const Item* _
 // 8 K of one order, sign and field, four neighbouring threads the 32 K of a tile row, so that they find the
 // row pair's power of two with two shuffles and store 16 bytes at a time.  Split-BF16: a warp takes a row
 // pair, a lane one K.  The rows of padding fields stay as tc_configure zeroed them.  Fields run in slices of Bs, slice z
-// in its own tile region of xslice bytes, and a CTA takes kPackFields rows' worth of fields of a slice
-// (blockIdx.z: slice and group of fields), which keeps the GPU filled at small band-limits too.  Bound by HBM
+// in its own tile region of xslice bytes, and a CTA takes `per` fields of a slice, an even number
+// (blockIdx.z: slice and group of fields): eight, or two where that leaves SMs without a CTA.  Bound by HBM
 // traffic (1.1 GB at L = 1024, B = 64: 0.16 ms) and by how many loads are in flight: six CTAs on an SM (40
 // registers) take 0.28 ms where three with the next fields' loads under way (80 registers) took 0.47 and
 // a CTA of 64 KB staging with bulk stores 0.66; at L = 512, B = 32 42 us, 68 before.
-constexpr int kPackFields = 8;
-static int pack_v_groups(int NC) { return (NC / 4 + kPackFields - 1) / kPackFields; }
 
 template <bool BF>
-__global__ void __launch_bounds__(256, 6) pack_v_kernel(int L, int s, int Btot, int Bs, size_t xslice, int NC,
+__global__ void __launch_bounds__(256, 6) pack_v_kernel(int L, int s, int Btot, int Bs, int per, size_t xslice, int NC,
                                                      const int* __restrict__ xc0, const long long* __restrict__ xoff,
                                                      const float2* __restrict__ flm, uint8_t* __restrict__ X,
                                                      float* __restrict__ XS) {
   __shared__ float2 sv[2][32][33];
-  const int half = NC / 2, nb = half / 2;  // nb: fields of a sign half, padded
-  const int groups = (nb + kPackFields - 1) / kPackFields, z = blockIdx.z / groups, bg = (blockIdx.z - z * groups) * kPackFields;
+  const int half = NC / 2, groups = (Bs + per - 1) / per, z = blockIdx.z / groups, bg = (blockIdx.z - z * groups) * per;
   const int B = min(Bs, Btot - z * Bs);
   const long long flm_n = (long long)Btot * L * L, flm0 = (long long)z * Bs * L * L;
   const long long x_tiles = (long long)(xslice / (kParts<BF> * (size_t)NC * 128));
@@ -186,7 +183,7 @@ __global__ void __launch_bounds__(256, 6) pack_v_kernel(int L, int s, int Btot, 
   const int as = s < 0 ? -s : s;
   const int part_bytes = NC * 128;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b_end = min(bg + kPackFields, B);
+  const int b_end = min(bg + per, B);
   // 32 degrees l x (orders m0 .. m0 + 15, then -m0 .. -m0 - 15) of a field: four values a thread, whose
   // places in a field are the same for every field
   int at[4];
@@ -824,12 +821,14 @@ cudaError_t tc_pack_a(TcPlan* p, int forward, const double* table, const float* 
 }
 
 cudaError_t tc_pack_data(TcPlan* p, const void* src, cudaStream_t st, int* launches) {
-  const dim3 g(p->nC, (p->L + 15) / 16, (unsigned)(p->nS * pack_v_groups(p->NC)));
+  // Two fields a CTA while eight would give fewer than two CTAs to an SM (L = 65, B = 8, kept Delta, inverse: split BF16 49.7 -> 39.7 us)
+  const int mb = (p->L + 15) / 16, per = p->nC * mb * p->nS * ((p->Bs + 7) / 8) < 2 * p->grid ? 2 : 8;
+  const dim3 g(p->nC, mb, (unsigned)(p->nS * ((p->Bs + per - 1) / per)));
   if (p->bf16)
-    pack_v_kernel<true><<<g, 256, 0, st>>>(p->L, p->s, p->B, p->Bs, p->xslice, p->NC, p->xc0, p->xoff,
+    pack_v_kernel<true><<<g, 256, 0, st>>>(p->L, p->s, p->B, p->Bs, per, p->xslice, p->NC, p->xc0, p->xoff,
                                            (const float2*)src, p->X, p->XS);
   else
-    pack_v_kernel<false><<<g, 256, 0, st>>>(p->L, p->s, p->B, p->Bs, p->xslice, p->NC, p->xc0, p->xoff,
+    pack_v_kernel<false><<<g, 256, 0, st>>>(p->L, p->s, p->B, p->Bs, per, p->xslice, p->NC, p->xc0, p->xoff,
                                             (const float2*)src, p->X, p->XS);
   *launches += 1;
   return cudaGetLastError();

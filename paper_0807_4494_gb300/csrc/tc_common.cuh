@@ -286,33 +286,29 @@ __device__ __forceinline__ float warp_power(float amax, float* scale) {
 }
 
 // Writes two rows (j, j + 1: a field's real and imaginary part) of a data tile if `store` (warp-uniform), the
-// warp's lanes holding K = lane of both (x, y).  Split-FP16: of x and y times the block's power of two `up`;
-// neighbouring lanes exchange a value, so that each lane splits and stores two K of one row (4-byte stores).
-// Split-BF16: three 2-byte parts a value and the zero half.
+// warp's lanes holding K = lane of both (x, y): neighbouring lanes exchange a value, so that each lane splits and
+// stores two K of one row (4-byte stores).  Split-FP16: of x and y times the block's power of two `up`.
+// Split-BF16: three parts; the half of the second part's row that none of them fills stays as it was zeroed.
 template <bool BF>
 __device__ __forceinline__ void put_rows2(uint8_t* tile, int part_bytes, int j, int lane, float x, float y, float up, bool store) {
+  const bool odd = lane & 1;
+  const float other = __shfl_xor_sync(0xffffffffu, odd ? x : y, 1);
+  const float a = odd ? other : x, b = odd ? y : other;
+  const uint32_t off = sw128(j + (lane & 1), 4 * (lane >> 1));
   if constexpr (BF) {
+    uint16_t h[2], m[2], l[2];
+    split_bf16x3(a, &h[0], &m[0], &l[0]);
+    split_bf16x3(b, &h[1], &m[1], &l[1]);
     if (!store) return;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      uint16_t h, m, l;
-      split_bf16x3(i ? y : x, &h, &m, &l);
-      const uint32_t off = sw128(j + i, 2 * lane);
-      *(uint16_t*)(tile + off) = h;
-      *(uint16_t*)(tile + (off ^ 64u)) = m;
-      *(uint16_t*)(tile + part_bytes + off) = l;
-      *(uint16_t*)(tile + part_bytes + (off ^ 64u)) = 0;
-    }
+    *(uint32_t*)(tile + off) = h[0] | (uint32_t)h[1] << 16;
+    *(uint32_t*)(tile + (off ^ 64u)) = m[0] | (uint32_t)m[1] << 16;
+    *(uint32_t*)(tile + part_bytes + off) = l[0] | (uint32_t)l[1] << 16;
   } else {
-    const bool odd = lane & 1;
-    const float other = __shfl_xor_sync(0xffffffffu, odd ? x : y, 1);
     uint32_t h, l;
-    split2(up * (odd ? other : x), up * (odd ? y : other), &h, &l);
-    const uint32_t off = sw128(j + (lane & 1), 4 * (lane >> 1));
-    if (store) {
-      *(uint32_t*)(tile + off) = h;
-      *(uint32_t*)(tile + (off ^ 64u)) = l;
-    }
+    split2(up * a, up * b, &h, &l);
+    if (!store) return;
+    *(uint32_t*)(tile + off) = h;
+    *(uint32_t*)(tile + (off ^ 64u)) = l;
   }
 }
 
