@@ -89,7 +89,7 @@ typedef enum {
                            * rounding; the default needs no hand-off between degrees and 2 FP64
                            * instructions an entry against about 9. */
 #define SSHT_FLAG_TUNE 4  /* tensor-core plans: at creation, time the contraction's shape candidates
-                           * (fields per GEMM launch 64/32/16, pipeline depth 2-4, work order) on the
+                           * (fields per slice 64/32/16, pipeline depth 2-4, work order) on the
                            * plan's own operands and keep the fastest; with the environment variable
                            * SSHT_TUNE_CACHE naming a file, choices are read from it (no timing) and
                            * appended to it after tuning, one JSON object per line keyed by
@@ -122,7 +122,7 @@ SSHT_API int ssht_plan(ssht_plan_t* out, int L, int s, int batch);
 /* Create a plan from a descriptor (precision and Delta mode).  With SSHT_DELTA_CACHE the
  * recursion runs here, synchronously, and its table stays resident in device memory.
  * The tensor-core precisions (SSHT_TF32X3, SSHT_BF16X6) take any batch: the contraction runs the
- * fields in slices of at most 64 (one GEMM launch each, all reading the same A operand). */
+ * fields in slices of at most 64 (one launch for all, which read the same A operand). */
 SSHT_API int ssht_plan_ex(ssht_plan_t* out, const ssht_plan_desc* desc);
 
 /* Release every resource of a plan (NULL is accepted).  Synchronises the device. */

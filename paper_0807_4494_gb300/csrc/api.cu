@@ -679,7 +679,7 @@ int pair_call(ssht_plan_t p, int which, const void* in, void* out, cudaStream_t 
 
 // ---------------------------------------------------------------------------------------------
 // Tile tuning of the tensor-core contraction (SSHT_FLAG_TUNE, and the tuned buckets of groups):
-// every shape candidate -- fields per GEMM launch, pipeline depth, work order -- is timed on the
+// every shape candidate -- fields per slice, pipeline depth, work order -- is timed on the
 // plan's own operands (inverse + forward contractions, CUDA events) and the fastest kept.  With
 // SSHT_TUNE_CACHE naming a file, choices are looked up there first and stored after tuning, one
 // JSON object per line: {"key": "L=1024 s=2 B=64 tf32x3", "slice": 64, "stages": 2, ...}.

@@ -73,12 +73,13 @@ struct Item {
 };
 
 struct TcArgs {
-  int L, s, B, NC;        // B: fields of this slice; NC = 2H: padded columns, H = 2 Bs rounded up to 16 (<= 128)
+  int L, s, B, Bs, NC;    // Bs: fields of a slice (blockIdx.y); NC = 2H: padded columns, H = 2 Bs rounded up to 16 (<= 128)
   int stages;             // pipeline depth
   const int* sched;       // CTA b runs items [sched[b], sched[b + 1]) in order
   const Item* items;
   const uint8_t* A;       // packed A tiles
-  const uint8_t* X;       // packed data tiles
+  const uint8_t* X;       // packed data tiles, xslice bytes a slice
+  size_t xslice;
   const float* XS;        // split-FP16: their scales, [tile][NC / 2]
   const long long* xoff;  // per m: data tile index of chunk xc0(m)
   const int* xc0;         // per m: first chunk stored for m
@@ -88,7 +89,8 @@ struct TcArgs {
   int rows;               // forward: half rows instead of flm
   int* status;
   long long wait_ns;      // spin limit of the pipeline waits
-  long long a_tiles, x_tiles, out_n;  // extents of A, this slice's data tiles and out (index checks)
+  long long a_tiles, x_tiles;  // extents of A and of a slice's data tiles (index checks)
+  long long out_field;         // elements of a field in out
 };
 
 __device__ __forceinline__ float2 ipow_signed(int s, int k) {
@@ -279,6 +281,9 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
   static_assert(SCALE_SLOTS > MAX_STAGES + 2 && (SCALE_SLOTS & (SCALE_SLOTS - 1)) == 0, "scale ring");
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
+  // this slice's outputs and fields (read again for every item: kept in registers, they cost the sums' loop some)
+  __shared__ float2* slice_out;
+  __shared__ int slice_fields;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == 1) tmem_alloc(&tmem_base, 512);
   if (threadIdx.x == 0) {
@@ -293,6 +298,9 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
     for (int k = 0; k < SCALE_SLOTS; ++k) mbar_init(&scale_full[k], 1);
     mbar_init(&done_bar, 1);
     abort_flag = 0;
+    const int first = blockIdx.y * a.Bs;
+    slice_out = a.out + first * a.out_field;
+    slice_fields = min(a.Bs, a.B - first);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   fence_before();
@@ -310,6 +318,8 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
       const bool one = elect_one();
       int s = 0, ph = 1, n = 0;     // stage, parity its empty barrier is waited for, chunk
       uint32_t used = 0, uph = 0;   // stages that were filled, and the parity of their last fill
+      const uint8_t* X = a.X + (size_t)blockIdx.y * a.xslice;
+      const float* XS = BF ? nullptr : a.XS + (size_t)blockIdx.y * a.x_tiles * (a.NC / 2);
       for (int w = w_begin; w < w_end && !*abort; ++w) {
         const Item itm = a.items[w];
         const long long x0 = FWD ? (long long)itm.m * nC : a.xoff[itm.m] - a.xc0[itm.m];
@@ -329,11 +339,11 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
             if constexpr (!BF) {
               const int slot = n & (SCALE_SLOTS - 1);
               mbar_expect_tx(&scale_full[slot], (uint32_t)(2 * a.NC));
-              bulk_g2s(scales[slot], a.XS + (size_t)xt * (a.NC / 2), (uint32_t)(2 * a.NC), &scale_full[slot]);
+              bulk_g2s(scales[slot], XS + (size_t)xt * (a.NC / 2), (uint32_t)(2 * a.NC), &scale_full[slot]);
             }
             mbar_expect_tx(&full[s], (uint32_t)(GA + gx));
             bulk_g2s(st, asrc, GA, &full[s]);
-            bulk_g2s(st + GA, a.X + (size_t)xt * gx, (uint32_t)gx, &full[s]);
+            bulk_g2s(st + GA, X + (size_t)xt * gx, (uint32_t)gx, &full[s]);
           }
           used |= 1u << s;
           uph = (uph & ~(1u << s)) | ((uint32_t)(ph ^ 1) << s);
@@ -407,7 +417,7 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
     const int q = warp & 3;            // tensor-memory lane quarter this warp may access
     const int cg = (warp - 4) >> 2;    // of the NC / 16 groups of 16 columns: cg, cg + 4, cg + 8, cg + 12
     const int r = q * 32 + lane;
-    const int L = a.L, Lp = L - 1, NT = 2 * L - 1, B = a.B, s = a.s;
+    const int L = a.L, Lp = L - 1, NT = 2 * L - 1, s = a.s;
     const int H = a.NC / 2;
     const uint32_t tq = tbase + ((uint32_t)(q * 32) << 16);
     int seg = 0, sph = 0, n = 0;
@@ -462,6 +472,8 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
       const int rowv = itm.i * TM + r;  // m' (inverse) or l (forward)
       const bool valid = FWD ? (rowv <= Lp && rowv >= m) : (rowv <= Lp);
       if (!valid) continue;
+      const int B = *(volatile int*)&slice_fields;
+      float2* const out = *(float2* volatile*)&slice_out;
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
         const int j = 16 * (4 * g + cg);
@@ -474,15 +486,15 @@ __global__ void __launch_bounds__(THREADS, 1) tc_gemm_kernel(TcArgs a) {
         const float rs = ((h && (rowv & 1)) ? -1.f : 1.f) * (BF ? 1.f : 16384.f / kAScale);
         const float2 pz = make_float2(rs * pu.x, rs * pu.y);
         const bool flat = FWD && !a.rows;
-        const long long o0 = flat ? (long long)rowv * rowv + rowv + mm : (long long)(mm + Lp) * L + rowv;
         const long long ob = flat ? (long long)L * L : (long long)NT * L;
+        const long long o0 = flat ? (long long)rowv * rowv + rowv + mm : (long long)(mm + Lp) * L + rowv;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int b = b0 + k;
           if (b >= B) break;
           const float xr = acc[16 * g + 2 * k], xi = acc[16 * g + 2 * k + 1];
           const long long o = o0 + b * ob;
-          if (in_bounds(o, a.out_n, kbGemmOut)) a.out[o] = make_float2(pz.x * xr - pz.y * xi, pz.x * xi + pz.y * xr);
+          if (in_bounds(o, B * a.out_field, kbGemmOut)) out[o] = make_float2(pz.x * xr - pz.y * xi, pz.x * xi + pz.y * xr);
         }
       }
     }
@@ -530,7 +542,7 @@ struct TcPlan {
   int L = 0, s = 0, B = 0, NC = 0, nC = 0, nI = 0;
   bool bf16 = false;  // split-BF16 (3 parts, 6 products) instead of split-FP16
   TcConfig cfg;
-  int Bs = 0, nS = 0;        // fields per slice (one GEMM launch each) and slices
+  int Bs = 0, nS = 0;        // fields per slice and slices
   size_t xslice = 0;         // bytes of one slice's data tiles
   std::vector<Item> inv_h, fwd_h;  // work items in creation order (re-sorted by the configuration)
   Item* items_inv = nullptr;  // in schedule order: CTA-major
@@ -856,43 +868,44 @@ constexpr long long kRowsFrom = 1ll << 22;
 cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, const void* ph, int* status, long long wait_ns,
                     cudaStream_t st, int* launches) {
   const bool via_rows = forward && rows && (long long)p->B * p->L * p->L >= kRowsFrom;
-  // one launch per slice of fields; every slice reads the same A tiles
-  for (int sl = 0; sl < p->nS; ++sl) {
-    TcArgs a;
-    a.L = p->L;
-    a.s = p->s;
-    a.B = std::min(p->Bs, p->B - sl * p->Bs);
-    a.NC = p->NC;
-    a.stages = p->cfg.stages;
-    a.sched = forward ? p->sched_fwd : p->sched_inv;
-    a.items = forward ? p->items_fwd : p->items_inv;
-    a.A = forward ? p->A : p->A_inv;
-    a.X = p->X + (size_t)sl * p->xslice;
-    a.XS = p->XS ? p->XS + (size_t)sl * (p->xslice / 256) : nullptr;
-    a.xoff = p->xoff;
-    a.xc0 = p->xc0;
-    a.ph = (const float2*)ph;
-    const size_t per_field = (forward && !via_rows) ? (size_t)p->L * p->L : (size_t)(2 * p->L - 1) * p->L;
-    a.out = (float2*)(via_rows ? rows : out) + (size_t)sl * p->Bs * per_field;
-    a.rows = via_rows;
-    a.status = status;
-    a.wait_ns = wait_ns;
-    a.a_tiles = forward ? p->tiles_A : p->tiles_inv;
-    a.x_tiles = (long long)(p->xslice / ((p->bf16 ? 2 : 1) * (size_t)p->NC * 128));
-    a.out_n = (long long)a.B * (long long)per_field;
-    const int grid = forward ? p->grid_fwd : p->grid_inv;
-    if (forward && p->bf16)
-      tc_gemm_kernel<true, true><<<grid, THREADS, p->smem, st>>>(a);
-    else if (forward)
-      tc_gemm_kernel<true, false><<<grid, THREADS, p->smem, st>>>(a);
-    else if (p->bf16)
-      tc_gemm_kernel<false, true><<<grid, THREADS, p->smem, st>>>(a);
-    else
-      tc_gemm_kernel<false, false><<<grid, THREADS, p->smem, st>>>(a);
-    *launches += 1;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  // all slices of fields in one launch, one after the other; every slice reads the same A tiles (a launch a slice took
+  // 8 to 10 us each at small band-limits: split BF16, L = 8, B = 8192 2607 us an inverse and a forward, now 173; tf32x3, L = 33,
+  // B = 8192 3661, now 1513)
+  TcArgs a;
+  a.L = p->L;
+  a.s = p->s;
+  a.B = p->B;
+  a.Bs = p->Bs;
+  a.NC = p->NC;
+  a.stages = p->cfg.stages;
+  a.sched = forward ? p->sched_fwd : p->sched_inv;
+  a.items = forward ? p->items_fwd : p->items_inv;
+  a.A = forward ? p->A : p->A_inv;
+  a.X = p->X;
+  a.xslice = p->xslice;
+  a.XS = p->XS;
+  a.xoff = p->xoff;
+  a.xc0 = p->xc0;
+  a.ph = (const float2*)ph;
+  a.out = (float2*)(via_rows ? rows : out);
+  a.rows = via_rows;
+  a.status = status;
+  a.wait_ns = wait_ns;
+  a.a_tiles = forward ? p->tiles_A : p->tiles_inv;
+  a.x_tiles = (long long)(p->xslice / ((p->bf16 ? 2 : 1) * (size_t)p->NC * 128));
+  a.out_field = (long long)((forward && !via_rows) ? p->L : 2 * p->L - 1) * p->L;
+  const dim3 grid((unsigned)(forward ? p->grid_fwd : p->grid_inv), (unsigned)p->nS);
+  if (forward && p->bf16)
+    tc_gemm_kernel<true, true><<<grid, THREADS, p->smem, st>>>(a);
+  else if (forward)
+    tc_gemm_kernel<true, false><<<grid, THREADS, p->smem, st>>>(a);
+  else if (p->bf16)
+    tc_gemm_kernel<false, true><<<grid, THREADS, p->smem, st>>>(a);
+  else
+    tc_gemm_kernel<false, false><<<grid, THREADS, p->smem, st>>>(a);
+  *launches += 1;
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   if (via_rows) {
     const int N = 2 * p->L - 1;
     // fields in z, at most 65535 a launch (the library's largest batch)

@@ -117,7 +117,7 @@ cudaError_t real_setup();
 // Tensor-core contractions (contract_tc.cu), split-FP16 (SSHT_TF32X3) or split-BF16
 // ---------------------------------------------------------------------------
 struct TcPlan;
-// The contraction's tunable shape: fields per GEMM launch (the N tile: 2 x 2 x slice real columns,
+// The contraction's tunable shape: fields per slice (the N tile: 2 x 2 x slice real columns,
 // padded to 16), pipeline depth (stages of A and data tiles in shared memory), and the order of the
 // work items (inverse: 0 grouped by m, 1 longest first; forward: 0 longest first, 1 grouped by m).
 struct TcConfig {

@@ -64,3 +64,18 @@ def test_one_field_takes_no_longer_than_eight(precision):
         us[B] = _us(lambda: plan.forward(f, out=out))
         plan.check()
     assert us[1] < 1.25 * us[8], us
+
+
+@pytest.mark.parametrize("precision", ["tf32x3", "bf16x6"])
+def test_time_grows_less_than_the_slices_of_fields(precision):
+    """64 slices of 64 fields at a small band-limit fill the GPU that one leaves empty: with a launch for each
+    slice they took 25 times as long.  Bound: 16 times."""
+    from paper_0807_4494_gb300 import ssht
+    us = {}
+    for B in (64, 4096):
+        plan = ssht.Plan(8, 0, B, precision=precision, delta_mode="cache")
+        x = torch.randn(B, 64, dtype=torch.complex64, device="cuda")
+        out = plan.inverse(x)
+        us[B] = _us(lambda: plan.inverse(x, out=out))
+        plan.check()
+    assert us[4096] < 16 * us[64], us
