@@ -103,10 +103,9 @@ struct ssht_plan_s {
   size_t w_bytes = 0;  // of W1 (FP64 plans: of W2 too)
   void* W3 = nullptr;
   size_t w3_bytes = 0;
-  void* ph = nullptr;       // phase table, element precision
-  double2* ph64 = nullptr;  // phase table, FP64
+  double2* ph64 = nullptr;  // phase table (the triangular forward's)
   cufftHandle fft_phi = 0, fft_theta = 0;
-  bool have_phi = false, have_theta = false, have_conv = false;
+  bool have_phi = false, have_theta = false;
   void* stage_in = nullptr;
   size_t stage_in_bytes = 0;
   void* stage_out = nullptr;
@@ -433,7 +432,7 @@ int tc_pack(ssht_plan_t p, const void* src, cudaStream_t st) {
 int tc_multiply(ssht_plan_t p, int forward, void* dst, cudaStream_t st) {
   int n = 0;
   StageScope sc(p, forward ? SSHT_STAGE_PROJECT : SSHT_STAGE_INVERSE, st);
-  SSHT_CUDA(tc_gemm(p->tc, forward, dst, forward ? p->W1 : nullptr, p->ph, p->delta.status, p->wait_ns, st, &n), "tensor-core contraction");
+  SSHT_CUDA(tc_gemm(p->tc, forward, dst, forward ? p->W1 : nullptr, p->delta.status, p->wait_ns, st, &n), "tensor-core contraction");
   p->launches += n;
   return 0;
 }
@@ -730,8 +729,8 @@ int time_contractions(ssht_plan_t p, cudaStream_t st, float* ms) {
   int n = 0, rc = 0;
   for (int it = 0; it < 4 && !rc; ++it) {
     if (it == 1) cudaEventRecord(e0, st);
-    cudaError_t e = tc_gemm(p->tc, 0, p->W1, nullptr, p->ph, p->delta.status, p->wait_ns, st, &n);
-    if (e == cudaSuccess) e = tc_gemm(p->tc, 1, p->W2, p->W1, p->ph, p->delta.status, p->wait_ns, st, &n);
+    cudaError_t e = tc_gemm(p->tc, 0, p->W1, nullptr, p->delta.status, p->wait_ns, st, &n);
+    if (e == cudaSuccess) e = tc_gemm(p->tc, 1, p->W2, p->W1, p->delta.status, p->wait_ns, st, &n);
     if (e != cudaSuccess) rc = fail(SSHT_ECUDA, std::string("tuning contraction: ") + cudaGetErrorString(e));
   }
   cudaEventRecord(e1, st);
@@ -827,7 +826,7 @@ void release(ssht_plan_t p) {
   if (p->have_theta) cufftDestroy(p->fft_theta);
   if (!p->delta_shared) delta_free(p->delta);
   lane_tables_free(p->lane);
-  void* ptrs[] = {p->U, p->Uf, p->W1, p->W2, p->W3, p->ph, p->ph64, p->stage_in, p->stage_out, p->rc, p->rg};
+  void* ptrs[] = {p->U, p->Uf, p->W1, p->W2, p->W3, p->ph64, p->stage_in, p->stage_out, p->rc, p->rg};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   delete p;
@@ -948,30 +947,21 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     if ((rc = dalloc(p, &p->W3, w3, "operand digits"))) return bail(rc);
     p->w3_bytes = w3;
   }
-  if ((rc = dalloc(p, &p->ph, (size_t)(2 * d.N - 1) * p->elem, "phase table"))) return bail(rc);
-  if ((rc = dalloc(p, (void**)&p->ph64, (size_t)(2 * d.N - 1) * sizeof(double2), "phase table"))) return bail(rc);
-
-  // Phase table e^{i pi k / N}, |k| < N, computed in FP64 on the host.
-  {
+  if (p->f64) {
+    // Phase table e^{i pi k / N}, |k| < N, computed in FP64 on the host.
+    if ((rc = dalloc(p, (void**)&p->ph64, (size_t)(2 * d.N - 1) * sizeof(double2), "phase table"))) return bail(rc);
     std::vector<double2> h(2 * d.N - 1);
-    std::vector<float2> hf(2 * d.N - 1);
     const double pi = 3.14159265358979323846;
     for (int k = -(d.N - 1); k <= d.N - 1; ++k) {
       // reduce the angle to [-pi/2, pi/2]-ish before cos/sin for accuracy: k/N in (-1, 1)
       const double a = pi * (double)k / (double)d.N;
       h[k + d.N - 1] = make_double2(std::cos(a), std::sin(a));
-      hf[k + d.N - 1] = make_float2((float)std::cos(a), (float)std::sin(a));
     }
     ce = cudaMemcpy(p->ph64, h.data(), h.size() * sizeof(double2), cudaMemcpyHostToDevice);
-    if (ce == cudaSuccess)
-      ce = cudaMemcpy(p->ph, p->f64 ? (const void*)h.data() : (const void*)hf.data(), h.size() * p->elem,
-                      cudaMemcpyHostToDevice);
     if (ce != cudaSuccess) {
       release(p);
       return fail(SSHT_ECUDA, std::string("phase table upload: ") + cudaGetErrorString(ce));
     }
-  }
-  if (p->f64) {
     if ((rc = make_fft(p, &p->fft_phi, &p->have_phi, d.N, (size_t)B * d.L, "cuFFT phi plan"))) return bail(rc);
     if ((rc = make_fft(p, &p->fft_theta, &p->have_theta, d.N, (size_t)B * d.N, "cuFFT theta plan"))) return bail(rc);
   }

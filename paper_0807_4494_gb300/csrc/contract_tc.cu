@@ -83,7 +83,6 @@ struct TcArgs {
   const float* XS;        // split-FP16: their scales, [tile][NC / 2]
   const long long* xoff;  // per m: data tile index of chunk xc0(m)
   const int* xc0;         // per m: first chunk stored for m
-  const float2* ph;       // e^{i pi k/N}, k in [-(N-1), N-1], at k + N - 1
   float2* out;            // half rows [B][N][L] (rows by signed order; inverse: F, columns m'; forward with
                           // `rows`: columns l >= |m|), or flm [B][L*L]
   int rows;               // forward: half rows instead of flm
@@ -865,7 +864,7 @@ TileOut tc_forward_tiles(const TcPlan* p) {
 // workspace and rows_to_flm_kernel transposes them (GB300, B = 64: the GEMM at L = 1024 1.68 ms direct, 0.69 by rows and 0.17 for the transposition).
 constexpr long long kRowsFrom = 1ll << 22;
 
-cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, const void* ph, int* status, long long wait_ns,
+cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, int* status, long long wait_ns,
                     cudaStream_t st, int* launches) {
   const bool via_rows = forward && rows && (long long)p->B * p->L * p->L >= kRowsFrom;
   // all slices of fields in one launch, one after the other; every slice reads the same A tiles (a launch a slice took
@@ -886,7 +885,6 @@ cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, const void* p
   a.XS = p->XS;
   a.xoff = p->xoff;
   a.xc0 = p->xc0;
-  a.ph = (const float2*)ph;
   a.out = (float2*)(via_rows ? rows : out);
   a.rows = via_rows;
   a.status = status;

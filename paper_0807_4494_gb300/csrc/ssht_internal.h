@@ -143,7 +143,7 @@ cudaError_t tc_pack_data(TcPlan* p, const void* src, cudaStream_t st, int* launc
 // The contraction: forward = 0 writes the half rows F (float2 [B][N][L], m' >= 0) of the inverse;
 // forward = 1 writes flm (float2 [B][L*L]), large outputs by way of the workspace rows (float2 [B][N][L];
 // null: always directly).  Timeouts set bit 2 of *status.
-cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, const void* ph, int* status, long long wait_ns,
+cudaError_t tc_gemm(TcPlan* p, int forward, void* out, void* rows, int* status, long long wait_ns,
                     cudaStream_t st, int* launches);
 // Where the forward theta pass writes the projection's data tiles directly (in place of H and
 // tc_pack_data): the tile array, its column count NC, chunks per m nC, and the split form

@@ -24,18 +24,6 @@ __host__ __device__ __forceinline__ uint32_t sw128(int row, int kbyte) {
   return (uint32_t)((row >> 3) * 1024 + (row & 7) * 128 + ((((kbyte >> 4) ^ row) & 7) << 4) + (kbyte & 15));
 }
 
-// Shared-memory matrix descriptor: start address, stride between 8-row groups (1024 bytes),
-// descriptor version 1, SWIZZLE_128B.
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)1 << 16;                   // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;         // stride byte offset
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
-}
-
 // Instruction descriptor: D = F32, A = B = BF16 (kind::f16), both K-major, shape M x N.
 __device__ __forceinline__ uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
@@ -163,7 +151,8 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
 }
-// kind::f16, one CTA or a pair, with the descriptors (desc_sw128) given by their low words -- the
+// kind::f16, one CTA or a pair.  The shared-memory matrix descriptors (SWIZZLE_128B, version 1, 1024 bytes between
+// 8-row groups, the leading offset unused for swizzled K-major tiles) are given by their low words -- the
 // start address in 16-byte units, kDescLow added -- so that stepping through a tile is one addition.
 constexpr uint32_t kDescLow = 1u << 16, kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);
 template <bool PAIR>
