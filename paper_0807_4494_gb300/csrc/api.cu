@@ -985,8 +985,20 @@ int create(ssht_plan_t* out, const ssht_plan_desc* desc, const DeltaWork* shared
     p->bytes += tc_bytes(p->tc);
   }
   if (tiles_direct(p)) {
-    // the spin column once: the table of one sweep, then U from it
-    if ((rc = run_delta(p, 0))) return bail(rc);
+    // the spin column once, from the table: a kept table, which ssht_wigner_delta hands out, is made whole (a group's
+    // shared one is), and one of a small band-limit, whose sweep takes less than the list of tasks; else only the
+    // entries that U reads (the sweep, L = 1024, s = 2: 0.95 -> 0.23 ms)
+    if (p->delta_mode == SSHT_DELTA_CACHE || p->delta_shared || L <= 512) {
+      if ((rc = run_delta(p, 0))) return bail(rc);
+    } else {
+      ce = column_run_spin(p->delta, L, s, 0);
+      if (ce == cudaSuccess) ce = delta_spin_column(p->delta.table, L, s, p->U, p->Uf, 0);
+      if (ce != cudaSuccess) {
+        release(p);
+        return fail(ce == cudaErrorMemoryAllocation ? SSHT_ENOMEM : SSHT_ECUDA, std::string("spin column: ") + cudaGetErrorString(ce));
+      }
+      p->launches += 2;
+    }
     p->u_fixed = true;
     // the calls' recursions run on the plan's non-blocking stream: U must be complete first
     ce = cudaDeviceSynchronize();

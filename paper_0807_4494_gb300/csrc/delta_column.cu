@@ -715,36 +715,52 @@ __global__ void lane_first_rows_kernel(int L, const double* __restrict__ sq, con
   }
 }
 
-// One thread per degree l walks m' = l .. 0: a(m'), b(m') from the sqrt tables (the products of
-// the unscaled relation), p(l, l) = p(l, l-1) = 1, p(l, m'-1) = b(m') p(l, m'+1) and
-// alpha(l, m') = 2 a(m') p(l, m') / p(l, m'-1) (alpha(l, 0) is never used: no step leaves m' = 0).
-// Written degree-major (l(l+1)/2 + m', the column recursion's chunks) and in the triangle layout
-// tri_idx(m', l) (the degree-lane recursion), with U_l[m'] transposed beside them.
-__global__ void rescale_tables_kernel(int L, const double* __restrict__ sq, const double* __restrict__ rsq,
-                                      const float* __restrict__ Uf, double* __restrict__ alc, float* __restrict__ pc,
-                                      double* __restrict__ alT, float* __restrict__ pT, float* __restrict__ ufT) {
+// The rescaled relation's tables, from the sqrt tables (the products of the unscaled relation): p(l, l) = p(l, l-1) = 1,
+// p(l, m'-1) = b(m') p(l, m'+1) and alpha(l, m') = 2 a(m') p(l, m') / p(l, m'-1) (alpha(l, 0) is never used: no step leaves
+// m' = 0).  Written degree-major (l(l+1)/2 + m', the column recursion's chunks) and in the triangle layout tri_idx(m', l) (the
+// degree-lane recursion), with U_l[m'] transposed beside them.  Only p is a chain: a thread a degree multiplies it up,
+// one FP64 instruction a step, between two kernels that make b and alpha for all entries at once (all in the chain's thread
+// they took 1.0 ms at L = 1024).
+__device__ __forceinline__ double rescale_a(int l, int mp, const double* __restrict__ rsq) {
+  return __dmul_rn(rsq[l - mp + 1], rsq[l + mp]);
+}
+// b(m') at tri_idx(m', l), m' >= 1.  blockIdx.y: m'.
+__global__ void rescale_b_kernel(int L, const double* __restrict__ sq, const double* __restrict__ rsq, double* __restrict__ b) {
+  const int mp = blockIdx.y, l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= L || l < mp || mp < 1) return;
+  b[tri_idx(mp, l, L)] = __dmul_rn(__dmul_rn(sq[l - mp], sq[l + mp + 1]), rescale_a(l, mp, rsq));
+}
+// p(l, m') at tri_idx(m', l), a thread a degree.
+__global__ void rescale_p_kernel(int L, const double* __restrict__ b, double* __restrict__ p) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= L) return;
-  const size_t row = (size_t)l * (l + 1) / 2;
-  double p_up = 1.0, p_cur = 1.0;  // p(l, m'+1) and p(l, m') at m' = l (the first is not used there)
-  for (int mp = l; mp >= 0; --mp) {
-    double p_dn = 0.0, al = 0.0;
-    if (mp >= 1) {
-      const double a = __dmul_rn(rsq[l - mp + 1], rsq[l + mp]);
-      const double b = __dmul_rn(__dmul_rn(sq[l - mp], sq[l + mp + 1]), a);
-      p_dn = mp == l ? 1.0 : __dmul_rn(b, p_up);
-      al = __ddiv_rn(__dmul_rn(2.0 * a, p_cur), p_dn);
-    }
-    const size_t kt = tri_idx(mp, l, L);
-    const float pf = __double2float_rn(p_cur);
-    alc[row + mp] = al;
-    pc[row + mp] = pf;
-    alT[kt] = al;
-    pT[kt] = pf;
-    ufT[kt] = Uf[row + mp];
-    p_up = p_cur;
-    p_cur = p_dn;
+  double up = 1.0, cur = 1.0;  // p(l, m'+1) and p(l, m') at m' = l - 1
+  p[tri_idx(l, l, L)] = 1.0;
+  if (l >= 1) p[tri_idx(l - 1, l, L)] = 1.0;
+#pragma unroll 4
+  for (int mp = l - 1; mp >= 1; --mp) {
+    const double dn = __dmul_rn(b[tri_idx(mp, l, L)], up);
+    p[tri_idx(mp - 1, l, L)] = dn;
+    up = cur;
+    cur = dn;
   }
+}
+// blockIdx.y: m'.
+__global__ void rescale_tables_kernel(int L, const double* __restrict__ rsq, const float* __restrict__ Uf, const double* __restrict__ p,
+                                      double* __restrict__ alc, float* __restrict__ pc, double* __restrict__ alT,
+                                      float* __restrict__ pT, float* __restrict__ ufT) {
+  const int mp = blockIdx.y, l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l >= L || l < mp) return;
+  const size_t row = (size_t)l * (l + 1) / 2, kt = tri_idx(mp, l, L);
+  const double cur = p[kt];
+  double al = 0.0;
+  if (mp >= 1) al = __ddiv_rn(__dmul_rn(2.0 * rescale_a(l, mp, rsq), cur), p[tri_idx(mp - 1, l, L)]);
+  const float pf = __double2float_rn(cur);
+  alc[row + mp] = al;
+  pc[row + mp] = pf;
+  alT[kt] = al;
+  pT[kt] = pf;
+  ufT[kt] = Uf[row + mp];
 }
 
 // ab2[M] = abase[M] - 2 i (i + 1), i = M / 128: the tile of (M, row block il, chunk c) of the
@@ -803,16 +819,17 @@ cudaError_t column_setup(DeltaWork& w, int L, int device) {
   return cudaMemcpy(w.sqrt_tab, sqv.data(), sqv.size() * sizeof(double), cudaMemcpyHostToDevice);
 }
 
-static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, const LaneTables* lt, ATiles t,
-                                 cudaStream_t st) {
+// tasks / ntasks: the tasks to run, all of w's by default.
+static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, const LaneTables* lt, ATiles t, cudaStream_t st,
+                                 const int2* tasks = nullptr, int ntasks = 0) {
   cudaError_t e;
   unsigned int* counter = lt ? lt->counter : w.barrier;
   if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned int), st)) != cudaSuccess) return e;
   ColumnParams P;
   P.L = L;
-  P.ntasks = w.ntasks;
+  P.ntasks = tasks ? ntasks : w.ntasks;
   P.sms = w.sms;
-  P.tasks = w.tasks;
+  P.tasks = tasks ? tasks : w.tasks;
   P.sq = w.sqrt_tab;
   P.rsq = w.sqrt_tab + (2 * (size_t)L + 4);
   P.table = w.table;
@@ -837,6 +854,23 @@ static cudaError_t column_launch(const DeltaWork& w, int L, const float* Uf, con
 
 cudaError_t column_run(const DeltaWork& w, int L, cudaStream_t st) {
   return column_launch(w, L, nullptr, nullptr, ATiles(), st);
+}
+
+// The entries (m', |s|) of the table come from the blocks of columns up to |s|'s: its own for the rows from its first
+// column on, and those before it (transposed) for the rows above.  For a small |s| that is one task a degree.
+cudaError_t column_run_spin(const DeltaWork& w, int L, int s, cudaStream_t st) {
+  if (w.method != kDeltaColumn) return cudaErrorInvalidValue;
+  const int last = (s < 0 ? -s : s) / 32;
+  std::vector<int2> tasks = column_tasks(L);
+  tasks.erase(std::remove_if(tasks.begin(), tasks.end(), [&](const int2& t) { return t.y > last; }), tasks.end());
+  int2* d = nullptr;
+  cudaError_t e = dev_malloc(&d, tasks.size() * sizeof(int2));
+  if (e != cudaSuccess) return e;
+  e = cudaMemcpy(d, tasks.data(), tasks.size() * sizeof(int2), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = column_launch(w, L, nullptr, nullptr, ATiles(), st, d, (int)tasks.size());
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  cudaFree(d);
+  return e;
 }
 
 void lane_tables_free(LaneTables& t) {
@@ -875,9 +909,13 @@ cudaError_t lane_tables_setup(LaneTables& t, const DeltaWork& w, int L, int s, c
     return e;
   const double* sq = w.sqrt_tab;
   const double* rsq = w.sqrt_tab + (2 * (size_t)L + 4);
-  lane_first_rows_kernel<<<dim3((unsigned)((L + 31) / 32 + 7) / 8, (unsigned)L), 256>>>(L, sq, rsq, t.t1m, t.t1e);
+  // b and p pass through the arrays of alpha and of the first rows
+  const dim3 all((unsigned)((L + 127) / 128), (unsigned)L);
+  rescale_b_kernel<<<all, 128>>>(L, sq, rsq, t.alT);
+  rescale_p_kernel<<<(unsigned)((L + 31) / 32), 32>>>(L, t.alT, t.t1m);
+  rescale_tables_kernel<<<all, 128>>>(L, rsq, Uf, t.t1m, t.alc, t.pc, t.alT, t.pT, t.ufT);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  rescale_tables_kernel<<<(unsigned)((L + 127) / 128), 128>>>(L, sq, rsq, Uf, t.alc, t.pc, t.alT, t.pT, t.ufT);
+  lane_first_rows_kernel<<<dim3((unsigned)((L + 31) / 32 + 7) / 8, (unsigned)L), 256>>>(L, sq, rsq, t.t1m, t.t1e);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   tile_base_kernel<<<(unsigned)((L + 127) / 128), 128>>>(L, abase, t.ab2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -79,6 +79,8 @@ cudaError_t delta_run(const DeltaWork& w, int L, cudaStream_t st, long long wait
 // The column method's setup and launch (delta_column.cu); delta_setup / delta_run dispatch.
 cudaError_t column_setup(DeltaWork& w, int L, int device);
 cudaError_t column_run(const DeltaWork& w, int L, cudaStream_t st);
+// Those entries of the table that the spin column of s reads (column method; synchronises the stream).
+cudaError_t column_run_spin(const DeltaWork& w, int L, int s, cudaStream_t st);
 // U[l][m'] = sqrt((2l+1)/4pi) Delta^l_{m',-s}, l < L, 0 <= m' <= l, at tri(l) + m'; Uf is the
 // same in FP32 (rounded to nearest).
 cudaError_t delta_spin_column(const double* table, int L, int s, double* U, float* Uf, cudaStream_t st);

@@ -12,21 +12,24 @@ static __global__ void node_table_kernel(int N, double2* cs) {
   if (r < 2 * N) cs[r] = make_double2(cospi((double)r / N), sinpi((double)r / N));
 }
 
-// Prefix sums over even p = 2q >= 0 of w_e(p) e^{ip x_t}, w_e(p) = 2/(1-p^2): T[q * L + t], q < L.
+// Prefix sums over even p = 2q >= 0 of w_e(p) e^{ip x_t}, w_e(p) = 2/(1-p^2): T[q * L + t], q < L.  A block is a warp,
+// whose lanes make the weights of 32 q's at a time (a division by every thread at every step took 0.47 ms at L = 1024).
 static __global__ void weight_prefix_kernel(int L, const double2* __restrict__ cs, double2* __restrict__ T) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, N = 2 * L - 1;
-  if (t >= L) return;
+  const int t = blockIdx.x * 32 + threadIdx.x, N = 2 * L - 1;
   double2 sum = make_double2(0.0, 0.0);
-  const int step = (int)((2ll * (2 * t + 1)) % (2 * N));
+  const int step = t < L ? (int)((2ll * (2 * t + 1)) % (2 * N)) : 0;
   int r = 0;
-  for (int q = 0; q < L; ++q) {
-    const double p = 2.0 * q, w = 2.0 / (1.0 - p * p);
-    const double2 e = cs[r];
-    sum.x += w * e.x;
-    sum.y += w * e.y;
-    T[(size_t)q * L + t] = sum;
-    r += step;
-    if (r >= 2 * N) r -= 2 * N;
+  for (int q0 = 0; q0 < L; q0 += 32) {
+    const double p = 2.0 * (q0 + (int)threadIdx.x), mine = 2.0 / (1.0 - p * p);
+    for (int i = 0; i < min(32, L - q0); ++i) {
+      const double w = __shfl_sync(0xffffffffu, mine, i);
+      const double2 e = cs[r];
+      sum.x += w * e.x;
+      sum.y += w * e.y;
+      if (t < L) T[(size_t)(q0 + i) * L + t] = sum;
+      r += step;
+      if (r >= 2 * N) r -= 2 * N;
+    }
   }
 }
 

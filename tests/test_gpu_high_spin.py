@@ -1,7 +1,7 @@
-"""Tensor-core plans above L = 1024 with spins near the band-limit, against FP64 plans.
-
-Such a plan has as few recursion tasks as one of small band-limit, but its first rows lie below the
-FP64 range and carry exponents of their own.  Bound 2e-6 max-norm, that of the L = 2048 tests."""
+"""Tensor-core plans with spins beyond the first block of columns, against FP64 plans: above L = 1024 near the
+band-limit, where a plan has as few recursion tasks as one of small band-limit, but first rows below the FP64 range
+that carry exponents of their own; and above L = 512, where plan creation makes only the part of the table that the
+spin column reads.  Bound 2e-6 max-norm, that of the L = 2048 tests."""
 import pytest
 import torch
 
@@ -16,8 +16,8 @@ def _built():
     __graft_entry__.build()
 
 
-@pytest.mark.parametrize("L,s", [(1100, 1040), (1280, 1200), (1280, -1200)])
-def test_tensor_core_plans_with_few_tasks_above_L1024(L, s):
+@pytest.mark.parametrize("L,s", [(600, 31), (600, -70), (1100, 1040), (1280, 1200), (1280, -1200)])
+def test_high_spins(L, s):
     from paper_0807_4494_gb300 import ssht
     x = torch.from_numpy(inputs.coeffs(L, s, 1, seed=1)).cuda()
     ref = ssht.Plan(L, s, 1, precision="fp64")
