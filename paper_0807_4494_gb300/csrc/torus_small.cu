@@ -312,11 +312,12 @@ struct SmallPlan {
 };
 
 // Where this form is the better one.  FP32-class plans, against the tensor-core products (which round a field up to units
-// of 128 rows and 64 K), inverse and forward in us, these and those: fp32 L = 16, B = 8192 166 + 225 and 776 + 716, L = 48,
-// B = 512 130 + 189 and 163 + 178, L = 49, B = 512 189 + 220 and 167 + 194, L = 64, B = 64 45 + 54 and 47 + 54, B = 128
-// 80 + 96 and 68 + 85, L = 65, B = 1 35 + 42 and 33 + 37 (its block of rings no longer fits beside another CTA's); tf32x3 L = 48,
-// B = 512 151 + 159 and 171 + 174, L = 64, B = 1 29 + 29 and 35 + 33, B = 128 72 + 70 and 62 + 62.  FP64 plans, against the
-// two-launch products (torus_direct.cu): L = 8, B = 8192 323 + 415 and 817 + 868, L = 32, B = 8192 5432 + 6481 and 6647 + 8007.
+// of 128 rows and 64 K), inverse and forward with a kept table in us, these and those: fp32 L = 16, B = 4096 83 + 114 and
+// 401 + 366, L = 48, B = 512 130 + 189 and 163 + 176, L = 49, B = 512 183 + 218 and 167 + 195, L = 64, B = 64 46 + 54 and
+// 48 + 54, B = 128 79 + 96 and 68 + 85, L = 65, B = 1 35 + 37 and 33 + 30 (phi of the last ring takes the CTA a second round);
+// tf32x3 L = 48, B = 512 93 + 99 and 113 + 113, L = 64, B = 1 29 + 29 and 33 + 31, B = 128 58 + 58 and 50 + 50.  FP64 plans,
+// against the two-launch products (torus_direct.cu): L = 8, B = 8192 323 + 415 and 817 + 868, L = 32, B = 8192 5432 + 6481 and
+// 6647 + 8007.
 bool small_wanted(int L, int B, bool f64) {
   return f64 ? L <= 32 : L <= 48 || (L <= 64 && (long long)B * L * L * L <= (1ll << 24));
 }
