@@ -7,8 +7,9 @@
 // spread over the GPU by their blocks.  A thread keeps 8 complex sums: the two signs of two orders of one parity in the
 // inverse's theta, four rings or four orders elsewhere, so that what it reads serves four times.
 //
-// What bounds it: 16 B L^3 flops a direction on the FP64 pipe, or in FP32 the shared-memory reads beside the
-// multiply-adds; a launch at the smallest sizes.  (Measured at small_wanted.)
+// What bounds it: 16 B L^3 flops a direction on the FP64 pipe (97 % of it: L = 32, B = 1024 554 us), or in FP32 the
+// shared-memory reads beside the multiply-adds (70 % of their rate: L = 16, B = 8192 38 us, L = 48, B = 512 58); a
+// launch at the smallest sizes.  (Against the other forms: small_wanted.)
 #include "bounds.cuh"
 #include "ssht_internal.h"
 #include "tc_common.cuh"
@@ -314,7 +315,7 @@ struct SmallPlan {
 // Where this form is the better one.  FP32-class plans, against the tensor-core products (which round a field up to units
 // of 128 rows and 64 K), inverse and forward with a kept table in us, these and those: fp32 L = 16, B = 4096 83 + 114 and
 // 401 + 366, L = 48, B = 512 130 + 189 and 163 + 176, L = 49, B = 512 183 + 218 and 167 + 195, L = 64, B = 64 46 + 54 and
-// 48 + 54, B = 128 79 + 96 and 68 + 85, L = 65, B = 1 35 + 37 and 33 + 30 (phi of the last ring takes the CTA a second round);
+// 48 + 54, B = 128 79 + 96 and 68 + 85, L = 65, B = 1 35 + 37 and 33 + 30 (its 17 quads of rings take the CTA two turns);
 // tf32x3 L = 48, B = 512 93 + 99 and 113 + 113, L = 64, B = 1 29 + 29 and 33 + 31, B = 128 58 + 58 and 50 + 50.  FP64 plans,
 // against the two-launch products (torus_direct.cu): L = 8, B = 8192 323 + 415 and 817 + 868, L = 32, B = 8192 5432 + 6481 and
 // 6647 + 8007.
