@@ -1,4 +1,4 @@
-// Torus passes of FP64 plans above L = 32 with little work: the folded cosine and sine products of the torus stage
+// Torus passes of FP64 plans with little work: the folded cosine and sine products of the torus stage
 // (torus_gemm.cu gives the identities) in FP64 on CUDA cores, four launches an inverse + forward.
 //
 // Matrices are stored [k][row], so that a warp's lanes (32 rows) read them coalesced, and a data column is
@@ -45,12 +45,12 @@ __device__ __forceinline__ Pair reduce_warps(Pair v, int warp, int lane) {
   return r;
 }
 
-// Element i of a buffer of n, zero outside (checked builds).
-__device__ __forceinline__ double2 load(const double2* p, long long i, long long n) {
-  return in_bounds(i, n, kbTorusIn) ? __ldg(&p[i]) : make_double2(0.0, 0.0);
+// Element i of a run that starts `at` elements into a buffer of n, zero outside (checked builds).
+__device__ __forceinline__ double2 load(const double2* run, size_t i, size_t at, long long n) {
+  return in_bounds((long long)(at + i), n, kbTorusIn) ? __ldg(&run[i]) : make_double2(0.0, 0.0);
 }
-__device__ __forceinline__ void store(double2* p, long long i, long long n, double2 v) {
-  if (in_bounds(i, n, kbTorusOut)) p[i] = v;
+__device__ __forceinline__ void store(double2* run, size_t i, size_t at, long long n, double2 v) {
+  if (in_bounds((long long)(at + i), n, kbTorusOut)) run[i] = v;
 }
 
 __device__ __forceinline__ void axpy(double2& acc, double a, double2 x) {
@@ -66,15 +66,17 @@ __global__ void __launch_bounds__(32 * kWarps) direct_theta_inverse_kernel(int L
   const int t = 32 * blockIdx.y + lane, b = blockIdx.x / L, m = blockIdx.x - b * L;
   const bool odd = (m + s) & 1;
   const double* A = M + (size_t)(odd ? kSinKX : kCosKX) * L * L;
-  const long long fp = ((long long)b * N + L - 1 + m) * L, fm = fp - 2ll * m * L;
+  const size_t fp = ((size_t)b * N + L - 1 + m) * L, fm = ((size_t)b * N + L - 1 - m) * L;
+  const double2* Fp = F + fp;
+  const double2* Fm = F + fm;
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = warp; k < L; k += kWarps) {
     double a = t < L ? __ldg(&A[(size_t)k * L + t]) : 0.0;
     if (k == 0) a *= 0.5;  // the sum is doubled below
-    axpy(v.a, a, load(F, fp + k, in_n));
-    axpy(v.b, a, load(F, fm + k, in_n));
+    axpy(v.a, a, load(Fp, k, fp, in_n));
+    axpy(v.b, a, load(Fm, k, fm, in_n));
   }
   v = reduce_warps(v, warp, lane);
   if (warp || t >= L) return;
@@ -87,9 +89,9 @@ __global__ void __launch_bounds__(32 * kWarps) direct_theta_inverse_kernel(int L
     e = make_double2(-e.y, e.x);
     o = make_double2(-o.y, o.x);
   }
-  const long long at = ((long long)b * L + m) * L + t;
-  store(work, at, out_n, make_double2(2.0 * e.x, 2.0 * e.y));
-  store(work, (long long)B * L * L + at, out_n, make_double2(2.0 * o.x, 2.0 * o.y));
+  const size_t at = ((size_t)b * L + m) * L + t;
+  store(work, at, 0, out_n, make_double2(2.0 * e.x, 2.0 * e.y));
+  store(work, (size_t)B * L * L + at, 0, out_n, make_double2(2.0 * o.x, 2.0 * o.y));
 }
 
 // phi inverse: E, O [2][b][m][t] -> f[b][t][p] = E + iO, f[b][t][N-1-p] = E - iO.
@@ -100,20 +102,23 @@ __global__ void __launch_bounds__(32 * kWarps) direct_phi_inverse_kernel(int L, 
   const int p = 32 * blockIdx.y + lane, b = blockIdx.x / L, t = blockIdx.x - b * L;
   const double* C = M + (size_t)kCosKX * L * L;
   const double* S = M + (size_t)kSinKX * L * L;
-  const long long e0 = (long long)b * L * L + t, o0 = e0 + (long long)B * L * L;
+  const size_t e0 = (size_t)b * L * L + t, o0 = e0 + (size_t)B * L * L;
+  const double2* E = work + e0;
+  const double2* O = work + o0;
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = warp; k < L; k += kWarps) {
     const double c = p < L ? __ldg(&C[(size_t)k * L + p]) : 0.0, sn = p < L ? __ldg(&S[(size_t)k * L + p]) : 0.0;
-    axpy(v.a, c, load(work, e0 + (long long)k * L, in_n));
-    axpy(v.b, sn, load(work, o0 + (long long)k * L, in_n));
+    axpy(v.a, c, load(E, (size_t)k * L, e0, in_n));
+    axpy(v.b, sn, load(O, (size_t)k * L, o0, in_n));
   }
   v = reduce_warps(v, warp, lane);
   if (warp || p >= L) return;
-  const long long row = ((long long)b * L + t) * N;
-  store(f, row + p, out_n, make_double2(v.a.x - v.b.y, v.a.y + v.b.x));
-  if (p < L - 1) store(f, row + N - 1 - p, out_n, make_double2(v.a.x + v.b.y, v.a.y - v.b.x));
+  const size_t r0 = ((size_t)b * L + t) * N;
+  double2* row = f + r0;
+  store(row, p, r0, out_n, make_double2(v.a.x - v.b.y, v.a.y + v.b.x));
+  if (p < L - 1) store(row, N - 1 - p, r0, out_n, make_double2(v.a.x + v.b.y, v.a.y - v.b.x));
 }
 
 // phi of forward and adjoint: f [b][t][p] -> P, Q [2][b][t][m].  A warp folds 32 of its k's at a time.
@@ -125,7 +130,8 @@ __global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, 
   const int m = 32 * blockIdx.y + lane, b = blockIdx.x / L, t = blockIdx.x - b * L;
   const double* C = M + (size_t)kCosXK * L * L;
   const double* S = M + (size_t)kSinXK * L * L;
-  const long long row = ((long long)b * L + t) * N;
+  const size_t r0 = ((size_t)b * L + t) * N;
+  const double2* row = f + r0;
   const int per = (L + kWarps - 1) / kWarps, k_end = min(L, (warp + 1) * per);
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
@@ -133,9 +139,9 @@ __global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, 
     const int p = k0 + lane;
     double2 e = make_double2(0.0, 0.0), o = e;
     if (p < k_end) {
-      e = load(f, row + p, in_n);
+      e = load(row, p, r0, in_n);
       if (p < L - 1) {
-        const double2 y = load(f, row + N - 1 - p, in_n);
+        const double2 y = load(row, N - 1 - p, r0, in_n);
         o = make_double2(e.x - y.x, e.y - y.y);
         e = make_double2(e.x + y.x, e.y + y.y);
       }
@@ -154,9 +160,9 @@ __global__ void __launch_bounds__(32 * kWarps) direct_phi_forward_kernel(int L, 
   }
   v = reduce_warps(v, warp, lane);
   if (warp || m >= L) return;
-  const long long at = ((long long)b * L + t) * L + m;
-  store(work, at, out_n, v.a);
-  store(work, (long long)B * L * L + at, out_n, v.b);
+  const size_t at = ((size_t)b * L + t) * L + m;
+  store(work, at, 0, out_n, v.a);
+  store(work, (size_t)B * L * L + at, 0, out_n, v.b);
 }
 
 // theta of forward (weight matrices) and adjoint (cosines and sines, the fold of m' < 0): P, Q -> H [b][m + Lp][m'].
@@ -168,14 +174,16 @@ __global__ void __launch_bounds__(32 * kWarps) direct_theta_forward_kernel(int L
   const int mp = 32 * blockIdx.y + lane, b = blockIdx.x / L, m = blockIdx.x - b * L;
   const bool odd = (m + s) & 1;
   const double* A = M + (size_t)(adjoint ? (odd ? kSinXK : kCosXK) : (odd ? kWeightO : kWeightE)) * L * L;
-  const long long p0 = (long long)b * L * L + m, q0 = p0 + (long long)B * L * L;
+  const size_t p0 = (size_t)b * L * L + m, q0 = p0 + (size_t)B * L * L;
+  const double2* P = work + p0;
+  const double2* Q = work + q0;
   Pair v;
   v.a = v.b = make_double2(0.0, 0.0);
 #pragma unroll 4
   for (int k = warp; k < L; k += kWarps) {
     const double a = mp < L ? __ldg(&A[(size_t)k * L + mp]) : 0.0;
-    axpy(v.a, a, load(work, p0 + (long long)k * L, in_n));
-    axpy(v.b, a, load(work, q0 + (long long)k * L, in_n));
+    axpy(v.a, a, load(P, (size_t)k * L, p0, in_n));
+    axpy(v.b, a, load(Q, (size_t)k * L, q0, in_n));
   }
   v = reduce_warps(v, warp, lane);
   if (warp || mp >= L) return;
@@ -185,8 +193,8 @@ __global__ void __launch_bounds__(32 * kWarps) direct_theta_forward_kernel(int L
     hp = make_double2(hp.y, -hp.x);
     hm = make_double2(hm.y, -hm.x);
   }
-  store(H, ((long long)b * N + L - 1 + m) * L + mp, out_n, hp);
-  if (m > 0) store(H, ((long long)b * N + L - 1 - m) * L + mp, out_n, hm);
+  store(H, ((size_t)b * N + L - 1 + m) * L + mp, 0, out_n, hp);
+  if (m > 0) store(H, ((size_t)b * N + L - 1 - m) * L + mp, 0, out_n, hm);
 }
 
 }  // namespace
@@ -197,11 +205,12 @@ struct DirectPlan {
   size_t bytes = 0;
 };
 
-// Where these products beat those of digits: for little work, where the digits' nine launches set the time.  (Up to
-// L = 32 one launch does both passes: torus_small.cu.)  GB300, torus stage of an inverse and a forward in us, digits against these: L = 64, B = 1
-// 95 and 43; L = 96, B = 1 101 and 56; L = 128, B = 1 107 and 102; beyond the line L = 96, B = 2 104 and 85, L = 64, B = 8
-// 98 and 103 (the two meet there); L = 144, B = 1 115 and 132; L = 128, B = 4 114 and 283.
-bool direct_wanted(int L, int B) { return (long long)B * L * L * L <= (1ll << 21); }
+// Where these products beat those of digits: for little work, where the digits' nine launches set the time, and
+// at band-limits that fill little of their tiles (many fields of those take torus_small.cu).  GB300, torus stage of an inverse
+// and a forward in us, digits against these: L = 64, B = 1 95 and 43; L = 96, B = 1 101 and 56; L = 128, B = 1 107 and 102;
+// L = 32, B = 128 193 and 185; beyond the line L = 96, B = 2 104 and 85, L = 64, B = 8 98 and 103 (the two meet there); L = 144,
+// B = 1 115 and 132; L = 128, B = 4 114 and 283.
+bool direct_wanted(int L, int B) { return L <= 32 || (long long)B * L * L * L <= (1ll << 21); }
 
 cudaError_t direct_setup(DirectPlan** out, int L) {
   *out = nullptr;

@@ -316,11 +316,12 @@ struct SmallPlan {
 // of 128 rows and 64 K), inverse and forward with a kept table in us, these and those: fp32 L = 16, B = 4096 83 + 114 and
 // 401 + 366, L = 48, B = 512 130 + 189 and 163 + 176, L = 49, B = 512 183 + 218 and 167 + 195, L = 64, B = 64 46 + 54 and
 // 48 + 54, B = 128 79 + 96 and 68 + 85, L = 65, B = 1 35 + 37 and 33 + 30 (its 17 quads of rings take the CTA two turns);
-// tf32x3 L = 48, B = 512 93 + 99 and 113 + 113, L = 64, B = 1 29 + 29 and 33 + 31, B = 128 58 + 58 and 50 + 50.  FP64 plans,
-// against the two-launch products (torus_direct.cu): L = 8, B = 8192 323 + 415 and 817 + 868, L = 32, B = 8192 5432 + 6481 and
-// 6647 + 8007.
+// tf32x3 L = 48, B = 512 93 + 99 and 113 + 113, L = 64, B = 1 29 + 29 and 33 + 31, B = 128 58 + 58 and 50 + 50.
+// FP64 plans, against the two-launch products (torus_direct.cu), which spread a few fields over more of the GPU's FP64 pipes:
+// L = 4, B = 1 31 and 29, B = 128 32 and 38; L = 8, B = 64 42 and 40, B = 128 48 and 64; L = 16, B = 32 66 and 51, B = 128 83 and 112;
+// L = 32, B = 32 131 and 104, B = 96 219 and 211, B = 128 236 and 265, B = 8192 5432 + 6481 and 6647 + 8007.
 bool small_wanted(int L, int B, bool f64) {
-  return f64 ? L <= 32 : L <= 48 || (L <= 64 && (long long)B * L * L * L <= (1ll << 24));
+  return f64 ? L <= 4 || (L <= 32 && B >= 128) : L <= 48 || (L <= 64 && (long long)B * L * L * L <= (1ll << 24));
 }
 
 // Rings or orders of a block: the sizes the kernels are made for.
@@ -380,12 +381,13 @@ void small_destroy(SmallPlan* p) {
 size_t small_bytes(const SmallPlan* p) { return p ? p->bytes : 0; }
 
 // Fields of a CTA: two rounds of theta work for its threads, but no more than leave two CTAs to every SM; the blocks of
-// rings or orders go to CTAs of their own while the fields alone do not fill the GPU.
+// rings or orders go to CTAs of their own while the fields alone do not fill the GPU -- in FP64, which the pipe bounds, until
+// eight CTAs an SM even out its share (L = 32, B = 512 989 -> 830 us an inverse and a forward against two).
 static dim3 small_grid(const SmallPlan* p, int B, int* nf) {
   const int tb = block_of(p->L), items = (p->L + 3) / 4 * 2 * tb, blocks = (p->L + tb - 1) / tb, want = 2 * p->sms;
   *nf = std::max(1, std::min({32, 2 * kThreads / items, B / want}));
-  const int gx = (B + *nf - 1) / *nf;
-  return dim3((unsigned)gx, (unsigned)std::min(blocks, (want + gx - 1) / gx));
+  const int gx = (B + *nf - 1) / *nf, ctas = (p->f64 ? 8 : 2) * p->sms;
+  return dim3((unsigned)gx, (unsigned)std::min(blocks, (ctas + gx - 1) / gx));
 }
 
 template <typename T>

@@ -24,10 +24,10 @@ def rel(a, b):
 
 
 # (L, s, B): the smallest sizes; edges of blocks of 8 and 16 rings and orders and of 32 m'; several fields a CTA with a last
-# one not full; the rule's lines: L = 32 and 33 (FP64), L = 48 and 49, L = 64 and 65, B L^3 = 2^24 at L = 49 (142 and 143
+# one not full; the rule's lines: L = 4 and 5 and 127 and 128 fields up to L = 32 (FP64), L = 48 and 49, L = 64 and 65, B L^3 = 2^24 at L = 49 (142 and 143
 # fields) and L = 64 (64 and 65)
-@pytest.mark.parametrize("L,s,B", [(1, 0, 2), (2, 1, 1), (3, -1, 33), (5, 2, 3), (8, 0, 1000), (8, -7, 2), (9, 1, 1), (15, -2, 309),
-                                   (16, 3, 1250), (17, -1, 2), (24, 0, 609), (31, 30, 3), (32, 2, 613), (32, -1, 1), (33, 0, 5),
+@pytest.mark.parametrize("L,s,B", [(1, 0, 2), (2, 1, 1), (3, -1, 33), (4, 1, 2), (5, 2, 3), (5, -4, 129), (8, 0, 1000), (8, -7, 2), (9, 1, 1), (15, -2, 309),
+                                   (16, 3, 1250), (17, -1, 2), (24, 0, 609), (28, 1, 127), (28, -2, 128), (31, 30, 3), (32, 2, 613), (32, -1, 1), (33, 0, 5),
                                    (47, -3, 2), (48, 1, 4), (49, -3, 142), (49, 2, 143), (63, 1, 1), (64, 0, 64), (64, -2, 65),
                                    (65, 1, 2)])
 @pytest.mark.parametrize("precision", ["fp64", "fp32", "tf32x3", "bf16x6"])
